@@ -249,8 +249,10 @@ void carve(Arena &a, const spin_config &cfg, const Geometry &g, DevCtx &d, spin_
   d.fetch_queue = a.take<FetchItem>((size_t)g.fetch_cap);
   d.fetch_count = a.take<int32_t>(1);
   d.att_part = a.take<float>(B * g.max_chunks * G * (kHeadDim + 2));
+  d.att_ml = reinterpret_cast<float2 *>(d.att_part + B * g.max_chunks * G * kHeadDim);
   d.att_count = a.take<int32_t>(B);
   d.sel_count = a.take<int32_t>(B);
+  d.link = a.take<int32_t>(64);
   d.score_queue = a.take<int32_t>(1);
   d.score_done = a.take<int32_t>(1);
   d.scored = a.take<int32_t>(B);
@@ -845,6 +847,7 @@ int spin_create(const spin_config *cfg, spin_ctx **out) {
   fill(d.score_xfer, 0xff, (size_t)g.max_batch_sets * g.max_cand * 4);       // every word "not written"
   fill(d.att_count, 0, (size_t)g.max_batch_sets * 4);
   fill(d.sel_count, 0, (size_t)g.max_batch_sets * 4);
+  fill(d.link, 0, 64 * 4);
   fill(d.score_queue, 0, 4);
   fill(d.score_done, 0, 4);
   fill(d.scored, 0, (size_t)g.max_batch_sets * 4);
@@ -1329,14 +1332,12 @@ static int step_impl(spin_ctx *ctx, int32_t layer, const int32_t *req_ids, int32
     }
   }
   int64_t max_cand = 0, max_pages = 0;
-  bool may_be_empty = false;
   for (int i = 0; i < n_req; ++i) {
     LayerHost &L = ctx->reqs[(size_t)req_ids[i]].layers[(size_t)layer];
     const int64_t cand = ctx->cfg.partition_kind == SPIN_PART_TOKEN_DOT ? (int64_t)L.n_partitions * kPageTokens : L.n_partitions;
     max_cand = std::max(max_cand, cand);
     int64_t pages = cluster ? ctx->g.max_pages : std::min<int64_t>(ctx->cfg.topk, L.n_partitions);
     max_pages = std::max(max_pages, pages + L.tail_pages);
-    may_be_empty = may_be_empty || L.n_tokens == 0;
     L.last_batch_pos = i;
     b.tail_pages[i] = (int16_t)L.tail_pages;
     b.tail_len[i] = (int16_t)L.tail_len;
@@ -1359,7 +1360,7 @@ static int step_impl(spin_ctx *ctx, int32_t layer, const int32_t *req_ids, int32
   b.append_in_grid = in_grid ? 1 : 0;
   ctx->launches += launch_select(ctx->d, b, qd, kk, vv, (int)max_cand, st, &ctx->prof);
   ctx->launches += launch_fetch(ctx->d, st, ctx->sm_count, &ctx->prof);
-  ctx->launches += launch_attention(ctx->d, b, qd, od, (int)max_pages, may_be_empty, st, &ctx->prof);
+  ctx->launches += launch_attention(ctx->d, b, qd, od, (int)max_pages, st, &ctx->prof);
   if (oc == 2) CK(cudaMemcpyAsync(out, ctx->stage_out, qbytes, cudaMemcpyDeviceToHost, st));
   CK(cudaGetLastError());
   return SPIN_OK;

@@ -1,20 +1,23 @@
 // Attention over the selected pages plus the local tail (Section 4.1 "Attention"), fused with
 // the page fetch of Retrieve step 4 (Section 5.2): paged GQA decode attention, split over
-// chunks of the page list and merged by log-sum-exp.
+// CTAs and merged by log-sum-exp.
 //
-// k_attn: one CTA (4 warps) per (set, chunk of 8 pages).  Each warp owns two pages of the
-// chunk.  It requests both pages at once with 16-byte cp.async copies into XOR-swizzled
-// shared memory (a page is one contiguous 8 KiB run: 16 K rows then 16 V rows) -- from an
-// HBM slot for a hit, straight from pinned host memory for a miss -- so every missed page of
-// the step is in flight on the host link while the hits are being attended from HBM.  A
-// missed page that was admitted to the cache is written from shared memory into its HBM
-// slot after use (that is the fetch); a bypassed page is only attended.  QK^T and PV run on
-// mma.sync m16n8k16 bf16 tiles with fp32 accumulators (query heads padded to M = 16, the
-// page's 16 tokens as N resp. K): at ~4 flop/byte the kernel is HBM/PCIe bound and tensor
-// tiles are used to take instruction issue off the critical path, which is also why the
-// 64..128-row tcgen05 tiles (>90% padding at GQA 4) are not.  The last CTA of a set to finish
-// (a counter cleared by the cache-manager kernel) merges the set's partials and writes bf16.
+// k_attn: a set's page list is dealt out to the warps of its CTAs (4 warps each), page by page in
+// turn, so every warp has its share of the missed pages (which lead the list) and of the hits.
+// A warp keeps two pages in flight in shared memory and one accumulator over all its pages; the
+// CTA writes one partial.  A page (8 KiB: 16 K rows, then 16 V rows) is brought in by one
+// instruction, a 256-byte bulk copy (TMA) per lane, each row to its own place at a stride of 272
+// bytes, which is what lets ldmatrix read 8 rows without a bank conflict; it comes from an HBM
+// slot for a hit and straight from pinned host memory for a miss, so the missed pages of the step
+// are on the host link while the hits are being attended from HBM.  A missed page that was
+// admitted to the cache goes from shared memory to its HBM slot by bulk copies too (that is the
+// fetch); a bypassed page is only attended.  K Q^T and V^T P^T run on mma.sync m16n8k16 bf16 tiles
+// with fp32 accumulators (the page's 16 tokens resp. 16 channels as M, the query heads as N = 8): at
+// ~4 flop/byte the kernel is HBM/PCIe bound and tensor tiles are used to take instruction issue
+// off the critical path, which is also why the 64..128-row tcgen05 tiles (>90% padding at GQA 4)
+// are not.  The last CTA of a set to finish merges the set's partials and writes bf16.
 #define SPIN_FILE_ID 4
+#include <atomic>
 #include <cstdio>
 
 #include "../../include/spin.h"
@@ -31,26 +34,25 @@ __device__ __forceinline__ void dbg_ta(int, int) {}
 
 namespace {
 
-constexpr int kAttnWarps = 4;
-constexpr int kPartStride = kHeadDim + 2;       // per head: 128 outputs, max, sum
+constexpr int kAttnWarps = 4, kAttnThreads = kAttnWarps * 32;
+constexpr int kStageRow = kRowBytes + 16;                  // a row of a staged page: 8 rows' 16-byte pieces fall into 8 bank groups
+constexpr int kStageBytes = 2 * kPageTokens * kStageRow;   // 32 rows
+constexpr int kWarpStages = 2;
+constexpr int kAttnSmem = kAttnWarps * kWarpStages * kStageBytes;
+static_assert(kAttnSmem == kAttnCtaSmem, "what the scoring launcher leaves room for");
+constexpr int kCtaPages = kChunkPages;                     // a set of n pages is split over at most ceil(n / 8) CTAs
+constexpr int kCombStride = kHeadDim + 4;                  // floats of a head's row in the warps' exchange area
 
 __device__ __forceinline__ uint32_t smem_u32(const void *p) {
   return static_cast<uint32_t>(__cvta_generic_to_shared(p));
 }
-__device__ __forceinline__ void cp_async16(uint32_t dst, const void *src) {
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(dst), "l"(src) : "memory");
-}
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
-template <int N> __device__ __forceinline__ void cp_async_wait() {
-  asm volatile("cp.async.wait_group %0;\n" ::"n"(N) : "memory");
-}
 __device__ __forceinline__ void ldmatrix_x4(uint32_t addr, uint32_t &r0, uint32_t &r1, uint32_t &r2, uint32_t &r3) {
   asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];\n"
-               : "=r"(r0), "=r"(r1), "=r"(r2), "=r"(r3) : "r"(addr));
+               : "=r"(r0), "=r"(r1), "=r"(r2), "=r"(r3) : "r"(addr) : "memory");
 }
 __device__ __forceinline__ void ldmatrix_x4_trans(uint32_t addr, uint32_t &r0, uint32_t &r1, uint32_t &r2, uint32_t &r3) {
   asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];\n"
-               : "=r"(r0), "=r"(r1), "=r"(r2), "=r"(r3) : "r"(addr));
+               : "=r"(r0), "=r"(r1), "=r"(r2), "=r"(r3) : "r"(addr) : "memory");
 }
 __device__ __forceinline__ void mma_bf16(float (&d)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3,
                                          uint32_t b0, uint32_t b1) {
@@ -58,408 +60,470 @@ __device__ __forceinline__ void mma_bf16(float (&d)[4], uint32_t a0, uint32_t a1
                : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
                : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
 }
+__device__ __forceinline__ uint32_t movmatrix_trans(uint32_t x) {
+  uint32_t y;
+  asm volatile("movmatrix.sync.aligned.m8n8.trans.b16 %0, %1;\n" : "=r"(y) : "r"(x));
+  return y;
+}
 __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
   __nv_bfloat162 v = __floats2bfloat162_rn(lo, hi);
   return *reinterpret_cast<uint32_t *>(&v);
 }
 
-// Byte offset of the 16-byte piece `chunk` (0..15) of row `row` (0..31: K rows, then V rows)
-// inside a page staged in shared memory.  Pieces are XOR-swizzled by the row so that the 8
-// rows an ldmatrix touches fall into 8 different bank groups.
-__device__ __forceinline__ uint32_t swz(int row, int chunk) {
-  return (uint32_t)(row * kRowBytes + ((chunk ^ (row & 7)) << 4));
+// One warp requests one page: lane r copies row r (256 bytes); the stage's mbarrier counts the bytes.
+__device__ __forceinline__ void request_page(uint32_t sdst, uint32_t bar, const uint8_t *src, int lane) {
+  if (lane == 0) asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n" ::"r"(bar), "r"(kPageBytes) : "memory");
+  __syncwarp();
+  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];\n"
+               ::"r"(sdst + lane * kStageRow), "l"(src + lane * kRowBytes), "r"(kRowBytes), "r"(bar) : "memory");
+}
+// Pages that other SMs have written with ordinary stores and announced by a flag may now be read by
+// bulk copies.
+__device__ __forceinline__ void pages_visible() { asm volatile("fence.proxy.async.global;\n" ::: "memory"); }
+__device__ __forceinline__ bool page_test(uint32_t bar, uint32_t parity) {
+  uint32_t done;
+  asm volatile("{\n.reg .pred p;\nmbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\nselp.u32 %0, 1, 0, p;\n}\n"
+               : "=r"(done) : "r"(bar), "r"(parity) : "memory");
+  return __all_sync(0xffffffffu, done);
+}
+// Bounded wait for a stage: false (reported by the caller) if its copies have not landed after seconds.
+__device__ __forceinline__ bool page_landed(uint32_t bar, uint32_t parity) {
+  uint32_t done = 0;
+#pragma unroll 1
+  for (int spin = 0; spin < (1 << 22) && !done; ++spin)
+    asm volatile("{\n.reg .pred p;\nmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\nselp.u32 %0, 1, 0, p;\n}\n"
+                 : "=r"(done) : "r"(bar), "r"(parity) : "memory");
+  return __all_sync(0xffffffffu, done);
 }
 
-// One warp requests one page: 16 copies of 16 bytes per lane, 512 contiguous bytes per instruction.
-__device__ __forceinline__ void request_page(uint32_t sdst, const uint8_t *src, int lane) {
-#pragma unroll
-  for (int j = 0; j < 16; ++j) {
-    const int piece = j * 32 + lane;              // 0..511
-    const int row = piece >> 4, chunk = piece & 15;
-    cp_async16(sdst + swz(row, chunk), src + (size_t)piece * 16);
-  }
-}
-
+// A warp's running state.  The tiles are transposed (tokens resp. channels as M = 16, the query
+// heads as N = 8): a head is a column, so no row of a tile is padding at 8 heads, and a page costs
+// 16 mma instead of the 32 (and the accumulators half the registers) of heads padded to M = 16.
 struct WarpAcc {
-  float m, l;                 // running max (base-2 logits) and partial sum of this lane's row
-  float o[16][4];             // 16 n-tiles of 8 channels; [.][0..1] = row lane/4, [.][2..3] = row+8 (unused, zero)
+  float m[2], l[2];           // heads (lane % 4) * 2 + {0, 1}: running max (base-2 logits), this lane's share of the sum
+  float o[8][4];              // 16-channel tiles: channels lane / 4 (+ 8), heads as above: [0], [1] resp. [2], [3]
 };
 
-// Attend one staged page: S = Q K^T (16 x 16), online softmax, O += P V.
-__device__ __forceinline__ void attend_page(uint32_t spage, const uint32_t (&qa)[8][2], uint32_t mask,
+// Attend one staged page: S^T = K Q^T (16 tokens x 8 heads), online softmax, O^T += V^T P^T.
+__device__ __forceinline__ void attend_page(uint32_t spage, const uint32_t (&qb)[8][2], uint32_t mask,
                                             float scale2, WarpAcc &acc, int lane) {
-  float s[2][4] = {{0.f, 0.f, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f}};
   const int mat = lane >> 3, r8 = lane & 7;
-  {
-    const int token = r8 + ((mat >> 1) << 3);
+  const uint32_t krow = spage + (uint32_t)((r8 + ((mat & 1) << 3)) * kStageRow + (mat >> 1) * 16);
+  const uint32_t vrow = spage + (uint32_t)((kPageTokens + r8 + ((mat >> 1) << 3)) * kStageRow + (mat & 1) * 16);
+  float s[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
-    for (int ks = 0; ks < 8; ++ks) {
-      uint32_t b0, b1, b2, b3;
-      ldmatrix_x4(spage + swz(token, 2 * ks + (mat & 1)), b0, b1, b2, b3);
-      mma_bf16(s[0], qa[ks][0], 0u, qa[ks][1], 0u, b0, b1);
-      mma_bf16(s[1], qa[ks][0], 0u, qa[ks][1], 0u, b2, b3);
-    }
+  for (int ks = 0; ks < 8; ++ks) {
+    uint32_t a0, a1, a2, a3;
+    ldmatrix_x4(krow + ks * 32, a0, a1, a2, a3);
+    mma_bf16(s, a0, a1, a2, a3, qb[ks][0], qb[ks][1]);
   }
-  // this lane's row = lane/4; its tokens: nt*8 + (lane%4)*2 + {0,1}
-  float p[2][2];
-  float mx = -INFINITY;
+  // this lane's tokens: lane / 4 (s[0], s[1]) and lane / 4 + 8 (s[2], s[3])
+  const bool t0 = (mask >> (lane >> 2)) & 1u, t1 = (mask >> ((lane >> 2) + 8)) & 1u;
+  float corr[2];
 #pragma unroll
-  for (int nt = 0; nt < 2; ++nt)
+  for (int h = 0; h < 2; ++h) {
+    s[h] = t0 ? s[h] * scale2 : -INFINITY;
+    s[2 + h] = t1 ? s[2 + h] * scale2 : -INFINITY;
+    float mx = fmaxf(s[h], s[2 + h]);
+    mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 4));
+    mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 8));
+    mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 16));
+    const float mn = fmaxf(acc.m[h], mx);
+    const float base = mn == -INFINITY ? 0.f : mn;         // all masked so far: every p is 0
+    corr[h] = exp2f(acc.m[h] - base);                      // acc.m = -inf -> 0
+    s[h] = exp2f(s[h] - base);
+    s[2 + h] = exp2f(s[2 + h] - base);
+    acc.l[h] = acc.l[h] * corr[h] + (s[h] + s[2 + h]);
+    acc.m[h] = mn;
+  }
+  // P (token rows, head columns) transposed into the B operand
+  const uint32_t b0 = movmatrix_trans(pack_bf16(s[0], s[1])), b1 = movmatrix_trans(pack_bf16(s[2], s[3]));
 #pragma unroll
-    for (int j = 0; j < 2; ++j) {
-      const int tok = nt * 8 + (lane & 3) * 2 + j;
-      const float v = ((mask >> tok) & 1u) ? s[nt][j] * scale2 : -INFINITY;
-      p[nt][j] = v;
-      mx = fmaxf(mx, v);
-    }
-  mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 1));
-  mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 2));
-  const float mn = fmaxf(acc.m, mx);
-  const float base = mn == -INFINITY ? 0.f : mn;           // all masked so far: every p is 0
-  const float corr = exp2f(acc.m - base);                  // acc.m = -inf -> 0
-  float psum = 0.f;
-#pragma unroll
-  for (int nt = 0; nt < 2; ++nt)
-#pragma unroll
-    for (int j = 0; j < 2; ++j) {
-      p[nt][j] = exp2f(p[nt][j] - base);
-      psum += p[nt][j];
-    }
-  acc.l = acc.l * corr + psum;
-  acc.m = mn;
-  const uint32_t pa0 = pack_bf16(p[0][0], p[0][1]), pa2 = pack_bf16(p[1][0], p[1][1]);
-  {
-    const int token = r8 + ((mat & 1) << 3);
-#pragma unroll
-    for (int nb = 0; nb < 8; ++nb) {
-      uint32_t b0, b1, b2, b3;
-      ldmatrix_x4_trans(spage + swz(kPageTokens + token, 2 * nb + (mat >> 1)), b0, b1, b2, b3);
-      acc.o[2 * nb][0] *= corr; acc.o[2 * nb][1] *= corr;
-      acc.o[2 * nb + 1][0] *= corr; acc.o[2 * nb + 1][1] *= corr;
-      mma_bf16(acc.o[2 * nb], pa0, 0u, pa2, 0u, b0, b1);
-      mma_bf16(acc.o[2 * nb + 1], pa0, 0u, pa2, 0u, b2, b3);
-    }
+  for (int nt = 0; nt < 8; ++nt) {
+    uint32_t a0, a1, a2, a3;
+    ldmatrix_x4_trans(vrow + nt * 32, a0, a1, a2, a3);
+    acc.o[nt][0] *= corr[0]; acc.o[nt][1] *= corr[1];
+    acc.o[nt][2] *= corr[0]; acc.o[nt][3] *= corr[1];
+    mma_bf16(acc.o[nt], a0, a1, a2, a3, b0, b1);
   }
 }
 
-// Retrieve step 4 for one admitted miss: the staged page goes to its HBM slot.
-__device__ __forceinline__ void store_page(const uint8_t *spage_generic, uint8_t *dst, int lane) {
-#pragma unroll
-  for (int j = 0; j < 16; ++j) {
-    const int piece = j * 32 + lane;
-    const int row = piece >> 4, chunk = piece & 15;
-    *reinterpret_cast<uint4 *>(dst + (size_t)piece * 16) =
-        *reinterpret_cast<const uint4 *>(spage_generic + swz(row, chunk));
-  }
+// Retrieve step 4 for one admitted miss: the staged page goes to its HBM slot, lane r moving row r.
+__device__ __forceinline__ void store_page(uint32_t spage, uint8_t *dst, int lane) {
+  asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;\ncp.async.bulk.commit_group;\n"
+               ::"l"(dst + lane * kRowBytes), "r"(spage + lane * kStageRow), "r"(kRowBytes) : "memory");
+}
+// The lane's copies out of shared memory have read their source.
+__device__ __forceinline__ void stores_read() { asm volatile("cp.async.bulk.wait_group.read 0;\n" ::: "memory"); }
+
+// Turns on the host link.  The link needs a few hundred KB of reads in flight; whatever is asked of
+// it beyond that waits inside the GPU's memory system, in front of everything else the same SMs
+// want from HBM: page lists, flags, hits.  So a page takes a turn before it is requested, and at
+// most kLinkWindow turns are open at a time; a page that has landed closes its own.  Both counters
+// only ever grow (modulo 2^32).  The lowest open turn never waits for a higher one.
+// Measured on the Llama-shaped step (64 sets, 396 missed pages): last set's list of missed pages
+// 75-86 us into the step without a limit, 35 us with one; step 112 us without, 106 / 102 / 103 / 107 us
+// with a window of 32 / 64 / 96 / 160 pages.
+constexpr int kLinkWindow = 64, kLinkDone = 32, kLinkPolls = 1 << 20;
+__device__ __forceinline__ int link_turn(const DevCtx &c, int lane) {
+  int t = 0;
+  if (lane == 0) t = atomicAdd(c.link, 1);
+  return __shfl_sync(0xffffffffu, t, 0);
+}
+__device__ __forceinline__ void link_close(const DevCtx &c, int lane) { if (lane == 0) atomicAdd(c.link + kLinkDone, 1); }
+__device__ __forceinline__ bool link_open(const DevCtx &c, int turn) {
+  int done;
+  asm volatile("ld.relaxed.gpu.global.s32 %0, [%1];\n" : "=r"(done) : "l"(c.link + kLinkDone) : "memory");
+  return __all_sync(0xffffffffu, (int)((unsigned)turn - (unsigned)done) < kLinkWindow);
 }
 
-// A page that came over the host link goes to the HBM slot it was admitted to.  With an early
-// descriptor (open_idx >= 0) the slot is read from page_src once the set's second flag is up
-// (long since, as a rule: the page took microseconds to arrive); a bypassed page has none.
-__device__ __forceinline__ void fetched_page_to_slot(const DevCtx &c, const Batch &bt, int b, size_t pl,
-                                                     const uint8_t *spage_generic, int slot_page, int open_idx,
-                                                     bool slots_known, int lane) {
-  if (open_idx >= 0) {
-    int ok = 1;
-    if (!slots_known) {
-      if (lane == 0) ok = flag_wait(c, c.ready + b, bt.epoch);
-      ok = __shfl_sync(0xffffffffu, ok, 0);
+// What a lane knows of one page of its warp.
+struct PageRef {
+  int src, fill, open_idx;    // HBM page (< 0: ~host page); host page to bring in (-1 none); list index of an open slot (-1 none)
+  uint32_t mask;
+};
+
+__device__ __forceinline__ PageRef page_ref(const DevCtx &c, const Batch &bt, int b, int i_req, int head, size_t pl, int pos) {
+  PageRef r{0, -1, -1, 0u};
+  if (c.page_desc) {                        // work-ordered descriptors written by the cache manager
+    const int4 dsc = __ldcg(c.page_desc + pl + pos);
+    r.src = dsc.x; r.fill = dsc.y; r.mask = (uint32_t)dsc.z;
+    const bool open = dsc.x == -3;          // early descriptor: page_src[dsc.w] names the slot later
+    if (open) { r.open_idx = dsc.w; r.src = 0; }
+    if (r.fill == -2) {
+      // Retrieve step 3 for a missed page: Partition Offset -> CPU page table, both in pinned
+      // host memory (two dependent reads over the host link)
+      const int set = set_index(c, bt.req[i_req], bt.layer, head);
+      const int32_t *off = off_lookup(c, set, c.page_part[pl + dsc.w]);
+      const int32_t *hp = off ? cpt_lookup(c, set, *off + c.page_pidx[pl + dsc.w]) : nullptr;
+      const int host_page = hp ? *hp : -1;
+      if (host_page < 0) { r.src = -1; r.fill = c.n_host_pages; }         // fails the range check below
+      else if (open || r.src >= 0) r.fill = host_page;                    // fetched (admitted, or not yet known)
+      else { r.src = ~host_page; r.fill = -1; }                           // bypassed: attend from host
     }
-    slot_page = ok ? __ldcg(c.page_src + pl + open_idx) : -1;
-    if (slot_page >= c.n_gpu_pages) { if (lane == 0) dev_error(c, kErrBounds); slot_page = -1; }
+    if (open && r.fill < 0) { r.src = -1; r.fill = c.n_host_pages; }      // an early descriptor always names a host page
+  } else {                                  // plain lists, attended in the order given
+    r.src = c.page_src[pl + pos];
+    r.mask = c.page_mask[pl + pos];
   }
-  if (slot_page >= 0) store_page(spage_generic, c.gpu_pages + (size_t)slot_page * kPageBytes, lane);
+  // a descriptor that points outside the pools is dropped (and reported), never followed
+  const bool ok = (r.src >= 0 ? r.src < c.n_gpu_pages : ~r.src < c.n_host_pages) && r.fill < c.n_host_pages;
+  if (!ok) { dev_error(c, kErrBounds); r = PageRef{0, -1, -1, 0u}; }
+  return r;
+}
+
+// Four outputs over their softmax denominator, as bf16; zero where nothing was attended.
+__device__ __forceinline__ uint2 normalised(float4 o, float l) {
+  if (!(l > 0.f)) return make_uint2(0u, 0u);
+  return make_uint2(pack_bf16(o.x / l, o.y / l), pack_bf16(o.z / l, o.w / l));
+}
+
+// Counts the calling CTA in as one of the set's n_rows; true for the last one.  One thread calls it,
+// between two CTA barriers: its release orders the CTA's partials before the count, its acquire the
+// count before the CTA's reads of the other rows' partials.  The counters of a decode step are
+// cleared by the set's cache manager.  Those of the allocation-free call are 64-bit words that start
+// a call at zero because the last row of the call before left them so; the call's number in the
+// upper half makes a word right again that an abandoned call has left behind.
+__device__ __forceinline__ bool last_row(const DevCtx &c, int b, int n_rows) {
+  if (c.att_words) {
+    unsigned long long *w = c.att_words + b, old;
+    const unsigned long long base = (unsigned long long)c.att_call << 32;
+    atomicMax(w, base);
+    asm volatile("atom.acq_rel.gpu.global.add.u64 %0, [%1], 1;\n" : "=l"(old) : "l"(w) : "memory");
+    const bool last = old - base == (unsigned long long)(n_rows - 1);
+    if (last) *w = 0ull;
+    return last;
+  }
+  int old;
+  asm volatile("atom.acq_rel.gpu.global.add.s32 %0, [%1], 1;\n" : "=r"(old) : "l"(c.att_count + b) : "memory");
+  return old == n_rows - 1;
+}
+
+// Merge of a set's partials (one per CTA row; n_rows of them) by the last CTA to finish.  A warp
+// owns a head (two of them for G = 8; for G < 4 the warps share a head's rows and meet in shared
+// memory at the end), a lane four channels of it: 16-byte loads, kB of them in flight per lane,
+// the first batch already while the rows' maxima are being reduced.  Rows are added in a fixed
+// order, so the result does not depend on which CTA came last.
+// Measured: 64 rows of 4 heads 10 us -> 4.5 us, 3 rows of 4 heads 3.7 -> 1 us.
+template <int G>
+__device__ __forceinline__ void merge_rows(const DevCtx &c, int b, int n_rows, __nv_bfloat16 *__restrict__ out_rows, float *s_comb) {
+  constexpr int kWph = G >= kAttnWarps ? 1 : kAttnWarps / G;               // warps per head
+  constexpr int kB = 16;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, sub = warp % kWph;
+  const int nk = n_rows > sub ? (n_rows - sub + kWph - 1) / kWph : 0;      // this warp's rows: sub, sub + kWph, ...
+#pragma unroll 1
+  for (int g = warp / kWph; g < G; g += kAttnWarps) {
+    const float2 *ml = c.att_ml + ((size_t)b * c.max_chunks + sub) * G + g;
+    const float4 *po = reinterpret_cast<const float4 *>(c.att_part) + (((size_t)b * c.max_chunks + sub) * G + g) * (kHeadDim / 4) + lane;
+    constexpr size_t kMlStep = (size_t)kWph * G, kPoStep = (size_t)kWph * G * (kHeadDim / 4);
+    float4 v[kB];
+    if (nk > 0) {
+#pragma unroll
+      for (int i = 0; i < kB; ++i) v[i] = __ldcg(po + (size_t)min(i, nk - 1) * kPoStep);
+    }
+    float2 first = make_float2(-INFINITY, 0.f);                            // rows 0..31 of the warp stay in registers
+    if (lane < nk) first = __ldcg(ml + (size_t)lane * kMlStep);
+    float mx = first.x;
+#pragma unroll 1
+    for (int k = lane + 32; k < nk; k += 32) mx = fmaxf(mx, __ldcg(ml + (size_t)k * kMlStep).x);
+#pragma unroll
+    for (int o = 16; o; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+    float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+    float den = 0.f, w = 0.f;
+#pragma unroll 1
+    for (int k0 = 0; k0 < nk; k0 += kB) {
+      if ((k0 & 31) == 0) {                                                // weights of the next 32 rows, one per lane
+        if (k0 > 0) first = k0 + lane < nk ? __ldcg(ml + (size_t)(k0 + lane) * kMlStep) : make_float2(-INFINITY, 0.f);
+        w = first.x == -INFINITY ? 0.f : exp2f(first.x - mx);
+        den += first.y * w;
+      }
+      if (k0 > 0) {
+#pragma unroll
+        for (int i = 0; i < kB; ++i) v[i] = __ldcg(po + (size_t)min(k0 + i, nk - 1) * kPoStep);
+      }
+#pragma unroll
+      for (int i = 0; i < kB; ++i) {
+        const float wi = __shfl_sync(0xffffffffu, w, (k0 & 31) + i);       // zero beyond the last row
+        acc.x = fmaf(v[i].x, wi, acc.x); acc.y = fmaf(v[i].y, wi, acc.y);
+        acc.z = fmaf(v[i].z, wi, acc.z); acc.w = fmaf(v[i].w, wi, acc.w);
+      }
+    }
+#pragma unroll
+    for (int o = 16; o; o >>= 1) den += __shfl_xor_sync(0xffffffffu, den, o);
+    if (kWph > 1) {
+      // s_comb: [warps][128 outputs, max, sum]
+      float *mine = s_comb + warp * kCombStride;
+      reinterpret_cast<float4 *>(mine)[lane] = acc;
+      if (lane == 0) { mine[kHeadDim] = mx; mine[kHeadDim + 1] = den; }
+      __syncthreads();
+      if (sub != 0) return;
+      float m_all = -INFINITY;
+#pragma unroll
+      for (int j = 0; j < kWph; ++j) m_all = fmaxf(m_all, mine[j * kCombStride + kHeadDim]);
+      acc = make_float4(0.f, 0.f, 0.f, 0.f);
+      den = 0.f;
+#pragma unroll
+      for (int j = 0; j < kWph; ++j) {
+        const float *o = mine + j * kCombStride;
+        const float a = o[kHeadDim] == -INFINITY ? 0.f : exp2f(o[kHeadDim] - m_all);
+        const float4 x = reinterpret_cast<const float4 *>(o)[lane];
+        acc.x = fmaf(x.x, a, acc.x); acc.y = fmaf(x.y, a, acc.y); acc.z = fmaf(x.z, a, acc.z); acc.w = fmaf(x.w, a, acc.w);
+        den = fmaf(o[kHeadDim + 1], a, den);
+      }
+    }
+    reinterpret_cast<uint2 *>(out_rows + (size_t)g * kHeadDim)[lane] = normalised(acc, den);
+  }
 }
 
 template <int G>
 __device__ __forceinline__ void attn_cta(const DevCtx &c, const Batch &bt, const __nv_bfloat16 *__restrict__ q,
-                                         __nv_bfloat16 *__restrict__ out, uint8_t *smem_pages) {
-  __shared__ float sh[kAttnWarps][G][kPartStride];
-  __shared__ int sh_last;
-  // launch order: chunk 0 of every set first (the chunks that hold the missed pages), or set by set
-  const int b = bt.attn_set_major ? blockIdx.y : blockIdx.x, chunk = bt.attn_set_major ? blockIdx.x : blockIdx.y;
-  const int first = chunk * kChunkPages;
+                                         __nv_bfloat16 *__restrict__ out, uint8_t *smem) {
+  __shared__ __align__(8) unsigned long long s_bar[kAttnWarps * kWarpStages];
+  __shared__ float s_m[kAttnWarps][G], s_l[kAttnWarps][G];
+  __shared__ int sh_ok, sh_np, sh_nm, sh_last;
+  // launch order: row 0 of every set first (the rows that own the first missed pages), or set by set
+  const int b = bt.attn_set_major ? blockIdx.y : blockIdx.x, row = bt.attn_set_major ? blockIdx.x : blockIdx.y;
+  const int max_rows = bt.attn_set_major ? gridDim.x : gridDim.y;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const uint32_t bar0 = smem_u32(&s_bar[kWarpStages * warp]), stage0 = smem_u32(smem) + (uint32_t)(kWarpStages * warp) * kStageBytes;
+  if (lane < kWarpStages) {
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" ::"r"(bar0 + 8 * lane) : "memory");
+    asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
+  }
   int np = 0, nm = 0;                      // pages in the set's list; how many of them are early descriptors
   if (c.ready) {
     // A set raises two flags.  The first says that its missed pages are listed (the leading
-    // n_miss descriptors, slot still open): a warp requests those of its pages at once, so the
+    // n_miss descriptors, slot still open): a warp requests its first missed page at once, so the
     // pages cross the host link while the cache manager is still freeing slots for them.  For
-    // its other pages a warp waits for the second flag (complete list) and for the tail page.
-    __shared__ int sh_ok, sh_np, sh_nm;
+    // everything else a warp waits for the second flag (complete list) and for the tail page.
     if (threadIdx.x == 0) {
       const int ok = flag_wait(c, c.ready1 + b, bt.epoch);
       // a count beyond the list's stride can neither read past the set's row nor leave the merge
-      // waiting for chunks that no CTA of the grid owns
-      sh_np = ok ? max(0, min(c.n_pages[b], c.max_pages + c.tail_cap)) : 0;
-      sh_nm = ok ? c.n_miss[b] : 0;
+      // waiting for rows that no CTA of the grid owns
+      sh_np = ok ? max(0, min(__ldcg(c.n_pages + b), c.max_pages + c.tail_cap)) : 0;
+      sh_nm = ok ? __ldcg(c.n_miss + b) : 0;
       sh_ok = ok;
     }
     __syncthreads();
     if (!sh_ok) return;
     np = sh_np; nm = sh_nm;
+    pages_visible();
   } else {
     pdl_wait_prev();
     np = max(0, min(c.n_pages[b], c.max_pages + c.tail_cap));
+    __syncwarp();
   }
-  if (chunk == 0) dbg_ta(b, 10);
-  if (first >= np) return;
-  const int last = min(np, first + kChunkPages);
+  if (row == 0) dbg_ta(b, 10);
   const int i_req = b / c.Hkv, head = b % c.Hkv;
+  __nv_bfloat16 *out_rows = out + ((size_t)i_req * c.Hq + head * G) * kHeadDim;
+  if (np == 0) {                           // nothing to attend: the set's rows are zero
+    if (row == 0)
+      for (int e = threadIdx.x; e < G * kHeadDim / 4; e += kAttnThreads) reinterpret_cast<uint2 *>(out_rows)[e] = make_uint2(0u, 0u);
+    return;
+  }
+  const int n_rows = min(max_rows, (np + kCtaPages - 1) / kCtaPages);       // CTAs that share this set
+  if (row >= n_rows) return;
   const size_t pl = (size_t)b * (c.max_pages + c.tail_cap);
+  const int stride = n_rows * kAttnWarps;                                   // the warp's pages: mine, mine + stride, ...
+  const int mine = row * kAttnWarps + warp;
 
-  // the warp's two pages.  Early descriptors lead the list, so the first page is early whenever
-  // the second is.  Requests go out, and are waited for, in this order: early pages, then (after
-  // the second flag) the others, of which the one that has to cross the host link comes last.
-  int pg[2] = {first + warp, first + warp + kAttnWarps};
-  int n_mine = (pg[0] < last) + (pg[1] < last);
-  const int n_early = (n_mine >= 1 && pg[0] < nm) + (n_mine >= 2 && pg[1] < nm);
-  int src[2] = {0, 0}, fill[2] = {-1, -1}, open_idx[2] = {-1, -1};
-  uint32_t mask[2] = {0, 0};
-  auto describe = [&](int i) {
-    if (c.page_desc) {                      // work-ordered descriptors written by the cache manager
-      const int4 dsc = c.page_desc[pl + pg[i]];
-      src[i] = dsc.x; fill[i] = dsc.y; mask[i] = (uint32_t)dsc.z;
-      const bool open = dsc.x == -3;        // early descriptor: page_src[dsc.w] names the slot later
-      if (open) { open_idx[i] = dsc.w; src[i] = 0; }
-      if (fill[i] == -2) {
-        // Retrieve step 3 for a missed page: Partition Offset -> CPU page table, both in pinned
-        // host memory (two dependent reads over the host link, all lanes read the same words)
-        const int set = set_index(c, bt.req[i_req], bt.layer, head);
-        const int32_t *off = off_lookup(c, set, c.page_part[pl + dsc.w]);
-        const int32_t *hp = off ? cpt_lookup(c, set, *off + c.page_pidx[pl + dsc.w]) : nullptr;
-        const int host_page = hp ? *hp : -1;
-        if (host_page < 0) { src[i] = -1; fill[i] = c.n_host_pages; }       // fails the range check below
-        else if (open || src[i] >= 0) fill[i] = host_page;                  // fetched (admitted, or not yet known)
-        else { src[i] = ~host_page; fill[i] = -1; }                         // bypassed: attend from host
-      }
-      if (open && fill[i] < 0) { src[i] = -1; fill[i] = c.n_host_pages; }   // an early descriptor always names a host page
-    } else {                                // plain lists, attended in the order given
-      src[i] = c.page_src[pl + pg[i]];
-      mask[i] = c.page_mask[pl + pg[i]];
-    }
-    // a descriptor that points outside the pools is dropped (and reported), never followed
-    const bool ok = (src[i] >= 0 ? src[i] < c.n_gpu_pages : ~src[i] < c.n_host_pages) && fill[i] < c.n_host_pages;
-    if (!ok) { if (lane == 0) dev_error(c, kErrBounds); src[i] = 0; fill[i] = -1; mask[i] = 0; open_idx[i] = -1; }
-  };
-  uint8_t *spage[2] = {smem_pages + (size_t)(2 * warp) * kPageBytes, smem_pages + (size_t)(2 * warp + 1) * kPageBytes};
-  auto request = [&](int i) {
-    const uint8_t *from = fill[i] >= 0 ? c.host_pages + (size_t)fill[i] * kPageBytes : page_ptr(c, src[i]);
-    request_page(smem_u32(spage[i]), from, lane);
-  };
-  // one cp.async group per page slot, in slot order (an empty group where the warp has no page)
-#pragma unroll
-  for (int i = 0; i < 2; ++i)
-    if (i < n_early) { describe(i); request(i); cp_async_commit(); }
-  if (n_early < n_mine) {
-    if (c.ready) {
-      int ok = 1;
-      if (lane == 0) ok = flag_wait(c, c.ready + b, bt.epoch) && flag_wait(c, c.tail_ready + b, bt.epoch);
-      ok = __shfl_sync(0xffffffffu, ok, 0);
-      if (!ok) n_mine = n_early;            // reported by the wait: the warp attends what it has and the CTA still arrives
-    }
-#pragma unroll
-    for (int i = 0; i < 2; ++i)
-      if (i >= n_early && i < n_mine) describe(i);
-    if (n_early == 0 && n_mine == 2 && (fill[0] >= 0 || src[0] < 0) && !(fill[1] >= 0 || src[1] < 0)) {
-      int t = src[0]; src[0] = src[1]; src[1] = t;
-      t = fill[0]; fill[0] = fill[1]; fill[1] = t;
-      t = open_idx[0]; open_idx[0] = open_idx[1]; open_idx[1] = t;
-      uint32_t u = mask[0]; mask[0] = mask[1]; mask[1] = u;
-    }
-#pragma unroll
-    for (int i = 0; i < 2; ++i)
-      if (i >= n_early && i < n_mine) { request(i); cp_async_commit(); }
-  }
-#pragma unroll
-  for (int i = 0; i < 2; ++i)
-    if (i >= n_mine) cp_async_commit();
-  if (chunk == 0) dbg_ta(b, 11);
-
-  // Q as A-operand fragments: row = lane/4 (query head, zero beyond G), 8 k-steps of 16 channels
-  uint32_t qa[8][2];
-  {
-    const int row = lane >> 2;
-    const uint32_t *qrow = reinterpret_cast<const uint32_t *>(q + ((size_t)i_req * c.Hq + head * G + (row < G ? row : 0)) * kHeadDim);
-#pragma unroll
-    for (int ks = 0; ks < 8; ++ks) {
-      qa[ks][0] = row < G ? qrow[ks * 8 + (lane & 3)] : 0u;
-      qa[ks][1] = row < G ? qrow[ks * 8 + 4 + (lane & 3)] : 0u;
-    }
-  }
+  // Q^T as B-operand fragments: column = lane/4 (query head, zero beyond G), 8 k-steps of 16 channels
+  uint32_t qb[8][2];
   WarpAcc acc;
-  acc.m = -INFINITY;
-  acc.l = 0.f;
+  acc.m[0] = acc.m[1] = -INFINITY;
+  acc.l[0] = acc.l[1] = 0.f;
 #pragma unroll
-  for (int i = 0; i < 16; ++i) { acc.o[i][0] = acc.o[i][1] = acc.o[i][2] = acc.o[i][3] = 0.f; }
+  for (int i = 0; i < 8; ++i) { acc.o[i][0] = acc.o[i][1] = acc.o[i][2] = acc.o[i][3] = 0.f; }
   const float scale2 = c.sm_scale * 1.4426950408889634f;
 
-  cp_async_wait<1>();
-  __syncwarp();
-  if (chunk == 0) dbg_ta(b, 12);
-  if (n_mine >= 1) {
-    attend_page(smem_u32(spage[0]), qa, mask[0], scale2, acc, lane);
-    if (fill[0] >= 0) fetched_page_to_slot(c, bt, b, pl, spage[0], src[0], open_idx[0], n_early < 1, lane);
-  }
-  cp_async_wait<0>();
-  __syncwarp();
-  if (chunk == 0) dbg_ta(b, 13);
-  if (n_mine >= 2) {
-    attend_page(smem_u32(spage[1]), qa, mask[1], scale2, acc, lane);
-    if (fill[1] >= 0) fetched_page_to_slot(c, bt, b, pl, spage[1], src[1], open_idx[1], n_early < 2, lane);
+  // The warp's pages in batches of 32, a lane per page (one batch as a rule).  Requests and waits
+  // of a batch: its first missed page is requested as soon as it is known and stays in stage 0;
+  // the hits go through stage 1 meanwhile (through both stages if nothing is missing), then the
+  // missed pages are attended.  The order in which a warp attends its pages is fixed.
+  uint32_t phases = 0;                     // parity of the next wait, a bit per stage
+  bool dead = false, listed = c.ready == nullptr;
+#pragma unroll 1
+  for (int p0 = mine; p0 < np && !dead; p0 += 32 * stride) {
+    const int pos = p0 + lane * stride;
+    PageRef ref{0, -1, -1, 0u};
+    int in0 = -1, in1 = -1;                // the pages (lanes) that have the two stages
+    int turn0 = 0, turn1 = 0;              // their turns on the host link
+    uint32_t issued = 0, on_link = 0;      // stages whose page has been requested; whose page has a turn on the link
+    auto request = [&](int stage, int j) {
+      const int src = __shfl_sync(0xffffffffu, ref.src, j), fill = __shfl_sync(0xffffffffu, ref.fill, j);
+      const uint8_t *from = fill >= 0 ? c.host_pages + (size_t)fill * kPageBytes : page_ptr(c, src);
+      request_page(stage0 + stage * kStageBytes, bar0 + 8 * stage, from, lane);
+      issued |= 1u << stage;
+    };
+    const bool early = pos < min(nm, np);
+    const bool early0 = p0 < nm && !listed;               // early pages lead the list: lane 0's is one of them
+    if (early0) { turn0 = link_turn(c, lane); on_link = 1u; in0 = 0; }
+    if (early) ref = page_ref(c, bt, b, i_req, head, pl, pos);
+    if (early0 && link_open(c, turn0)) request(0, 0);
+    if (p0 == mine) {
+      const int qr = lane >> 2;
+      const uint32_t *qrow = reinterpret_cast<const uint32_t *>(q + ((size_t)i_req * c.Hq + head * G + (qr < G ? qr : 0)) * kHeadDim);
+#pragma unroll
+      for (int ks = 0; ks < 8; ++ks) {
+        qb[ks][0] = qr < G ? qrow[ks * 8 + (lane & 3)] : 0u;
+        qb[ks][1] = qr < G ? qrow[ks * 8 + 4 + (lane & 3)] : 0u;
+      }
+    }
+    if (!listed) {
+      int ok = 1;
+      if (lane == 0) ok = flag_wait2(c, c.ready + b, c.tail_ready + b, bt.epoch);
+      listed = __shfl_sync(0xffffffffu, ok, 0) != 0;
+      pages_visible();
+      dead = !listed;                      // reported by the wait: the warp only sees off the copy it has in flight, and the CTA still arrives
+    }
+    if (pos < np && !early && !dead) ref = page_ref(c, bt, b, i_req, head, pl, pos);
+    // the slot of a page that is brought in; an early descriptor's is known by now (negative: bypassed, attended only)
+    int slot_page = ref.fill >= 0 ? ref.src : -1;
+    if (ref.open_idx >= 0 && !dead) slot_page = __ldcg(c.page_src + pl + ref.open_idx);
+    const bool from_host = ref.fill >= 0 || ref.src < 0;
+    const uint32_t hosted = __ballot_sync(0xffffffffu, pos < np && from_host);
+    uint32_t misses = hosted, hits = __ballot_sync(0xffffffffu, pos < np && !from_host);
+    if (early0) { misses &= ~1u; hits &= ~1u; }           // (a dropped early descriptor is attended with an empty mask)
+    if (dead) misses = hits = 0u;
+    auto pop = [](uint32_t &m) { const int j = __ffs(m) - 1; m &= m - 1; return j; };
+    auto next = [&]() { return hits ? pop(hits) : misses ? pop(misses) : -1; };
+    // the page that has a stage: an HBM page is requested at once, a host page takes its turn on the link
+    auto take0 = [&](int j) { in0 = j; if (j >= 0) { if ((hosted >> j) & 1u) { turn0 = link_turn(c, lane); on_link |= 1u; } else request(0, j); } };
+    auto take1 = [&](int j) { in1 = j; if (j >= 0) { if ((hosted >> j) & 1u) { turn1 = link_turn(c, lane); on_link |= 2u; } else request(1, j); } };
+    if (in0 < 0) take0(misses ? pop(misses) : next());
+    int hits_in1 = (on_link & 1u) ? __popc(hits) : 0;     // hits still to come through stage 1 while stage 0 holds a missed page
+    take1(next());
+    if (row == 0 && p0 == mine) dbg_ta(b, 11);
+    int cur = hits_in1 > 0 ? 1 : 0, polls = 0;
+#pragma unroll 1
+    for (;;) {
+      const int j = cur ? in1 : in0;
+      if (j < 0) break;
+      if ((on_link & ~issued) != 0u && !dead) {
+        if ((on_link & ~issued & 1u) && link_open(c, turn0)) request(0, in0);
+        if ((on_link & ~issued & 2u) && link_open(c, turn1)) request(1, in1);
+      }
+      // a missed page that has landed behind the hits gives its turn on
+      if (hits_in1 > 0 && (on_link & issued & 1u) && page_test(bar0, phases & 1u)) { link_close(c, lane); on_link &= ~1u; }
+      if (!((issued >> cur) & 1u)) {
+        if (!dead && ++polls < kLinkPolls) { __nanosleep(100); continue; }
+        if (!dead && lane == 0) dev_error(c, kErrTimeout);
+        dead = true;
+      } else {
+        if (!page_landed(bar0 + 8 * cur, (phases >> cur) & 1u)) {           // its stage may still be written to: no more requests
+          if (lane == 0) dev_error(c, kErrTimeout);
+          dead = true;
+        }
+        phases ^= 1u << cur;
+      }
+      if (row == 0 && p0 == mine) dbg_ta(b, 12);
+      if ((on_link >> cur) & 1u) link_close(c, lane);
+      on_link &= ~(1u << cur);
+      issued &= ~(1u << cur);
+      const uint32_t spage = stage0 + cur * kStageBytes;
+      if (!dead) {
+        attend_page(spage, qb, __shfl_sync(0xffffffffu, ref.mask, j), scale2, acc, lane);
+        const int slot = __shfl_sync(0xffffffffu, slot_page, j);
+        if (slot >= c.n_gpu_pages) { if (lane == 0) dev_error(c, kErrBounds); }
+        else if (slot >= 0) { store_page(spage, c.gpu_pages + (size_t)slot * kPageBytes, lane); stores_read(); }
+      }
+      __syncwarp();                        // every lane has read the stage
+      const int nx = dead ? -1 : next();
+      if (cur) take1(nx); else take0(nx);
+      if (hits_in1 > 0) { if (--hits_in1 == 0) cur = 0; }
+      else cur ^= 1;
+    }
   }
 
-  // row sums live in the 4 lanes of a quad
-  acc.l += __shfl_xor_sync(0xffffffffu, acc.l, 1);
-  acc.l += __shfl_xor_sync(0xffffffffu, acc.l, 2);
-  {
-    const int row = lane >> 2;
-    if (row < G) {
+  if (row == 0) dbg_ta(b, 13);
+  // a head's sum lives in the 8 lanes of its column; the warps meet in their own (now idle) stage 0
+  float *comb = reinterpret_cast<float *>(smem);
+  constexpr int kWarpComb = kWarpStages * kStageBytes / 4;                  // floats between the warps' areas
+  static_assert(G * kCombStride * 4 <= kStageBytes, "a warp's outputs fit its first stage");
 #pragma unroll
-      for (int nt = 0; nt < 16; ++nt) {
-        sh[warp][row][nt * 8 + (lane & 3) * 2] = acc.o[nt][0];
-        sh[warp][row][nt * 8 + (lane & 3) * 2 + 1] = acc.o[nt][1];
-      }
-      if ((lane & 3) == 0) { sh[warp][row][kHeadDim] = acc.m; sh[warp][row][kHeadDim + 1] = acc.l; }
+  for (int h = 0; h < 2; ++h) {
+#pragma unroll
+    for (int o = 4; o < 32; o <<= 1) acc.l[h] += __shfl_xor_sync(0xffffffffu, acc.l[h], o);
+    const int hr = (lane & 3) * 2 + h;
+    if (hr < G) {
+      float *w = comb + warp * kWarpComb + hr * kCombStride + (lane >> 2);
+#pragma unroll
+      for (int nt = 0; nt < 8; ++nt) { w[nt * 16] = acc.o[nt][h]; w[nt * 16 + 8] = acc.o[nt][2 + h]; }
+      if (lane < 4) { s_m[warp][hr] = acc.m[h]; s_l[warp][hr] = acc.l[h]; }
     }
   }
   __syncthreads();
-  const int n_chunks = (np + kChunkPages - 1) / kChunkPages;
-  float *part = c.att_part + ((size_t)b * c.max_chunks + chunk) * G * kPartStride;
-  for (int e = threadIdx.x; e < G * kHeadDim; e += kAttnWarps * 32) {
-    const int g = e / kHeadDim, ch = e % kHeadDim;
+#pragma unroll 1
+  for (int e = threadIdx.x; e < G * (kHeadDim / 4); e += kAttnThreads) {
+    const int g = e / (kHeadDim / 4), col = e % (kHeadDim / 4);
     float mn = -INFINITY;
 #pragma unroll
-    for (int w = 0; w < kAttnWarps; ++w) mn = fmaxf(mn, sh[w][g][kHeadDim]);
-    float a_o = 0.f, a_l = 0.f;
+    for (int w = 0; w < kAttnWarps; ++w) mn = fmaxf(mn, s_m[w][g]);
+    float4 o = make_float4(0.f, 0.f, 0.f, 0.f);
+    float l = 0.f;
 #pragma unroll
     for (int w = 0; w < kAttnWarps; ++w) {
-      const float mw = sh[w][g][kHeadDim];
-      const float a = mw == -INFINITY ? 0.f : exp2f(mw - mn);
-      a_o += sh[w][g][ch] * a;
-      a_l += sh[w][g][kHeadDim + 1] * a;
+      const float mw = s_m[w][g], a = mw == -INFINITY ? 0.f : exp2f(mw - mn);
+      const float4 x = reinterpret_cast<const float4 *>(comb + w * kWarpComb + g * kCombStride)[col];
+      o.x = fmaf(x.x, a, o.x); o.y = fmaf(x.y, a, o.y); o.z = fmaf(x.z, a, o.z); o.w = fmaf(x.w, a, o.w);
+      l = fmaf(s_l[w][g], a, l);
     }
-    if (n_chunks == 1) {
-      // only chunk of the set: finish here
-      out[((size_t)i_req * c.Hq + head * G + g) * kHeadDim + ch] = __float2bfloat16(a_l > 0.f ? a_o / a_l : 0.f);
+    if (n_rows == 1) {                     // the set's only CTA finishes here
+      reinterpret_cast<uint2 *>(out_rows)[e] = normalised(o, l);
     } else {
-      part[g * kPartStride + ch] = a_o;
-      if (ch == 0) { part[g * kPartStride + kHeadDim] = mn; part[g * kPartStride + kHeadDim + 1] = a_l; }
+      const size_t at = ((size_t)b * c.max_chunks + row) * G + g;
+      reinterpret_cast<float4 *>(c.att_part)[at * (kHeadDim / 4) + col] = o;
+      if (col == 0) c.att_ml[at] = make_float2(mn, l);
     }
   }
-  if (n_chunks == 1) return;
+  if (n_rows == 1) return;
   // the last CTA of the set to get here merges all partials (log-sum-exp)
-  __threadfence();
   __syncthreads();
-  if (threadIdx.x == 0) sh_last = atomicAdd(&c.att_count[b], 1) == n_chunks - 1;
+  if (threadIdx.x == 0) sh_last = last_row(c, b, n_rows);
   __syncthreads();
   if (!sh_last) return;
   dbg_ta(b, 14);
-  __threadfence();
-  // merge.  Nothing here grows with the number of chunks: the per-chunk (max, sum) pairs are
-  // reduced to the set's max and denominator first (a thread's pairs all belong to one head,
-  // the stride being a multiple of the group), then the outputs are accumulated over tiles of
-  // kMergeTile chunks whose weights exp2(m_k - m) sit in shared memory.
-  constexpr int kThreads = kAttnWarps * 32, kMergeTile = 512;
-  static_assert(kThreads == kHeadDim, "thread t of the merge owns channel t of every head");
-  const float *parts = c.att_part + (size_t)b * c.max_chunks * G * kPartStride;
-  float *s_red = reinterpret_cast<float *>(smem_pages);           // [kThreads]
-  float *s_mx = s_red + kThreads;                                 // [G] the set's max per head
-  float *s_den = s_mx + G;                                        // [G]
-  float *s_scale = s_den + G;                                     // [kMergeTile][G]
-  float *s_sum = s_scale + kMergeTile * G;                        // [kMergeTile][G] (single-tile form only)
-  // A set of at most kMergeTile chunks (every decode step of the benchmark configurations) reads
-  // its (max, sum) pairs from memory once, all loads of a thread in flight together; larger
-  // sets take three passes over them, tile by tile.
-  const bool one_tile = n_chunks <= kMergeTile;
-  {
-    float mx = -INFINITY;
-    if (one_tile) {
-#pragma unroll 4
-      for (int e = threadIdx.x; e < n_chunks * G; e += kThreads) {
-        const float *pp = parts + (size_t)e * kPartStride + kHeadDim;
-        const float mk = __ldcg(pp), lk = __ldcg(pp + 1);
-        s_scale[e] = mk;
-        s_sum[e] = lk;
-        mx = fmaxf(mx, mk);
-      }
-    } else {
-      for (int e = threadIdx.x; e < n_chunks * G; e += kThreads)
-        mx = fmaxf(mx, __ldcg(parts + (size_t)e * kPartStride + kHeadDim));
-    }
-    s_red[threadIdx.x] = mx;
-    __syncthreads();
-    if (threadIdx.x < G) {
-      float m_ = -INFINITY;
-      for (int i = threadIdx.x; i < kThreads; i += G) m_ = fmaxf(m_, s_red[i]);
-      s_mx[threadIdx.x] = m_;
-    }
-    __syncthreads();
-    const float mn = s_mx[threadIdx.x % G];
-    float den = 0.f;
-    if (one_tile) {
-      // a thread's own entries: the chunk's maximum gives way to its weight in place
-      for (int e = threadIdx.x; e < n_chunks * G; e += kThreads) {
-        const float mk = s_scale[e], w = mk == -INFINITY ? 0.f : exp2f(mk - mn);
-        s_scale[e] = w;
-        den += mk == -INFINITY ? 0.f : s_sum[e] * w;
-      }
-    } else {
-      for (int e = threadIdx.x; e < n_chunks * G; e += kThreads) {
-        const float *pp = parts + (size_t)e * kPartStride;
-        const float mk = __ldcg(pp + kHeadDim);
-        den += mk == -INFINITY ? 0.f : __ldcg(pp + kHeadDim + 1) * exp2f(mk - mn);
-      }
-    }
-    s_red[threadIdx.x] = den;
-    __syncthreads();
-    if (threadIdx.x < G) {
-      float d_ = 0.f;
-      for (int i = threadIdx.x; i < kThreads; i += G) d_ += s_red[i];
-      s_den[threadIdx.x] = d_;
-    }
-  }
-  float a_o[G];                                                   // this thread's outputs: e = tid + j * kThreads
-#pragma unroll
-  for (int j = 0; j < G; ++j) a_o[j] = 0.f;
-  for (int k0 = 0; k0 < n_chunks; k0 += kMergeTile) {
-    const int kn = min(kMergeTile, n_chunks - k0);
-    __syncthreads();                                              // the previous tile's weights have been used (one tile: the weights are all written)
-    if (!one_tile) {
-      for (int e = threadIdx.x; e < kn * G; e += kThreads) {
-        const float mk = __ldcg(parts + ((size_t)k0 * G + e) * kPartStride + kHeadDim);
-        s_scale[e] = mk == -INFINITY ? 0.f : exp2f(mk - s_mx[e % G]);
-      }
-      __syncthreads();
-    }
-    // a thread's G outputs are channel `threadIdx.x` of every head: the loads of a batch of chunks
-    // for all G heads are issued together (their L2 latency is paid once per batch, not once per head)
-    const float *pt = parts + (size_t)k0 * G * kPartStride + threadIdx.x;
-    // 64 loads in flight per thread; the last batch is padded with its last chunk at weight zero
-    // (one loop, no chunk-by-chunk remainder whose loads would each wait for the one before)
-    constexpr int kB = G >= 8 ? 8 : G == 4 ? 16 : 32;
-#pragma unroll 1
-    for (int k = 0; k < kn; k += kB) {
-      float v[G][kB];
-#pragma unroll
-      for (int j = 0; j < G; ++j)
-#pragma unroll
-        for (int i = 0; i < kB; ++i) v[j][i] = __ldcg(pt + ((size_t)min(k + i, kn - 1) * G + j) * kPartStride);
-#pragma unroll
-      for (int j = 0; j < G; ++j)
-#pragma unroll
-        for (int i = 0; i < kB; ++i) {
-          const float w = k + i < kn ? s_scale[(k + i) * G + j] : 0.f;
-          a_o[j] = fmaf(v[j][i], w, a_o[j]);
-        }
-    }
-  }
-#pragma unroll
-  for (int j = 0; j < G; ++j) {
-    const int e = threadIdx.x + j * kThreads, g = e / kHeadDim, ch = e % kHeadDim;
-    const float den = s_den[g];
-    out[((size_t)i_req * c.Hq + head * G + g) * kHeadDim + ch] = __float2bfloat16(den > 0.f ? a_o[j] / den : 0.f);
-  }
+  merge_rows<G>(c, b, n_rows, out_rows, comb);
   dbg_ta(b, 15);
 }
 
@@ -468,57 +532,53 @@ __device__ __forceinline__ void attn_cta(const DevCtx &c, const Batch &bt, const
 // before it exits, this grid cannot complete ahead of that one, and whatever the stream runs
 // next (the next step's scoring kernel waits for this grid) comes after all of its writes.
 template <int G>
-__global__ void __launch_bounds__(kAttnWarps * 32)
+__global__ void __launch_bounds__(kAttnThreads, 3)
 k_attn(DevCtx c, Batch bt, const __nv_bfloat16 *__restrict__ q, __nv_bfloat16 *__restrict__ out) {
-  extern __shared__ __align__(128) uint8_t smem_pages[];          // [8][8192]
+  extern __shared__ __align__(128) uint8_t smem[];                // [warps][2] staged pages
   pdl_launch_next();
-  attn_cta<G>(c, bt, q, out, smem_pages);
+  attn_cta<G>(c, bt, q, out, smem);
   if (blockIdx.x == 0 && blockIdx.y == 0) pdl_wait_prev();
 }
 
-// Sets whose page list is empty get a zero output (no CTA of k_attn reaches them).
-__global__ void k_attn_zero_empty(DevCtx c, __nv_bfloat16 *__restrict__ out, int n_sets) {
-  const int b = blockIdx.x;
-  if (b >= n_sets || c.n_pages[b] > 0) return;
-  const int i_req = b / c.Hkv, head = b % c.Hkv;
-  for (int e = threadIdx.x; e < c.G * kHeadDim; e += blockDim.x)
-    out[((size_t)i_req * c.Hq + head * c.G) * kHeadDim + e] = __float2bfloat16(0.f);
-}
-
 template <int G>
-void launch_attn_g(const DevCtx &c, const Batch &b, const __nv_bfloat16 *q, __nv_bfloat16 *out, dim3 grid,
-                   cudaStream_t st) {
-  static bool configured_dev[kMaxDevices] = {};
-  bool &configured = configured_dev[current_device_slot()];
-  constexpr int smem = kChunkPages * kPageBytes;
-  if (!configured) {
-    cudaFuncSetAttribute(k_attn<G>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+void launch_attn_g(const DevCtx &c, const Batch &b, const __nv_bfloat16 *q, __nv_bfloat16 *out, int n_sets, int max_pages, cudaStream_t st) {
+  static int resident_dev[kMaxDevices] = {};
+  int &resident = resident_dev[current_device_slot()];
+  if (!resident) {
+    cudaFuncSetAttribute(k_attn<G>, cudaFuncAttributeMaxDynamicSharedMemorySize, kAttnSmem);
     cudaFuncSetAttribute(k_attn<G>, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
-    configured = true;
+    int dev = 0, sms = 0, per_sm = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_attn<G>, kAttnThreads, kAttnSmem);
+    resident = sms * per_sm > 0 ? sms * per_sm : 148;
   }
-  launch_pdl(k_attn<G>, grid, dim3(kAttnWarps * 32), (size_t)smem, st, 1, c, b, q, out);
+  // As many CTAs per set as the GPU holds at once (444), and at least 8 pages for each: every CTA is
+  // resident, its pages stream through its stages, and CTAs share HBM by what they have in flight,
+  // so equal shares end together.  256 sets of 56 pages, 8 heads: 57.7 us with a CTA per 8 pages
+  // (four waves), 35.3 us with one CTA per set; 128 sets of 65 pages: lists complete to merged
+  // 34 us -> 20 us.
+  int rows = resident / n_sets;
+  rows = rows < (max_pages + kCtaPages - 1) / kCtaPages ? rows : (max_pages + kCtaPages - 1) / kCtaPages;
+  if (rows > c.max_chunks) rows = c.max_chunks;
+  if (rows < 1) rows = 1;
+  const dim3 grid = b.attn_set_major ? dim3(rows, n_sets) : dim3(n_sets, rows);
+  launch_pdl(k_attn<G>, grid, dim3(kAttnThreads), (size_t)kAttnSmem, st, 1, c, b, q, out);
 }
 
 }  // namespace
 
 int launch_attention(const DevCtx &c, const Batch &b, const __nv_bfloat16 *q,
-                     __nv_bfloat16 *out, int max_pages_hint, bool may_be_empty, cudaStream_t st, Prof *prof) {
+                     __nv_bfloat16 *out, int max_pages_hint, cudaStream_t st, Prof *prof) {
   const int n_sets = b.n_req * c.Hkv;
-  int chunks = (max_pages_hint + kChunkPages - 1) / kChunkPages;
-  if (chunks < 1) chunks = 1;
-  if (chunks > c.max_chunks) chunks = c.max_chunks;
-  dim3 grid(n_sets, chunks);
-  if (b.attn_set_major) grid = dim3(chunks, n_sets);
-  int launched = 1;
-  if (may_be_empty) { k_attn_zero_empty<<<n_sets, 128, 0, st>>>(c, out, n_sets); ++launched; }
   switch (c.G) {
-    case 1: launch_attn_g<1>(c, b, q, out, grid, st); break;
-    case 2: launch_attn_g<2>(c, b, q, out, grid, st); break;
-    case 4: launch_attn_g<4>(c, b, q, out, grid, st); break;
-    default: launch_attn_g<8>(c, b, q, out, grid, st); break;
+    case 1: launch_attn_g<1>(c, b, q, out, n_sets, max_pages_hint, st); break;
+    case 2: launch_attn_g<2>(c, b, q, out, n_sets, max_pages_hint, st); break;
+    case 4: launch_attn_g<4>(c, b, q, out, n_sets, max_pages_hint, st); break;
+    default: launch_attn_g<8>(c, b, q, out, n_sets, max_pages_hint, st); break;
   }
   prof_mark(prof, st, kProfAttnSplit);
-  return launched;
+  return 1;
 }
 
 }  // namespace spin
@@ -535,7 +595,12 @@ namespace spin {
 namespace {
 constexpr size_t kStaticPartialFloats = (size_t)2 << 20;                  // 8 MiB of fp32
 __device__ __align__(256) static float g_static_partials[kStaticPartialFloats];
+// Arrival words, one per set: the size limit admits fewer sets than this (130 floats and a counter each).
+constexpr int kStaticSets = (int)(kStaticPartialFloats / (kHeadDim + 2 + 1)) + 1;
+__device__ static unsigned long long g_static_words[kStaticSets];         // zero between calls (see last_row)
 float *g_static_partials_addr[kMaxDevices] = {};                          // per device, set up once
+unsigned long long *g_static_words_addr[kMaxDevices] = {};
+std::atomic<uint32_t> g_static_calls{0};
 }  // namespace
 }  // namespace spin
 
@@ -554,7 +619,8 @@ extern "C" int spin_paged_attention_static(const void *q, const void *page_pool,
     return SPIN_ERR_INVALID;
   }
   const int chunks = (list_stride + kChunkPages - 1) / kChunkPages;
-  // layout of the built-in array: [n_sets] arrival counters (as int32), then the partials
+  // room in the built-in array for one partial per 8 pages of every list (and, as ever, a word per
+  // set): more than the call uses, since a CTA writes one partial for all its pages
   const size_t counter_floats = ((size_t)n_sets + 63) / 64 * 64;
   const size_t need = counter_floats + (size_t)n_sets * chunks * group * (kHeadDim + 2);
   if (need > kStaticPartialFloats) {
@@ -570,14 +636,17 @@ extern "C" int spin_paged_attention_static(const void *q, const void *page_pool,
     return SPIN_ERR_CUDA;
   }
   if (!g_static_partials_addr[dev]) {
-    // In host code the array's name is only a stand-in for the symbol: the address the
-    // kernels can use has to be asked for, once per device, with that device current.
+    // In host code the arrays' names are only stand-ins for the symbols: the addresses the
+    // kernels can use have to be asked for, once per device, with that device current.
     float *p = nullptr;
+    unsigned long long *w = nullptr;
     cudaError_t e = cudaGetSymbolAddress(reinterpret_cast<void **>(&p), g_static_partials);
-    if (e != cudaSuccess || !p) {
+    if (e == cudaSuccess) e = cudaGetSymbolAddress(reinterpret_cast<void **>(&w), g_static_words);
+    if (e != cudaSuccess || !p || !w) {
       fprintf(stderr, "spin_paged_attention_static: cudaGetSymbolAddress failed: %s\n", cudaGetErrorString(e));
       return SPIN_ERR_CUDA;
     }
+    g_static_words_addr[dev] = w;
     g_static_partials_addr[dev] = p;
   }
   DevCtx c{};
@@ -597,21 +666,16 @@ extern "C" int spin_paged_attention_static(const void *q, const void *page_pool,
   c.tail_ready = nullptr;
   c.ready1 = nullptr;
   c.n_miss = nullptr;
-  c.att_count = reinterpret_cast<int32_t *>(g_static_partials_addr[dev]);
-  c.att_part = g_static_partials_addr[dev] + counter_floats;
+  c.att_part = g_static_partials_addr[dev];
+  c.att_ml = reinterpret_cast<float2 *>(c.att_part + (size_t)n_sets * chunks * group * kHeadDim);
+  c.att_words = g_static_words_addr[dev];
+  c.att_call = g_static_calls.fetch_add(1u, std::memory_order_relaxed) + 1u;
   cudaStream_t st = reinterpret_cast<cudaStream_t>(cuda_stream);
-  // the array still holds the previous call's counters: they are the one thing that must
-  // start at zero (a memset of library memory, not an allocation)
-  cudaError_t e = cudaMemsetAsync(c.att_count, 0, counter_floats * sizeof(float), st);
-  if (e != cudaSuccess) {
-    fprintf(stderr, "spin_paged_attention_static: clearing the counters failed: %s\n", cudaGetErrorString(e));
-    return SPIN_ERR_CUDA;
-  }
   Batch b{};
   b.n_req = n_sets;
   launch_attention(c, b, reinterpret_cast<const __nv_bfloat16 *>(q), reinterpret_cast<__nv_bfloat16 *>(out),
-                   list_stride, true, st, nullptr);
-  e = cudaGetLastError();
+                   list_stride, st, nullptr);
+  const cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) {
     fprintf(stderr, "spin_paged_attention_static: launch failed: %s\n", cudaGetErrorString(e));
     return SPIN_ERR_CUDA;

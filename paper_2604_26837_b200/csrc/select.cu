@@ -999,7 +999,7 @@ int launch_select(const DevCtx &c, Batch &b, const __nv_bfloat16 *q, const __nv_
     // shared memory of an SM: this kernel's ring beside ONE more CTA, an attention CTA (64 KiB of
     // pages and its per-warp partials) or a selection CTA (smaller); the selection CTAs, one per
     // set, take some SMs and the first attention CTAs the others.  1 KiB per CTA is the system's.
-    const int attn_smem = kChunkPages * kPageBytes + 4 * c.G * (kHeadDim + 2) * 4 + 1024;
+    const int attn_smem = kAttnCtaSmem + 4 * 1024;
     int n_stages = 227 * 1024 - attn_smem - 8 * 1024;
     if (n_stages > 160 * 1024) n_stages = 160 * 1024;
     b.attn_set_major = sg.n_items > 24 * sm_count_of_device() ? 1 : 0;   // a long scoring phase: sets become ready one after the other

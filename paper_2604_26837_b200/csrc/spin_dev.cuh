@@ -22,7 +22,8 @@ constexpr int kMaxBuckets = 64;
 enum : int { kKindPage = 0, kKindToken = 1, kKindCluster = 2, kKindPageMean = 3 };
 // sticky device error bits (same values as SPIN_DEV_ERR_* of the public header)
 constexpr unsigned kErrBounds = 1u, kErrPageList = 2u, kErrTimeout = 4u, kErrState = 8u;
-constexpr int kChunkPages = 8;                              // pages per attention split
+constexpr int kChunkPages = 8;                              // a set of n pages has room for ceil(n / 8) attention partials
+constexpr int kAttnCtaSmem = 8 * 2 * kPageTokens * (kRowBytes + 16);   // staged pages of an attention CTA
 
 // Per-set scalars (device resident, updated only by kernels).
 struct SetState {
@@ -102,8 +103,12 @@ struct DevCtx {
   FetchItem *fetch_queue;       // misses of the whole batch
   int32_t *fetch_count;
   int32_t fetch_cap;
-  float *att_part;              // split-K partials [b][max_chunks][G][kHeadDim + 2]
-  int32_t *att_count;           // [b] chunks of the set that have finished (zero before attention)
+  float *att_part;              // split-K partials: outputs [b][max_chunks][G][kHeadDim]
+  float2 *att_ml;               // ... and their (max, sum) [b][max_chunks][G]
+  int32_t *att_count;           // [b] CTAs of the set that have finished (zero before attention)
+  unsigned long long *att_words;   // the same for the allocation-free call (null in a context), with
+  uint32_t att_call;            //   the call's number in the upper half of each word
+  int32_t *link;                // turns on the host link: [0] taken, [32] done (words of their own lines)
   int32_t *sel_count;           // [b] scoring CTAs of the set that have finished (zero between steps)
   int32_t *score_queue;         // next work item of the resident scoring grid (zero between steps)
   int32_t *score_done;          // CTAs of that grid that have left (zero between steps)
@@ -239,6 +244,20 @@ __device__ __forceinline__ bool flag_wait(const DevCtx &c, const int32_t *flag, 
   return false;
 }
 
+// The same for two flags, polled together.
+__device__ __forceinline__ bool flag_wait2(const DevCtx &c, const int32_t *flag0, const int32_t *flag1, int32_t value) {
+  unsigned pause = 32;
+  for (int spin = 0; spin < kFlagWaitPolls; ++spin) {
+    int32_t v0, v1;
+    asm volatile("ld.acquire.gpu.global.s32 %0, [%2];\nld.acquire.gpu.global.s32 %1, [%3];" : "=&r"(v0), "=r"(v1) : "l"(flag0), "l"(flag1) : "memory");
+    if (v0 == value && v1 == value) return true;
+    __nanosleep(pause);
+    if (pause < 256) pause <<= 1;
+  }
+  dev_error(c, kErrTimeout);
+  return false;
+}
+
 // Scores handed from the streaming scoring kernel to a set's selection without a fence: a score
 // is one naturally aligned 4-byte store, so the word itself says whether it has arrived.  The
 // buffer holds kScoreUnset (a NaN pattern no finite computation produces) in every word between
@@ -345,6 +364,6 @@ int launch_reindex_apply(const DevCtx &c, int req, int layer, int n_clusters, in
                          const uint32_t *touched, cudaStream_t st);
 size_t cache_smem_bytes(const DevCtx &c);
 int launch_attention(const DevCtx &c, const Batch &b, const __nv_bfloat16 *q,
-                     __nv_bfloat16 *out, int max_pages_hint, bool may_be_empty, cudaStream_t st, Prof *prof);
+                     __nv_bfloat16 *out, int max_pages_hint, cudaStream_t st, Prof *prof);
 
 }  // namespace spin
