@@ -174,6 +174,7 @@ struct spin_ctx {
   int sm_count = 148;
   uint64_t launches = 0;
   size_t dir_bytes_in_use = 0;
+  std::vector<DirUpdate> dir_updates;   // directory entries mapped by the call in progress, not yet on the device (see flush_dirs)
   Prof prof;
   int32_t epoch = 0;                 // decode calls so far (value of the per-set ready flags)
   uint32_t floor_calls = 0;          // spin_debug_launch_floor calls (their flag values)
@@ -306,10 +307,10 @@ inline SetHost &set_of(spin_ctx *ctx, int req, int layer, int head) {
   return ctx->sets[(size_t)set_index(ctx->d, req, layer, head)];
 }
 
-// Map the second-level segment holding entry `idx` of one table if it is not mapped yet, and
-// push the directory entry to the device (stream ordered).  Returns the segment or -1.
+// Map the second-level segment holding entry `idx` of one table if it is not mapped yet, and note
+// the directory entry for the device (flush_dirs).  Returns the segment or -1.
 int ensure_seg(spin_ctx *ctx, BitmapPool &pool, std::vector<int32_t> &dir, int32_t *dev_dir_row,
-               int64_t idx, int shift, cudaStream_t st) {
+               int64_t idx, int shift) {
   const size_t di = (size_t)(idx >> shift);
   if (di >= dir.size()) return -1;
   if (dir[di] < 0) {
@@ -317,9 +318,19 @@ int ensure_seg(spin_ctx *ctx, BitmapPool &pool, std::vector<int32_t> &dir, int32
     if (s < 0) return -1;
     dir[di] = (int32_t)s;
     ctx->dir_bytes_in_use += 4;
-    if (cudaMemcpyAsync(dev_dir_row + di, &dir[di], 4, cudaMemcpyHostToDevice, st) != cudaSuccess) return -1;
+    ctx->dir_updates.push_back(DirUpdate{(int32_t)(dev_dir_row + di - ctx->d.dir_meta), (int32_t)s});
   }
   return dir[di];
+}
+
+// Push the directory entries that ensure_seg has noted to the device (stream ordered), all of a
+// call's in one launch as a rule: an append of 2048 pages to 8 heads maps some 320 segments, and
+// as 320 four-byte copies they cost ~1 ms before the first page could move.  No entry is left
+// over when a call returns.
+void flush_dirs(spin_ctx *ctx, cudaStream_t st) {
+  if (ctx->dir_updates.empty()) return;
+  ctx->launches += launch_dir_update(ctx->d, ctx->dir_updates.data(), (int)ctx->dir_updates.size(), st);
+  ctx->dir_updates.clear();
 }
 
 int validate_req_layer(spin_ctx *ctx, int req, int layer) {
@@ -333,7 +344,7 @@ int validate_req_layer(spin_ctx *ctx, int req, int layer) {
 // Host-side Index/Offload bookkeeping of the page-sized kinds for one (request, layer) that
 // grows from n0 to n1 tokens: allocate host pages, fill CPU page table / Partition Offset
 // entries, map the segments the kernels will write.
-int grow_paged(spin_ctx *ctx, int req, int layer, int64_t n1, cudaStream_t st) {
+int grow_paged(spin_ctx *ctx, int req, int layer, int64_t n1) {
   LayerHost &L = ctx->reqs[(size_t)req].layers[(size_t)layer];
   const Geometry &g = ctx->g;
   const DevCtx &d = ctx->d;
@@ -344,27 +355,36 @@ int grow_paged(spin_ctx *ctx, int req, int layer, int64_t n1, cudaStream_t st) {
   const int64_t new_pages = j_end - first_new_page + 1;
   if (new_pages > 0 && ctx->host_page_pool.available() < new_pages * ctx->cfg.num_kv_heads)
     return fail(ctx, SPIN_ERR_OOM_HOST, "out of host pages");
+  // segment by segment: the tables' entries of a segment are consecutive in the pinned pools
   for (int h = 0; h < ctx->cfg.num_kv_heads; ++h) {
     const int set = set_index(d, req, layer, h);
     SetHost &S = ctx->sets[(size_t)set];
-    for (int64_t j = first_new_page; j <= j_end; ++j) {
-      int seg = ensure_seg(ctx, ctx->cpt_segs, S.dir_cpt, d.dir_cpt + (size_t)set * g.dir_page, j, g.seg_shift, st);
+    for (int64_t j = first_new_page; j <= j_end;) {
+      const int64_t end = std::min(j_end + 1, ((j >> g.seg_shift) + 1) << g.seg_shift);
+      const int seg = ensure_seg(ctx, ctx->cpt_segs, S.dir_cpt, d.dir_cpt + (size_t)set * g.dir_page, j, g.seg_shift);
       if (seg < 0) return fail(ctx, SPIN_ERR_OOM_HOST, "out of CPU page table segments");
-      const int64_t hp = ctx->host_page_pool.alloc();
-      ctx->h_cpt_pool[((size_t)seg << g.seg_shift) + (j & (g.seg - 1))] = (int32_t)hp;
-      S.host_pages.push_back((int32_t)hp);
+      int32_t *cpt = ctx->h_cpt_pool + ((size_t)seg << g.seg_shift);
+      for (; j < end; ++j) {
+        const int32_t hp = (int32_t)ctx->host_page_pool.alloc();
+        cpt[j & (g.seg - 1)] = hp;
+        S.host_pages.push_back(hp);
+      }
     }
     // partitions L.n_partitions .. j_end-1 get indexed by this call
-    for (int64_t p = L.n_partitions; p < j_end; ++p) {
-      if (ensure_seg(ctx, ctx->meta_segs, S.dir_meta, d.dir_meta + (size_t)set * g.dir_part, p, g.seg_shift, st) < 0)
+    for (int64_t p = L.n_partitions; p < j_end;) {
+      const int64_t end = std::min(j_end, ((p >> g.seg_shift) + 1) << g.seg_shift);
+      if (ensure_seg(ctx, ctx->meta_segs, S.dir_meta, d.dir_meta + (size_t)set * g.dir_part, p, g.seg_shift) < 0)
         return fail(ctx, SPIN_ERR_OOM_DEVICE, "out of Meta-partition segments");
-      int seg = ensure_seg(ctx, ctx->off_segs, S.dir_off, d.dir_off + (size_t)set * g.dir_part, p, g.seg_shift, st);
+      const int seg = ensure_seg(ctx, ctx->off_segs, S.dir_off, d.dir_off + (size_t)set * g.dir_part, p, g.seg_shift);
       if (seg < 0) return fail(ctx, SPIN_ERR_OOM_HOST, "out of Partition Offset segments");
-      ctx->h_off_pool[((size_t)seg << g.seg_shift) + (p & (g.seg - 1))] = (int32_t)p;
-      const int64_t e = ctx->cfg.partition_kind == SPIN_PART_TOKEN_DOT ? p * kPageTokens : p;
-      if (ensure_seg(ctx, ctx->sum_segs, S.dir_sum, d.dir_sumseg + (size_t)set * g.dir_sum, e, g.sum_shift, st) < 0)
-        return fail(ctx, SPIN_ERR_OOM_DEVICE, "out of summary segments");
+      int32_t *off = ctx->h_off_pool + ((size_t)seg << g.seg_shift);
+      for (; p < end; ++p) off[p & (g.seg - 1)] = (int32_t)p;
     }
+    const int64_t per_page = ctx->cfg.partition_kind == SPIN_PART_TOKEN_DOT ? kPageTokens : 1;
+    const int64_t e_end = j_end * per_page;
+    for (int64_t e = L.n_partitions * per_page; e < e_end; e = ((e >> g.sum_shift) + 1) << g.sum_shift)
+      if (ensure_seg(ctx, ctx->sum_segs, S.dir_sum, d.dir_sumseg + (size_t)set * g.dir_sum, e, g.sum_shift) < 0)
+        return fail(ctx, SPIN_ERR_OOM_DEVICE, "out of summary segments");
   }
   L.n_tokens = n1;
   L.n_partitions = (int32_t)j_end;
@@ -376,7 +396,7 @@ int grow_paged(spin_ctx *ctx, int req, int layer, int64_t n1, cudaStream_t st) {
 }
 
 // Decode tokens of a clustered (request, layer): they extend the tail.
-int grow_cluster_tail(spin_ctx *ctx, int req, int layer, int64_t n_new, cudaStream_t st) {
+int grow_cluster_tail(spin_ctx *ctx, int req, int layer, int64_t n_new) {
   LayerHost &L = ctx->reqs[(size_t)req].layers[(size_t)layer];
   const Geometry &g = ctx->g;
   const DevCtx &d = ctx->d;
@@ -389,7 +409,7 @@ int grow_cluster_tail(spin_ctx *ctx, int req, int layer, int64_t n_new, cudaStre
         const int set = set_index(d, req, layer, h);
         SetHost &S = ctx->sets[(size_t)set];
         const int64_t j = L.tail_first + L.tail_pages;
-        int seg = ensure_seg(ctx, ctx->cpt_segs, S.dir_cpt, d.dir_cpt + (size_t)set * g.dir_page, j, g.seg_shift, st);
+        int seg = ensure_seg(ctx, ctx->cpt_segs, S.dir_cpt, d.dir_cpt + (size_t)set * g.dir_page, j, g.seg_shift);
         if (seg < 0) return fail(ctx, SPIN_ERR_OOM_HOST, "out of CPU page table segments");
         const int64_t hp = ctx->host_page_pool.alloc();
         ctx->h_cpt_pool[((size_t)seg << g.seg_shift) + (j & (g.seg - 1))] = (int32_t)hp;
@@ -463,7 +483,8 @@ int append_paged_device(spin_ctx *ctx, int req, int layer, const __nv_bfloat16 *
   LayerHost &L = ctx->reqs[(size_t)req].layers[(size_t)layer];
   const int64_t n0 = L.n_tokens;
   const int64_t j0 = n0 > 0 ? (n0 - 1) / kPageTokens : -1;
-  int rc = grow_paged(ctx, req, layer, n0 + n, st);
+  int rc = grow_paged(ctx, req, layer, n0 + n);
+  flush_dirs(ctx, st);
   if (rc) return rc;
   const int64_t j_end = (n0 + n - 1) / kPageTokens;
   // pages strictly between the old tail page and the newest page: complete, all rows new
@@ -523,8 +544,8 @@ int append_paged_device(spin_ctx *ctx, int req, int layer, const __nv_bfloat16 *
   return SPIN_OK;
 }
 
-int prefill_clustered(spin_ctx *ctx, int req, int layer, const void *k, const void *v, int64_t n,
-                      const int32_t *token_partition, const void *centroids, cudaStream_t st) {
+int prefill_clustered_impl(spin_ctx *ctx, int req, int layer, const void *k, const void *v, int64_t n,
+                           const int32_t *token_partition, const void *centroids, cudaStream_t st) {
   LayerHost &L = ctx->reqs[(size_t)req].layers[(size_t)layer];
   const Geometry &g = ctx->g;
   const DevCtx &d = ctx->d;
@@ -556,16 +577,16 @@ int prefill_clustered(spin_ctx *ctx, int req, int layer, const void *k, const vo
       const int32_t m = count[(size_t)h * C + c], npg = (m + kPageTokens - 1) / kPageTokens;
       first_row_page[(size_t)h * C + c] = off;
       meta[(size_t)c] = MetaEntry{m, 0};
-      int seg = ensure_seg(ctx, ctx->off_segs, S.dir_off, d.dir_off + (size_t)set * g.dir_part, c, g.seg_shift, st);
+      int seg = ensure_seg(ctx, ctx->off_segs, S.dir_off, d.dir_off + (size_t)set * g.dir_part, c, g.seg_shift);
       if (seg < 0) return fail(ctx, SPIN_ERR_OOM_HOST, "out of Partition Offset segments");
       ctx->h_off_pool[((size_t)seg << g.seg_shift) + (c & (g.seg - 1))] = off;
-      if (ensure_seg(ctx, ctx->meta_segs, S.dir_meta, d.dir_meta + (size_t)set * g.dir_part, c, g.seg_shift, st) < 0)
+      if (ensure_seg(ctx, ctx->meta_segs, S.dir_meta, d.dir_meta + (size_t)set * g.dir_part, c, g.seg_shift) < 0)
         return fail(ctx, SPIN_ERR_OOM_DEVICE, "out of Meta-partition segments");
-      if (ensure_seg(ctx, ctx->sum_segs, S.dir_sum, d.dir_sumseg + (size_t)set * g.dir_sum, c, g.sum_shift, st) < 0)
+      if (ensure_seg(ctx, ctx->sum_segs, S.dir_sum, d.dir_sumseg + (size_t)set * g.dir_sum, c, g.sum_shift) < 0)
         return fail(ctx, SPIN_ERR_OOM_DEVICE, "out of summary segments");
       for (int i = 0; i < npg; ++i) {
         const int64_t j = off + i;
-        int cs = ensure_seg(ctx, ctx->cpt_segs, S.dir_cpt, d.dir_cpt + (size_t)set * g.dir_page, j, g.seg_shift, st);
+        int cs = ensure_seg(ctx, ctx->cpt_segs, S.dir_cpt, d.dir_cpt + (size_t)set * g.dir_page, j, g.seg_shift);
         if (cs < 0) return fail(ctx, SPIN_ERR_OOM_HOST, "out of CPU page table segments");
         const int64_t hp = ctx->host_page_pool.alloc();
         ctx->h_cpt_pool[((size_t)cs << g.seg_shift) + (j & (g.seg - 1))] = (int32_t)hp;
@@ -626,6 +647,7 @@ int prefill_clustered(spin_ctx *ctx, int req, int layer, const void *k, const vo
       const int32_t hp = S.host_pages[(size_t)(first_row_page[(size_t)h * C + c] + r / kPageTokens)];
       dest[(size_t)t * H + h] = (int64_t)hp * kPageTokens + r % kPageTokens;
     }
+  flush_dirs(ctx, st);
   // centroids -> summary segments
   const __nv_bfloat16 *cen = reinterpret_cast<const __nv_bfloat16 *>(centroids);
   void *cen_tmp = nullptr;
@@ -709,6 +731,13 @@ int prefill_clustered(spin_ctx *ctx, int req, int layer, const void *k, const vo
   L.tail_len = 0;
   L.clustered = true;
   return SPIN_OK;
+}
+
+int prefill_clustered(spin_ctx *ctx, int req, int layer, const void *k, const void *v, int64_t n,
+                      const int32_t *token_partition, const void *centroids, cudaStream_t st) {
+  const int rc = prefill_clustered_impl(ctx, req, layer, k, v, n, token_partition, centroids, st);
+  flush_dirs(ctx, st);                      // a call that failed half way leaves no entry behind either
+  return rc;
 }
 
 }  // namespace
@@ -915,41 +944,49 @@ int spin_request_open(spin_ctx *ctx, int64_t slots, int32_t *out_req) {
     return fail(ctx, SPIN_ERR_BUDGET, "budget needs %lld GPU pages, %lld free", (long long)(slots * sets_per_req), (long long)ctx->gpu_page_pool.available());
   if (ctx->gpt_segs.available() < segs_per_set * sets_per_req)
     return fail(ctx, SPIN_ERR_OOM_DEVICE, "out of GPU page table segments");
-  std::vector<GptEntry> ent((size_t)g.seg);
-  for (int l = 0; l < ctx->cfg.num_layers; ++l)
-    for (int h = 0; h < ctx->cfg.num_kv_heads; ++h) {
-      const int set = set_index(d, req, l, h);
-      SetHost &S = ctx->sets[(size_t)set];
-      S = SetHost();
-      S.dir_meta.assign((size_t)g.dir_part, -1);
-      S.dir_off.assign((size_t)g.dir_part, -1);
-      S.dir_gpt.assign((size_t)g.dir_slot, -1);
-      S.dir_cpt.assign((size_t)g.dir_page, -1);
-      S.dir_sum.assign((size_t)g.dir_sum, -1);
-      for (int64_t s0 = 0; s0 < slots; s0 += g.seg) {
-        const int64_t seg = ctx->gpt_segs.alloc();
-        S.dir_gpt[(size_t)(s0 >> g.seg_shift)] = (int32_t)seg;
-        ctx->dir_bytes_in_use += 4;
-        const int cnt = (int)std::min<int64_t>(g.seg, slots - s0);
-        for (int i = 0; i < g.seg; ++i) {
-          int32_t phys = -1;
-          if (i < cnt) { phys = (int32_t)ctx->gpu_page_pool.alloc(); S.gpu_pages.push_back(phys); }
-          ent[(size_t)i] = GptEntry{-1, phys, 0, -1};
-        }
-        CK(cudaMemcpy(d.gpt_pool + ((size_t)seg << g.seg_shift), ent.data(), (size_t)g.seg * sizeof(GptEntry), cudaMemcpyHostToDevice));
+  // All sets of a request are consecutive (layer by layer, head by head), so each table's rows go up
+  // in one copy, and the page table segments in one copy per run of consecutive segments.  The
+  // directories of the other tables hold nothing but "unmapped" since spin_create or the last close.
+  const int set0 = set_index(d, req, 0, 0), n_sets = (int)sets_per_req;
+  std::vector<GptEntry> ent;
+  std::vector<int32_t> dir_gpt((size_t)n_sets * g.dir_slot, -1), tails((size_t)n_sets * g.tail_cap);
+  std::vector<SetState> states((size_t)n_sets);
+  int64_t run_seg = -1;                                     // first segment of the entries collected so far
+  auto upload = [&]() {
+    cudaError_t e = ent.empty() ? cudaSuccess : cudaMemcpy(d.gpt_pool + ((size_t)run_seg << g.seg_shift), ent.data(), ent.size() * sizeof(GptEntry), cudaMemcpyHostToDevice);
+    ent.clear();
+    return e;
+  };
+  for (int i = 0; i < n_sets; ++i) {
+    const int set = set0 + i;
+    SetHost &S = ctx->sets[(size_t)set];
+    S = SetHost();
+    S.dir_meta.assign((size_t)g.dir_part, -1);
+    S.dir_off.assign((size_t)g.dir_part, -1);
+    S.dir_gpt.assign((size_t)g.dir_slot, -1);
+    S.dir_cpt.assign((size_t)g.dir_page, -1);
+    S.dir_sum.assign((size_t)g.dir_sum, -1);
+    for (int64_t s0 = 0; s0 < slots; s0 += g.seg) {
+      const int64_t seg = ctx->gpt_segs.alloc();
+      S.dir_gpt[(size_t)(s0 >> g.seg_shift)] = (int32_t)seg;
+      dir_gpt[(size_t)i * g.dir_slot + (size_t)(s0 >> g.seg_shift)] = (int32_t)seg;
+      ctx->dir_bytes_in_use += 4;
+      if (!ent.empty() && seg != run_seg + (int64_t)(ent.size() >> g.seg_shift)) CK(upload());
+      if (ent.empty()) run_seg = seg;
+      const int cnt = (int)std::min<int64_t>(g.seg, slots - s0);
+      for (int k = 0; k < g.seg; ++k) {
+        int32_t phys = -1;
+        if (k < cnt) { phys = (int32_t)ctx->gpu_page_pool.alloc(); S.gpu_pages.push_back(phys); }
+        ent.push_back(GptEntry{-1, phys, 0, -1});
       }
-      CK(cudaMemcpy(d.dir_gpt + (size_t)set * g.dir_slot, S.dir_gpt.data(), (size_t)g.dir_slot * 4, cudaMemcpyHostToDevice));
-      CK(cudaMemcpy(d.dir_meta + (size_t)set * g.dir_part, S.dir_meta.data(), (size_t)g.dir_part * 4, cudaMemcpyHostToDevice));
-      CK(cudaMemcpy(d.dir_off + (size_t)set * g.dir_part, S.dir_off.data(), (size_t)g.dir_part * 4, cudaMemcpyHostToDevice));
-      CK(cudaMemcpy(d.dir_cpt + (size_t)set * g.dir_page, S.dir_cpt.data(), (size_t)g.dir_page * 4, cudaMemcpyHostToDevice));
-      CK(cudaMemcpy(d.dir_sumseg + (size_t)set * g.dir_sum, S.dir_sum.data(), (size_t)g.dir_sum * 4, cudaMemcpyHostToDevice));
-      std::vector<int32_t> tails((size_t)g.tail_cap);
-      for (int j = 0; j < g.tail_cap; ++j) tails[(size_t)j] = (int32_t)(ctx->cfg.gpu_cache_pages + (int64_t)set * g.tail_cap + j);
-      CK(cudaMemcpy(d.tail_phys + (size_t)set * g.tail_cap, tails.data(), (size_t)g.tail_cap * 4, cudaMemcpyHostToDevice));
-      SetState s{};
-      s.slots = (int32_t)slots;
-      CK(cudaMemcpy(d.state + set, &s, sizeof s, cudaMemcpyHostToDevice));
     }
+    for (int j = 0; j < g.tail_cap; ++j) tails[(size_t)i * g.tail_cap + j] = (int32_t)(ctx->cfg.gpu_cache_pages + (int64_t)set * g.tail_cap + j);
+    states[(size_t)i].slots = (int32_t)slots;
+  }
+  CK(upload());
+  CK(cudaMemcpy(d.dir_gpt + (size_t)set0 * g.dir_slot, dir_gpt.data(), dir_gpt.size() * 4, cudaMemcpyHostToDevice));
+  CK(cudaMemcpy(d.tail_phys + (size_t)set0 * g.tail_cap, tails.data(), tails.size() * 4, cudaMemcpyHostToDevice));
+  CK(cudaMemcpy(d.state + set0, states.data(), states.size() * sizeof(SetState), cudaMemcpyHostToDevice));
   RequestHost &R = ctx->reqs[(size_t)req];
   R.open = true;
   R.slots = slots;
@@ -958,7 +995,7 @@ int spin_request_open(spin_ctx *ctx, int64_t slots, int32_t *out_req) {
   return SPIN_OK;
 }
 
-int spin_reindex(spin_ctx *ctx, int32_t req, int32_t layer, void *cuda_stream) {
+static int reindex_impl(spin_ctx *ctx, int32_t req, int32_t layer, void *cuda_stream) {
   int rc = validate_req_layer(ctx, req, layer);
   if (rc) return rc;
   if (ctx->cfg.partition_kind != SPIN_PART_CLUSTER_CENTROID)
@@ -1037,7 +1074,7 @@ int spin_reindex(spin_ctx *ctx, int32_t req, int32_t layer, void *cuda_stream) {
     SetHost &S = ctx->sets[(size_t)set];
     S.host_pages.assign((size_t)(total_max + n_rem), -1);
     auto put = [&](int64_t j, int32_t hp) -> bool {
-      const int cs = ensure_seg(ctx, ctx->cpt_segs, S.dir_cpt, d.dir_cpt + (size_t)set * g.dir_page, j, g.seg_shift, st);
+      const int cs = ensure_seg(ctx, ctx->cpt_segs, S.dir_cpt, d.dir_cpt + (size_t)set * g.dir_page, j, g.seg_shift);
       if (cs < 0) return false;
       ctx->h_cpt_pool[((size_t)cs << g.seg_shift) + (j & (g.seg - 1))] = hp;
       S.host_pages[(size_t)j] = hp;
@@ -1063,6 +1100,7 @@ int spin_reindex(spin_ctx *ctx, int32_t req, int32_t layer, void *cuda_stream) {
   CK(cudaMemcpyAsync(ctx->stage_dest, dest.data(), dest.size() * 8, cudaMemcpyHostToDevice, st));
   CK(cudaMemcpyAsync(d_new_tokens, new_tokens.data(), new_tokens.size() * 4, cudaMemcpyHostToDevice, st));
   CK(cudaMemcpyAsync(d_touched, touched.data(), touched.size() * 4, cudaMemcpyHostToDevice, st));
+  flush_dirs(ctx, st);
   ctx->launches += launch_move_rows(d, req, layer, ctx->stage_dest, n_tok, st);
   ctx->launches += launch_reindex_apply(d, req, layer, C, n_full, total_max, n_rem, n_rem ? L.tail_len : 0,
                                         total_max + n_rem, d_new_tokens, d_touched, st);
@@ -1083,6 +1121,13 @@ int spin_reindex(spin_ctx *ctx, int32_t req, int32_t layer, void *cuda_stream) {
   CK(cudaGetLastError());
   return SPIN_OK;
 }
+
+int spin_reindex(spin_ctx *ctx, int32_t req, int32_t layer, void *cuda_stream) {
+  const int rc = reindex_impl(ctx, req, layer, cuda_stream);
+  if (ctx) flush_dirs(ctx, reinterpret_cast<cudaStream_t>(cuda_stream));   // a call that failed half way leaves no entry behind either
+  return rc;
+}
+
 int spin_request_close(spin_ctx *ctx, int32_t req) {
   if (!ctx) return SPIN_ERR_INVALID;
   if (req < 0 || req >= ctx->cfg.max_requests) return fail(ctx, SPIN_ERR_INVALID, "request id %d out of range", req);
@@ -1105,14 +1150,16 @@ int spin_request_close(spin_ctx *ctx, int32_t req) {
       drop(ctx->off_segs, S.dir_off);
       drop(ctx->cpt_segs, S.dir_cpt);
       drop(ctx->sum_segs, S.dir_sum);
-      CK(cudaMemset(d.dir_gpt + (size_t)set * g.dir_slot, 0xff, (size_t)g.dir_slot * 4));
-      CK(cudaMemset(d.dir_meta + (size_t)set * g.dir_part, 0xff, (size_t)g.dir_part * 4));
-      CK(cudaMemset(d.dir_off + (size_t)set * g.dir_part, 0xff, (size_t)g.dir_part * 4));
-      CK(cudaMemset(d.dir_cpt + (size_t)set * g.dir_page, 0xff, (size_t)g.dir_page * 4));
-      CK(cudaMemset(d.dir_sumseg + (size_t)set * g.dir_sum, 0xff, (size_t)g.dir_sum * 4));
-      CK(cudaMemset(d.state + set, 0, sizeof(SetState)));
       S = SetHost();
     }
+  // the rows of a request's sets are consecutive in every table
+  const size_t set0 = (size_t)set_index(d, req, 0, 0), n = (size_t)ctx->cfg.num_layers * ctx->cfg.num_kv_heads;
+  CK(cudaMemset(d.dir_gpt + set0 * g.dir_slot, 0xff, n * g.dir_slot * 4));
+  CK(cudaMemset(d.dir_meta + set0 * g.dir_part, 0xff, n * g.dir_part * 4));
+  CK(cudaMemset(d.dir_off + set0 * g.dir_part, 0xff, n * g.dir_part * 4));
+  CK(cudaMemset(d.dir_cpt + set0 * g.dir_page, 0xff, n * g.dir_page * 4));
+  CK(cudaMemset(d.dir_sumseg + set0 * g.dir_sum, 0xff, n * g.dir_sum * 4));
+  CK(cudaMemset(d.state + set0, 0, n * sizeof(SetState)));
   R = RequestHost();
   return SPIN_OK;
 }
@@ -1209,7 +1256,8 @@ int spin_append_kv(spin_ctx *ctx, int32_t req, int32_t layer, const void *k, con
       vv = ctx->stage_v;
     }
     if (cluster) {
-      rc = grow_cluster_tail(ctx, req, layer, m, st);
+      rc = grow_cluster_tail(ctx, req, layer, m);
+      flush_dirs(ctx, st);
       if (rc) return rc;
       AppendEdgeArgs a{};
       a.n_req = 1; a.layer = layer; a.req[0] = req;
@@ -1246,10 +1294,11 @@ int spin_append_kv_batch(spin_ctx *ctx, int32_t layer, const int32_t *req_ids, i
   // all checks passed: from here on the call changes state
   for (int i = 0; i < n_req; ++i) {
     LayerHost &L = ctx->reqs[(size_t)req_ids[i]].layers[(size_t)layer];
-    int rc = cluster ? grow_cluster_tail(ctx, req_ids[i], layer, 1, st) : grow_paged(ctx, req_ids[i], layer, L.n_tokens + 1, st);
-    if (rc) return rc;
+    int rc = cluster ? grow_cluster_tail(ctx, req_ids[i], layer, 1) : grow_paged(ctx, req_ids[i], layer, L.n_tokens + 1);
+    if (rc) { flush_dirs(ctx, st); return rc; }
     a.n_tokens[i] = (int32_t)(L.n_tokens - 1);
   }
+  flush_dirs(ctx, st);
   const __nv_bfloat16 *kk = reinterpret_cast<const __nv_bfloat16 *>(k), *vv = reinterpret_cast<const __nv_bfloat16 *>(v);
   if (!k_dev) {
     const size_t bytes = (size_t)n_req * ctx->cfg.num_kv_heads * kRowBytes;
@@ -1302,9 +1351,10 @@ static int step_impl(spin_ctx *ctx, int32_t layer, const int32_t *req_ids, int32
   if (with_append) {
     for (int i = 0; i < n_req; ++i) {
       LayerHost &L = ctx->reqs[(size_t)req_ids[i]].layers[(size_t)layer];
-      int rc = cluster ? grow_cluster_tail(ctx, req_ids[i], layer, 1, st) : grow_paged(ctx, req_ids[i], layer, L.n_tokens + 1, st);
-      if (rc) return rc;
+      int rc = cluster ? grow_cluster_tail(ctx, req_ids[i], layer, 1) : grow_paged(ctx, req_ids[i], layer, L.n_tokens + 1);
+      if (rc) { flush_dirs(ctx, st); return rc; }
     }
+    flush_dirs(ctx, st);
     kk = reinterpret_cast<const __nv_bfloat16 *>(k);
     vv = reinterpret_cast<const __nv_bfloat16 *>(v);
     if (kc == 2) {

@@ -105,6 +105,14 @@ k_copy_centroids(DevCtx c, int req, int layer, const __nv_bfloat16 *__restrict__
   }
 }
 
+// Directory entries, carried in the kernel's parameters.
+constexpr int kDirBatch = 448;                       // 3.5 KB of parameters
+struct DirBatch { int32_t n; DirUpdate u[kDirBatch]; };
+__global__ void __launch_bounds__(256)
+k_dir_update(int32_t *__restrict__ dirs, const __grid_constant__ DirBatch a) {
+  for (int i = threadIdx.x; i < a.n; i += 256) dirs[a.u[i].at] = a.u[i].value;
+}
+
 // Step inputs that live in pinned host memory (q, new k/v) are brought into the staging
 // buffers by one small kernel of zero-copy reads instead of one copy-engine transfer each.
 __global__ void __launch_bounds__(256)
@@ -131,6 +139,17 @@ int launch_stage_in(void *dq, const void *sq, size_t q_bytes, void *dk, const vo
              reinterpret_cast<uint4 *>(dk), reinterpret_cast<const uint4 *>(sk), reinterpret_cast<uint4 *>(dv),
              reinterpret_cast<const uint4 *>(sv), nkv);
   return 1;
+}
+
+int launch_dir_update(const DevCtx &c, const DirUpdate *u, int n, cudaStream_t st) {
+  int launched = 0;
+  for (int i = 0; i < n; i += kDirBatch, ++launched) {
+    DirBatch a;
+    a.n = n - i < kDirBatch ? n - i : kDirBatch;
+    for (int j = 0; j < a.n; ++j) a.u[j] = u[i + j];
+    k_dir_update<<<1, 256, 0, st>>>(c.dir_meta, a);
+  }
+  return launched;
 }
 
 int launch_append_bulk(const DevCtx &c, int req, int layer, const __nv_bfloat16 *k,

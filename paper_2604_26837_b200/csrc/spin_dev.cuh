@@ -335,6 +335,8 @@ struct AppendEdgeArgs {     // one (request) per entry; all its kv heads are pro
   int32_t req[kMaxBatch];
   int32_t n_tokens[kMaxBatch];   // tokens of the request before this append, as the host has counted them
 };
+struct DirUpdate { int32_t at, value; };   // a directory entry: index from dir_meta (the five directories share one region), new value
+int launch_dir_update(const DevCtx &c, const DirUpdate *u, int n, cudaStream_t st);
 int launch_append_bulk(const DevCtx &c, int req, int layer, const __nv_bfloat16 *k,
                        const __nv_bfloat16 *v, int first_page, int n_pages, int first_token_of_call,
                        cudaStream_t st, Prof *prof, uint8_t *stage = nullptr, const int32_t *stage_hp = nullptr);
