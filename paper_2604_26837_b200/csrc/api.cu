@@ -170,7 +170,7 @@ struct spin_ctx {
   uint8_t *h_pages = nullptr;
   // staging for host-pointer arguments
   __nv_bfloat16 *stage_q = nullptr, *stage_out = nullptr, *stage_k = nullptr, *stage_v = nullptr;
-  int64_t *stage_dest = nullptr;
+  int64_t *stage_dest = nullptr;        // spin_reindex: destination rows of the folded tokens
   int sm_count = 148;
   uint64_t launches = 0;
   size_t dir_bytes_in_use = 0;
@@ -183,7 +183,11 @@ struct spin_ctx {
   static constexpr int kOffloadSlots = 4;
   uint8_t *offload_stage = nullptr;
   int32_t *offload_hp = nullptr;     // per staged unit: its host page id (what the kernel records in the mirror)
-  int32_t *offload_lrow = nullptr;   // cluster prefill: row places of one prefill's tokens (see prefill_clustered)
+  // cluster prefill (see prefill_clustered): every token row's place in its set's page order; per
+  // (head, cluster) token counts (behind one 64-bit word: the first bad entry), first pages, running counts
+  int32_t *cl_place = nullptr, *cl_base = nullptr, *cl_run = nullptr;
+  unsigned long long *cl_bad = nullptr;
+  int32_t *cl_count = nullptr;
   int64_t offload_slot_units = 0;    // (page, kv head) units of 8 KiB per slot; 0 = write-through
   cudaStream_t offload_stream = nullptr;
   cudaEvent_t ev_staged[kOffloadSlots] = {}, ev_done[kOffloadSlots] = {};
@@ -273,10 +277,17 @@ void carve(Arena &a, const spin_config &cfg, const Geometry &g, DevCtx &d, spin_
     const int64_t units = cfg.offload_stage_bytes / spin_ctx::kOffloadSlots / kPageBytes;
     uint8_t *os = a.take<uint8_t>((size_t)units * spin_ctx::kOffloadSlots * kPageBytes);
     int32_t *oh = a.take<int32_t>((size_t)units * spin_ctx::kOffloadSlots);
-    // cluster granularity: where every (token, head) row of a prefill goes in its set's page order
-    int32_t *ol = cfg.partition_kind == SPIN_PART_CLUSTER_CENTROID
-                      ? a.take<int32_t>((size_t)cfg.max_context_tokens * cfg.num_kv_heads) : nullptr;
-    if (ctx) { ctx->offload_stage = os; ctx->offload_hp = oh; ctx->offload_slot_units = units; ctx->offload_lrow = ol; }
+    if (ctx) { ctx->offload_stage = os; ctx->offload_hp = oh; ctx->offload_slot_units = units; }
+  }
+  if (cfg.partition_kind == SPIN_PART_CLUSTER_CENTROID) {
+    const size_t hc = (size_t)cfg.num_kv_heads * cfg.num_clusters;
+    int32_t *place = a.take<int32_t>((size_t)cfg.max_context_tokens * cfg.num_kv_heads);
+    int32_t *count = a.take<int32_t>(2 + hc), *base = a.take<int32_t>(hc), *run = a.take<int32_t>(hc);
+    if (ctx) {
+      ctx->cl_place = place; ctx->cl_base = base; ctx->cl_run = run;
+      ctx->cl_bad = reinterpret_cast<unsigned long long *>(count);
+      ctx->cl_count = count + 2;
+    }
   }
 }
 
@@ -544,6 +555,10 @@ int append_paged_device(spin_ctx *ctx, int req, int layer, const __nv_bfloat16 *
   return SPIN_OK;
 }
 
+// Cluster prefill.  The GPU counts the clusters' tokens, the host (which hands out the pages) lays
+// the sets' pages out from the counts, the GPU does everything that is per token: ranks the
+// tokens within their clusters, fills the tables' HBM copies and moves the rows.  (Counting and
+// placing 262144 rows on the host and uploading a place per row took 2.8 ms of a 5.4 ms prefill.)
 int prefill_clustered_impl(spin_ctx *ctx, int req, int layer, const void *k, const void *v, int64_t n,
                            const int32_t *token_partition, const void *centroids, cudaStream_t st) {
   LayerHost &L = ctx->reqs[(size_t)req].layers[(size_t)layer];
@@ -552,103 +567,75 @@ int prefill_clustered_impl(spin_ctx *ctx, int req, int layer, const void *k, con
   const int H = ctx->cfg.num_kv_heads, C = ctx->cfg.num_clusters;
   if (L.n_tokens != 0) return fail(ctx, SPIN_ERR_STATE, "cluster prefill must be the first append of (request, layer)");
   if (n > ctx->cfg.max_context_tokens) return fail(ctx, SPIN_ERR_INVALID, "prefill exceeds max_context_tokens");
+  const size_t rows = (size_t)n * H, hc = (size_t)H * C;
+  // 1. token counts of every cluster (and the first entry that is no cluster, if any)
+  const int32_t *tp = token_partition;
+  if (!is_device_ptr(tp)) {
+    CK(cudaMemcpyAsync(ctx->cl_place, tp, rows * 4, cudaMemcpyDefault, st));
+    tp = ctx->cl_place;                                       // the places are written over the clusters they are made from
+  }
+  CK(cudaMemsetAsync(ctx->cl_bad, 0xff, 8, st));
+  CK(cudaMemsetAsync(ctx->cl_count, 0, hc * 4, st));
+  ctx->launches += launch_cluster_count(tp, rows, H, C, ctx->cl_count, ctx->cl_bad, st);
+  std::vector<int32_t> blob(2 + hc);
+  CK(cudaMemcpyAsync(blob.data(), ctx->cl_bad, blob.size() * 4, cudaMemcpyDeviceToHost, st));
   CK(cudaStreamSynchronize(st));
-  // partition specification on the host
-  std::vector<int32_t> tp((size_t)n * H);
-  CK(cudaMemcpy(tp.data(), token_partition, tp.size() * 4, cudaMemcpyDefault));
-  std::vector<int32_t> count((size_t)H * C, 0);
-  for (int64_t t = 0; t < n; ++t)
-    for (int h = 0; h < H; ++h) {
-      const int32_t c = tp[(size_t)t * H + h];
-      if (c < 0 || c >= C) return fail(ctx, SPIN_ERR_INVALID, "token_partition[%lld][%d] = %d out of range", (long long)t, h, c);
-      ++count[(size_t)h * C + c];
-    }
+  uint64_t bad;
+  memcpy(&bad, blob.data(), 8);
+  if (bad != ~0ull) {
+    int32_t c = 0;
+    CK(cudaMemcpy(&c, token_partition + bad, 4, cudaMemcpyDefault));
+    return fail(ctx, SPIN_ERR_INVALID, "token_partition[%lld][%d] = %d out of range", (long long)(bad / H), (int)(bad % H), c);
+  }
+  const int32_t *count = blob.data() + 2;
   int64_t pages_needed = 0;
-  for (size_t i = 0; i < count.size(); ++i) pages_needed += (count[i] + kPageTokens - 1) / kPageTokens;
+  for (size_t i = 0; i < hc; ++i) pages_needed += (count[i] + kPageTokens - 1) / kPageTokens;
   if (ctx->host_page_pool.available() < pages_needed) return fail(ctx, SPIN_ERR_OOM_HOST, "out of host pages");
-  std::vector<int32_t> first_row_page((size_t)H * C);       // CPU-page-table offset of each cluster
-  std::vector<MetaEntry> meta((size_t)C);
+  // 2. the sets' pages, clusters in order, each one's pages together
+  std::vector<int32_t> base(hc);                              // CPU-page-table offset of each cluster
   int32_t total_pages_max = 0;
   for (int h = 0; h < H; ++h) {
     const int set = set_index(d, req, layer, h);
     SetHost &S = ctx->sets[(size_t)set];
+    const int32_t *cnt = count + (size_t)h * C;
     int32_t off = 0;
-    for (int c = 0; c < C; ++c) {
-      const int32_t m = count[(size_t)h * C + c], npg = (m + kPageTokens - 1) / kPageTokens;
-      first_row_page[(size_t)h * C + c] = off;
-      meta[(size_t)c] = MetaEntry{m, 0};
-      int seg = ensure_seg(ctx, ctx->off_segs, S.dir_off, d.dir_off + (size_t)set * g.dir_part, c, g.seg_shift);
+    for (int c0 = 0; c0 < C; c0 += g.seg) {
+      const int seg = ensure_seg(ctx, ctx->off_segs, S.dir_off, d.dir_off + (size_t)set * g.dir_part, c0, g.seg_shift);
       if (seg < 0) return fail(ctx, SPIN_ERR_OOM_HOST, "out of Partition Offset segments");
-      ctx->h_off_pool[((size_t)seg << g.seg_shift) + (c & (g.seg - 1))] = off;
-      if (ensure_seg(ctx, ctx->meta_segs, S.dir_meta, d.dir_meta + (size_t)set * g.dir_part, c, g.seg_shift) < 0)
+      if (ensure_seg(ctx, ctx->meta_segs, S.dir_meta, d.dir_meta + (size_t)set * g.dir_part, c0, g.seg_shift) < 0)
         return fail(ctx, SPIN_ERR_OOM_DEVICE, "out of Meta-partition segments");
-      if (ensure_seg(ctx, ctx->sum_segs, S.dir_sum, d.dir_sumseg + (size_t)set * g.dir_sum, c, g.sum_shift) < 0)
-        return fail(ctx, SPIN_ERR_OOM_DEVICE, "out of summary segments");
-      for (int i = 0; i < npg; ++i) {
-        const int64_t j = off + i;
-        int cs = ensure_seg(ctx, ctx->cpt_segs, S.dir_cpt, d.dir_cpt + (size_t)set * g.dir_page, j, g.seg_shift);
-        if (cs < 0) return fail(ctx, SPIN_ERR_OOM_HOST, "out of CPU page table segments");
-        const int64_t hp = ctx->host_page_pool.alloc();
-        ctx->h_cpt_pool[((size_t)cs << g.seg_shift) + (j & (g.seg - 1))] = (int32_t)hp;
-        S.host_pages.push_back((int32_t)hp);
+      int32_t *h_off = ctx->h_off_pool + ((size_t)seg << g.seg_shift);
+      for (int c = c0; c < std::min(C, c0 + g.seg); ++c) {
+        base[(size_t)h * C + c] = off;
+        h_off[c - c0] = off;
+        off += (cnt[c] + kPageTokens - 1) / kPageTokens;
       }
-      off += npg;
+    }
+    for (int c0 = 0; c0 < C; c0 += g.sum_entries)
+      if (ensure_seg(ctx, ctx->sum_segs, S.dir_sum, d.dir_sumseg + (size_t)set * g.dir_sum, c0, g.sum_shift) < 0)
+        return fail(ctx, SPIN_ERR_OOM_DEVICE, "out of summary segments");
+    for (int32_t j = 0; j < off;) {
+      const int32_t end = std::min<int32_t>(off, ((j >> g.seg_shift) + 1) << g.seg_shift);
+      const int cs = ensure_seg(ctx, ctx->cpt_segs, S.dir_cpt, d.dir_cpt + (size_t)set * g.dir_page, j, g.seg_shift);
+      if (cs < 0) return fail(ctx, SPIN_ERR_OOM_HOST, "out of CPU page table segments");
+      int32_t *cpt = ctx->h_cpt_pool + ((size_t)cs << g.seg_shift);
+      for (; j < end; ++j) {
+        const int32_t hp = (int32_t)ctx->host_page_pool.alloc();
+        cpt[j & (g.seg - 1)] = hp;
+        S.host_pages.push_back(hp);
+      }
     }
     total_pages_max = std::max(total_pages_max, off);
-    S.cl_tokens.assign(count.begin() + (size_t)h * C, count.begin() + (size_t)(h + 1) * C);
-    // Meta-partition entries, segment by segment
-    for (int c0 = 0; c0 < C; c0 += g.seg) {
-      const int cnt = std::min(g.seg, C - c0);
-      CK(cudaMemcpyAsync(d.meta_pool + ((size_t)S.dir_meta[(size_t)(c0 >> g.seg_shift)] << g.seg_shift),
-                         meta.data() + c0, (size_t)cnt * sizeof(MetaEntry), cudaMemcpyHostToDevice, st));
-      CK(cudaStreamSynchronize(st));
-    }
-    SetState s{};
-    s.n_tokens = (int32_t)n;
-    s.n_partitions = C;
-    s.n_host_pages = off;
-    s.tail_first = off;
-    s.slots = (int32_t)ctx->reqs[(size_t)req].slots;
-    SetState cur{};
-    CK(cudaMemcpy(&cur, d.state + set, sizeof cur, cudaMemcpyDeviceToHost));
-    s.step = cur.step;
-    CK(cudaMemcpy(d.state + set, &s, sizeof s, cudaMemcpyHostToDevice));
+    S.cl_tokens.assign(cnt, cnt + C);
   }
   // all heads of a (request, layer) share one tail position: use the largest page count so
   // that tail pages never collide with cluster pages of any head
-  for (int h = 0; h < H; ++h) {
-    const int set = set_index(d, req, layer, h);
-    SetHost &S = ctx->sets[(size_t)set];
-    while ((int32_t)S.host_pages.size() < total_pages_max) S.host_pages.push_back(-1);
-    SetState s{};
-    CK(cudaMemcpy(&s, d.state + set, sizeof s, cudaMemcpyDeviceToHost));
-    s.tail_first = total_pages_max;
-    s.n_host_pages = total_pages_max;
-    CK(cudaMemcpy(d.state + set, &s, sizeof s, cudaMemcpyHostToDevice));
-  }
-  // the decode kernels read the two host tables through their HBM mirror
-  if (d.off_mirror) {
-    for (int h = 0; h < H; ++h) {
-      const SetHost &S = set_of(ctx, req, layer, h);
-      for (int32_t seg : S.dir_off)
-        if (seg >= 0) CK(cudaMemcpyAsync(d.off_mirror + ((size_t)seg << g.seg_shift), ctx->h_off_pool + ((size_t)seg << g.seg_shift), (size_t)g.seg * 4, cudaMemcpyHostToDevice, st));
-      for (int32_t seg : S.dir_cpt)
-        if (seg >= 0) CK(cudaMemcpyAsync(d.cpt_mirror + ((size_t)seg << g.seg_shift), ctx->h_cpt_pool + ((size_t)seg << g.seg_shift), (size_t)g.seg * 4, cudaMemcpyHostToDevice, st));
-    }
-  }
-  // destination row of every (token, head): clusters keep their tokens in arrival order
-  std::vector<int32_t> filled((size_t)H * C, 0);
-  std::vector<int64_t> dest((size_t)n * H);
-  for (int64_t t = 0; t < n; ++t)
-    for (int h = 0; h < H; ++h) {
-      const int32_t c = tp[(size_t)t * H + h];
-      const int32_t r = filled[(size_t)h * C + c]++;
-      const SetHost &S = set_of(ctx, req, layer, h);
-      const int32_t hp = S.host_pages[(size_t)(first_row_page[(size_t)h * C + c] + r / kPageTokens)];
-      dest[(size_t)t * H + h] = (int64_t)hp * kPageTokens + r % kPageTokens;
-    }
+  for (int h = 0; h < H; ++h) set_of(ctx, req, layer, h).host_pages.resize((size_t)total_pages_max, -1);
   flush_dirs(ctx, st);
-  // centroids -> summary segments
+  // 3. tables, places, centroids
+  CK(cudaMemcpyAsync(ctx->cl_base, base.data(), hc * 4, cudaMemcpyHostToDevice, st));
+  ctx->launches += launch_cluster_tables(d, req, layer, C, total_pages_max, (int)n, ctx->cl_count, (int)ctx->reqs[(size_t)req].slots, st);
+  ctx->launches += launch_cluster_place(tp, n, H, C, ctx->cl_base, ctx->cl_run, ctx->cl_place, st);
   const __nv_bfloat16 *cen = reinterpret_cast<const __nv_bfloat16 *>(centroids);
   void *cen_tmp = nullptr;
   if (!is_device_ptr(centroids)) {
@@ -657,22 +644,14 @@ int prefill_clustered_impl(spin_ctx *ctx, int req, int layer, const void *k, con
     cen = reinterpret_cast<const __nv_bfloat16 *>(cen_tmp);
   }
   ctx->launches += launch_copy_centroids(d, req, layer, cen, C, st);
+  // 4. rows to their pages
   const bool dev_kv = is_device_ptr(k);
+  const __nv_bfloat16 *kd = reinterpret_cast<const __nv_bfloat16 *>(k), *vd = reinterpret_cast<const __nv_bfloat16 *>(v);
   if (dev_kv && ctx->offload_slot_units > 0) {
     // Asynchronous offload (Section 4.1): the rows are packed into pages in HBM staging slots on
     // the caller's stream, at HBM speed, range by range of the sets' logical pages; each slot
     // then moves to host memory by copy-engine transfers (one per run of consecutive host
     // pages) on the library's stream, behind this call.
-    std::vector<int32_t> lrow((size_t)n * H);
-    std::fill(filled.begin(), filled.end(), 0);
-    for (int64_t t = 0; t < n; ++t)
-      for (int h = 0; h < H; ++h) {
-        const int32_t c = tp[(size_t)t * H + h];
-        const int32_t r = filled[(size_t)h * C + c]++;
-        lrow[(size_t)t * H + h] = (first_row_page[(size_t)h * C + c] + r / kPageTokens) * kPageTokens + r % kPageTokens;
-      }
-    int32_t *d_lrow = ctx->offload_lrow;                    // this call ends with the stream idle: no earlier prefill still reads it
-    CK(cudaMemcpyAsync(d_lrow, lrow.data(), lrow.size() * 4, cudaMemcpyHostToDevice, st));
     const int64_t per = ctx->offload_slot_units / H;
     for (int64_t p0 = 0; p0 < total_pages_max; p0 += per) {
       const int m = (int)std::min<int64_t>(per, total_pages_max - p0), slot = ctx->offload_next;
@@ -680,8 +659,7 @@ int prefill_clustered_impl(spin_ctx *ctx, int req, int layer, const void *k, con
       if (ctx->slot_used[slot]) CK(cudaStreamWaitEvent(st, ctx->ev_done[slot], 0));     // ring full: wait for the drain
       uint8_t *stage = ctx->offload_stage + (size_t)slot * ctx->offload_slot_units * kPageBytes;
       CK(cudaMemsetAsync(stage, 0, (size_t)H * m * kPageBytes, st));                   // rows past a cluster's last token stay zero
-      ctx->launches += launch_cluster_scatter_staged(d, reinterpret_cast<const __nv_bfloat16 *>(k),
-                                                     reinterpret_cast<const __nv_bfloat16 *>(v), d_lrow, (int)n, (int)p0, m, stage, st);
+      ctx->launches += launch_cluster_scatter_staged(d, kd, vd, ctx->cl_place, (int)n, (int)p0, m, stage, st);
       CK(cudaEventRecord(ctx->ev_staged[slot], st));
       CK(cudaStreamWaitEvent(ctx->offload_stream, ctx->ev_staged[slot], 0));
       for (int h = 0; h < H; ++h) {
@@ -701,26 +679,21 @@ int prefill_clustered_impl(spin_ctx *ctx, int req, int layer, const void *k, con
       ctx->offload_last = slot;
       ++ctx->offload_gen;
     }
-    CK(cudaStreamSynchronize(st));          // the host-side sources of this call's copies end here; the drain goes on
+  } else if (dev_kv) {
+    ctx->launches += launch_cluster_scatter(d, req, layer, kd, vd, ctx->cl_place, n, st);
   } else {
-  // rows -> host pages, in chunks through the staging buffers
-  const int64_t chunk = g.stage_tokens;
-  for (int64_t t0 = 0; t0 < n; t0 += chunk) {
-    const int64_t m = std::min(chunk, n - t0);
-    const size_t rows = (size_t)m * H;
-    const __nv_bfloat16 *kk = reinterpret_cast<const __nv_bfloat16 *>(k) + (size_t)t0 * H * kHeadDim;
-    const __nv_bfloat16 *vv = reinterpret_cast<const __nv_bfloat16 *>(v) + (size_t)t0 * H * kHeadDim;
-    if (!dev_kv) {
-      CK(cudaMemcpyAsync(ctx->stage_k, kk, rows * kRowBytes, cudaMemcpyHostToDevice, st));
-      CK(cudaMemcpyAsync(ctx->stage_v, vv, rows * kRowBytes, cudaMemcpyHostToDevice, st));
-      kk = ctx->stage_k;
-      vv = ctx->stage_v;
+    // host rows come in through the staging buffers, chunk by chunk
+    const int64_t chunk = g.stage_tokens;
+    for (int64_t t0 = 0; t0 < n; t0 += chunk) {
+      const int64_t m = std::min(chunk, n - t0);
+      const size_t at = (size_t)t0 * H * kHeadDim, bytes = (size_t)m * H * kRowBytes;
+      CK(cudaMemcpyAsync(ctx->stage_k, kd + at, bytes, cudaMemcpyHostToDevice, st));
+      CK(cudaMemcpyAsync(ctx->stage_v, vd + at, bytes, cudaMemcpyHostToDevice, st));
+      ctx->launches += launch_cluster_scatter(d, req, layer, ctx->stage_k, ctx->stage_v, ctx->cl_place + (size_t)t0 * H, m, st);
+      CK(cudaStreamSynchronize(st));
     }
-    CK(cudaMemcpyAsync(ctx->stage_dest, dest.data() + (size_t)t0 * H, rows * 8, cudaMemcpyHostToDevice, st));
-    ctx->launches += launch_cluster_scatter(d, req, layer, kk, vv, ctx->stage_dest, (int)m, st);
-    CK(cudaStreamSynchronize(st));
   }
-  }
+  CK(cudaStreamSynchronize(st));            // the prefill form synchronises: its scratch is free again (a drain goes on)
   if (cen_tmp) CK(cudaFree(cen_tmp));
   CK(cudaGetLastError());
   L.n_tokens = n;

@@ -56,33 +56,119 @@ k_append_edge(DevCtx c, AppendEdgeArgs a, const __nv_bfloat16 *__restrict__ k,
   append_edge_body(c, set_index(c, a.req[i], a.layer, head), i, head, k, v, n_new, a.n_tokens[i], -1, krows);
 }
 
-// Cluster prefill: row `tok` of head `h` goes to row dest[tok][h] of the host tier (page id *
-// 16 + row), where the host runtime has packed each cluster's tokens in their original order.
+// ---- cluster prefill ------------------------------------------------------------------------
+// token_partition [n_tokens][Hkv] -> tokens per (head, cluster); bad = the first entry that names no
+// cluster (all ones if none does).
 __global__ void __launch_bounds__(256)
-k_cluster_scatter(DevCtx c, const __nv_bfloat16 *__restrict__ k, const __nv_bfloat16 *__restrict__ v,
-                  const int64_t *__restrict__ dest, int n_tokens) {
+k_cluster_count(const int32_t *__restrict__ tp, size_t rows, int H, int C, int32_t *__restrict__ count, unsigned long long *bad) {
+  for (size_t i = (size_t)blockIdx.x * 256 + threadIdx.x; i < rows; i += (size_t)gridDim.x * 256) {
+    const int32_t cl = tp[i];
+    if (cl < 0 || cl >= C) atomicMin(bad, (unsigned long long)i);
+    else atomicAdd(count + (size_t)(i % H) * C + cl, 1);
+  }
+}
+
+// A row's place in its set's logical page order: (first page of its cluster) * 16 + its rank among
+// the cluster's tokens (arrival order).  One CTA per kv head, a warp per run of consecutive tokens
+// with counters of its own in shared memory: count, prefix over the warps, then 32 tokens at a
+// time, the lanes of a cluster ranked by match_any.  Where even one warp's counters exceed shared
+// memory a single warp counts in `run` (global).  tp and place may be the same array: an entry is
+// read by the thread that overwrites it, after every count has been taken.
+// Latency-bound (a warp's steps follow one another): ~30 us for 32768 tokens and 512 clusters,
+// beside 2.6 ms for their rows on the host link.
+constexpr int kPlaceWarps = 16, kPlaceSmem = 160 * 1024;
+__global__ void __launch_bounds__(kPlaceWarps * 32)
+k_cluster_place(const int32_t *tp, int64_t n, int H, int C, const int32_t *__restrict__ base, int32_t *__restrict__ run,
+                int n_warps, int in_smem, int32_t *place) {
+  extern __shared__ int32_t s_run[];
+  const int head = blockIdx.x, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  int32_t *cnt = in_smem ? s_run + (size_t)warp * C : run + (size_t)head * C;
+  const int64_t per = (n + n_warps - 1) / n_warps, lo = warp < n_warps ? min(n, warp * per) : n, hi = warp < n_warps ? min(n, lo + per) : n;
+  const int32_t *mine = tp + head;
+  if (in_smem) {
+    for (int c = threadIdx.x; c < n_warps * C; c += blockDim.x) s_run[c] = 0;
+    __syncthreads();
+#pragma unroll 4
+    for (int64_t t = lo + lane; t < hi; t += 32) atomicAdd(cnt + mine[(size_t)t * H], 1);
+    __syncthreads();
+    for (int c = threadIdx.x; c < C; c += blockDim.x) {
+      int32_t sum = 0;
+      for (int w = 0; w < n_warps; ++w) { const int32_t x = s_run[(size_t)w * C + c]; s_run[(size_t)w * C + c] = sum; sum += x; }
+    }
+    __syncthreads();
+  } else {
+    for (int c = threadIdx.x; c < C; c += blockDim.x) cnt[c] = 0;
+    __syncthreads();
+    if (warp >= n_warps) return;
+  }
+  int64_t t = lo + lane;
+  int cl = t < hi ? mine[(size_t)t * H] : -1;
+#pragma unroll 1
+  for (int64_t t0 = lo; t0 < hi; t0 += 32) {
+    const int64_t t_next = t + 32;
+    const int cl_next = t_next < hi ? mine[(size_t)t_next * H] : -1;       // in flight while these 32 are ranked
+    const uint32_t same = __match_any_sync(0xffffffffu, cl);
+    const int32_t seen = cl >= 0 ? cnt[cl] : 0;
+    __syncwarp();
+    if (cl >= 0) {
+      place[(size_t)t * H + head] = base[(size_t)head * C + cl] * kPageTokens + seen + __popc(same & ((1u << lane) - 1u));
+      if ((same >> lane) == 1u) cnt[cl] = seen + __popc(same);             // the cluster's last lane
+    }
+    __syncwarp();
+    t = t_next;
+    cl = cl_next;
+  }
+}
+
+// What follows from the layout, for every kv head's set: Meta-partition entries, the HBM copies of
+// the Partition Offset and CPU page tables (read from the pinned originals) and the set's scalars.
+__global__ void __launch_bounds__(256)
+k_cluster_tables(DevCtx c, int req, int layer, int C, int n_pages, int n_tokens, const int32_t *__restrict__ count, int slots) {
+  const int head = blockIdx.y, set = set_index(c, req, layer, head), e = blockIdx.x * 256 + threadIdx.x;
+  if (e < C) {
+    MetaEntry *m = meta_at(c, set, e);
+    if (m) *m = MetaEntry{count[(size_t)head * C + e], 0}; else dev_error(c, kErrBounds);
+  }
+  mirror_tables(c, set, e, C, n_pages);
+  if (e == 0) {
+    SetState *s = c.state + set;
+    s->n_tokens = n_tokens;
+    s->n_partitions = C;
+    s->n_host_pages = n_pages;
+    s->tail_first = n_pages;
+    s->tail_pages = 0;
+    s->tail_len = 0;
+    s->slots = slots;
+  }
+}
+
+// Row (token, head) -> its place in the host tier.
+__global__ void __launch_bounds__(256)
+k_cluster_scatter(DevCtx c, int req, int layer, const __nv_bfloat16 *__restrict__ k, const __nv_bfloat16 *__restrict__ v,
+                  const int32_t *__restrict__ place, size_t rows) {
   const int piece = threadIdx.x & 15;
-  const size_t rows = (size_t)n_tokens * c.Hkv;
   for (size_t row = (size_t)blockIdx.x * 16 + (threadIdx.x >> 4); row < rows; row += (size_t)gridDim.x * 16) {
-    const int64_t d = dest[row];
-    uint8_t *dst = c.host_pages + (size_t)(d >> 4) * kPageBytes + (size_t)(d & 15) * kRowBytes + piece * 16;
+    const int32_t d = place[row];
+    const int32_t *hp = cpt_lookup(c, set_index(c, req, layer, (int)(row % c.Hkv)), d >> 4);
+    const int32_t host_page = hp ? *hp : -1;
+    if (host_page < 0 || host_page >= c.n_host_pages) { if (piece == 0) dev_error(c, kErrBounds); continue; }
+    uint8_t *dst = c.host_pages + (size_t)host_page * kPageBytes + (size_t)(d & 15) * kRowBytes + piece * 16;
     st16(dst, ld16(reinterpret_cast<const uint8_t *>(k) + row * kRowBytes + piece * 16));
     st16(dst + kHalfPageBytes, ld16(reinterpret_cast<const uint8_t *>(v) + row * kRowBytes + piece * 16));
   }
 }
 
-// The same through a staging slot in HBM (asynchronous offload): lrow[token][head] = the row's
-// place in its set's logical page order (CPU-page-table index * 16 + row); the rows whose page
+// The same through a staging slot in HBM (asynchronous offload): the rows whose page
 // lies in [p0, p0 + m) go to the slot, laid out head-major ([head][page - p0], the order in
 // which copy-engine transfers then move the pages to host memory), the others are left for
 // another pass.
 __global__ void __launch_bounds__(256)
 k_cluster_scatter_staged(DevCtx c, const __nv_bfloat16 *__restrict__ k, const __nv_bfloat16 *__restrict__ v,
-                         const int32_t *__restrict__ lrow, int n_tokens, int p0, int m, uint8_t *__restrict__ stage) {
+                         const int32_t *__restrict__ place, int n_tokens, int p0, int m, uint8_t *__restrict__ stage) {
   const int piece = threadIdx.x & 15;
   const size_t rows = (size_t)n_tokens * c.Hkv;
   for (size_t row = (size_t)blockIdx.x * 16 + (threadIdx.x >> 4); row < rows; row += (size_t)gridDim.x * 16) {
-    const int32_t d = lrow[row];
+    const int32_t d = place[row];
     const int lp = d >> 4;
     if (lp < p0 || lp >= p0 + m) continue;
     const int head = (int)(row % c.Hkv);
@@ -168,22 +254,47 @@ int launch_append_edge(const DevCtx &c, const AppendEdgeArgs &a, const __nv_bflo
   return 1;
 }
 
-int launch_cluster_scatter(const DevCtx &c, int req, int layer, const __nv_bfloat16 *k,
-                           const __nv_bfloat16 *v, const int64_t *dest_row, int n_tokens,
-                           cudaStream_t st) {
-  size_t rows = (size_t)n_tokens * c.Hkv;
-  int grid = (int)((rows + 15) / 16 < 148 * 16 ? (rows + 15) / 16 : 148 * 16);
-  if (grid < 1) grid = 1;
-  k_cluster_scatter<<<grid, 256, 0, st>>>(c, k, v, dest_row, n_tokens);
+int launch_cluster_count(const int32_t *tp, size_t rows, int H, int C, int32_t *count, unsigned long long *bad, cudaStream_t st) {
+  const size_t want = (rows + 255) / 256;
+  k_cluster_count<<<(int)(want < 148 * 8 ? want : 148 * 8), 256, 0, st>>>(tp, rows, H, C, count, bad);
   return 1;
 }
 
-int launch_cluster_scatter_staged(const DevCtx &c, const __nv_bfloat16 *k, const __nv_bfloat16 *v, const int32_t *lrow,
+int launch_cluster_place(const int32_t *tp, int64_t n, int H, int C, const int32_t *base, int32_t *run, int32_t *place, cudaStream_t st) {
+  // as many warps as have room for their counters; one, counting in global memory, where none has
+  int warps = kPlaceSmem / 4 / C;
+  const int in_smem = warps >= 1;
+  warps = warps < 1 ? 1 : warps > kPlaceWarps ? kPlaceWarps : warps;
+  const size_t smem = in_smem ? (size_t)warps * C * 4 : 0;
+  static bool configured_dev[kMaxDevices] = {};
+  bool &configured = configured_dev[current_device_slot()];
+  if (!configured) { cudaFuncSetAttribute(k_cluster_place, cudaFuncAttributeMaxDynamicSharedMemorySize, kPlaceSmem); configured = true; }
+  k_cluster_place<<<H, kPlaceWarps * 32, smem, st>>>(tp, n, H, C, base, run, warps, in_smem, place);
+  return 1;
+}
+
+int launch_cluster_tables(const DevCtx &c, int req, int layer, int C, int n_pages, int n_tokens, const int32_t *count, int slots, cudaStream_t st) {
+  const int n = C > n_pages ? C : n_pages;
+  k_cluster_tables<<<dim3((n + 255) / 256, c.Hkv), 256, 0, st>>>(c, req, layer, C, n_pages, n_tokens, count, slots);
+  return 1;
+}
+
+int launch_cluster_scatter(const DevCtx &c, int req, int layer, const __nv_bfloat16 *k,
+                           const __nv_bfloat16 *v, const int32_t *place, int64_t n_tokens,
+                           cudaStream_t st) {
+  const size_t rows = (size_t)n_tokens * c.Hkv;
+  int grid = (int)((rows + 15) / 16 < 148 * 16 ? (rows + 15) / 16 : 148 * 16);
+  if (grid < 1) grid = 1;
+  k_cluster_scatter<<<grid, 256, 0, st>>>(c, req, layer, k, v, place, rows);
+  return 1;
+}
+
+int launch_cluster_scatter_staged(const DevCtx &c, const __nv_bfloat16 *k, const __nv_bfloat16 *v, const int32_t *place,
                                   int n_tokens, int p0, int m, uint8_t *stage, cudaStream_t st) {
   size_t rows = (size_t)n_tokens * c.Hkv;
   int grid = (int)((rows + 15) / 16 < 148 * 16 ? (rows + 15) / 16 : 148 * 16);
   if (grid < 1) grid = 1;
-  k_cluster_scatter_staged<<<grid, 256, 0, st>>>(c, k, v, lrow, n_tokens, p0, m, stage);
+  k_cluster_scatter_staged<<<grid, 256, 0, st>>>(c, k, v, place, n_tokens, p0, m, stage);
   return 1;
 }
 

@@ -200,6 +200,12 @@ __device__ __forceinline__ void cpt_mirror_set(const DevCtx &c, int set, int i, 
   int seg = c.dir_cpt[(size_t)set * c.dir_page + (i >> c.seg_shift)];
   if (seg >= 0) c.cpt_mirror[((size_t)seg << c.seg_shift) + (i & ((1 << c.seg_shift) - 1))] = v;
 }
+// Entry e of both host tables of a set -> their HBM copies.
+__device__ __forceinline__ void mirror_tables(const DevCtx &c, int set, int e, int n_part, int n_pages) {
+  if (!c.off_mirror) return;
+  if (e < n_part) { const int32_t *o = off_at(c, set, e); if (o) off_mirror_set(c, set, e, *o); }
+  if (e < n_pages) { const int32_t *p = cpt_at(c, set, e); if (p) cpt_mirror_set(c, set, e, *p); }
+}
 __device__ __forceinline__ uint8_t *summary_at(const DevCtx &c, int set, int e) {
   int seg = c.dir_sumseg[(size_t)set * c.dir_sum + (e >> c.sum_shift)];
   return seg < 0 ? nullptr
@@ -342,10 +348,12 @@ int launch_append_bulk(const DevCtx &c, int req, int layer, const __nv_bfloat16 
                        cudaStream_t st, Prof *prof, uint8_t *stage = nullptr, const int32_t *stage_hp = nullptr);
 int launch_append_edge(const DevCtx &c, const AppendEdgeArgs &a, const __nv_bfloat16 *k,
                        const __nv_bfloat16 *v, int n_new, cudaStream_t st, Prof *prof);
-int launch_cluster_scatter(const DevCtx &c, int req, int layer, const __nv_bfloat16 *k,
-                           const __nv_bfloat16 *v, const int64_t *dest_row, int n_tokens,
-                           cudaStream_t st);
-int launch_cluster_scatter_staged(const DevCtx &c, const __nv_bfloat16 *k, const __nv_bfloat16 *v, const int32_t *lrow,
+int launch_cluster_count(const int32_t *tp, size_t rows, int H, int C, int32_t *count, unsigned long long *bad, cudaStream_t st);
+int launch_cluster_place(const int32_t *tp, int64_t n, int H, int C, const int32_t *base, int32_t *run, int32_t *place, cudaStream_t st);
+int launch_cluster_tables(const DevCtx &c, int req, int layer, int C, int n_pages, int n_tokens, const int32_t *count, int slots, cudaStream_t st);
+int launch_cluster_scatter(const DevCtx &c, int req, int layer, const __nv_bfloat16 *k, const __nv_bfloat16 *v,
+                           const int32_t *place, int64_t n_tokens, cudaStream_t st);
+int launch_cluster_scatter_staged(const DevCtx &c, const __nv_bfloat16 *k, const __nv_bfloat16 *v, const int32_t *place,
                                   int n_tokens, int p0, int m, uint8_t *stage, cudaStream_t st);
 int launch_stage_in(void *dq, const void *sq, size_t q_bytes, void *dk, const void *sk, void *dv, const void *sv,
                     size_t kv_bytes, cudaStream_t st);
