@@ -1005,87 +1005,84 @@ static int reindex_impl(spin_ctx *ctx, int32_t req, int32_t layer, void *cuda_st
     }
   }
   if (ctx->host_page_pool.available() < need) return fail(ctx, SPIN_ERR_OOM_HOST, "out of host pages");
+  const size_t stage_bytes = (size_t)std::max<int64_t>(g.stage_tokens, ctx->cfg.max_requests) * H * kRowBytes;
+  if ((size_t)H * (C + (C + 31) / 32) * 4 > stage_bytes) return fail(ctx, SPIN_ERR_INVALID, "too many clusters for the staging buffer");
+  // 3. The sets' Partition Offset and CPU page tables: clusters in order, each one's pages together,
+  // what is left of the tail behind the longest head's clusters.  A head's page list is the old one
+  // with the new pages put in behind their clusters' last ones: runs between them are copied whole.
+  const int n_rem = L.tail_pages - n_full;
   std::vector<int64_t> dest((size_t)n_tok * H);
-  std::vector<int32_t> new_tokens((size_t)H * C);
-  const int words = (C + 31) / 32;
-  std::vector<uint32_t> touched((size_t)H * words, 0u);
-  std::vector<std::vector<int32_t>> old_tail((size_t)H);
-  std::vector<std::vector<std::vector<int32_t>>> lists((size_t)H);
+  std::vector<std::vector<int32_t>> pages((size_t)H), tails((size_t)H);
+  std::vector<std::vector<std::pair<int32_t, int32_t>>> grown((size_t)H);      // (cluster, new pages), clusters ascending
   int32_t total_max = 0;
   for (int h = 0; h < H; ++h) {
     SetHost &S = set_of(ctx, req, layer, h);
-    for (int i = 0; i < L.tail_pages; ++i) old_tail[(size_t)h].push_back(S.host_pages[(size_t)(L.tail_first + i)]);
-    auto &ls = lists[(size_t)h];
-    ls.resize((size_t)C);
-    for (int c = 0; c < C; ++c) {
-      const int32_t seg = S.dir_off[(size_t)(c >> g.seg_shift)];
-      const int32_t off = ctx->h_off_pool[((size_t)seg << g.seg_shift) + (c & (g.seg - 1))];
-      const int npg = (S.cl_tokens[(size_t)c] + kPageTokens - 1) / kPageTokens;
-      ls[(size_t)c].assign(S.host_pages.begin() + off, S.host_pages.begin() + off + npg);
+    auto off_of = [&](int c) { return ctx->h_off_pool[((size_t)S.dir_off[(size_t)(c >> g.seg_shift)] << g.seg_shift) + (c & (g.seg - 1))]; };
+    auto npages = [](int32_t m) { return (m + kPageTokens - 1) / kPageTokens; };
+    tails[(size_t)h].assign(S.host_pages.begin() + L.tail_first, S.host_pages.begin() + L.tail_first + L.tail_pages);
+    // tokens by cluster, arrival order within a cluster
+    std::vector<std::pair<int32_t, int32_t>> by((size_t)n_tok);
+    for (int t = 0; t < n_tok; ++t) by[(size_t)t] = {assign[(size_t)t * H + h], t};
+    std::sort(by.begin(), by.end());
+    auto &out = pages[(size_t)h];
+    int32_t from = 0;                                          // old entries taken over so far
+    for (size_t i = 0; i < by.size();) {
+      const int32_t c = by[i].first, off = off_of(c), had = npages(S.cl_tokens[(size_t)c]);
+      out.insert(out.end(), S.host_pages.begin() + from, S.host_pages.begin() + off + had);
+      from = off + had;
+      const size_t first = out.size() - (size_t)had;           // the cluster's pages in the new list
+      int32_t m = S.cl_tokens[(size_t)c];
+      for (; i < by.size() && by[i].first == c; ++i, ++m) {
+        if (m % kPageTokens == 0) out.push_back((int32_t)ctx->host_page_pool.alloc());
+        dest[(size_t)by[i].second * H + h] = (int64_t)out[first + (size_t)(m / kPageTokens)] * kPageTokens + m % kPageTokens;
+      }
+      S.cl_tokens[(size_t)c] = m;
+      if (npages(m) > had) grown[(size_t)h].push_back({c, npages(m) - had});
     }
-    for (int t = 0; t < n_tok; ++t) {
-      const int32_t c = assign[(size_t)t * H + h];
-      const int32_t m = S.cl_tokens[(size_t)c];
-      if (m % kPageTokens == 0) ls[(size_t)c].push_back((int32_t)ctx->host_page_pool.alloc());
-      dest[(size_t)t * H + h] = (int64_t)ls[(size_t)c][(size_t)(m / kPageTokens)] * kPageTokens + m % kPageTokens;
-      S.cl_tokens[(size_t)c] = m + 1;
-      touched[(size_t)h * words + (c >> 5)] |= 1u << (c & 31);
-    }
-    int32_t total = 0;
-    for (int c = 0; c < C; ++c) total += (int32_t)ls[(size_t)c].size();
-    total_max = std::max(total_max, total);
-    std::copy(S.cl_tokens.begin(), S.cl_tokens.end(), new_tokens.begin() + (size_t)h * C);
+    // the rest of the old list ends with the last cluster, whose old page count the list's own growth gives
+    int32_t last_npg = npages(S.cl_tokens[(size_t)C - 1]);
+    if (!grown[(size_t)h].empty() && grown[(size_t)h].back().first == C - 1) last_npg -= grown[(size_t)h].back().second;
+    out.insert(out.end(), S.host_pages.begin() + from, S.host_pages.begin() + off_of(C - 1) + last_npg);
+    total_max = std::max(total_max, (int32_t)out.size());
   }
-
-  // 3. the sets' Partition Offset and CPU page tables laid out afresh (clusters in order, each
-  //    one's pages together), what is left of the tail behind the longest head's clusters
-  const int n_rem = L.tail_pages - n_full;
   if ((int64_t)total_max + g.tail_cap > (int64_t)g.dir_page * g.seg)
     return fail(ctx, SPIN_ERR_INVALID, "request %d outgrew its CPU page table", req);
   for (int h = 0; h < H; ++h) {
     const int set = set_index(d, req, layer, h);
     SetHost &S = ctx->sets[(size_t)set];
-    S.host_pages.assign((size_t)(total_max + n_rem), -1);
-    auto put = [&](int64_t j, int32_t hp) -> bool {
-      const int cs = ensure_seg(ctx, ctx->cpt_segs, S.dir_cpt, d.dir_cpt + (size_t)set * g.dir_page, j, g.seg_shift);
-      if (cs < 0) return false;
-      ctx->h_cpt_pool[((size_t)cs << g.seg_shift) + (j & (g.seg - 1))] = hp;
-      S.host_pages[(size_t)j] = hp;
+    // entries from `lo` on: into the pinned table, segment by segment
+    auto put = [&](const int32_t *src, int32_t lo, int32_t hi) -> bool {
+      for (int32_t j = lo; j < hi;) {
+        const int32_t end = std::min<int32_t>(hi, ((j >> g.seg_shift) + 1) << g.seg_shift);
+        const int cs = ensure_seg(ctx, ctx->cpt_segs, S.dir_cpt, d.dir_cpt + (size_t)set * g.dir_page, j, g.seg_shift);
+        if (cs < 0) return false;
+        memcpy(ctx->h_cpt_pool + ((size_t)cs << g.seg_shift) + (j & (g.seg - 1)), src + (j - lo), (size_t)(end - j) * 4);
+        j = end;
+      }
       return true;
     };
-    int32_t off = 0;
-    for (int c = 0; c < C; ++c) {
-      const int32_t seg = S.dir_off[(size_t)(c >> g.seg_shift)];
-      ctx->h_off_pool[((size_t)seg << g.seg_shift) + (c & (g.seg - 1))] = off;
-      for (int32_t hp : lists[(size_t)h][(size_t)c])
-        if (!put(off++, hp)) return fail(ctx, SPIN_ERR_OOM_HOST, "out of CPU page table segments");
+    auto &list = pages[(size_t)h];
+    const int32_t own = (int32_t)list.size();
+    int32_t add = 0;                                           // offsets move behind the first cluster that has grown
+    for (size_t i = 0; i < grown[(size_t)h].size(); ++i) {
+      add += grown[(size_t)h][i].second;
+      const int32_t c_end = i + 1 < grown[(size_t)h].size() ? grown[(size_t)h][i + 1].first + 1 : C;
+      for (int32_t c = grown[(size_t)h][i].first + 1; c < c_end; ++c) ctx->h_off_pool[((size_t)S.dir_off[(size_t)(c >> g.seg_shift)] << g.seg_shift) + (c & (g.seg - 1))] += add;
     }
-    for (int i = 0; i < n_rem; ++i)
-      if (!put((int64_t)total_max + i, old_tail[(size_t)h][(size_t)(n_full + i)])) return fail(ctx, SPIN_ERR_OOM_HOST, "out of CPU page table segments");
-    for (int i = 0; i < n_full; ++i) ctx->host_page_pool.release(old_tail[(size_t)h][(size_t)i]);   // their rows live in the clusters now
+    list.resize((size_t)total_max, -1);
+    for (int i = 0; i < n_rem; ++i) list.push_back(tails[(size_t)h][(size_t)(n_full + i)]);
+    if (!put(list.data(), 0, own) || !put(list.data() + total_max, total_max, total_max + n_rem))
+      return fail(ctx, SPIN_ERR_OOM_HOST, "out of CPU page table segments");
+    S.host_pages.swap(list);
+    for (int i = 0; i < n_full; ++i) ctx->host_page_pool.release(tails[(size_t)h][(size_t)i]);   // their rows live in the clusters now
   }
 
   // 4. device side: rows to their places; counts, residency and tail; the tables' HBM copies
-  int32_t *d_new_tokens = reinterpret_cast<int32_t *>(ctx->stage_v);
-  uint32_t *d_touched = reinterpret_cast<uint32_t *>(d_new_tokens + new_tokens.size());
-  const size_t stage_bytes = (size_t)std::max<int64_t>(g.stage_tokens, ctx->cfg.max_requests) * H * kRowBytes;
-  if ((new_tokens.size() + touched.size()) * 4 > stage_bytes) return fail(ctx, SPIN_ERR_INVALID, "too many clusters for the staging buffer");
   CK(cudaMemcpyAsync(ctx->stage_dest, dest.data(), dest.size() * 8, cudaMemcpyHostToDevice, st));
-  CK(cudaMemcpyAsync(d_new_tokens, new_tokens.data(), new_tokens.size() * 4, cudaMemcpyHostToDevice, st));
-  CK(cudaMemcpyAsync(d_touched, touched.data(), touched.size() * 4, cudaMemcpyHostToDevice, st));
   flush_dirs(ctx, st);
   ctx->launches += launch_move_rows(d, req, layer, ctx->stage_dest, n_tok, st);
   ctx->launches += launch_reindex_apply(d, req, layer, C, n_full, total_max, n_rem, n_rem ? L.tail_len : 0,
-                                        total_max + n_rem, d_new_tokens, d_touched, st);
-  if (d.off_mirror) {
-    for (int h = 0; h < H; ++h) {
-      const SetHost &S = set_of(ctx, req, layer, h);
-      for (int32_t seg : S.dir_off)
-        if (seg >= 0) CK(cudaMemcpyAsync(d.off_mirror + ((size_t)seg << g.seg_shift), ctx->h_off_pool + ((size_t)seg << g.seg_shift), (size_t)g.seg * 4, cudaMemcpyHostToDevice, st));
-      for (int32_t seg : S.dir_cpt)
-        if (seg >= 0) CK(cudaMemcpyAsync(d.cpt_mirror + ((size_t)seg << g.seg_shift), ctx->h_cpt_pool + ((size_t)seg << g.seg_shift), (size_t)g.seg * 4, cudaMemcpyHostToDevice, st));
-    }
-  }
+                                        total_max + n_rem, d_assign, st);
   L.tail_first = total_max;
   L.tail_pages = n_rem;
   if (n_rem == 0) L.tail_len = 0;

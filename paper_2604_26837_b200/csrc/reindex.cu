@@ -9,7 +9,9 @@
 //   k_move_rows      K/V rows from the HBM tail pages to their rows in pinned host memory
 //   k_reindex_apply  new token counts in the Meta-partition table; a cluster that took a
 //                    token loses its (stale) GPU residency: flag and slots cleared; the tail
-//                    shrinks to the partly filled newest page
+//                    shrinks to the partly filled newest page; the HBM copies of the two host
+//                    tables are read afresh from the pinned originals (a request of 131072 tokens
+//                    has some 320 segments of them: one copy each was half of a 1.9 ms call)
 #define SPIN_FILE_ID 5
 #include "spin_dev.cuh"
 
@@ -43,20 +45,34 @@ k_assign(DevCtx c, int req, int layer, int n_clusters, int32_t *__restrict__ ass
   unpack8(*reinterpret_cast<const uint4 *>(krow + lane16 * 16), kf);
   float best = -INFINITY;
   int arg = 0x7fffffff;
-  for (int cl = grp; cl < n_clusters; cl += 16) {
-    const uint8_t *srow = summary_at(c, set, cl);
-    if (!srow) { if (lane16 == 0) dev_error(c, kErrBounds); continue; }
-    float x[8];
-    unpack8(*reinterpret_cast<const uint4 *>(srow + lane16 * 16), x);
-    float s = kf[0] * x[0];
+  // kU centroids at a time: their directory entries, then their rows, are in flight together
+  constexpr int kU = 8;
+#pragma unroll 1
+  for (int c0 = grp; c0 < n_clusters; c0 += 16 * kU) {
+    uint4 raw[kU];
+    bool have[kU];
 #pragma unroll
-    for (int i = 1; i < 8; ++i) s = fmaf(kf[i], x[i], s);
-    s = s + __shfl_xor_sync(row_mask, s, 1);
-    s = s + __shfl_xor_sync(row_mask, s, 2);
-    s = s + __shfl_xor_sync(row_mask, s, 4);
-    s = s + __shfl_xor_sync(row_mask, s, 8);
-    s = s + 0.0f;
-    if (s > best) { best = s; arg = cl; }          // ascending ids: the first maximum stays
+    for (int u = 0; u < kU; ++u) {
+      const int cl = c0 + 16 * u;
+      const uint8_t *srow = cl < n_clusters ? summary_at(c, set, cl) : nullptr;
+      if (cl < n_clusters && !srow && lane16 == 0) dev_error(c, kErrBounds);
+      have[u] = srow != nullptr;
+      raw[u] = srow ? *reinterpret_cast<const uint4 *>(srow + lane16 * 16) : make_uint4(0, 0, 0, 0);
+    }
+#pragma unroll
+    for (int u = 0; u < kU; ++u) {
+      float x[8];
+      unpack8(raw[u], x);
+      float s = kf[0] * x[0];
+#pragma unroll
+      for (int i = 1; i < 8; ++i) s = fmaf(kf[i], x[i], s);
+      s = s + __shfl_xor_sync(row_mask, s, 1);
+      s = s + __shfl_xor_sync(row_mask, s, 2);
+      s = s + __shfl_xor_sync(row_mask, s, 4);
+      s = s + __shfl_xor_sync(row_mask, s, 8);
+      s = s + 0.0f;
+      if (have[u] && s > best) { best = s; arg = c0 + 16 * u; }   // ascending ids: the first maximum stays
+    }
   }
   if (lane16 == 0) { s_best[grp] = best; s_arg[grp] = arg; }
   __syncthreads();
@@ -91,19 +107,27 @@ struct ReindexArgs {
   int32_t tail_first, tail_pages, tail_len, n_host_pages;      // the sets' tail after the fold
 };
 
-// One CTA per kv head.  new_tokens: [Hkv][n_clusters]; touched: [Hkv][ceil(n_clusters / 32)].
+// grid (blocks, Hkv): every block takes its share of the tables' copies; block 0 of a head also does
+// the rest, from the tokens' clusters (assign: [n_tokens][Hkv]).
 __global__ void __launch_bounds__(256)
-k_reindex_apply(DevCtx c, ReindexArgs a, const int32_t *__restrict__ new_tokens, const uint32_t *__restrict__ touched) {
-  extern __shared__ int32_t s_tail[];
-  const int head = blockIdx.x, set = set_index(c, a.req, a.layer, head), tid = threadIdx.x;
+k_reindex_apply(DevCtx c, ReindexArgs a, const int32_t *__restrict__ assign) {
+  extern __shared__ int32_t s_tail[];                              // [tail_cap], then a bit per cluster that took a token
+  const int head = blockIdx.y, set = set_index(c, a.req, a.layer, head), tid = threadIdx.x;
+  mirror_tables(c, set, blockIdx.x * 256 + tid, a.n_clusters, a.n_host_pages);
+  if (blockIdx.x != 0) return;
   const int words = (a.n_clusters + 31) / 32;
-  const uint32_t *mine = touched + (size_t)head * words;
-  for (int cl = tid; cl < a.n_clusters; cl += 256) {
-    MetaEntry *m = meta_at(c, set, cl);
+  uint32_t *mine = reinterpret_cast<uint32_t *>(s_tail + c.tail_cap);
+  for (int i = tid; i < words; i += 256) mine[i] = 0;
+  __syncthreads();
+  for (int t = tid; t < a.n_folded_pages * kPageTokens; t += 256) {
+    const int cl = assign[(size_t)t * c.Hkv + head];
+    MetaEntry *m = cl >= 0 && cl < a.n_clusters ? meta_at(c, set, cl) : nullptr;
     if (!m) { dev_error(c, kErrBounds); continue; }
-    m->tokens = new_tokens[(size_t)head * a.n_clusters + cl];
-    if ((mine[cl >> 5] >> (cl & 31)) & 1u) m->resident = 0;
+    atomicAdd(&m->tokens, 1);
+    m->resident = 0;
+    atomicOr(&mine[cl >> 5], 1u << (cl & 31));
   }
+  __syncthreads();
   const int S = c.state[set].slots;
   for (int s = tid; s < S; s += 256) {
     GptEntry *e = gpt_at(c, set, s);
@@ -143,10 +167,11 @@ int launch_move_rows(const DevCtx &c, int req, int layer, const int64_t *dest, i
 }
 
 int launch_reindex_apply(const DevCtx &c, int req, int layer, int n_clusters, int n_folded_pages, int tail_first,
-                         int tail_pages, int tail_len, int n_host_pages, const int32_t *new_tokens,
-                         const uint32_t *touched, cudaStream_t st) {
+                         int tail_pages, int tail_len, int n_host_pages, const int32_t *assign, cudaStream_t st) {
   ReindexArgs a{req, layer, n_clusters, n_folded_pages, tail_first, tail_pages, tail_len, n_host_pages};
-  k_reindex_apply<<<c.Hkv, 256, (size_t)c.tail_cap * 4, st>>>(c, a, new_tokens, touched);
+  const int n = n_clusters > n_host_pages ? n_clusters : n_host_pages;
+  const size_t smem = (size_t)c.tail_cap * 4 + (size_t)((n_clusters + 31) / 32) * 4;
+  k_reindex_apply<<<dim3((n + 255) / 256, c.Hkv), 256, smem, st>>>(c, a, assign);
   return 1;
 }
 
