@@ -23,6 +23,7 @@ namespace {
 
 constexpr int kScoreThreads = 256;
 constexpr int kTopkThreads = 512;
+constexpr int kTopkSmem = 204 * 1024;      // dynamic shared memory of k_topk: 227 KB less its 19 KB of static
 
 __device__ __forceinline__ void unpack8(uint4 raw, float *f) {
   const uint32_t w[4] = {raw.x, raw.y, raw.z, raw.w};
@@ -977,7 +978,13 @@ int launch_select(const DevCtx &c, Batch &b, const __nv_bfloat16 *q, const __nv_
   // starts set by set, on the flag the last scoring CTA of a set raises (fuse 3)
   int mgr_tbl_cap = 0;
   size_t mgr_smem = 0;
-  const int manage = !fuse && plan_cache_fast(c, b, 160 * 1024, &mgr_tbl_cap, &mgr_smem) ? 1 : 0;
+  // cluster size of the stand-alone top-k from the largest candidate count: slices of at most 8192
+  // keys stay in shared memory, and the cache manager's tables beside them as far as they fit
+  int C = 1;
+  while (C < 8 && (max_cand + C - 1) / C > 8192) C *= 2;
+  int kc = (((max_cand + C - 1) / C) + 31) & ~31;       // a CTA's slice: whole rows of 32 keys
+  if (kc > 16384) kc = 0;                                // too many for shared memory: re-read from L2
+  const int manage = !fuse && plan_cache_fast(c, b, kTopkSmem - (size_t)kc * 4 - 16, &mgr_tbl_cap, &mgr_smem) ? 1 : 0;
   if (manage) fuse = 3;
   // work items: a tail item per set, then every request's segments head by head (segment 0
   // always runs: arrival counter)
@@ -1042,11 +1049,6 @@ int launch_select(const DevCtx &c, Batch &b, const __nv_bfloat16 *q, const __nv_
   }
   if (fuse == 1 || fuse == 2) return 1;
   {
-    // cluster size from the largest candidate count: slices of at most 8192 keys stay in smem
-    int C = 1;
-    while (C < 8 && (max_cand + C - 1) / C > 8192) C *= 2;
-    int kc = (((max_cand + C - 1) / C) + 31) & ~31;     // a CTA's slice: whole rows of 32 keys
-    if (kc > 16384) kc = 0;                              // too many for shared memory: re-read from L2
     static int smem_set_dev[kMaxDevices] = {};
     int &smem_set = smem_set_dev[current_device_slot()];
     int ksmem = kc * 4;

@@ -1018,7 +1018,7 @@ __device__ __forceinline__ void cache_stage(const DevCtx &c, int b, int set, int
 // cp.async while the radix select runs, the compaction and the free-slot scan need one block
 // scan each, and the page table is written back once at the end.  The time this takes is the
 // time before the set's missed pages can start to cross the host link.
-constexpr int kFastSlots = 1024;
+constexpr int kFastSlots = 4096;
 
 
 constexpr int kFastDigitBits = 11, kFastBins = 1 << kFastDigitBits;
@@ -1057,7 +1057,7 @@ inline bool plan_cache_fast(const DevCtx &c, const Batch &b, size_t smem_limit, 
   const size_t fs = fast_smem_bytes(0, max_slots_batch, c.dir_part, c.dir_slot, c.dir_page, c.max_parts, c.max_pages, 0);
   *tbl_cap = 0;
   *smem = fs;
-  if (max_slots_batch > 1024 || fs > 96 * 1024) return false;
+  if (max_slots_batch > kFastSlots || fs > smem_limit) return false;
   if (c.kind != kKindCluster && max_parts_batch > 0) {
     const size_t ft = fast_smem_bytes(0, max_slots_batch, c.dir_part, c.dir_slot, c.dir_page, c.max_parts, c.max_pages, max_parts_batch);
     if (ft <= smem_limit) { *tbl_cap = max_parts_batch; *smem = ft; }
