@@ -110,13 +110,17 @@ __device__ __forceinline__ void attend_page(uint32_t spage, const uint32_t (&qb)
   const int mat = lane >> 3, r8 = lane & 7;
   const uint32_t krow = spage + (uint32_t)((r8 + ((mat & 1) << 3)) * kStageRow + (mat >> 1) * 16);
   const uint32_t vrow = spage + (uint32_t)((kPageTokens + r8 + ((mat >> 1) << 3)) * kStageRow + (mat & 1) * 16);
-  float s[4] = {0.f, 0.f, 0.f, 0.f};
+  float s[4] = {0.f, 0.f, 0.f, 0.f}, s_odd[4] = {0.f, 0.f, 0.f, 0.f};      // two chains: half the serial mma latency
 #pragma unroll
-  for (int ks = 0; ks < 8; ++ks) {
-    uint32_t a0, a1, a2, a3;
+  for (int ks = 0; ks < 8; ks += 2) {
+    uint32_t a0, a1, a2, a3, b0, b1, b2, b3;
     ldmatrix_x4(krow + ks * 32, a0, a1, a2, a3);
+    ldmatrix_x4(krow + ks * 32 + 32, b0, b1, b2, b3);
     mma_bf16(s, a0, a1, a2, a3, qb[ks][0], qb[ks][1]);
+    mma_bf16(s_odd, b0, b1, b2, b3, qb[ks + 1][0], qb[ks + 1][1]);
   }
+#pragma unroll
+  for (int i = 0; i < 4; ++i) s[i] += s_odd[i];
   // this lane's tokens: lane / 4 (s[0], s[1]) and lane / 4 + 8 (s[2], s[3])
   const bool t0 = (mask >> (lane >> 2)) & 1u, t1 = (mask >> ((lane >> 2) + 8)) & 1u;
   float corr[2];
@@ -165,16 +169,15 @@ __device__ __forceinline__ void stores_read() { asm volatile("cp.async.bulk.wait
 // 75-86 us into the step without a limit, 35 us with one; step 112 us without, 106 / 102 / 103 / 107 us
 // with a window of 32 / 64 / 96 / 160 pages.
 constexpr int kLinkWindow = 64, kLinkDone = 32, kLinkPolls = 1 << 20;
-__device__ __forceinline__ int link_turn(const DevCtx &c, int lane) {
-  int t = 0;
-  if (lane == 0) t = atomicAdd(c.link, 1);
-  return __shfl_sync(0xffffffffu, t, 0);
-}
+__device__ __forceinline__ int link_turn(const DevCtx &c, int lane) { return lane == 0 ? atomicAdd(c.link, 1) : 0; }   // lane 0's
 __device__ __forceinline__ void link_close(const DevCtx &c, int lane) { if (lane == 0) atomicAdd(c.link + kLinkDone, 1); }
-__device__ __forceinline__ bool link_open(const DevCtx &c, int turn) {
+__device__ __forceinline__ int link_closed(const DevCtx &c) {
   int done;
   asm volatile("ld.relaxed.gpu.global.s32 %0, [%1];\n" : "=r"(done) : "l"(c.link + kLinkDone) : "memory");
-  return __all_sync(0xffffffffu, (int)((unsigned)turn - (unsigned)done) < kLinkWindow);
+  return done;
+}
+__device__ __forceinline__ bool link_open(int turn, int closed) {   // turn: lane 0's
+  return __shfl_sync(0xffffffffu, (int)((unsigned)turn - (unsigned)closed), 0) < kLinkWindow;
 }
 
 // What a lane knows of one page of its warp.
@@ -332,17 +335,18 @@ __device__ __forceinline__ void attn_cta(const DevCtx &c, const Batch &bt, const
   }
   int np = 0, nm = 0;                      // pages in the set's list; how many of them are early descriptors
   if (c.ready) {
-    // A set raises two flags.  The first says that its missed pages are listed (the leading
-    // n_miss descriptors, slot still open): a warp requests its first missed page at once, so the
-    // pages cross the host link while the cache manager is still freeing slots for them.  For
-    // everything else a warp waits for the second flag (complete list) and for the tail page.
+    // A set raises three flags.  The first says that its missed pages are listed (the leading
+    // descriptors, slot still open): a warp requests its first missed page at once, so the
+    // pages cross the host link while the cache manager is still busy.  For the hits a warp waits
+    // for the second flag (complete list) and for the tail page, for the slot of a page that has
+    // come over the link for the third.
     if (threadIdx.x == 0) {
-      const int ok = flag_wait(c, c.ready1 + b, bt.epoch);
+      uint32_t word = 0;
+      sh_ok = first_flag_wait(c, c.ready1 + b, bt.epoch, &word);
       // a count beyond the list's stride can neither read past the set's row nor leave the merge
       // waiting for rows that no CTA of the grid owns
-      sh_np = ok ? max(0, min(__ldcg(c.n_pages + b), c.max_pages + c.tail_cap)) : 0;
-      sh_nm = ok ? __ldcg(c.n_miss + b) : 0;
-      sh_ok = ok;
+      sh_np = min((int)(word >> 12), c.max_pages + c.tail_cap);
+      sh_nm = (int)(word & 4095u);
     }
     __syncthreads();
     if (!sh_ok) return;
@@ -376,30 +380,27 @@ __device__ __forceinline__ void attn_cta(const DevCtx &c, const Batch &bt, const
   for (int i = 0; i < 8; ++i) { acc.o[i][0] = acc.o[i][1] = acc.o[i][2] = acc.o[i][3] = 0.f; }
   const float scale2 = c.sm_scale * 1.4426950408889634f;
 
-  // The warp's pages in batches of 32, a lane per page (one batch as a rule).  Requests and waits
-  // of a batch: its first missed page is requested as soon as it is known and stays in stage 0;
-  // the hits go through stage 1 meanwhile (through both stages if nothing is missing), then the
-  // missed pages are attended.  The order in which a warp attends its pages is fixed.
+  // The warp's pages in batches of 32, a lane per page (one batch as a rule).  The order in which a
+  // warp attends its pages is fixed: the hits of a batch, then its missed pages.
   uint32_t phases = 0;                     // parity of the next wait, a bit per stage
-  bool dead = false, listed = c.ready == nullptr;
+  bool dead = false, listed = c.ready == nullptr, slots_known = listed;
 #pragma unroll 1
   for (int p0 = mine; p0 < np && !dead; p0 += 32 * stride) {
     const int pos = p0 + lane * stride;
     PageRef ref{0, -1, -1, 0u};
-    int in0 = -1, in1 = -1;                // the pages (lanes) that have the two stages
-    int turn0 = 0, turn1 = 0;              // their turns on the host link
-    uint32_t issued = 0, on_link = 0;      // stages whose page has been requested; whose page has a turn on the link
     auto request = [&](int stage, int j) {
       const int src = __shfl_sync(0xffffffffu, ref.src, j), fill = __shfl_sync(0xffffffffu, ref.fill, j);
-      const uint8_t *from = fill >= 0 ? c.host_pages + (size_t)fill * kPageBytes : page_ptr(c, src);
-      request_page(stage0 + stage * kStageBytes, bar0 + 8 * stage, from, lane);
-      issued |= 1u << stage;
+      request_page(stage0 + stage * kStageBytes, bar0 + 8 * stage, fill >= 0 ? c.host_pages + (size_t)fill * kPageBytes : page_ptr(c, src), lane);
     };
+    // a missed page is requested as soon as it is known (early pages lead the list: lane 0's is one of
+    // them): its turn, its descriptor and the count of closed turns are asked for together
     const bool early = pos < min(nm, np);
-    const bool early0 = p0 < nm && !listed;               // early pages lead the list: lane 0's is one of them
-    if (early0) { turn0 = link_turn(c, lane); on_link = 1u; in0 = 0; }
+    const bool early0 = p0 < nm && !listed;
+    int turn0 = 0, turn1 = 0, closed = 0;  // the stages' turns on the host link (lane 0's)
+    uint32_t issued = 0, on_link = 0;      // stages whose page has been requested; whose page has a turn on the link
+    if (early0) { turn0 = link_turn(c, lane); closed = link_closed(c); on_link = 1u; }
     if (early) ref = page_ref(c, bt, b, i_req, head, pl, pos);
-    if (early0 && link_open(c, turn0)) request(0, 0);
+    if (early0 && link_open(turn0, closed)) { request(0, 0); issued = 1u; }
     if (p0 == mine) {
       const int qr = lane >> 2;
       const uint32_t *qrow = reinterpret_cast<const uint32_t *>(q + ((size_t)i_req * c.Hq + head * G + (qr < G ? qr : 0)) * kHeadDim);
@@ -417,31 +418,65 @@ __device__ __forceinline__ void attn_cta(const DevCtx &c, const Batch &bt, const
       dead = !listed;                      // reported by the wait: the warp only sees off the copy it has in flight, and the CTA still arrives
     }
     if (pos < np && !early && !dead) ref = page_ref(c, bt, b, i_req, head, pl, pos);
-    // the slot of a page that is brought in; an early descriptor's is known by now (negative: bypassed, attended only)
-    int slot_page = ref.fill >= 0 ? ref.src : -1;
-    if (ref.open_idx >= 0 && !dead) slot_page = __ldcg(c.page_src + pl + ref.open_idx);
     const bool from_host = ref.fill >= 0 || ref.src < 0;
-    const uint32_t hosted = __ballot_sync(0xffffffffu, pos < np && from_host);
-    uint32_t misses = hosted, hits = __ballot_sync(0xffffffffu, pos < np && !from_host);
-    if (early0) { misses &= ~1u; hits &= ~1u; }           // (a dropped early descriptor is attended with an empty mask)
-    if (dead) misses = hits = 0u;
+    const uint32_t here = __ballot_sync(0xffffffffu, pos < np && !dead), host = __ballot_sync(0xffffffffu, from_host) & here;
+    if (row == 0 && p0 == mine) dbg_ta(b, 11);
+    if (host == 0 && !early0) {
+      // nothing to bring in (the usual batch): pages 0, 1, 2, ... through the two stages in turn
+      const int n = __popc(here);
+      request(0, 0);
+      if (n > 1) request(1, 1);
+#pragma unroll 1
+      for (int j = 0; j < n; ++j) {
+        const int st = j & 1;
+        const uint32_t mask = __shfl_sync(0xffffffffu, ref.mask, j);
+        if (!page_landed(bar0 + 8 * st, (phases >> st) & 1u)) {             // the stages may still be written to: no more requests
+          if (lane == 0) dev_error(c, kErrTimeout);
+          dead = true;
+          break;
+        }
+        phases ^= 1u << st;
+        attend_page(stage0 + st * kStageBytes, qb, mask, scale2, acc, lane);
+        __syncwarp();                      // every lane has read the stage
+        if (j + 2 < n) request(st, j + 2);
+      }
+      if (row == 0 && p0 == mine) dbg_ta(b, 12);
+      continue;
+    }
+    // The first missed page has stage 0 from the start; the hits go through stage 1 meanwhile, then
+    // the other missed pages through both.
+    const uint32_t hosted = host | (early0 ? 1u : 0u);    // (a dropped early descriptor keeps its turn and is attended with an empty mask)
+    uint32_t misses = hosted & here, hits = here & ~hosted;
     auto pop = [](uint32_t &m) { const int j = __ffs(m) - 1; m &= m - 1; return j; };
     auto next = [&]() { return hits ? pop(hits) : misses ? pop(misses) : -1; };
-    // the page that has a stage: an HBM page is requested at once, a host page takes its turn on the link
-    auto take0 = [&](int j) { in0 = j; if (j >= 0) { if ((hosted >> j) & 1u) { turn0 = link_turn(c, lane); on_link |= 1u; } else request(0, j); } };
-    auto take1 = [&](int j) { in1 = j; if (j >= 0) { if ((hosted >> j) & 1u) { turn1 = link_turn(c, lane); on_link |= 2u; } else request(1, j); } };
-    if (in0 < 0) take0(misses ? pop(misses) : next());
-    int hits_in1 = (on_link & 1u) ? __popc(hits) : 0;     // hits still to come through stage 1 while stage 0 holds a missed page
-    take1(next());
-    if (row == 0 && p0 == mine) dbg_ta(b, 11);
-    int cur = hits_in1 > 0 ? 1 : 0, polls = 0;
+    int in0 = early0 ? 0 : -1, in1 = -1;   // the pages (lanes) that have the two stages
+    if (early0) misses &= ~1u;
+    else { in0 = pop(misses); turn0 = link_turn(c, lane); on_link = 1u; }
+    int hits_in1 = __popc(hits), cur = hits_in1 > 0 ? 1 : 0, polls = 0;     // hits still to come through stage 1
+    bool refill1 = true, refill0 = false;
+    int slot_page = ref.fill >= 0 ? ref.src : -1;         // where a page that is brought in goes
+    if (ref.open_idx >= 0) slot_page = slots_known ? __ldcg(c.page_src + pl + ref.open_idx) : -1;
 #pragma unroll 1
     for (;;) {
+      // a free stage takes the next page: an HBM page is requested at once, a host page takes a turn on the link
+      if (refill1) {
+        in1 = dead ? -1 : next();
+        if (in1 >= 0 && ((hosted >> in1) & 1u)) { turn1 = link_turn(c, lane); on_link |= 2u; }
+        else if (in1 >= 0) { request(1, in1); issued |= 2u; }
+        refill1 = false;
+      }
+      if (refill0) {                       // (no hits are left by then)
+        in0 = dead ? -1 : next();
+        if (in0 >= 0) { turn0 = link_turn(c, lane); on_link |= 1u; }
+        refill0 = false;
+      }
       const int j = cur ? in1 : in0;
       if (j < 0) break;
-      if ((on_link & ~issued) != 0u && !dead) {
-        if ((on_link & ~issued & 1u) && link_open(c, turn0)) request(0, in0);
-        if ((on_link & ~issued & 2u) && link_open(c, turn1)) request(1, in1);
+      const uint32_t waiting = on_link & ~issued;
+      if (waiting && !dead) {
+        closed = link_closed(c);
+        if ((waiting & 1u) && link_open(turn0, closed)) { request(0, in0); issued |= 1u; }
+        if ((waiting & 2u) && link_open(turn1, closed)) { request(1, in1); issued |= 2u; }
       }
       // a missed page that has landed behind the hits gives its turn on
       if (hits_in1 > 0 && (on_link & issued & 1u) && page_test(bar0, phases & 1u)) { link_close(c, lane); on_link &= ~1u; }
@@ -450,6 +485,12 @@ __device__ __forceinline__ void attn_cta(const DevCtx &c, const Batch &bt, const
         if (!dead && lane == 0) dev_error(c, kErrTimeout);
         dead = true;
       } else {
+        if (((hosted >> j) & 1u) && !slots_known && !dead) {                // while the page is on its way
+          int ok = 1;
+          if (lane == 0) ok = flag_wait(c, c.slots_ready + b, bt.epoch);
+          slots_known = __shfl_sync(0xffffffffu, ok, 0) != 0;               // else reported: open pages are attended, not kept
+          slot_page = ref.open_idx < 0 ? slot_page : slots_known ? __ldcg(c.page_src + pl + ref.open_idx) : -1;   // negative: bypassed, attended only
+        }
         if (!page_landed(bar0 + 8 * cur, (phases >> cur) & 1u)) {           // its stage may still be written to: no more requests
           if (lane == 0) dev_error(c, kErrTimeout);
           dead = true;
@@ -463,13 +504,14 @@ __device__ __forceinline__ void attn_cta(const DevCtx &c, const Batch &bt, const
       const uint32_t spage = stage0 + cur * kStageBytes;
       if (!dead) {
         attend_page(spage, qb, __shfl_sync(0xffffffffu, ref.mask, j), scale2, acc, lane);
-        const int slot = __shfl_sync(0xffffffffu, slot_page, j);
-        if (slot >= c.n_gpu_pages) { if (lane == 0) dev_error(c, kErrBounds); }
-        else if (slot >= 0) { store_page(spage, c.gpu_pages + (size_t)slot * kPageBytes, lane); stores_read(); }
+        if ((hosted >> j) & 1u) {
+          const int slot = __shfl_sync(0xffffffffu, slot_page, j);
+          if (slot >= c.n_gpu_pages) { if (lane == 0) dev_error(c, kErrBounds); }
+          else if (slot >= 0) { store_page(spage, c.gpu_pages + (size_t)slot * kPageBytes, lane); stores_read(); }
+        }
       }
       __syncwarp();                        // every lane has read the stage
-      const int nx = dead ? -1 : next();
-      if (cur) take1(nx); else take0(nx);
+      if (cur) refill1 = true; else refill0 = true;
       if (hits_in1 > 0) { if (--hits_in1 == 0) cur = 0; }
       else cur ^= 1;
     }
@@ -665,7 +707,7 @@ extern "C" int spin_paged_attention_static(const void *q, const void *page_pool,
   c.ready = nullptr;                                        // plain stream order: no per-set flags
   c.tail_ready = nullptr;
   c.ready1 = nullptr;
-  c.n_miss = nullptr;
+  c.slots_ready = nullptr;
   c.att_part = g_static_partials_addr[dev];
   c.att_ml = reinterpret_cast<float2 *>(c.att_part + (size_t)n_sets * chunks * group * kHeadDim);
   c.att_words = g_static_words_addr[dev];

@@ -113,10 +113,11 @@ struct DevCtx {
   int32_t *score_queue;         // next work item of the resident scoring grid (zero between steps)
   int32_t *score_done;          // CTAs of that grid that have left (zero between steps)
   int32_t *scored;              // [b] epoch of the last step whose scores are complete (stand-alone top-k waits on it)
-  int32_t *ready;               // [b] epoch of the last step whose page list is complete
+  int32_t *ready;               // [b] epoch of the last step whose page list is complete (slots of missed pages may be open)
   int32_t *tail_ready;          // [b] epoch of the last step whose appended rows are in the tail page
-  int32_t *ready1;              // [b] epoch of the last step whose missed pages are listed (before their slots are known)
-  int32_t *n_miss;              // [b] leading descriptors of the page list that may be followed once ready1 is set
+  unsigned long long *ready1;   // [b] first flag: epoch of the last step whose missed pages are listed (upper half), with the
+                                //   length of the page list and its early descriptors (see first_flag)
+  int32_t *slots_ready;         // [b] epoch of the last step whose missed pages have their slots (page_src)
   int32_t max_chunks;
   int32_t fetch_mode;           // 0: misses are fetched by the attention kernel; 1: by k_fetch
   int32_t evict_exact;          // 1: exact-demand eviction variant (see spin_config)
@@ -232,6 +233,15 @@ __device__ __forceinline__ void flag_publish(int32_t *flag, int32_t value) {
   // before the call: the other threads' writes too) is visible to whoever acquires the flag
   asm volatile("st.release.gpu.global.s32 [%0], %1;" ::"l"(flag), "r"(value) : "memory");
 }
+// The first flag of a set carries what its consumers need first: the pages in its list (20 bits; a
+// list has at most 50 K selected and 32 K tail pages) and how many of them lead it as early
+// descriptors (12 bits; a count beyond that is only a smaller head start).
+__device__ __forceinline__ unsigned long long first_flag(int epoch, int n_pages, int n_early) {
+  return (unsigned long long)(uint32_t)epoch << 32 | (uint32_t)n_pages << 12 | (uint32_t)min(n_early, 4095);
+}
+__device__ __forceinline__ void first_flag_publish(unsigned long long *flag, unsigned long long value) {
+  asm volatile("st.release.gpu.global.u64 [%0], %1;" ::"l"(flag), "l"(value) : "memory");
+}
 constexpr int kFlagWaitPolls = 1 << 19;          // ~0.1 s of polls at the capped back-off
 __device__ __forceinline__ bool flag_wait(const DevCtx &c, const int32_t *flag, int32_t value,
                                           int max_polls = kFlagWaitPolls) {
@@ -243,6 +253,21 @@ __device__ __forceinline__ bool flag_wait(const DevCtx &c, const int32_t *flag, 
     int32_t v;
     asm volatile("ld.acquire.gpu.global.s32 %0, [%1];" : "=r"(v) : "l"(flag) : "memory");
     if (v == value) return true;
+    __nanosleep(pause);
+    if (pause < 256) pause <<= 1;
+  }
+  dev_error(c, kErrTimeout);
+  return false;
+}
+
+// The same for a set's first flag; its lower half in *word.
+__device__ __forceinline__ bool first_flag_wait(const DevCtx &c, const unsigned long long *flag, int32_t epoch, uint32_t *word) {
+  unsigned pause = 32;
+  for (int spin = 0; spin < kFlagWaitPolls; ++spin) {
+    unsigned long long v;
+    asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(flag) : "memory");
+    *word = (uint32_t)v;
+    if ((int32_t)(v >> 32) == epoch) return true;
     __nanosleep(pause);
     if (pause < 256) pause <<= 1;
   }

@@ -1004,9 +1004,10 @@ __device__ __forceinline__ void cache_stage(const DevCtx &c, int b, int set, int
     atomicAdd(&k->miss_pages, (unsigned long long)miss_pages);
     atomicAdd(&k->evicted_pages, (unsigned long long)sh.evicted);
     atomicAdd(&k->bypass_pages, (unsigned long long)sh.bypass_pages);
-    c.n_miss[b] = 0;                             // no early list on this path: both flags go up together
-    flag_publish(c.ready1 + b, epoch);
-    flag_publish(c.ready + b, epoch);            // attention may start on this set
+    // no early list on this path: all flags go up together, and attention may start on this set
+    first_flag_publish(c.ready1 + b, first_flag(epoch, total_pages + tail_pages, 0));
+    flag_publish(c.ready + b, epoch);
+    flag_publish(c.slots_ready + b, epoch);
   }
 }
 
@@ -1520,12 +1521,24 @@ __device__ __forceinline__ void cache_fast(const DevCtx &c, const Batch &bt, int
   __syncthreads();
   if (tid == 0) {
     c.n_pages[b] = total_pages + tail_pages;
-    c.n_miss[b] = early ? demand : 0;
-    flag_publish(c.ready1 + b, bt.epoch);
+    first_flag_publish(c.ready1 + b, first_flag(bt.epoch, total_pages + tail_pages, early ? demand : 0));
   }
 
   dbg_ts(b, 19);
-  // ---- step 2: one pass over the page table copy: promote, demote, histogram ----------------
+#pragma unroll 1
+  for (int j = tid; j < tail_pages; j += T) {
+    const int idx = total_pages + j;
+    const int src = c.tail_phys[(size_t)set * c.tail_cap + j];
+    const uint32_t m = j == tail_pages - 1 ? ((1u << tail_len) - 1u) : 0xffffu;
+    page_src[idx] = src;
+    page_mask[idx] = m;
+    page_slot[idx] = -2;
+    page_fill[idx] = -1;
+    page_desc[idx] = make_int4(src, -1, (int)m, idx);
+    page_part[idx] = -1;
+    page_pidx[idx] = j;
+  }
+  // ---- step 2: one pass over the page table copy: promote, demote, histogram; the hits are listed -
 #pragma unroll 1
   for (int s_ = tid; s_ < S; s_ += T) {
     int4 e = s_gpt[s_];
@@ -1541,6 +1554,9 @@ __device__ __forceinline__ void cache_fast(const DevCtx &c, const Batch &bt, int
       const int idx = s_pageoff[r] + e.z;
       page_src[idx] = e.y;
       page_slot[idx] = s_;
+      const int valid = min(kPageTokens, s_tokens[r] - e.z * kPageTokens);
+      const uint32_t pmask = c.kind == kKindToken ? c.part_mask[(size_t)b * c.max_parts + r] : ((1u << valid) - 1u);
+      page_desc[demand + (s_pageoff[r] - s_missbefore[r]) + e.z] = make_int4(e.y, -1, (int)pmask, idx);
     } else {
       if (t > nb - 1 && e.w > 0) --e.w;
       atomicAdd(&sh.lhist[e.w + 1], 1u);
@@ -1548,6 +1564,10 @@ __device__ __forceinline__ void cache_fast(const DevCtx &c, const Batch &bt, int
     s_gpt[s_] = e;
   }
   __syncthreads();
+  // The list is complete but for the missed pages' slots, which nobody needs before such a page has
+  // arrived: attention may go on to the hits while slots are being freed (a step without misses
+  // has nothing left to wait for).
+  if (tid == 0 && early) flag_publish(c.ready + b, bt.epoch);
 
   dbg_ts(b, 5);
   // ---- step 3: threshold, eviction, free slots in ascending order (one scan) ----------------
@@ -1668,7 +1688,7 @@ __device__ __forceinline__ void cache_fast(const DevCtx &c, const Batch &bt, int
     page_pidx[idx] = i;
     page_fill[idx] = -1;
     const int pos = state == kHit ? demand + (s_pageoff[r] - s_missbefore[r]) + i : s_missbefore[r] + i;
-    if (state == kHit) { page_desc[pos] = make_int4(page_src[idx], -1, (int)pmask, idx); continue; }
+    if (state == kHit) continue;
     const int mi = s_missbefore[r] + i;
     // the CPU page id found for the early list (-2: left to the fetching warp, which then reads
     // the two pinned host tables itself, so that no page list waits on the host link)
@@ -1704,26 +1724,14 @@ __device__ __forceinline__ void cache_fast(const DevCtx &c, const Batch &bt, int
   dbg_ts(b, 24);
   if (my_admit) atomicAdd(&sh.admit_pages, my_admit);
   if (my_bypass) atomicAdd(&sh.bypass_pages, my_bypass);
-#pragma unroll 1
-  for (int j = tid; j < tail_pages; j += T) {
-    const int idx = total_pages + j;
-    const int src = c.tail_phys[(size_t)set * c.tail_cap + j];
-    const uint32_t m = j == tail_pages - 1 ? ((1u << tail_len) - 1u) : 0xffffu;
-    page_src[idx] = src;
-    page_mask[idx] = m;
-    page_slot[idx] = -2;
-    page_fill[idx] = -1;
-    page_desc[idx] = make_int4(src, -1, (int)m, idx);
-    page_part[idx] = -1;
-    page_pidx[idx] = j;
-  }
   __syncthreads();
   dbg_ts(b, 7);
   if (tid == 0) {
     c.n_pages[b] = total_pages + tail_pages;
     c.n_parts[b] = np;
     c.state[set].step = t + 1;
-    flag_publish(c.ready + b, bt.epoch);
+    if (!early) flag_publish(c.ready + b, bt.epoch);
+    flag_publish(c.slots_ready + b, bt.epoch);
     // the counters go last: the flag's fence should not have to wait for them
     Counters *kc = c.counters;
     const int miss_pages = sh.admit_pages + sh.bypass_pages;
