@@ -1307,8 +1307,7 @@ static int step_impl(spin_ctx *ctx, int32_t layer, const int32_t *req_ids, int32
   const void *k_alias = nullptr, *v_alias = nullptr, *q_alias = nullptr, *out_alias = nullptr;
   const size_t kv_bytes = (size_t)n_req * ctx->cfg.num_kv_heads * kRowBytes;
   const size_t qbytes = (size_t)n_req * ctx->cfg.num_q_heads * kRowBytes;
-  bool in_grid = false, kv_pinned = false;
-  // q and new k/v in pinned host memory: one zero-copy staging kernel brings them in
+  bool in_grid = false;
   const int qc = classify_ptr(q, &q_alias), oc = classify_ptr(out, &out_alias);
   int kc = 0;
   if (with_append) {
@@ -1331,14 +1330,12 @@ static int step_impl(spin_ctx *ctx, int32_t layer, const int32_t *req_ids, int32
       CK(cudaMemcpyAsync(ctx->stage_k, k, kv_bytes, cudaMemcpyHostToDevice, st));
       CK(cudaMemcpyAsync(ctx->stage_v, v, kv_bytes, cudaMemcpyHostToDevice, st));
     }
-    if (kc != 0) { kk = ctx->stage_k; vv = ctx->stage_v; }
-    kv_pinned = kc == 1;
+    if (kc == 2) { kk = ctx->stage_k; vv = ctx->stage_v; }
+    // rows in pinned host memory are read where they are (each by the one CTA that appends it)
+    if (kc == 1) { kk = reinterpret_cast<const __nv_bfloat16 *>(k_alias); vv = reinterpret_cast<const __nv_bfloat16 *>(v_alias); }
     // An append that completes no page cannot change what Select sees: it then runs inside
     // the scoring kernel (one extra CTA per set).  Otherwise it runs first, on its own.
     in_grid = !completes_page;
-    if (kv_pinned || qc == 1)
-      ctx->launches += launch_stage_in(ctx->stage_q, qc == 1 ? q_alias : nullptr, qc == 1 ? qbytes : 0, ctx->stage_k,
-                                       k_alias, ctx->stage_v, v_alias, kv_pinned ? kv_bytes : 0, st);
     if (!in_grid) {
       AppendEdgeArgs a{};
       a.n_req = n_req;
@@ -1348,7 +1345,7 @@ static int step_impl(spin_ctx *ctx, int32_t layer, const int32_t *req_ids, int32
         a.n_tokens[i] = (int32_t)(ctx->reqs[(size_t)req_ids[i]].layers[(size_t)layer].n_tokens - 1);
       }
       prof_mark(&ctx->prof, st, -1);
-      ctx->launches += launch_append_edge(ctx->d, a, kk, vv, 1, st, &ctx->prof);
+      ctx->launches += launch_append_edge(ctx->d, a, kk, vv, 1, st, &ctx->prof, ctx->stage_q, qc == 1 ? q_alias : nullptr, qbytes);
     }
   }
   int64_t max_cand = 0, max_pages = 0;
@@ -1369,8 +1366,7 @@ static int step_impl(spin_ctx *ctx, int32_t layer, const int32_t *req_ids, int32
   const __nv_bfloat16 *qd = reinterpret_cast<const __nv_bfloat16 *>(q);
   __nv_bfloat16 *od = reinterpret_cast<__nv_bfloat16 *>(out);
   if (qc == 2) CK(cudaMemcpyAsync(ctx->stage_q, q, qbytes, cudaMemcpyHostToDevice, st));
-  if (qc == 1 && !with_append)
-    ctx->launches += launch_stage_in(ctx->stage_q, q_alias, qbytes, nullptr, nullptr, nullptr, nullptr, 0, st);
+  if (qc == 1 && (in_grid || !with_append)) ctx->launches += launch_stage_in(ctx->stage_q, q_alias, qbytes, st);
   if (qc != 0) qd = ctx->stage_q;
   // pinned host output: the attention kernel writes it directly (visible once the stream is synchronised)
   if (oc == 1) od = reinterpret_cast<__nv_bfloat16 *>(const_cast<void *>(out_alias));

@@ -24,6 +24,7 @@ k_append_bulk(DevCtx c, int req, int layer, const __nv_bfloat16 *__restrict__ k,
   const size_t in_off = (tok * c.Hkv + head) * kHeadDim * 2 + piece * 16;
   uint4 kk = ld16(reinterpret_cast<const uint8_t *>(k) + in_off);
   uint4 vv = ld16(reinterpret_cast<const uint8_t *>(v) + in_off);
+  const IndexPlace at = index_place(c, set, page);
   const size_t unit = (size_t)head * gridDim.x + blockIdx.x;        // head-major, as host pages are handed out
   int32_t host_page;
   if (stage) {
@@ -42,17 +43,24 @@ k_append_bulk(DevCtx c, int req, int layer, const __nv_bfloat16 *__restrict__ k,
   st16(dst + kHalfPageBytes, vv);
   st16(reinterpret_cast<uint8_t *>(krows[r]) + piece * 16, kk);
   __syncthreads();
-  index_page(c, set, page, krows, tid);
+  index_page(c, set, page, at, krows, tid);
 }
 
-// Stand-alone edge append: one CTA per (kv head, request).
+// Stand-alone edge append: one CTA per (kv head, request).  The rows of CTAs beyond the requests
+// bring in the step's queries where they live in pinned host memory (nq pieces of 16 bytes), beside
+// the append instead of in a launch in front of it; the new K/V rows are read where they are.
 __global__ void __launch_bounds__(256)
 k_append_edge(DevCtx c, AppendEdgeArgs a, const __nv_bfloat16 *__restrict__ k,
-              const __nv_bfloat16 *__restrict__ v, int n_new) {
+              const __nv_bfloat16 *__restrict__ v, int n_new, uint4 *dq, const uint4 *sq, int nq) {
   __shared__ __align__(16) __nv_bfloat16 krows[kPageTokens][kHeadDim];
   const int head = blockIdx.x, i = blockIdx.y;
   pdl_launch_next();
   pdl_wait_prev();
+  if (i >= a.n_req) {
+    const int first = ((i - a.n_req) * (int)gridDim.x + head) * 256 + threadIdx.x, step = ((int)gridDim.y - a.n_req) * (int)gridDim.x * 256;
+    for (int e = first; e < nq; e += step) dq[e] = sq[e];
+    return;
+  }
   append_edge_body(c, set_index(c, a.req[i], a.layer, head), i, head, k, v, n_new, a.n_tokens[i], -1, krows);
 }
 
@@ -199,31 +207,21 @@ k_dir_update(int32_t *__restrict__ dirs, const __grid_constant__ DirBatch a) {
   for (int i = threadIdx.x; i < a.n; i += 256) dirs[a.u[i].at] = a.u[i].value;
 }
 
-// Step inputs that live in pinned host memory (q, new k/v) are brought into the staging
-// buffers by one small kernel of zero-copy reads instead of one copy-engine transfer each.
+// A step's queries that live in pinned host memory are brought into the staging buffer by a small
+// kernel of zero-copy reads instead of a copy-engine transfer.
 __global__ void __launch_bounds__(256)
-k_stage_in(uint4 *dq, const uint4 *sq, int nq, uint4 *dk, const uint4 *sk, uint4 *dv, const uint4 *sv, int nkv) {
+k_stage_in(uint4 *dq, const uint4 *sq, int nq) {
   pdl_launch_next();
   pdl_wait_prev();
-  const int total = nq + 2 * nkv;
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < total; i += gridDim.x * blockDim.x) {
-    if (i < nq) dq[i] = sq[i];
-    else if (i < nq + nkv) dk[i - nq] = sk[i - nq];
-    else dv[i - nq - nkv] = sv[i - nq - nkv];
-  }
+  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < nq; i += gridDim.x * blockDim.x) dq[i] = sq[i];
 }
 
 }  // namespace
 
-int launch_stage_in(void *dq, const void *sq, size_t q_bytes, void *dk, const void *sk, void *dv, const void *sv,
-                    size_t kv_bytes, cudaStream_t st) {
-  const int nq = (int)(q_bytes / 16), nkv = (int)(kv_bytes / 16);
-  if (nq + nkv == 0) return 0;
-  int grid = (nq + 2 * nkv + 255) / 256;
-  if (grid > 64) grid = 64;
-  launch_pdl(k_stage_in, dim3(grid), dim3(256), 0, st, 1, reinterpret_cast<uint4 *>(dq), reinterpret_cast<const uint4 *>(sq), nq,
-             reinterpret_cast<uint4 *>(dk), reinterpret_cast<const uint4 *>(sk), reinterpret_cast<uint4 *>(dv),
-             reinterpret_cast<const uint4 *>(sv), nkv);
+int launch_stage_in(void *dq, const void *sq, size_t q_bytes, cudaStream_t st) {
+  const int nq = (int)(q_bytes / 16);
+  const int grid = (nq + 255) / 256 < 64 ? (nq + 255) / 256 : 64;
+  launch_pdl(k_stage_in, dim3(grid), dim3(256), 0, st, 1, reinterpret_cast<uint4 *>(dq), reinterpret_cast<const uint4 *>(sq), nq);
   return 1;
 }
 
@@ -248,8 +246,11 @@ int launch_append_bulk(const DevCtx &c, int req, int layer, const __nv_bfloat16 
 }
 
 int launch_append_edge(const DevCtx &c, const AppendEdgeArgs &a, const __nv_bfloat16 *k,
-                       const __nv_bfloat16 *v, int n_new, cudaStream_t st, Prof *prof) {
-  launch_pdl(k_append_edge, dim3(c.Hkv, a.n_req), dim3(256), 0, st, 1, c, a, k, v, n_new);
+                       const __nv_bfloat16 *v, int n_new, cudaStream_t st, Prof *prof, void *dq, const void *sq, size_t q_bytes) {
+  const int nq = sq ? (int)(q_bytes / 16) : 0;
+  int q_ctas = (nq + 255) / 256 < 64 ? (nq + 255) / 256 : 64;
+  launch_pdl(k_append_edge, dim3(c.Hkv, a.n_req + (q_ctas + c.Hkv - 1) / c.Hkv), dim3(256), 0, st, 1, c, a, k, v, n_new,
+             reinterpret_cast<uint4 *>(dq), reinterpret_cast<const uint4 *>(sq), nq);
   prof_mark(prof, st, kProfAppend);
   return 1;
 }

@@ -372,7 +372,8 @@ int launch_append_bulk(const DevCtx &c, int req, int layer, const __nv_bfloat16 
                        const __nv_bfloat16 *v, int first_page, int n_pages, int first_token_of_call,
                        cudaStream_t st, Prof *prof, uint8_t *stage = nullptr, const int32_t *stage_hp = nullptr);
 int launch_append_edge(const DevCtx &c, const AppendEdgeArgs &a, const __nv_bfloat16 *k,
-                       const __nv_bfloat16 *v, int n_new, cudaStream_t st, Prof *prof);
+                       const __nv_bfloat16 *v, int n_new, cudaStream_t st, Prof *prof,
+                       void *dq = nullptr, const void *sq = nullptr, size_t q_bytes = 0);
 int launch_cluster_count(const int32_t *tp, size_t rows, int H, int C, int32_t *count, unsigned long long *bad, cudaStream_t st);
 int launch_cluster_place(const int32_t *tp, int64_t n, int H, int C, const int32_t *base, int32_t *run, int32_t *place, cudaStream_t st);
 int launch_cluster_tables(const DevCtx &c, int req, int layer, int C, int n_pages, int n_tokens, const int32_t *count, int slots, cudaStream_t st);
@@ -380,8 +381,7 @@ int launch_cluster_scatter(const DevCtx &c, int req, int layer, const __nv_bfloa
                            const int32_t *place, int64_t n_tokens, cudaStream_t st);
 int launch_cluster_scatter_staged(const DevCtx &c, const __nv_bfloat16 *k, const __nv_bfloat16 *v, const int32_t *place,
                                   int n_tokens, int p0, int m, uint8_t *stage, cudaStream_t st);
-int launch_stage_in(void *dq, const void *sq, size_t q_bytes, void *dk, const void *sk, void *dv, const void *sv,
-                    size_t kv_bytes, cudaStream_t st);
+int launch_stage_in(void *dq, const void *sq, size_t q_bytes, cudaStream_t st);
 int launch_copy_centroids(const DevCtx &c, int req, int layer, const __nv_bfloat16 *cen,
                           int n_clusters, cudaStream_t st);
 int launch_select(const DevCtx &c, Batch &b, const __nv_bfloat16 *q, const __nv_bfloat16 *k_new,
