@@ -6,8 +6,11 @@
 // turn, so every warp has its share of the missed pages (which lead the list) and of the hits.
 // A warp keeps two pages in flight in shared memory and one accumulator over all its pages; the
 // CTA writes one partial.  A page (8 KiB: 16 K rows, then 16 V rows) is brought in by one
-// instruction, a 256-byte bulk copy (TMA) per lane, each row to its own place at a stride of 272
-// bytes, which is what lets ldmatrix read 8 rows without a bank conflict; it comes from an HBM
+// instruction, a 512-byte bulk copy (TMA) per lane of half the warp, each pair of rows to its own
+// place at a stride of 528 bytes; a tile takes the even tokens as its rows 0..7 and the odd ones as
+// rows 8..15, so ldmatrix reads 8 rows without a bank conflict.  (256 sets of 56 pages, 8 heads:
+// 24.0 us; with a copy per row, twice as many for the SM's one copy unit, 32; per four rows, at a
+// two-way conflict, 26.5; per page, at an eight-way conflict, 59.)  The page comes from an HBM
 // slot for a hit and straight from pinned host memory for a miss, so the missed pages of the step
 // are on the host link while the hits are being attended from HBM.  A missed page that was
 // admitted to the cache goes from shared memory to its HBM slot by bulk copies too (that is the
@@ -35,8 +38,9 @@ __device__ __forceinline__ void dbg_ta(int, int) {}
 namespace {
 
 constexpr int kAttnWarps = 4, kAttnThreads = kAttnWarps * 32;
-constexpr int kStageRow = kRowBytes + 16;                  // a row of a staged page: 8 rows' 16-byte pieces fall into 8 bank groups
-constexpr int kStageBytes = 2 * kPageTokens * kStageRow;   // 32 rows
+constexpr int kPairs = kPageTokens, kPairBytes = 2 * kRowBytes;   // pairs of rows of a page: 8 of K, 8 of V
+constexpr int kPairStride = kPairBytes + 16;               // 8 pairs' 16-byte pieces fall into 8 bank groups
+constexpr int kStageBytes = kPairs * kPairStride;
 constexpr int kWarpStages = 2;
 constexpr int kAttnSmem = kAttnWarps * kWarpStages * kStageBytes;
 static_assert(kAttnSmem == kAttnCtaSmem, "what the scoring launcher leaves room for");
@@ -70,12 +74,13 @@ __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
   return *reinterpret_cast<uint32_t *>(&v);
 }
 
-// One warp requests one page: lane r copies row r (256 bytes); the stage's mbarrier counts the bytes.
+// One warp requests one page: lane i copies pair i of its rows; the stage's mbarrier counts the bytes.
 __device__ __forceinline__ void request_page(uint32_t sdst, uint32_t bar, const uint8_t *src, int lane) {
   if (lane == 0) asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n" ::"r"(bar), "r"(kPageBytes) : "memory");
   __syncwarp();
-  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];\n"
-               ::"r"(sdst + lane * kStageRow), "l"(src + lane * kRowBytes), "r"(kRowBytes), "r"(bar) : "memory");
+  if (lane < kPairs)
+    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];\n"
+                 ::"r"(sdst + lane * kPairStride), "l"(src + lane * kPairBytes), "r"(kPairBytes), "r"(bar) : "memory");
 }
 // Pages that other SMs have written with ordinary stores and announced by a flag may now be read by
 // bulk copies.
@@ -108,8 +113,8 @@ struct WarpAcc {
 __device__ __forceinline__ void attend_page(uint32_t spage, const uint32_t (&qb)[8][2], uint32_t mask,
                                             float scale2, WarpAcc &acc, int lane) {
   const int mat = lane >> 3, r8 = lane & 7;
-  const uint32_t krow = spage + (uint32_t)((r8 + ((mat & 1) << 3)) * kStageRow + (mat >> 1) * 16);
-  const uint32_t vrow = spage + (uint32_t)((kPageTokens + r8 + ((mat >> 1) << 3)) * kStageRow + (mat & 1) * 16);
+  const uint32_t krow = spage + (uint32_t)(r8 * kPairStride + (mat & 1) * kRowBytes + (mat >> 1) * 16);
+  const uint32_t vrow = spage + (uint32_t)((kPairs / 2 + r8) * kPairStride + (mat >> 1) * kRowBytes + (mat & 1) * 16);
   float s[4] = {0.f, 0.f, 0.f, 0.f}, s_odd[4] = {0.f, 0.f, 0.f, 0.f};      // two chains: half the serial mma latency
 #pragma unroll
   for (int ks = 0; ks < 8; ks += 2) {
@@ -121,8 +126,9 @@ __device__ __forceinline__ void attend_page(uint32_t spage, const uint32_t (&qb)
   }
 #pragma unroll
   for (int i = 0; i < 4; ++i) s[i] += s_odd[i];
-  // this lane's tokens: lane / 4 (s[0], s[1]) and lane / 4 + 8 (s[2], s[3])
-  const bool t0 = (mask >> (lane >> 2)) & 1u, t1 = (mask >> ((lane >> 2) + 8)) & 1u;
+  // this lane's tokens: 2 * (lane / 4) (tile row lane / 4: s[0], s[1]) and the next (row + 8: s[2], s[3])
+  const uint32_t pair = mask >> (2 * (lane >> 2));
+  const bool t0 = pair & 1u, t1 = pair & 2u;
   float corr[2];
 #pragma unroll
   for (int h = 0; h < 2; ++h) {
@@ -152,10 +158,11 @@ __device__ __forceinline__ void attend_page(uint32_t spage, const uint32_t (&qb)
   }
 }
 
-// Retrieve step 4 for one admitted miss: the staged page goes to its HBM slot, lane r moving row r.
+// Retrieve step 4 for one admitted miss: the staged page goes to its HBM slot, lane i moving pair i.
 __device__ __forceinline__ void store_page(uint32_t spage, uint8_t *dst, int lane) {
-  asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;\ncp.async.bulk.commit_group;\n"
-               ::"l"(dst + lane * kRowBytes), "r"(spage + lane * kStageRow), "r"(kRowBytes) : "memory");
+  if (lane < kPairs)
+    asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;\ncp.async.bulk.commit_group;\n"
+                 ::"l"(dst + lane * kPairBytes), "r"(spage + lane * kPairStride), "r"(kPairBytes) : "memory");
 }
 // The lane's copies out of shared memory have read their source.
 __device__ __forceinline__ void stores_read() { asm volatile("cp.async.bulk.wait_group.read 0;\n" ::: "memory"); }
@@ -598,8 +605,8 @@ void launch_attn_g(const DevCtx &c, const Batch &b, const __nv_bfloat16 *q, __nv
   // As many CTAs per set as the GPU holds at once (444), and at least 8 pages for each: every CTA is
   // resident, its pages stream through its stages, and CTAs share HBM by what they have in flight,
   // so equal shares end together.  256 sets of 56 pages, 8 heads: 57.7 us with a CTA per 8 pages
-  // (four waves), 35.3 us with one CTA per set; 128 sets of 65 pages: lists complete to merged
-  // 34 us -> 20 us.
+  // (four waves), 24 us with one CTA per set; 128 sets of 65 pages: lists complete to merged
+  // 34 us -> 17 us.
   int rows = resident / n_sets;
   rows = rows < (max_pages + kCtaPages - 1) / kCtaPages ? rows : (max_pages + kCtaPages - 1) / kCtaPages;
   if (rows > c.max_chunks) rows = c.max_chunks;

@@ -23,7 +23,7 @@ enum : int { kKindPage = 0, kKindToken = 1, kKindCluster = 2, kKindPageMean = 3 
 // sticky device error bits (same values as SPIN_DEV_ERR_* of the public header)
 constexpr unsigned kErrBounds = 1u, kErrPageList = 2u, kErrTimeout = 4u, kErrState = 8u;
 constexpr int kChunkPages = 8;                              // a set of n pages has room for ceil(n / 8) attention partials
-constexpr int kAttnCtaSmem = 8 * 2 * kPageTokens * (kRowBytes + 16);   // staged pages of an attention CTA
+constexpr int kAttnCtaSmem = 8 * kPageTokens * (2 * kRowBytes + 16);   // staged pages of an attention CTA
 
 // Per-set scalars (device resident, updated only by kernels).
 struct SetState {
