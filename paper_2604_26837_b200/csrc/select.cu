@@ -259,14 +259,19 @@ __device__ __forceinline__ void score_item(const DevCtx &c, const Batch &bt, con
   // ---- fused continuation: the last CTA of the set to arrive selects and manages the cache ----
   __shared__ union { struct { TopkShared t; CacheShared c; } staged; FastShared fast; } shm;
   __shared__ int s_last;
-  __threadfence();
+  // (one thread's release and acquire, between two barriers, order every thread's scores before the
+  // count and the count before every thread's reads: a fence by all threads on either side costs
+  // the set ~1 us)
   __syncthreads();
-  if (threadIdx.x == 0) s_last = atomicAdd(&c.sel_count[b], 1) == segs_here - 1;
+  if (threadIdx.x == 0) {
+    int before;
+    asm volatile("atom.acq_rel.gpu.global.add.s32 %0, [%1], 1;\n" : "=r"(before) : "l"(c.sel_count + b) : "memory");
+    s_last = before == segs_here - 1;
+    if (s_last) c.sel_count[b] = 0;                         // ready for the next step
+  }
   __syncthreads();
   if (!s_last) return;
   dbg_ts(b, 9);
-  __threadfence();
-  if (threadIdx.x == 0) c.sel_count[b] = 0;                 // ready for the next step
   if (fuse == 3) {
     // selection runs in the cluster kernel behind this one: tell it that this set is scored
     if (threadIdx.x == 0) flag_publish(c.scored + b, bt.epoch);
