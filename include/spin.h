@@ -325,7 +325,7 @@ SPIN_API int spin_debug_read_page(spin_ctx *ctx, int32_t req, int32_t layer, int
  * memory budget, or on a path where touching an allocator is forbidden -- and therefore
  * cannot create a context, whose scratch comes out of a caller-allocated pool).
  * It runs the same split-K attention + log-sum-exp merge as spin_decode_step's last stage over
- * page lists the caller supplies; the split-K partials and counters use an 8 MiB array built into the
+ * page lists the caller supplies; the split-K partials use an 8 MiB array built into the
  * library image (every GPU that loads the library holds it until the process exits).
  *   q, out      bf16 [n_sets][group][128], device pointers (out is written)
  *   page_pool   device pointer to 8 KiB pages: 16 K rows then 16 V rows of 128 bf16
@@ -342,10 +342,10 @@ SPIN_API int spin_debug_read_page(spin_ctx *ctx, int32_t req, int32_t layer, int
  * nothing is launched.
  * The first call on each device looks up the built-in array's device address (no allocation);
  * make that first call outside any stream capture.  Asynchronous on cuda_stream.  All calls
- * share the one array and it keeps the previous call's contents; the call clears the per-set
- * arrival counters at its start (the only part that must begin at zero) and overwrites what
- * else it later reads, but two calls whose kernels can overlap on the GPU (different streams,
- * no ordering) would race on it. */
+ * share the one array and it keeps the previous call's contents; a call overwrites what it later
+ * reads (the per-set arrival words, which have an array of their own, are zero between calls),
+ * but two calls whose kernels can overlap on the GPU (different streams, no ordering) would race
+ * on it. */
 SPIN_API int spin_paged_attention_static(const void *q, const void *page_pool,
                                          const int32_t *page_ids, const uint32_t *page_masks,
                                          const int32_t *n_pages, int32_t n_sets,

@@ -228,6 +228,16 @@ __device__ __forceinline__ uint2 normalised(float4 o, float l) {
   return make_uint2(pack_bf16(o.x / l, o.y / l), pack_bf16(o.z / l, o.w / l));
 }
 
+// Four outputs to the caller's buffer, which need not be aligned to more than an element.
+__device__ __forceinline__ void store_out(__nv_bfloat16 *dst, uint2 v) {
+  if ((reinterpret_cast<uintptr_t>(dst) & 7) == 0) {
+    *reinterpret_cast<uint2 *>(dst) = v;
+  } else {
+    uint16_t *d = reinterpret_cast<uint16_t *>(dst);
+    d[0] = (uint16_t)v.x; d[1] = (uint16_t)(v.x >> 16); d[2] = (uint16_t)v.y; d[3] = (uint16_t)(v.y >> 16);
+  }
+}
+
 // Counts the calling CTA in as one of the set's n_rows; true for the last one.  One thread calls it,
 // between two CTA barriers: its release orders the CTA's partials before the count, its acquire the
 // count before the CTA's reads of the other rows' partials.  The counters of a decode step are
@@ -321,7 +331,7 @@ __device__ __forceinline__ void merge_rows(const DevCtx &c, int b, int n_rows, _
         den = fmaf(o[kHeadDim + 1], a, den);
       }
     }
-    reinterpret_cast<uint2 *>(out_rows + (size_t)g * kHeadDim)[lane] = normalised(acc, den);
+    store_out(out_rows + (size_t)g * kHeadDim + 4 * lane, normalised(acc, den));
   }
 }
 
@@ -369,7 +379,7 @@ __device__ __forceinline__ void attn_cta(const DevCtx &c, const Batch &bt, const
   __nv_bfloat16 *out_rows = out + ((size_t)i_req * c.Hq + head * G) * kHeadDim;
   if (np == 0) {                           // nothing to attend: the set's rows are zero
     if (row == 0)
-      for (int e = threadIdx.x; e < G * kHeadDim / 4; e += kAttnThreads) reinterpret_cast<uint2 *>(out_rows)[e] = make_uint2(0u, 0u);
+      for (int e = threadIdx.x; e < G * kHeadDim / 4; e += kAttnThreads) store_out(out_rows + 4 * e, make_uint2(0u, 0u));
     return;
   }
   const int n_rows = min(max_rows, (np + kCtaPages - 1) / kCtaPages);       // CTAs that share this set
@@ -558,7 +568,7 @@ __device__ __forceinline__ void attn_cta(const DevCtx &c, const Batch &bt, const
       l = fmaf(s_l[w][g], a, l);
     }
     if (n_rows == 1) {                     // the set's only CTA finishes here
-      reinterpret_cast<uint2 *>(out_rows)[e] = normalised(o, l);
+      store_out(out_rows + 4 * e, normalised(o, l));
     } else {
       const size_t at = ((size_t)b * c.max_chunks + row) * G + g;
       reinterpret_cast<float4 *>(c.att_part)[at * (kHeadDim / 4) + col] = o;

@@ -171,6 +171,7 @@ int launch_reindex_apply(const DevCtx &c, int req, int layer, int n_clusters, in
   ReindexArgs a{req, layer, n_clusters, n_folded_pages, tail_first, tail_pages, tail_len, n_host_pages};
   const int n = n_clusters > n_host_pages ? n_clusters : n_host_pages;
   const size_t smem = (size_t)c.tail_cap * 4 + (size_t)((n_clusters + 31) / 32) * 4;
+  if (smem > 48 * 1024) cudaFuncSetAttribute(k_reindex_apply, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   k_reindex_apply<<<dim3((n + 255) / 256, c.Hkv), 256, smem, st>>>(c, a, assign);
   return 1;
 }

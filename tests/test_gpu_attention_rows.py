@@ -46,3 +46,24 @@ def test_attention_split_edges(sets, group, pages):
     assert err <= 2.0 ** -8 * max(1.0, want.abs().max().item()) * 2, err
     if sets > 4:
         assert not out[4].any()
+
+
+@pytest.mark.parametrize("sets,pages", [(3, 5), (2, 40)])
+def test_outputs_need_no_more_than_element_alignment(sets, pages):
+    import paper_2604_26837_b200 as P
+    g = torch.Generator(device="cuda").manual_seed(sets)
+    pool = torch.randn(sets * pages, 2, 16, 128, dtype=torch.bfloat16, device="cuda", generator=g)
+    ids = torch.arange(sets * pages, dtype=torch.int32, device="cuda").view(sets, pages)
+    masks = torch.full((sets, pages), 0xFFFF, dtype=torch.int32, device="cuda")
+    counts = torch.full((sets,), pages, dtype=torch.int32, device="cuda")
+    counts[-1] = 0
+    q = torch.randn(sets, 4, 128, device="cuda", generator=g).to(torch.bfloat16)
+    outs = []
+    for offset in (0, 1):                    # whole pieces; one element further on
+        buf = torch.full((q.numel() + 8,), 7.0, dtype=torch.bfloat16, device="cuda")
+        out = buf[offset:offset + q.numel()]
+        assert P.spin_paged_attention_static(q, pool, ids, masks, counts, sets, pages, 4, 0.0, out) == 0
+        torch.cuda.synchronize()
+        assert (buf[:offset] == 7).all() and (buf[offset + q.numel():] == 7).all()
+        outs.append(out.clone())
+    assert torch.equal(outs[0], outs[1])
