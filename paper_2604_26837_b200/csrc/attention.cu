@@ -109,7 +109,7 @@ struct WarpAcc {
   float o[8][4];              // 16-channel tiles: channels lane / 4 (+ 8), heads as above: [0], [1] resp. [2], [3]
 };
 
-// Attend one staged page: S^T = K Q^T (16 tokens x 8 heads), online softmax, O^T += V^T P^T.
+// Attend one staged page: S^T = K Q^T (16 tokens x 8 heads), online softmax, O^T = corr O^T + beta V^T P^T.
 __device__ __forceinline__ void attend_page(uint32_t spage, const uint32_t (&qb)[8][2], uint32_t mask,
                                             float scale2, WarpAcc &acc, int lane) {
   const int mat = lane >> 3, r8 = lane & 7;
@@ -129,7 +129,12 @@ __device__ __forceinline__ void attend_page(uint32_t spage, const uint32_t (&qb)
   // this lane's tokens: 2 * (lane / 4) (tile row lane / 4: s[0], s[1]) and the next (row + 8: s[2], s[3])
   const uint32_t pair = mask >> (2 * (lane >> 2));
   const bool t0 = pair & 1u, t1 = pair & 2u;
-  float corr[2];
+  // A page's probabilities are taken against the page's own maximum, and its outputs then scaled into
+  // the accumulator in 32 bits: the heaviest token of every page enters the bf16 tiles as exactly 1,
+  // so what bf16 costs does not grow with the length of a warp's list.  (Against fp64, 256 sets of 56
+  // pages, 8 heads, relative 2-norm: 2.12e-3 with a running maximum over the list, 1.95e-3 with this, at 24.8 us
+  // instead of 24.0.)
+  float corr[2], beta[2];
 #pragma unroll
   for (int h = 0; h < 2; ++h) {
     s[h] = t0 ? s[h] * scale2 : -INFINITY;
@@ -140,10 +145,12 @@ __device__ __forceinline__ void attend_page(uint32_t spage, const uint32_t (&qb)
     mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 16));
     const float mn = fmaxf(acc.m[h], mx);
     const float base = mn == -INFINITY ? 0.f : mn;         // all masked so far: every p is 0
+    const float own = mx == -INFINITY ? 0.f : mx;
     corr[h] = exp2f(acc.m[h] - base);                      // acc.m = -inf -> 0
-    s[h] = exp2f(s[h] - base);
-    s[2 + h] = exp2f(s[2 + h] - base);
-    acc.l[h] = acc.l[h] * corr[h] + (s[h] + s[2 + h]);
+    beta[h] = exp2f(mx - base);                            // the page all masked -> 0
+    s[h] = exp2f(s[h] - own);
+    s[2 + h] = exp2f(s[2 + h] - own);
+    acc.l[h] = acc.l[h] * corr[h] + (s[h] + s[2 + h]) * beta[h];
     acc.m[h] = mn;
   }
   // P (token rows, head columns) transposed into the B operand
@@ -152,9 +159,10 @@ __device__ __forceinline__ void attend_page(uint32_t spage, const uint32_t (&qb)
   for (int nt = 0; nt < 8; ++nt) {
     uint32_t a0, a1, a2, a3;
     ldmatrix_x4_trans(vrow + nt * 32, a0, a1, a2, a3);
-    acc.o[nt][0] *= corr[0]; acc.o[nt][1] *= corr[1];
-    acc.o[nt][2] *= corr[0]; acc.o[nt][3] *= corr[1];
-    mma_bf16(acc.o[nt], a0, a1, a2, a3, b0, b1);
+    float d[4] = {0.f, 0.f, 0.f, 0.f};
+    mma_bf16(d, a0, a1, a2, a3, b0, b1);
+    acc.o[nt][0] = fmaf(d[0], beta[0], acc.o[nt][0] * corr[0]); acc.o[nt][1] = fmaf(d[1], beta[1], acc.o[nt][1] * corr[1]);
+    acc.o[nt][2] = fmaf(d[2], beta[0], acc.o[nt][2] * corr[0]); acc.o[nt][3] = fmaf(d[3], beta[1], acc.o[nt][3] * corr[1]);
   }
 }
 

@@ -67,3 +67,33 @@ def test_outputs_need_no_more_than_element_alignment(sets, pages):
         assert (buf[:offset] == 7).all() and (buf[offset + q.numel():] == 7).all()
         outs.append(out.clone())
     assert torch.equal(outs[0], outs[1])
+
+
+@pytest.mark.parametrize("sets,group,pages,sharpness", [(256, 8, 56, 1.0), (256, 2, 64, 1.0), (60, 1, 200, 1.0), (230, 8, 60, 2.0), (8, 4, 40, 1.0)])
+def test_rounding_of_probabilities_does_not_grow_with_the_list(sets, group, pages, sharpness):
+    """Error against fp64, beside that of the same sums with probabilities rounded to bf16 against the
+    largest of every 32 tokens (a warp's two pages of eight): the kernel's may not be larger.  Both are sums of many
+    independent roundings, so over sets * group * 128 >= 4096 outputs they agree to 1 / sqrt(2 * 4096) ~ 1 %."""
+    import paper_2604_26837_b200 as P
+    g = torch.Generator(device="cuda").manual_seed(sets + pages)
+    pool = torch.randn(sets * pages, 2, 16, 128, dtype=torch.bfloat16, device="cuda", generator=g)
+    ids = torch.randperm(sets * pages, device="cuda", generator=g).to(torch.int32).view(sets, pages).contiguous()
+    masks = torch.full((sets, pages), 0xFFFF, dtype=torch.int32, device="cuda")
+    counts = torch.full((sets,), pages, dtype=torch.int32, device="cuda")
+    q = (torch.randn(sets, group, 128, device="cuda", generator=g) * sharpness).to(torch.bfloat16)
+    out = torch.empty_like(q)
+    assert P.spin_paged_attention_static(q, pool, ids, masks, counts, sets, pages, group, 0.0, out) == 0
+    torch.cuda.synchronize()
+    err, err32, norm = 0.0, 0.0, 0.0
+    for i in range(sets):
+        rows = pool[ids[i].long()].double()
+        k, v = rows[:, 0].reshape(-1, 128), rows[:, 1].reshape(-1, 128)
+        s = q[i].double() @ k.T / np.sqrt(128.0)
+        want = torch.softmax(s, dim=-1) @ v
+        base = s.view(group, -1, 32).amax(-1, keepdim=True).expand(-1, -1, 32).reshape(s.shape)
+        p, scale = torch.exp(s - base), torch.exp(base - s.amax(-1, keepdim=True))
+        rounded = ((p.to(torch.bfloat16).double() * scale) @ v / (p * scale).sum(-1, keepdim=True)).to(torch.bfloat16)
+        err += (out[i].double() - want).square().sum().item()
+        err32 += (rounded.double() - want).square().sum().item()
+        norm += want.square().sum().item()
+    assert err <= err32 * 1.02, ((err / norm) ** 0.5, (err32 / norm) ** 0.5)
