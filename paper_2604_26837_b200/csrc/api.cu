@@ -329,7 +329,7 @@ int ensure_seg(spin_ctx *ctx, BitmapPool &pool, std::vector<int32_t> &dir, int32
     if (s < 0) return -1;
     dir[di] = (int32_t)s;
     ctx->dir_bytes_in_use += 4;
-    ctx->dir_updates.push_back(DirUpdate{(int32_t)(dev_dir_row + di - ctx->d.dir_meta), (int32_t)s});
+    ctx->dir_updates.push_back(dir_update(ctx->d.dir_meta, dev_dir_row + di, (int32_t)s));
   }
   return dir[di];
 }

@@ -200,11 +200,11 @@ k_copy_centroids(DevCtx c, int req, int layer, const __nv_bfloat16 *__restrict__
 }
 
 // Directory entries, carried in the kernel's parameters.
-constexpr int kDirBatch = 448;                       // 3.5 KB of parameters
-struct DirBatch { int32_t n; DirUpdate u[kDirBatch]; };
+constexpr int kDirBatch = 336;                       // 4 KB of parameters
+struct DirBatch { int64_t at[kDirBatch]; int32_t value[kDirBatch]; int32_t n; };
 __global__ void __launch_bounds__(256)
 k_dir_update(int32_t *__restrict__ dirs, const __grid_constant__ DirBatch a) {
-  for (int i = threadIdx.x; i < a.n; i += 256) dirs[a.u[i].at] = a.u[i].value;
+  for (int i = threadIdx.x; i < a.n; i += 256) dirs[a.at[i]] = a.value[i];
 }
 
 // A step's queries that live in pinned host memory are brought into the staging buffer by a small
@@ -230,7 +230,7 @@ int launch_dir_update(const DevCtx &c, const DirUpdate *u, int n, cudaStream_t s
   for (int i = 0; i < n; i += kDirBatch, ++launched) {
     DirBatch a;
     a.n = n - i < kDirBatch ? n - i : kDirBatch;
-    for (int j = 0; j < a.n; ++j) a.u[j] = u[i + j];
+    for (int j = 0; j < a.n; ++j) { a.at[j] = u[i + j].at; a.value[j] = u[i + j].value; }
     k_dir_update<<<1, 256, 0, st>>>(c.dir_meta, a);
   }
   return launched;

@@ -366,7 +366,11 @@ struct AppendEdgeArgs {     // one (request) per entry; all its kv heads are pro
   int32_t req[kMaxBatch];
   int32_t n_tokens[kMaxBatch];   // tokens of the request before this append, as the host has counted them
 };
-struct DirUpdate { int32_t at, value; };   // a directory entry: index from dir_meta (the five directories share one region), new value
+// A directory entry to be written: its index from dir_meta (the five directories follow one another in the
+// context's pool) and its value.  The index is 64 bits wide: 256 requests of 80 layers and 8 heads with a million
+// tokens each and 16-entry segments have 3.4e9 words of directories.
+struct DirUpdate { int64_t at; int32_t value; };
+inline DirUpdate dir_update(const int32_t *dirs, const int32_t *entry, int32_t value) { return DirUpdate{(int64_t)(entry - dirs), value}; }
 int launch_dir_update(const DevCtx &c, const DirUpdate *u, int n, cudaStream_t st);
 int launch_append_bulk(const DevCtx &c, int req, int layer, const __nv_bfloat16 *k,
                        const __nv_bfloat16 *v, int first_page, int n_pages, int first_token_of_call,
