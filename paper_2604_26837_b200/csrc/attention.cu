@@ -92,10 +92,16 @@ __device__ __forceinline__ bool page_test(uint32_t bar, uint32_t parity) {
   return __all_sync(0xffffffffu, done);
 }
 // Bounded wait for a stage: false (reported by the caller) if its copies have not landed after seconds.
-__device__ __forceinline__ bool page_landed(uint32_t bar, uint32_t parity) {
+// A warp that gives a page up waits once more, with the second limit, before its stages are used for
+// anything else (see the end of the page loop).
+#ifndef SPIN_LANDED_POLLS
+#define SPIN_LANDED_POLLS (1 << 22)
+#endif
+constexpr int kLandedPolls = SPIN_LANDED_POLLS, kDrainPolls = 1 << 22;
+__device__ __forceinline__ bool page_landed(uint32_t bar, uint32_t parity, int polls = kLandedPolls) {
   uint32_t done = 0;
 #pragma unroll 1
-  for (int spin = 0; spin < (1 << 22) && !done; ++spin)
+  for (int spin = 0; spin < polls && !done; ++spin)
     asm volatile("{\n.reg .pred p;\nmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\nselp.u32 %0, 1, 0, p;\n}\n"
                  : "=r"(done) : "r"(bar), "r"(parity) : "memory");
   return __all_sync(0xffffffffu, done);
@@ -408,7 +414,8 @@ __device__ __forceinline__ void attn_cta(const DevCtx &c, const Batch &bt, const
   // The warp's pages in batches of 32, a lane per page (one batch as a rule).  The order in which a
   // warp attends its pages is fixed: the hits of a batch, then its missed pages.
   uint32_t phases = 0;                     // parity of the next wait, a bit per stage
-  bool dead = false, listed = c.ready == nullptr, slots_known = listed;
+  bool dead = false, listed = c.ready == nullptr, slots_known = listed;    // dead: a wait has run out
+  uint32_t issued = 0, on_link = 0;        // stages whose page has been requested and not seen to land; whose page has a turn on the link
 #pragma unroll 1
   for (int p0 = mine; p0 < np && !dead; p0 += 32 * stride) {
     const int pos = p0 + lane * stride;
@@ -422,7 +429,6 @@ __device__ __forceinline__ void attn_cta(const DevCtx &c, const Batch &bt, const
     const bool early = pos < min(nm, np);
     const bool early0 = p0 < nm && !listed;
     int turn0 = 0, turn1 = 0, closed = 0;  // the stages' turns on the host link (lane 0's)
-    uint32_t issued = 0, on_link = 0;      // stages whose page has been requested; whose page has a turn on the link
     if (early0) { turn0 = link_turn(c, lane); closed = link_closed(c); on_link = 1u; }
     if (early) ref = page_ref(c, bt, b, i_req, head, pl, pos);
     if (early0 && link_open(turn0, closed)) { request(0, 0); issued = 1u; }
@@ -440,11 +446,11 @@ __device__ __forceinline__ void attn_cta(const DevCtx &c, const Batch &bt, const
       if (lane == 0) ok = flag_wait2(c, c.ready + b, c.tail_ready + b, bt.epoch);
       listed = __shfl_sync(0xffffffffu, ok, 0) != 0;
       pages_visible();
-      dead = !listed;                      // reported by the wait: the warp only sees off the copy it has in flight, and the CTA still arrives
+      if (!listed) { dead = true; break; } // reported by the wait: nothing more is requested
     }
-    if (pos < np && !early && !dead) ref = page_ref(c, bt, b, i_req, head, pl, pos);
+    if (pos < np && !early) ref = page_ref(c, bt, b, i_req, head, pl, pos);
     const bool from_host = ref.fill >= 0 || ref.src < 0;
-    const uint32_t here = __ballot_sync(0xffffffffu, pos < np && !dead), host = __ballot_sync(0xffffffffu, from_host) & here;
+    const uint32_t here = __ballot_sync(0xffffffffu, pos < np), host = __ballot_sync(0xffffffffu, from_host) & here;   // (lane 0 is here)
     if (row == 0 && p0 == mine) dbg_ta(b, 11);
     if (host == 0 && !early0) {
       // nothing to bring in (the usual batch): pages 0, 1, 2, ... through the two stages in turn
@@ -455,8 +461,9 @@ __device__ __forceinline__ void attn_cta(const DevCtx &c, const Batch &bt, const
       for (int j = 0; j < n; ++j) {
         const int st = j & 1;
         const uint32_t mask = __shfl_sync(0xffffffffu, ref.mask, j);
-        if (!page_landed(bar0 + 8 * st, (phases >> st) & 1u)) {             // the stages may still be written to: no more requests
+        if (!page_landed(bar0 + 8 * st, (phases >> st) & 1u)) {
           if (lane == 0) dev_error(c, kErrTimeout);
+          issued = 1u << st | (j + 1 < n ? 2u >> st : 0u);
           dead = true;
           break;
         }
@@ -485,20 +492,20 @@ __device__ __forceinline__ void attn_cta(const DevCtx &c, const Batch &bt, const
     for (;;) {
       // a free stage takes the next page: an HBM page is requested at once, a host page takes a turn on the link
       if (refill1) {
-        in1 = dead ? -1 : next();
+        in1 = next();
         if (in1 >= 0 && ((hosted >> in1) & 1u)) { turn1 = link_turn(c, lane); on_link |= 2u; }
         else if (in1 >= 0) { request(1, in1); issued |= 2u; }
         refill1 = false;
       }
       if (refill0) {                       // (no hits are left by then)
-        in0 = dead ? -1 : next();
+        in0 = next();
         if (in0 >= 0) { turn0 = link_turn(c, lane); on_link |= 1u; }
         refill0 = false;
       }
       const int j = cur ? in1 : in0;
       if (j < 0) break;
       const uint32_t waiting = on_link & ~issued;
-      if (waiting && !dead) {
+      if (waiting) {
         closed = link_closed(c);
         if ((waiting & 1u) && link_open(turn0, closed)) { request(0, in0); issued |= 1u; }
         if ((waiting & 2u) && link_open(turn1, closed)) { request(1, in1); issued |= 2u; }
@@ -506,34 +513,34 @@ __device__ __forceinline__ void attn_cta(const DevCtx &c, const Batch &bt, const
       // a missed page that has landed behind the hits gives its turn on
       if (hits_in1 > 0 && (on_link & issued & 1u) && page_test(bar0, phases & 1u)) { link_close(c, lane); on_link &= ~1u; }
       if (!((issued >> cur) & 1u)) {
-        if (!dead && ++polls < kLinkPolls) { __nanosleep(100); continue; }
-        if (!dead && lane == 0) dev_error(c, kErrTimeout);
+        if (++polls < kLinkPolls) { __nanosleep(100); continue; }
+        if (lane == 0) dev_error(c, kErrTimeout);
         dead = true;
-      } else {
-        if (((hosted >> j) & 1u) && !slots_known && !dead) {                // while the page is on its way
-          int ok = 1;
-          if (lane == 0) ok = flag_wait(c, c.slots_ready + b, bt.epoch);
-          slots_known = __shfl_sync(0xffffffffu, ok, 0) != 0;               // else reported: open pages are attended, not kept
-          slot_page = ref.open_idx < 0 ? slot_page : slots_known ? __ldcg(c.page_src + pl + ref.open_idx) : -1;   // negative: bypassed, attended only
-        }
-        if (!page_landed(bar0 + 8 * cur, (phases >> cur) & 1u)) {           // its stage may still be written to: no more requests
-          if (lane == 0) dev_error(c, kErrTimeout);
-          dead = true;
-        }
-        phases ^= 1u << cur;
+        break;
       }
+      if (((hosted >> j) & 1u) && !slots_known) {                           // while the page is on its way
+        int ok = 1;
+        if (lane == 0) ok = flag_wait(c, c.slots_ready + b, bt.epoch);
+        slots_known = __shfl_sync(0xffffffffu, ok, 0) != 0;
+        if (!slots_known) { dead = true; break; }                           // reported by the wait
+        if (ref.open_idx >= 0) slot_page = __ldcg(c.page_src + pl + ref.open_idx);   // negative: bypassed, attended only
+      }
+      if (!page_landed(bar0 + 8 * cur, (phases >> cur) & 1u)) {
+        if (lane == 0) dev_error(c, kErrTimeout);
+        dead = true;
+        break;
+      }
+      phases ^= 1u << cur;
       if (row == 0 && p0 == mine) dbg_ta(b, 12);
       if ((on_link >> cur) & 1u) link_close(c, lane);
       on_link &= ~(1u << cur);
       issued &= ~(1u << cur);
       const uint32_t spage = stage0 + cur * kStageBytes;
-      if (!dead) {
-        attend_page(spage, qb, __shfl_sync(0xffffffffu, ref.mask, j), scale2, acc, lane);
-        if ((hosted >> j) & 1u) {
-          const int slot = __shfl_sync(0xffffffffu, slot_page, j);
-          if (slot >= c.n_gpu_pages) { if (lane == 0) dev_error(c, kErrBounds); }
-          else if (slot >= 0) { store_page(spage, c.gpu_pages + (size_t)slot * kPageBytes, lane); stores_read(); }
-        }
+      attend_page(spage, qb, __shfl_sync(0xffffffffu, ref.mask, j), scale2, acc, lane);
+      if ((hosted >> j) & 1u) {
+        const int slot = __shfl_sync(0xffffffffu, slot_page, j);
+        if (slot >= c.n_gpu_pages) { if (lane == 0) dev_error(c, kErrBounds); }
+        else if (slot >= 0) { store_page(spage, c.gpu_pages + (size_t)slot * kPageBytes, lane); stores_read(); }
       }
       __syncwarp();                        // every lane has read the stage
       if (cur) refill1 = true; else refill0 = true;
@@ -542,6 +549,15 @@ __device__ __forceinline__ void attn_cta(const DevCtx &c, const Batch &bt, const
     }
   }
 
+  // Every way out of the loops above leads here: the list is done (no copy in flight, no turn open), or
+  // a wait has run out, for the list (at most stage 0's early page is in flight), for a turn, for the slots
+  // or for a page (one or both stages).  A copy in flight writes to a stage that the outputs are exchanged through
+  // below, so it is seen off first.
+  if (dead)
+    for (int st = 0; st < kWarpStages; ++st) {
+      if ((issued >> st) & 1u) page_landed(bar0 + 8 * st, (phases >> st) & 1u, kDrainPolls);
+      if ((on_link >> st) & 1u) link_close(c, lane);
+    }
   if (row == 0) dbg_ta(b, 13);
   // a head's sum lives in the 8 lanes of its column; the warps meet in their own (now idle) stage 0
   float *comb = reinterpret_cast<float *>(smem);
