@@ -445,6 +445,7 @@ __device__ __forceinline__ void attn_cta(const DevCtx &c, const Batch &bt, const
       int ok = 1;
       if (lane == 0) ok = flag_wait2(c, c.ready + b, c.tail_ready + b, bt.epoch);
       listed = __shfl_sync(0xffffffffu, ok, 0) != 0;
+      __syncwarp();                        // lane 0's acquire comes before every lane's reads of the list
       pages_visible();
       if (!listed) { dead = true; break; } // reported by the wait: nothing more is requested
     }
@@ -523,6 +524,7 @@ __device__ __forceinline__ void attn_cta(const DevCtx &c, const Batch &bt, const
         if (lane == 0) ok = flag_wait(c, c.slots_ready + b, bt.epoch);
         slots_known = __shfl_sync(0xffffffffu, ok, 0) != 0;
         if (!slots_known) { dead = true; break; }                           // reported by the wait
+        __syncwarp();                                                       // (as above)
         if (ref.open_idx >= 0) slot_page = __ldcg(c.page_src + pl + ref.open_idx);   // negative: bypassed, attended only
       }
       if (!page_landed(bar0 + 8 * cur, (phases >> cur) & 1u)) {
