@@ -1348,13 +1348,16 @@ static int step_impl(spin_ctx *ctx, int32_t layer, const int32_t *req_ids, int32
       ctx->launches += launch_append_edge(ctx->d, a, kk, vv, 1, st, &ctx->prof, ctx->stage_q, qc == 1 ? q_alias : nullptr, qbytes);
     }
   }
-  int64_t max_cand = 0, max_pages = 0;
+  int64_t max_cand = 0, max_pages = 0, est_pages = 0;
   for (int i = 0; i < n_req; ++i) {
     LayerHost &L = ctx->reqs[(size_t)req_ids[i]].layers[(size_t)layer];
     const int64_t cand = ctx->cfg.partition_kind == SPIN_PART_TOKEN_DOT ? (int64_t)L.n_partitions * kPageTokens : L.n_partitions;
     max_cand = std::max(max_cand, cand);
     int64_t pages = cluster ? ctx->g.max_pages : std::min<int64_t>(ctx->cfg.topk, L.n_partitions);
     max_pages = std::max(max_pages, pages + L.tail_pages);
+    // the clusters' average size is all the host knows of what topk of them will hold
+    const int64_t about = cluster ? ctx->cfg.topk * (L.n_tokens / ctx->cfg.num_clusters / kPageTokens + 1) : pages;
+    est_pages += (std::min(pages, about) + L.tail_pages) * ctx->cfg.num_kv_heads;
     L.last_batch_pos = i;
     b.tail_pages[i] = (int16_t)L.tail_pages;
     b.tail_len[i] = (int16_t)L.tail_len;
@@ -1376,7 +1379,7 @@ static int step_impl(spin_ctx *ctx, int32_t layer, const int32_t *req_ids, int32
   b.append_in_grid = in_grid ? 1 : 0;
   ctx->launches += launch_select(ctx->d, b, qd, kk, vv, (int)max_cand, st, &ctx->prof);
   ctx->launches += launch_fetch(ctx->d, st, ctx->sm_count, &ctx->prof);
-  ctx->launches += launch_attention(ctx->d, b, qd, od, (int)max_pages, st, &ctx->prof);
+  ctx->launches += launch_attention(ctx->d, b, qd, od, (int)max_pages, est_pages, st, &ctx->prof);
   if (oc == 2) CK(cudaMemcpyAsync(out, ctx->stage_out, qbytes, cudaMemcpyDeviceToHost, st));
   CK(cudaGetLastError());
   return SPIN_OK;

@@ -349,15 +349,75 @@ __device__ __forceinline__ void merge_rows(const DevCtx &c, int b, int n_rows, _
   }
 }
 
+// CTAs that share a list of np pages.  As a rule the set's part of the GPU; a list that would leave more than
+// `share` pages to each of those gets more, up to the grid's rows.
+__device__ __forceinline__ int attn_rows_of(const Batch &bt, int np, int share, int max_rows) {
+  const int most = min(max_rows, (np + kCtaPages - 1) / kCtaPages);
+  return min(most, max(bt.attn_rows, (np + share - 1) / share));
+}
+// Half as much again as a CTA's part of an average list.
+__host__ __device__ inline long long share_of(long long pages, long long n_sets, int rows) {
+  return (3 * pages + 2 * n_sets * rows - 1) / (2 * n_sets * rows);
+}
+
+// Lists whose lengths only the device knows (a set per request): every CTA takes the average from all
+// counts.  With half as much again as the average for a share, the further rows of all long lists
+// together are at most two thirds of the sets' own, and the grid has that many CTAs behind those,
+// which look up what is theirs.
+__device__ __forceinline__ int count_of(const DevCtx &c, int i) { return max(0, min(c.n_pages[i], c.max_pages)); }
+__device__ __forceinline__ int share_by_counts(const DevCtx &c, const Batch &bt, int *s_sum) {
+  int sum = 0;
+#pragma unroll 4
+  for (int i = threadIdx.x; i < bt.n_req; i += kAttnThreads) sum += count_of(c, i);
+  sum = __reduce_add_sync(0xffffffffu, sum);
+  if ((threadIdx.x & 31) == 0) s_sum[threadIdx.x >> 5] = sum;
+  __syncthreads();
+  long long pages = 0;
+#pragma unroll
+  for (int w = 0; w < kAttnWarps; ++w) pages += s_sum[w];
+  return max(bt.attn_share, (int)min(share_of(pages, bt.n_req, bt.attn_rows), 1ll << 30));
+}
+// The further row that is CTA x's to do, in the order of the sets; false: none.
+__device__ __forceinline__ bool further_row(const DevCtx &c, const Batch &bt, int share, int x, int *s_sum, int *s_at, int *b, int *row) {
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int per = (bt.n_req + kAttnThreads - 1) / kAttnThreads, first = threadIdx.x * per, last = min(bt.n_req, first + per);
+  auto further = [&](int i) { return max(0, attn_rows_of(bt, count_of(c, i), share, c.max_chunks) - bt.attn_rows); };
+  int mine = 0;
+#pragma unroll 4
+  for (int i = first; i < last; ++i) mine += further(i);
+  int before = mine;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int t = __shfl_up_sync(0xffffffffu, before, o);
+    if (lane >= o) before += t;
+  }
+  __syncthreads();                         // the sums have been read
+  if (lane == 31) s_sum[warp] = before;
+  if (threadIdx.x == 0) s_at[0] = -1;
+  __syncthreads();
+  before -= mine;
+  for (int w = 0; w < warp; ++w) before += s_sum[w];
+  if (x >= before && x < before + mine)
+    for (int i = first; i < last; ++i) {
+      const int more = further(i);
+      if (x < before + more) { s_at[0] = i; s_at[1] = bt.attn_rows + x - before; break; }
+      before += more;
+    }
+  __syncthreads();
+  *b = s_at[0]; *row = s_at[1];
+  return *b >= 0;
+}
+
 template <int G>
-__device__ __forceinline__ void attn_cta(const DevCtx &c, const Batch &bt, const __nv_bfloat16 *__restrict__ q,
-                                         __nv_bfloat16 *__restrict__ out, uint8_t *smem) {
+__device__ __forceinline__ void attn_row(const DevCtx &c, const Batch &bt, const __nv_bfloat16 *__restrict__ q,
+                                         __nv_bfloat16 *__restrict__ out, uint8_t *smem, int b, int row, int max_rows, int share) {
   __shared__ __align__(8) unsigned long long s_bar[kAttnWarps * kWarpStages];
   __shared__ float s_m[kAttnWarps][G], s_l[kAttnWarps][G];
   __shared__ int sh_ok, sh_np, sh_nm, sh_last;
-  // launch order: row 0 of every set first (the rows that own the first missed pages), or set by set
-  const int b = bt.attn_set_major ? blockIdx.y : blockIdx.x, row = bt.attn_set_major ? blockIdx.x : blockIdx.y;
-  const int max_rows = bt.attn_set_major ? gridDim.x : gridDim.y;
+  const int i_req = b / c.Hkv, head = b % c.Hkv;
+  int np_most = c.max_pages + c.tail_cap;  // pages that the set's list may have
+  if (c.ready && c.kind != kKindCluster) np_most = min(np_most, min(c.topk, bt.n_partitions[i_req]) + bt.tail_pages[i_req]);
+  if (row > 0 && row >= attn_rows_of(bt, np_most, bt.attn_share, max_rows)) return;       // no list of this set reaches this row
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const uint32_t bar0 = smem_u32(&s_bar[kWarpStages * warp]), stage0 = smem_u32(smem) + (uint32_t)(kWarpStages * warp) * kStageBytes;
   if (lane < kWarpStages) {
@@ -374,9 +434,9 @@ __device__ __forceinline__ void attn_cta(const DevCtx &c, const Batch &bt, const
     if (threadIdx.x == 0) {
       uint32_t word = 0;
       sh_ok = first_flag_wait(c, c.ready1 + b, bt.epoch, &word);
-      // a count beyond the list's stride can neither read past the set's row nor leave the merge
-      // waiting for rows that no CTA of the grid owns
-      sh_np = min((int)(word >> 12), c.max_pages + c.tail_cap);
+      // a count beyond what the set's list can have can neither read past the set's row nor leave
+      // the merge waiting for rows that have left
+      sh_np = min((int)(word >> 12), np_most);
       sh_nm = (int)(word & 4095u);
     }
     __syncthreads();
@@ -385,18 +445,17 @@ __device__ __forceinline__ void attn_cta(const DevCtx &c, const Batch &bt, const
     pages_visible();
   } else {
     pdl_wait_prev();
-    np = max(0, min(c.n_pages[b], c.max_pages + c.tail_cap));
+    np = max(0, min(c.n_pages[b], np_most));
     __syncwarp();
   }
   if (row == 0) dbg_ta(b, 10);
-  const int i_req = b / c.Hkv, head = b % c.Hkv;
   __nv_bfloat16 *out_rows = out + ((size_t)i_req * c.Hq + head * G) * kHeadDim;
   if (np == 0) {                           // nothing to attend: the set's rows are zero
     if (row == 0)
       for (int e = threadIdx.x; e < G * kHeadDim / 4; e += kAttnThreads) store_out(out_rows + 4 * e, make_uint2(0u, 0u));
     return;
   }
-  const int n_rows = min(max_rows, (np + kCtaPages - 1) / kCtaPages);       // CTAs that share this set
+  const int n_rows = attn_rows_of(bt, np, share, max_rows);
   if (row >= n_rows) return;
   const size_t pl = (size_t)b * (c.max_pages + c.tail_cap);
   const int stride = n_rows * kAttnWarps;                                   // the warp's pages: mine, mine + stride, ...
@@ -616,26 +675,40 @@ __device__ __forceinline__ void attn_cta(const DevCtx &c, const Batch &bt, const
 // go by the per-set flags never wait for the scoring kernel as a whole; with one CTA doing so
 // before it exits, this grid cannot complete ahead of that one, and whatever the stream runs
 // next (the next step's scoring kernel waits for this grid) comes after all of its writes.
-template <int G>
+template <int G, bool kCounted>
 __global__ void __launch_bounds__(kAttnThreads, 3)
 k_attn(DevCtx c, Batch bt, const __nv_bfloat16 *__restrict__ q, __nv_bfloat16 *__restrict__ out) {
   extern __shared__ __align__(128) uint8_t smem[];                // [warps][2] staged pages
   pdl_launch_next();
-  attn_cta<G>(c, bt, q, out, smem);
+  if (!kCounted) {
+    // launch order: row 0 of every set first (the rows that own the first missed pages), or set by set
+    const int b = bt.attn_set_major ? blockIdx.y : blockIdx.x, row = bt.attn_set_major ? blockIdx.x : blockIdx.y;
+    attn_row<G>(c, bt, q, out, smem, b, row, bt.attn_set_major ? gridDim.x : gridDim.y, bt.attn_share);
+  } else {
+    __shared__ int s_sum[kAttnWarps], s_at[2];
+    int b = blockIdx.x % bt.n_req, row = blockIdx.x / bt.n_req;
+    pdl_wait_prev();
+    const int share = share_by_counts(c, bt, s_sum), own = bt.n_req * bt.attn_rows;
+    if ((int)blockIdx.x < own || further_row(c, bt, share, (int)blockIdx.x - own, s_sum, s_at, &b, &row))
+      attn_row<G>(c, bt, q, out, smem, b, row, c.max_chunks, share);
+  }
   if (blockIdx.x == 0 && blockIdx.y == 0) pdl_wait_prev();
 }
 
+constexpr int kSharePages = 32, kExtraCtas = 2048;
 template <int G>
-void launch_attn_g(const DevCtx &c, const Batch &b, const __nv_bfloat16 *q, __nv_bfloat16 *out, int n_sets, int max_pages, cudaStream_t st) {
+void launch_attn_g(const DevCtx &c, Batch b, const __nv_bfloat16 *q, __nv_bfloat16 *out, int n_sets, int max_pages, long long est_pages, cudaStream_t st) {
   static int resident_dev[kMaxDevices] = {};
   int &resident = resident_dev[current_device_slot()];
   if (!resident) {
-    cudaFuncSetAttribute(k_attn<G>, cudaFuncAttributeMaxDynamicSharedMemorySize, kAttnSmem);
-    cudaFuncSetAttribute(k_attn<G>, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
+    for (auto kernel : {k_attn<G, false>, k_attn<G, true>}) {
+      cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kAttnSmem);
+      cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
+    }
     int dev = 0, sms = 0, per_sm = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_attn<G>, kAttnThreads, kAttnSmem);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_attn<G, false>, kAttnThreads, kAttnSmem);
     resident = sms * per_sm > 0 ? sms * per_sm : 148;
   }
   // As many CTAs per set as the GPU holds at once (444), and at least 8 pages for each: every CTA is
@@ -643,24 +716,43 @@ void launch_attn_g(const DevCtx &c, const Batch &b, const __nv_bfloat16 *q, __nv
   // so equal shares end together.  256 sets of 56 pages, 8 heads: 57.7 us with a CTA per 8 pages
   // (four waves), 24 us with one CTA per set; 128 sets of 65 pages: lists complete to merged
   // 34 us -> 17 us.
-  int rows = resident / n_sets;
-  rows = rows < (max_pages + kCtaPages - 1) / kCtaPages ? rows : (max_pages + kCtaPages - 1) / kCtaPages;
-  if (rows > c.max_chunks) rows = c.max_chunks;
-  if (rows < 1) rows = 1;
+  // Lists are not always equal.  One that leaves a CTA more than kSharePages and more than half as much
+  // again as the average list does is split further (256 lists, one of 500 pages and the rest of 8: 128 us
+  // without that, 17 with, 31 with a CTA per 8 pages; decode, 32 requests x 8 heads, one of 8192 tokens
+  // and the rest of 130: 152 us, 46, 74).  Below that a further split only costs: 256 lists of 56 pages, two
+  // CTAs each: 35 us instead of 25.  In a decode step the average is the host's estimate, and the grid has
+  // rows for the longest list it may meet, at most kExtraCtas of them, which leave at once where they
+  // are not needed (~1 ns each).  Where only the device knows the lengths, CTAs take the average from the
+  // counts, and fewer spare ones find out from them what is theirs; looking at the counts costs a call ~1 us
+  // (256 even lists of 56 pages: 26.0 us instead of 25.0), so it is done where a list may leave a CTA more than
+  // 2 kSharePages (445 lists, one of 64 pages and the rest of 8: 19 us without, 22 with).
+  auto clamp = [](long long x, long long lo, long long hi) { return (int)(x > hi ? hi : x < lo ? lo : x); };
+  const int chunks = clamp((max_pages + kCtaPages - 1) / kCtaPages, 1, c.max_chunks);
+  b.attn_rows = clamp(resident / n_sets, 1, chunks);
+  b.attn_share = clamp(share_of(est_pages, n_sets, b.attn_rows), kSharePages, 1 << 30);
+  int rows = clamp((max_pages + b.attn_share - 1) / b.attn_share, b.attn_rows, chunks);
+  if (!c.ready && max_pages > 2 * kSharePages * b.attn_rows) {
+    const int own = n_sets * b.attn_rows;
+    launch_pdl(k_attn<G, true>, dim3(own + own * 2 / 3), dim3(kAttnThreads), (size_t)kAttnSmem, st, 1, c, b, q, out);
+    return;
+  }
+  if (!c.ready) rows = b.attn_rows;
+  rows = clamp(rows, b.attn_rows, clamp(kExtraCtas / n_sets, b.attn_rows, chunks));
+  b.attn_share = clamp((max_pages + rows - 1) / rows, b.attn_share, 1 << 30);
   const dim3 grid = b.attn_set_major ? dim3(rows, n_sets) : dim3(n_sets, rows);
-  launch_pdl(k_attn<G>, grid, dim3(kAttnThreads), (size_t)kAttnSmem, st, 1, c, b, q, out);
+  launch_pdl(k_attn<G, false>, grid, dim3(kAttnThreads), (size_t)kAttnSmem, st, 1, c, b, q, out);
 }
 
 }  // namespace
 
 int launch_attention(const DevCtx &c, const Batch &b, const __nv_bfloat16 *q,
-                     __nv_bfloat16 *out, int max_pages_hint, cudaStream_t st, Prof *prof) {
+                     __nv_bfloat16 *out, int max_pages_hint, long long est_pages, cudaStream_t st, Prof *prof) {
   const int n_sets = b.n_req * c.Hkv;
   switch (c.G) {
-    case 1: launch_attn_g<1>(c, b, q, out, n_sets, max_pages_hint, st); break;
-    case 2: launch_attn_g<2>(c, b, q, out, n_sets, max_pages_hint, st); break;
-    case 4: launch_attn_g<4>(c, b, q, out, n_sets, max_pages_hint, st); break;
-    default: launch_attn_g<8>(c, b, q, out, n_sets, max_pages_hint, st); break;
+    case 1: launch_attn_g<1>(c, b, q, out, n_sets, max_pages_hint, est_pages, st); break;
+    case 2: launch_attn_g<2>(c, b, q, out, n_sets, max_pages_hint, est_pages, st); break;
+    case 4: launch_attn_g<4>(c, b, q, out, n_sets, max_pages_hint, est_pages, st); break;
+    default: launch_attn_g<8>(c, b, q, out, n_sets, max_pages_hint, est_pages, st); break;
   }
   prof_mark(prof, st, kProfAttnSplit);
   return 1;
@@ -759,7 +851,7 @@ extern "C" int spin_paged_attention_static(const void *q, const void *page_pool,
   Batch b{};
   b.n_req = n_sets;
   launch_attention(c, b, reinterpret_cast<const __nv_bfloat16 *>(q), reinterpret_cast<__nv_bfloat16 *>(out),
-                   list_stride, st, nullptr);
+                   list_stride, 0, st, nullptr);
   const cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) {
     fprintf(stderr, "spin_paged_attention_static: launch failed: %s\n", cudaGetErrorString(e));

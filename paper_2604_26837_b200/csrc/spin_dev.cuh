@@ -142,7 +142,8 @@ struct Batch {
   int32_t epoch;            // number of this decode call: value of the ready flags it sets
   int32_t append_in_grid;   // the scoring kernel's tail CTAs append this step's tokens
   int32_t attn_set_major;   // attention CTAs ordered set by set (sets become ready one after the
-                            // other over a long scoring phase) instead of chunk 0 of every set first
+                            // other over a long scoring phase) instead of row 0 of every set first
+  int32_t attn_rows, attn_share;   // attention: CTAs of a set as a rule; pages per CTA beyond which a list gets more (see attn_rows_of)
 };
 
 __host__ __device__ inline int set_index(const DevCtx &c, int req, int layer, int head) {
@@ -402,6 +403,6 @@ int launch_reindex_apply(const DevCtx &c, int req, int layer, int n_clusters, in
                          int tail_pages, int tail_len, int n_host_pages, const int32_t *assign, cudaStream_t st);
 size_t cache_smem_bytes(const DevCtx &c);
 int launch_attention(const DevCtx &c, const Batch &b, const __nv_bfloat16 *q,
-                     __nv_bfloat16 *out, int max_pages_hint, cudaStream_t st, Prof *prof);
+                     __nv_bfloat16 *out, int max_pages_hint, long long est_pages, cudaStream_t st, Prof *prof);   // est_pages: of all sets' lists together, about
 
 }  // namespace spin

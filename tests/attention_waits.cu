@@ -23,7 +23,7 @@ template <typename T> void put(T *d, const std::vector<T> &h) { cudaMemcpy(d, h.
 void scene(const char *name, int list, int slots, int early, int n_miss, int closed, bool timeout, bool zeros) {
   DevCtx c{};
   c.num_layers = 1; c.Hkv = 2; c.G = kG; c.Hq = 2 * kG;
-  c.max_pages = kList; c.tail_cap = 1; c.max_chunks = (kStride + kChunkPages - 1) / kChunkPages;
+  c.max_pages = c.topk = kList; c.tail_cap = 1; c.max_chunks = (kStride + kChunkPages - 1) / kChunkPages;
   c.sm_scale = 0.088f;
   c.n_gpu_pages = kGpuPages; c.n_host_pages = kHostPages;
   c.gpu_pages = device<uint8_t>((size_t)kGpuPages * kPageBytes, 0x3f);          // bf16 0.747
@@ -58,10 +58,11 @@ void scene(const char *name, int list, int slots, int early, int n_miss, int clo
   c.counters = device<Counters>(1);
   Batch bt{};
   bt.n_req = kSets / c.Hkv; bt.epoch = kEpoch;
+  for (int i = 0; i < bt.n_req; ++i) bt.n_partitions[i] = kList;
   __nv_bfloat16 *q = device<__nv_bfloat16>(kSets * kG * kHeadDim, 0x3c), *out = device<__nv_bfloat16>(kSets * kG * kHeadDim, 0x55);
   for (int call = 0; call < 2; ++call) {                                        // the second meets what the first has left
     cudaMemset(c.att_count, 0, kSets * 4);
-    launch_attention(c, bt, q, out, kList, nullptr, nullptr);
+    launch_attention(c, bt, q, out, kList, (long long)kSets * kList, nullptr, nullptr);
     cudaDeviceSynchronize();
   }
   const cudaError_t e = cudaDeviceSynchronize();

@@ -97,3 +97,92 @@ def test_rounding_of_probabilities_does_not_grow_with_the_list(sets, group, page
         err32 += (rounded.double() - want).square().sum().item()
         norm += want.square().sum().item()
     assert err <= err32 * 1.02, ((err / norm) ** 0.5, (err32 / norm) ** 0.5)
+
+
+def _lists(sets, group, pages, counts, seed=5):
+    g = torch.Generator(device="cuda").manual_seed(seed)
+    pool = torch.randn(sets * pages, 2, 16, 128, dtype=torch.bfloat16, device="cuda", generator=g)
+    ids = torch.randperm(sets * pages, device="cuda", generator=g).to(torch.int32).view(sets, pages).contiguous()
+    masks = torch.full((sets, pages), 0xFFFF, dtype=torch.int32, device="cuda")
+    q = torch.randn(sets, group, 128, device="cuda", generator=g).to(torch.bfloat16)
+    return q, pool, ids, masks, torch.tensor(counts, dtype=torch.int32, device="cuda")
+
+
+@pytest.mark.parametrize("sets,group,pages,short,long", [
+    (256, 1, 500, 8, {17: 500, 200: 499}),                  # 16 rows where one is the rule, done by other lists' CTAs
+    (256, 1, 500, 8, {i: 500 for i in range(100, 256, 2)}), # further rows of many lists
+    (64, 1, 500, 9, {0: 500, 63: 65}),                      # 16 rows where six are the rule
+    (64, 8, 248, 9, {0: 248, 63: 65}),                      # lists too short for the counts to be looked at
+    (700, 1, 180, 3, {0: 180, 1: 33, 698: 95, 699: 97}),    # more sets than CTAs at once
+    (223, 2, 280, 0, {5: 280}),                             # nothing in the other lists
+    (1790, 1, 72, 1, {0: 72, 1789: 33}), (2048, 1, 56, 1, {0: 56, 2047: 33}),   # the most sets that the built-in arrays take with such lists
+])
+def test_uneven_lists(sets, group, pages, short, long):
+    import paper_2604_26837_b200 as P
+    counts = [long.get(i, short) for i in range(sets)]
+    q, pool, ids, masks, n = _lists(sets, group, pages, counts)
+    out = torch.full_like(q, 7.0)
+    for _ in range(2):
+        assert P.spin_paged_attention_static(q, pool, ids, masks, n, sets, pages, group, 0.0, out) == 0
+    torch.cuda.synchronize()
+    for i in list(long) + [2, 3, sets // 2]:
+        rows = pool[ids[i, :counts[i]].long()].double()
+        s = q[i].double() @ rows[:, 0].reshape(-1, 128).T / np.sqrt(128.0)
+        want = torch.softmax(s, dim=-1) @ rows[:, 1].reshape(-1, 128)
+        assert (out[i].double() - want).abs().max().item() <= 2.0 ** -7 * max([1.0] + want.abs().flatten().tolist()), i
+
+
+def _best_us(f, calls=20):
+    best = 1e9
+    for _ in range(6):
+        e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+        torch.cuda.synchronize()
+        e0.record()
+        for _ in range(calls):
+            f()
+        e1.record()
+        torch.cuda.synchronize()
+        best = min(best, e0.elapsed_time(e1) * 1e3 / calls)
+    return best
+
+
+def test_a_long_list_among_short_ones_is_shared():
+    """The batch takes about what its long list and its short ones take by themselves, not what four warps need for 500 pages
+    (measured: 25 us, 8 + 7 apart, 128 where every set had one CTA)."""
+    import paper_2604_26837_b200 as P
+
+    def us(sets, counts):
+        a = _lists(sets, 1, 500, counts)
+        out = torch.empty_like(a[0])
+        return _best_us(lambda: P.spin_paged_attention_static(*a, sets, 500, 1, 0.0, out))
+    both, alone = us(256, [8] * 100 + [500] + [8] * 155), us(1, [500]) + us(256, [8] * 256)
+    assert both <= 3 * alone, (both, alone)
+
+
+def test_a_long_request_among_short_ones():
+    """Decode: outputs of an uneven batch against those of the same requests one at a time."""
+    import paper_2604_26837_b200 as P
+    lengths, H, topk = [3000] + [37 + i for i in range(31)], 8, 170
+    g = torch.Generator(device="cuda").manual_seed(3)
+    kv = [torch.randn(2, n, H, 128, dtype=torch.bfloat16, device="cuda", generator=g) for n in lengths]
+    q = torch.randn(4, len(lengths), 2 * H, 128, device="cuda", generator=g).to(torch.bfloat16)
+    new = torch.randn(2, 4, len(lengths), H, 128, dtype=torch.bfloat16, device="cuda", generator=g)
+    outs = []
+    for together in (True, False):
+        cfg = P.make_config(device=0, num_layers=1, num_q_heads=2 * H, num_kv_heads=H, max_requests=len(lengths), max_context_tokens=3100,
+                            partition_kind=0, topk=topk, lru_buckets=8, gpu_cache_pages=H * (len(lengths) + 1) * 180,
+                            host_pages=H * sum(n // 16 + 2 for n in lengths))
+        s = P.Spin(cfg)
+        reqs = [s.request_open(180) for _ in lengths]
+        for r, x in zip(reqs, kv):
+            s.append_kv(r, 0, x[0], x[1], x.shape[1])
+        out = torch.zeros_like(q)
+        for t in range(4):
+            for i in ([slice(None)] if together else [slice(i, i + 1) for i in range(len(lengths))]):
+                s.decode_step_append(0, s.req_array(reqs[i]), new[0, t, i], new[1, t, i], q[t, i], out[t, i])
+        torch.cuda.synchronize()
+        assert s.stats()["error_bits"] == 0
+        outs.append(out.double())
+        s.close()
+    # two sums in different orders, each within 2^-8 of the exact one (bf16 probabilities, bf16 outputs)
+    assert (outs[0] - outs[1]).abs().max().item() <= 2.0 ** -7 * max(1.0, outs[1].abs().max().item())
