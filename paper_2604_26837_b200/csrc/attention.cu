@@ -408,11 +408,12 @@ __device__ __forceinline__ bool further_row(const DevCtx &c, const Batch &bt, in
   return *b >= 0;
 }
 
-template <int G>
+// One row of a set by a CTA of W warps (kAttnWarps; 1 for lists that fit one, which have a single row).
+template <int G, int W>
 __device__ __forceinline__ void attn_row(const DevCtx &c, const Batch &bt, const __nv_bfloat16 *__restrict__ q,
                                          __nv_bfloat16 *__restrict__ out, uint8_t *smem, int b, int row, int max_rows, int share) {
-  __shared__ __align__(8) unsigned long long s_bar[kAttnWarps * kWarpStages];
-  __shared__ float s_m[kAttnWarps][G], s_l[kAttnWarps][G];
+  __shared__ __align__(8) unsigned long long s_bar[W * kWarpStages];
+  __shared__ float s_m[W][G], s_l[W][G];
   __shared__ int sh_ok, sh_np, sh_nm, sh_last;
   const int i_req = b / c.Hkv, head = b % c.Hkv;
   int np_most = c.max_pages + c.tail_cap;  // pages that the set's list may have
@@ -452,14 +453,14 @@ __device__ __forceinline__ void attn_row(const DevCtx &c, const Batch &bt, const
   __nv_bfloat16 *out_rows = out + ((size_t)i_req * c.Hq + head * G) * kHeadDim;
   if (np == 0) {                           // nothing to attend: the set's rows are zero
     if (row == 0)
-      for (int e = threadIdx.x; e < G * kHeadDim / 4; e += kAttnThreads) store_out(out_rows + 4 * e, make_uint2(0u, 0u));
+      for (int e = threadIdx.x; e < G * kHeadDim / 4; e += W * 32) store_out(out_rows + 4 * e, make_uint2(0u, 0u));
     return;
   }
   const int n_rows = attn_rows_of(bt, np, share, max_rows);
   if (row >= n_rows) return;
   const size_t pl = (size_t)b * (c.max_pages + c.tail_cap);
-  const int stride = n_rows * kAttnWarps;                                   // the warp's pages: mine, mine + stride, ...
-  const int mine = row * kAttnWarps + warp;
+  const int stride = n_rows * W;                                   // the warp's pages: mine, mine + stride, ...
+  const int mine = row * W + warp;
 
   // Q^T as B-operand fragments: column = lane/4 (query head, zero beyond G), 8 k-steps of 16 channels
   uint32_t qb[8][2];
@@ -638,15 +639,15 @@ __device__ __forceinline__ void attn_row(const DevCtx &c, const Batch &bt, const
   }
   __syncthreads();
 #pragma unroll 1
-  for (int e = threadIdx.x; e < G * (kHeadDim / 4); e += kAttnThreads) {
+  for (int e = threadIdx.x; e < G * (kHeadDim / 4); e += W * 32) {
     const int g = e / (kHeadDim / 4), col = e % (kHeadDim / 4);
     float mn = -INFINITY;
 #pragma unroll
-    for (int w = 0; w < kAttnWarps; ++w) mn = fmaxf(mn, s_m[w][g]);
+    for (int w = 0; w < W; ++w) mn = fmaxf(mn, s_m[w][g]);
     float4 o = make_float4(0.f, 0.f, 0.f, 0.f);
     float l = 0.f;
 #pragma unroll
-    for (int w = 0; w < kAttnWarps; ++w) {
+    for (int w = 0; w < W; ++w) {
       const float mw = s_m[w][g], a = mw == -INFINITY ? 0.f : exp2f(mw - mn);
       const float4 x = reinterpret_cast<const float4 *>(comb + w * kWarpComb + g * kCombStride)[col];
       o.x = fmaf(x.x, a, o.x); o.y = fmaf(x.y, a, o.y); o.z = fmaf(x.z, a, o.z); o.w = fmaf(x.w, a, o.w);
@@ -660,7 +661,7 @@ __device__ __forceinline__ void attn_row(const DevCtx &c, const Batch &bt, const
       if (col == 0) c.att_ml[at] = make_float2(mn, l);
     }
   }
-  if (n_rows == 1) return;
+  if (W < kAttnWarps || n_rows == 1) return;
   // the last CTA of the set to get here merges all partials (log-sum-exp)
   __syncthreads();
   if (threadIdx.x == 0) sh_last = last_row(c, b, n_rows);
@@ -675,22 +676,22 @@ __device__ __forceinline__ void attn_row(const DevCtx &c, const Batch &bt, const
 // go by the per-set flags never wait for the scoring kernel as a whole; with one CTA doing so
 // before it exits, this grid cannot complete ahead of that one, and whatever the stream runs
 // next (the next step's scoring kernel waits for this grid) comes after all of its writes.
-template <int G, bool kCounted>
-__global__ void __launch_bounds__(kAttnThreads, 3)
+template <int G, int W, bool kCounted>
+__global__ void __launch_bounds__(W * 32, 3 * kAttnWarps / W)
 k_attn(DevCtx c, Batch bt, const __nv_bfloat16 *__restrict__ q, __nv_bfloat16 *__restrict__ out) {
   extern __shared__ __align__(128) uint8_t smem[];                // [warps][2] staged pages
   pdl_launch_next();
   if (!kCounted) {
     // launch order: row 0 of every set first (the rows that own the first missed pages), or set by set
     const int b = bt.attn_set_major ? blockIdx.y : blockIdx.x, row = bt.attn_set_major ? blockIdx.x : blockIdx.y;
-    attn_row<G>(c, bt, q, out, smem, b, row, bt.attn_set_major ? gridDim.x : gridDim.y, bt.attn_share);
+    attn_row<G, W>(c, bt, q, out, smem, b, row, bt.attn_set_major ? gridDim.x : gridDim.y, bt.attn_share);
   } else {
     __shared__ int s_sum[kAttnWarps], s_at[2];
     int b = blockIdx.x % bt.n_req, row = blockIdx.x / bt.n_req;
     pdl_wait_prev();
     const int share = share_by_counts(c, bt, s_sum), own = bt.n_req * bt.attn_rows;
     if ((int)blockIdx.x < own || further_row(c, bt, share, (int)blockIdx.x - own, s_sum, s_at, &b, &row))
-      attn_row<G>(c, bt, q, out, smem, b, row, c.max_chunks, share);
+      attn_row<G, W>(c, bt, q, out, smem, b, row, c.max_chunks, share);
   }
   if (blockIdx.x == 0 && blockIdx.y == 0) pdl_wait_prev();
 }
@@ -701,14 +702,14 @@ void launch_attn_g(const DevCtx &c, Batch b, const __nv_bfloat16 *q, __nv_bfloat
   static int resident_dev[kMaxDevices] = {};
   int &resident = resident_dev[current_device_slot()];
   if (!resident) {
-    for (auto kernel : {k_attn<G, false>, k_attn<G, true>}) {
+    for (auto kernel : {k_attn<G, kAttnWarps, false>, k_attn<G, kAttnWarps, true>, k_attn<G, 1, false>}) {
       cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kAttnSmem);
       cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
     }
     int dev = 0, sms = 0, per_sm = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_attn<G, false>, kAttnThreads, kAttnSmem);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_attn<G, kAttnWarps, false>, kAttnThreads, kAttnSmem);
     resident = sms * per_sm > 0 ? sms * per_sm : 148;
   }
   // As many CTAs per set as the GPU holds at once (444), and at least 8 pages for each: every CTA is
@@ -731,16 +732,22 @@ void launch_attn_g(const DevCtx &c, Batch b, const __nv_bfloat16 *q, __nv_bfloat
   b.attn_rows = clamp(resident / n_sets, 1, chunks);
   b.attn_share = clamp(share_of(est_pages, n_sets, b.attn_rows), kSharePages, 1 << 30);
   int rows = clamp((max_pages + b.attn_share - 1) / b.attn_share, b.attn_rows, chunks);
+  // More sets than the GPU holds CTAs, and lists of one page or two per stage: a CTA of one warp each,
+  // four times as many at once.  (16000 lists of one page: 134 us with four warps, 41 with one.)
+  if (max_pages <= 2 * kWarpStages && n_sets > resident) {
+    launch_pdl(k_attn<G, 1, false>, b.attn_set_major ? dim3(1, n_sets) : dim3(n_sets, 1), dim3(32), (size_t)kAttnSmem / kAttnWarps, st, 1, c, b, q, out);
+    return;
+  }
   if (!c.ready && max_pages > 2 * kSharePages * b.attn_rows) {
     const int own = n_sets * b.attn_rows;
-    launch_pdl(k_attn<G, true>, dim3(own + own * 2 / 3), dim3(kAttnThreads), (size_t)kAttnSmem, st, 1, c, b, q, out);
+    launch_pdl(k_attn<G, kAttnWarps, true>, dim3(own + own * 2 / 3), dim3(kAttnThreads), (size_t)kAttnSmem, st, 1, c, b, q, out);
     return;
   }
   if (!c.ready) rows = b.attn_rows;
   rows = clamp(rows, b.attn_rows, clamp(kExtraCtas / n_sets, b.attn_rows, chunks));
   b.attn_share = clamp((max_pages + rows - 1) / rows, b.attn_share, 1 << 30);
   const dim3 grid = b.attn_set_major ? dim3(rows, n_sets) : dim3(n_sets, rows);
-  launch_pdl(k_attn<G, false>, grid, dim3(kAttnThreads), (size_t)kAttnSmem, st, 1, c, b, q, out);
+  launch_pdl(k_attn<G, kAttnWarps, false>, grid, dim3(kAttnThreads), (size_t)kAttnSmem, st, 1, c, b, q, out);
 }
 
 }  // namespace

@@ -186,3 +186,27 @@ def test_a_long_request_among_short_ones():
         s.close()
     # two sums in different orders, each within 2^-8 of the exact one (bf16 probabilities, bf16 outputs)
     assert (outs[0] - outs[1]).abs().max().item() <= 2.0 ** -7 * max(1.0, outs[1].abs().max().item())
+
+
+@pytest.mark.parametrize("sets,group,pages", [(445, 4, 4), (445, 8, 1), (600, 1, 3), (445, 2, 5), (444, 4, 4)])
+def test_short_lists_of_many_sets(sets, group, pages):
+    # a warp to itself for each list of up to four pages, from 445 sets on
+    test_attention_split_edges(sets, group, pages)
+
+
+def test_short_lists_of_many_sets_in_a_decode_step():
+    import workloads as W
+    from test_gpu_parity import _wl, run_parity
+    w = _wl(W.PART_PAGE_MINMAX, num_layers=1, batch=60, num_q_heads=16, num_kv_heads=8, context=16 * 9 + 3, topk=3, slots_per_set=5, steps=6)
+    assert run_parity(w, one_call=True, oracle_reqs=[0, 59])["stats"]["error_bits"] == 0
+
+
+def test_many_one_page_lists_take_little_more_than_as_many_pages_in_longer_lists():
+    import paper_2604_26837_b200 as P
+
+    def us(sets, pages):
+        a = _lists(sets, 1, pages, [pages] * sets)
+        out = torch.empty_like(a[0])
+        return _best_us(lambda: P.spin_paged_attention_static(*a, sets, pages, 1, 0.0, out))
+    one, eight = us(16000, 1), us(2000, 8)
+    assert one <= 2.5 * eight, (one, eight)
