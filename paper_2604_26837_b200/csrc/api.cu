@@ -170,7 +170,8 @@ struct spin_ctx {
   uint8_t *h_pages = nullptr;
   // staging for host-pointer arguments
   __nv_bfloat16 *stage_q = nullptr, *stage_out = nullptr, *stage_k = nullptr, *stage_v = nullptr;
-  int64_t *stage_dest = nullptr;        // spin_reindex: destination rows of the folded tokens
+  int64_t *stage_dest = nullptr;        // spin_reindex: destination rows of the folded tokens; cluster prefill: token counts
+  size_t stage_dest_bytes = 0;
   int sm_count = 148;
   uint64_t launches = 0;
   size_t dir_bytes_in_use = 0;
@@ -183,11 +184,7 @@ struct spin_ctx {
   static constexpr int kOffloadSlots = 4;
   uint8_t *offload_stage = nullptr;
   int32_t *offload_hp = nullptr;     // per staged unit: its host page id (what the kernel records in the mirror)
-  // cluster prefill (see prefill_clustered): every token row's place in its set's page order; per
-  // (head, cluster) token counts (behind one 64-bit word: the first bad entry), first pages, running counts
-  int32_t *cl_place = nullptr, *cl_base = nullptr, *cl_run = nullptr;
-  unsigned long long *cl_bad = nullptr;
-  int32_t *cl_count = nullptr;
+  int32_t *offload_place = nullptr;  // cluster prefill: every token row's place in its set's page order (see prefill_clustered)
   int64_t offload_slot_units = 0;    // (page, kv head) units of 8 KiB per slot; 0 = write-through
   cudaStream_t offload_stream = nullptr;
   cudaEvent_t ev_staged[kOffloadSlots] = {}, ev_done[kOffloadSlots] = {};
@@ -257,14 +254,14 @@ void carve(Arena &a, const spin_config &cfg, const Geometry &g, DevCtx &d, spin_
   d.att_ml = reinterpret_cast<float2 *>(d.att_part + B * g.max_chunks * G * kHeadDim);
   d.att_count = a.take<int32_t>(B);
   d.sel_count = a.take<int32_t>(B);
-  d.link = a.take<int32_t>(64);
-  d.score_queue = a.take<int32_t>(1);
-  d.score_done = a.take<int32_t>(1);
+  // four counters that many CTAs add to, 128 bytes apart
+  d.score_queue = a.take<int32_t>(32 * 3 + 1);
+  d.link = d.score_queue + 32;
+  d.score_done = d.score_queue + 64;
   d.scored = a.take<int32_t>(B);
   d.ready = a.take<int32_t>(B);
   d.tail_ready = a.take<int32_t>(B);
   d.ready1 = a.take<unsigned long long>(B);
-  d.slots_ready = a.take<int32_t>(B);
   d.counters = a.take<Counters>(1);
   __nv_bfloat16 *sq = a.take<__nv_bfloat16>((size_t)cfg.max_requests * cfg.num_q_heads * kHeadDim);
   __nv_bfloat16 *so = a.take<__nv_bfloat16>((size_t)cfg.max_requests * cfg.num_q_heads * kHeadDim);
@@ -272,22 +269,15 @@ void carve(Arena &a, const spin_config &cfg, const Geometry &g, DevCtx &d, spin_
   __nv_bfloat16 *sk = a.take<__nv_bfloat16>(stage_rows * kHeadDim);
   __nv_bfloat16 *sv = a.take<__nv_bfloat16>(stage_rows * kHeadDim);
   int64_t *sd = a.take<int64_t>(stage_rows);
-  if (ctx) { ctx->stage_q = sq; ctx->stage_out = so; ctx->stage_k = sk; ctx->stage_v = sv; ctx->stage_dest = sd; }
+  if (ctx) { ctx->stage_q = sq; ctx->stage_out = so; ctx->stage_k = sk; ctx->stage_v = sv; ctx->stage_dest = sd; ctx->stage_dest_bytes = stage_rows * sizeof(int64_t); }
   if (cfg.offload_stage_bytes > 0) {
     const int64_t units = cfg.offload_stage_bytes / spin_ctx::kOffloadSlots / kPageBytes;
     uint8_t *os = a.take<uint8_t>((size_t)units * spin_ctx::kOffloadSlots * kPageBytes);
     int32_t *oh = a.take<int32_t>((size_t)units * spin_ctx::kOffloadSlots);
-    if (ctx) { ctx->offload_stage = os; ctx->offload_hp = oh; ctx->offload_slot_units = units; }
-  }
-  if (cfg.partition_kind == SPIN_PART_CLUSTER_CENTROID) {
-    const size_t hc = (size_t)cfg.num_kv_heads * cfg.num_clusters;
-    int32_t *place = a.take<int32_t>((size_t)cfg.max_context_tokens * cfg.num_kv_heads);
-    int32_t *count = a.take<int32_t>(2 + hc), *base = a.take<int32_t>(hc), *run = a.take<int32_t>(hc);
-    if (ctx) {
-      ctx->cl_place = place; ctx->cl_base = base; ctx->cl_run = run;
-      ctx->cl_bad = reinterpret_cast<unsigned long long *>(count);
-      ctx->cl_count = count + 2;
-    }
+    // cluster granularity: where every (token, head) row of a prefill goes in its set's page order
+    int32_t *op = cfg.partition_kind == SPIN_PART_CLUSTER_CENTROID
+                      ? a.take<int32_t>((size_t)cfg.max_context_tokens * cfg.num_kv_heads) : nullptr;
+    if (ctx) { ctx->offload_stage = os; ctx->offload_hp = oh; ctx->offload_slot_units = units; ctx->offload_place = op; }
   }
 }
 
@@ -555,10 +545,32 @@ int append_paged_device(spin_ctx *ctx, int req, int layer, const __nv_bfloat16 *
   return SPIN_OK;
 }
 
+// HBM that a cluster prefill of (request, layer) may use until it returns: the cache slots and tail pages
+// of the sets it fills, which hold nothing before it.  The tail pages of a layer's sets are consecutive, the
+// slots are as a rule (pages are handed out lowest first); the longest run is taken.
+struct PrefillRoom { int32_t *words; int64_t tokens; };       // a word per (token, head) for so many tokens
+PrefillRoom prefill_room(spin_ctx *ctx, int req, int layer, int64_t n) {
+  const Geometry &g = ctx->g;
+  const int H = ctx->cfg.num_kv_heads;
+  const int64_t enough = (n * H * 4 + kPageBytes - 1) / kPageBytes;
+  int64_t at = ctx->cfg.gpu_cache_pages + (int64_t)set_index(ctx->d, req, layer, 0) * g.tail_cap, len = (int64_t)H * g.tail_cap;
+  int64_t first = 0, run = 0;
+  for (int h = 0; h < H && len < enough; ++h)
+    for (int32_t p : set_of(ctx, req, layer, h).gpu_pages) {
+      if (run == 0 || p != first + run) { first = p; run = 0; }
+      if (++run > len) { at = first; len = run; }
+      if (len >= enough) break;
+    }
+  return PrefillRoom{reinterpret_cast<int32_t *>(ctx->d.gpu_pages + at * kPageBytes), len * (kPageBytes / 4) / H};
+}
+
 // Cluster prefill.  The GPU counts the clusters' tokens, the host (which hands out the pages) lays
 // the sets' pages out from the counts, the GPU does everything that is per token: ranks the
 // tokens within their clusters, fills the tables' HBM copies and moves the rows.  (Counting and
 // placing 262144 rows on the host and uploading a place per row took 2.8 ms of a 5.4 ms prefill.)
+// It has no HBM of its own: counts go through stage_dest, as many clusters at a time as it holds,
+// places through the sets' own pages, as many tokens at a time as those hold (one go as a rule; the
+// clusters' running counts wait in the residency words, zero before and after).
 int prefill_clustered_impl(spin_ctx *ctx, int req, int layer, const void *k, const void *v, int64_t n,
                            const int32_t *token_partition, const void *centroids, cudaStream_t st) {
   LayerHost &L = ctx->reqs[(size_t)req].layers[(size_t)layer];
@@ -567,37 +579,52 @@ int prefill_clustered_impl(spin_ctx *ctx, int req, int layer, const void *k, con
   const int H = ctx->cfg.num_kv_heads, C = ctx->cfg.num_clusters;
   if (L.n_tokens != 0) return fail(ctx, SPIN_ERR_STATE, "cluster prefill must be the first append of (request, layer)");
   if (n > ctx->cfg.max_context_tokens) return fail(ctx, SPIN_ERR_INVALID, "prefill exceeds max_context_tokens");
-  const size_t rows = (size_t)n * H, hc = (size_t)H * C;
+  const size_t hc = (size_t)H * C;
+  const bool dev_kv = is_device_ptr(k), dev_tp = is_device_ptr(token_partition), ring = dev_kv && ctx->offload_slot_units > 0;
+  PrefillRoom room = prefill_room(ctx, req, layer, n);
+  if (ring) room = PrefillRoom{ctx->offload_place, n};        // its rows are taken up several times, all places at once
+  const int64_t chunk = dev_kv ? std::min(n, room.tokens) : std::min({n, room.tokens, g.stage_tokens});
+  // a chunk's clusters [tokens][H] on the device
+  auto clusters_of = [&](int64_t t0, int64_t m, const int32_t **tp) {
+    *tp = dev_tp ? token_partition + (size_t)t0 * H : room.words;
+    return dev_tp ? cudaSuccess : cudaMemcpyAsync(room.words, token_partition + (size_t)t0 * H, (size_t)m * H * 4, cudaMemcpyDefault, st);
+  };
+  const int32_t *tp = nullptr;
   // 1. token counts of every cluster (and the first entry that is no cluster, if any)
-  const int32_t *tp = token_partition;
-  if (!is_device_ptr(tp)) {
-    CK(cudaMemcpyAsync(ctx->cl_place, tp, rows * 4, cudaMemcpyDefault, st));
-    tp = ctx->cl_place;                                       // the places are written over the clusters they are made from
+  unsigned long long *d_bad = reinterpret_cast<unsigned long long *>(ctx->stage_dest);
+  int32_t *d_count = reinterpret_cast<int32_t *>(d_bad + 1);
+  const int slice = (int)std::min<int64_t>(C, (int64_t)((ctx->stage_dest_bytes - 8) / 4 / H));
+  std::vector<int32_t> count(hc), part((size_t)2 + (size_t)H * slice);          // [H][C]; the bad entry, then [H][clusters of a slice]
+  for (int c0 = 0; c0 < C; c0 += slice) {
+    const int nc = std::min(slice, C - c0);
+    const size_t words = 2 + (size_t)H * nc;
+    CK(cudaMemsetAsync(d_bad, 0xff, 8, st));
+    CK(cudaMemsetAsync(d_count, 0, (words - 2) * 4, st));
+    for (int64_t t0 = 0, m; t0 < n; t0 += m) {
+      m = std::min(dev_tp ? n : room.tokens, n - t0);
+      CK(clusters_of(t0, m, &tp));
+      ctx->launches += launch_cluster_count(tp, (size_t)t0 * H, (size_t)m * H, H, C, c0, nc, d_count, d_bad, st);
+    }
+    CK(cudaMemcpyAsync(part.data(), d_bad, words * 4, cudaMemcpyDeviceToHost, st));
+    CK(cudaStreamSynchronize(st));
+    uint64_t bad;
+    memcpy(&bad, part.data(), 8);
+    if (bad != ~0ull) {
+      int32_t c = 0;
+      CK(cudaMemcpy(&c, token_partition + bad, 4, cudaMemcpyDefault));
+      return fail(ctx, SPIN_ERR_INVALID, "token_partition[%lld][%d] = %d out of range", (long long)(bad / H), (int)(bad % H), c);
+    }
+    for (int h = 0; h < H; ++h) std::copy_n(part.begin() + 2 + (ptrdiff_t)h * nc, nc, count.begin() + (ptrdiff_t)h * C + c0);
   }
-  CK(cudaMemsetAsync(ctx->cl_bad, 0xff, 8, st));
-  CK(cudaMemsetAsync(ctx->cl_count, 0, hc * 4, st));
-  ctx->launches += launch_cluster_count(tp, rows, H, C, ctx->cl_count, ctx->cl_bad, st);
-  std::vector<int32_t> blob(2 + hc);
-  CK(cudaMemcpyAsync(blob.data(), ctx->cl_bad, blob.size() * 4, cudaMemcpyDeviceToHost, st));
-  CK(cudaStreamSynchronize(st));
-  uint64_t bad;
-  memcpy(&bad, blob.data(), 8);
-  if (bad != ~0ull) {
-    int32_t c = 0;
-    CK(cudaMemcpy(&c, token_partition + bad, 4, cudaMemcpyDefault));
-    return fail(ctx, SPIN_ERR_INVALID, "token_partition[%lld][%d] = %d out of range", (long long)(bad / H), (int)(bad % H), c);
-  }
-  const int32_t *count = blob.data() + 2;
   int64_t pages_needed = 0;
   for (size_t i = 0; i < hc; ++i) pages_needed += (count[i] + kPageTokens - 1) / kPageTokens;
   if (ctx->host_page_pool.available() < pages_needed) return fail(ctx, SPIN_ERR_OOM_HOST, "out of host pages");
   // 2. the sets' pages, clusters in order, each one's pages together
-  std::vector<int32_t> base(hc);                              // CPU-page-table offset of each cluster
   int32_t total_pages_max = 0;
   for (int h = 0; h < H; ++h) {
     const int set = set_index(d, req, layer, h);
     SetHost &S = ctx->sets[(size_t)set];
-    const int32_t *cnt = count + (size_t)h * C;
+    const int32_t *cnt = count.data() + (size_t)h * C;
     int32_t off = 0;
     for (int c0 = 0; c0 < C; c0 += g.seg) {
       const int seg = ensure_seg(ctx, ctx->off_segs, S.dir_off, d.dir_off + (size_t)set * g.dir_part, c0, g.seg_shift);
@@ -606,7 +633,6 @@ int prefill_clustered_impl(spin_ctx *ctx, int req, int layer, const void *k, con
         return fail(ctx, SPIN_ERR_OOM_DEVICE, "out of Meta-partition segments");
       int32_t *h_off = ctx->h_off_pool + ((size_t)seg << g.seg_shift);
       for (int c = c0; c < std::min(C, c0 + g.seg); ++c) {
-        base[(size_t)h * C + c] = off;
         h_off[c - c0] = off;
         off += (cnt[c] + kPageTokens - 1) / kPageTokens;
       }
@@ -632,10 +658,16 @@ int prefill_clustered_impl(spin_ctx *ctx, int req, int layer, const void *k, con
   // that tail pages never collide with cluster pages of any head
   for (int h = 0; h < H; ++h) set_of(ctx, req, layer, h).host_pages.resize((size_t)total_pages_max, -1);
   flush_dirs(ctx, st);
-  // 3. tables, places, centroids
-  CK(cudaMemcpyAsync(ctx->cl_base, base.data(), hc * 4, cudaMemcpyHostToDevice, st));
-  ctx->launches += launch_cluster_tables(d, req, layer, C, total_pages_max, (int)n, ctx->cl_count, (int)ctx->reqs[(size_t)req].slots, st);
-  ctx->launches += launch_cluster_place(tp, n, H, C, ctx->cl_base, ctx->cl_run, ctx->cl_place, st);
+  // 3. tables (from the counts, which are still on the device where one slice holds them all), centroids
+  for (int c0 = 0; c0 < C; c0 += slice) {
+    const int nc = std::min(slice, C - c0);
+    if (slice < C) {
+      for (int h = 0; h < H; ++h) std::copy_n(count.begin() + (ptrdiff_t)h * C + c0, nc, part.begin() + (ptrdiff_t)h * nc);
+      CK(cudaMemcpyAsync(d_count, part.data(), (size_t)H * nc * 4, cudaMemcpyHostToDevice, st));
+    }
+    ctx->launches += launch_cluster_tables(d, req, layer, C, c0, nc, total_pages_max, (int)n, d_count, (int)ctx->reqs[(size_t)req].slots, st);
+    if (slice < C) CK(cudaStreamSynchronize(st));
+  }
   const __nv_bfloat16 *cen = reinterpret_cast<const __nv_bfloat16 *>(centroids);
   void *cen_tmp = nullptr;
   if (!is_device_ptr(centroids)) {
@@ -645,9 +677,10 @@ int prefill_clustered_impl(spin_ctx *ctx, int req, int layer, const void *k, con
   }
   ctx->launches += launch_copy_centroids(d, req, layer, cen, C, st);
   // 4. rows to their pages
-  const bool dev_kv = is_device_ptr(k);
   const __nv_bfloat16 *kd = reinterpret_cast<const __nv_bfloat16 *>(k), *vd = reinterpret_cast<const __nv_bfloat16 *>(v);
-  if (dev_kv && ctx->offload_slot_units > 0) {
+  if (ring) {
+    CK(clusters_of(0, n, &tp));
+    ctx->launches += launch_cluster_place(d, req, layer, tp, n, C, true, true, room.words, st);
     // Asynchronous offload (Section 4.1): the rows are packed into pages in HBM staging slots on
     // the caller's stream, at HBM speed, range by range of the sets' logical pages; each slot
     // then moves to host memory by copy-engine transfers (one per run of consecutive host
@@ -659,7 +692,7 @@ int prefill_clustered_impl(spin_ctx *ctx, int req, int layer, const void *k, con
       if (ctx->slot_used[slot]) CK(cudaStreamWaitEvent(st, ctx->ev_done[slot], 0));     // ring full: wait for the drain
       uint8_t *stage = ctx->offload_stage + (size_t)slot * ctx->offload_slot_units * kPageBytes;
       CK(cudaMemsetAsync(stage, 0, (size_t)H * m * kPageBytes, st));                   // rows past a cluster's last token stay zero
-      ctx->launches += launch_cluster_scatter_staged(d, kd, vd, ctx->cl_place, (int)n, (int)p0, m, stage, st);
+      ctx->launches += launch_cluster_scatter_staged(d, kd, vd, room.words, (int)n, (int)p0, m, stage, st);
       CK(cudaEventRecord(ctx->ev_staged[slot], st));
       CK(cudaStreamWaitEvent(ctx->offload_stream, ctx->ev_staged[slot], 0));
       for (int h = 0; h < H; ++h) {
@@ -679,18 +712,18 @@ int prefill_clustered_impl(spin_ctx *ctx, int req, int layer, const void *k, con
       ctx->offload_last = slot;
       ++ctx->offload_gen;
     }
-  } else if (dev_kv) {
-    ctx->launches += launch_cluster_scatter(d, req, layer, kd, vd, ctx->cl_place, n, st);
   } else {
-    // host rows come in through the staging buffers, chunk by chunk
-    const int64_t chunk = g.stage_tokens;
     for (int64_t t0 = 0; t0 < n; t0 += chunk) {
       const int64_t m = std::min(chunk, n - t0);
       const size_t at = (size_t)t0 * H * kHeadDim, bytes = (size_t)m * H * kRowBytes;
-      CK(cudaMemcpyAsync(ctx->stage_k, kd + at, bytes, cudaMemcpyHostToDevice, st));
-      CK(cudaMemcpyAsync(ctx->stage_v, vd + at, bytes, cudaMemcpyHostToDevice, st));
-      ctx->launches += launch_cluster_scatter(d, req, layer, ctx->stage_k, ctx->stage_v, ctx->cl_place + (size_t)t0 * H, m, st);
-      CK(cudaStreamSynchronize(st));
+      CK(clusters_of(t0, m, &tp));
+      ctx->launches += launch_cluster_place(d, req, layer, tp, m, C, t0 == 0, t0 + m == n, room.words, st);
+      if (!dev_kv) {                          // host rows come in through the staging buffers
+        CK(cudaMemcpyAsync(ctx->stage_k, kd + at, bytes, cudaMemcpyHostToDevice, st));
+        CK(cudaMemcpyAsync(ctx->stage_v, vd + at, bytes, cudaMemcpyHostToDevice, st));
+      }
+      ctx->launches += launch_cluster_scatter(d, req, layer, dev_kv ? kd + at : ctx->stage_k, dev_kv ? vd + at : ctx->stage_v, room.words, m, st);
+      if (!dev_kv) CK(cudaStreamSynchronize(st));
     }
   }
   CK(cudaStreamSynchronize(st));            // the prefill form synchronises: its scratch is free again (a drain goes on)
@@ -849,14 +882,11 @@ int spin_create(const spin_config *cfg, spin_ctx **out) {
   fill(d.score_xfer, 0xff, (size_t)g.max_batch_sets * g.max_cand * 4);       // every word "not written"
   fill(d.att_count, 0, (size_t)g.max_batch_sets * 4);
   fill(d.sel_count, 0, (size_t)g.max_batch_sets * 4);
-  fill(d.link, 0, 64 * 4);
-  fill(d.score_queue, 0, 4);
-  fill(d.score_done, 0, 4);
+  fill(d.score_queue, 0, (32 * 3 + 1) * 4);
   fill(d.scored, 0, (size_t)g.max_batch_sets * 4);
   fill(d.ready, 0, (size_t)g.max_batch_sets * 4);
   fill(d.tail_ready, 0, (size_t)g.max_batch_sets * 4);
   fill(d.ready1, 0, (size_t)g.max_batch_sets * 8);
-  fill(d.slots_ready, 0, (size_t)g.max_batch_sets * 4);
   fill(d.state, 0, (size_t)g.n_sets * sizeof(SetState));
   fill(d.counters, 0, sizeof(Counters));
   fill(d.fetch_count, 0, 4);

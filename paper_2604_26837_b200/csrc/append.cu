@@ -65,49 +65,59 @@ k_append_edge(DevCtx c, AppendEdgeArgs a, const __nv_bfloat16 *__restrict__ k,
 }
 
 // ---- cluster prefill ------------------------------------------------------------------------
-// token_partition [n_tokens][Hkv] -> tokens per (head, cluster); bad = the first entry that names no
-// cluster (all ones if none does).
+// token_partition [n_tokens][Hkv] from entry `first` on -> tokens per (head, cluster), for the clusters
+// [c0, c0 + nc); bad = the first entry that names no cluster (all ones if none does).
 __global__ void __launch_bounds__(256)
-k_cluster_count(const int32_t *__restrict__ tp, size_t rows, int H, int C, int32_t *__restrict__ count, unsigned long long *bad) {
+k_cluster_count(const int32_t *__restrict__ tp, size_t first, size_t rows, int H, int C, int c0, int nc, int32_t *__restrict__ count,
+                unsigned long long *bad) {
   for (size_t i = (size_t)blockIdx.x * 256 + threadIdx.x; i < rows; i += (size_t)gridDim.x * 256) {
     const int32_t cl = tp[i];
-    if (cl < 0 || cl >= C) atomicMin(bad, (unsigned long long)i);
-    else atomicAdd(count + (size_t)(i % H) * C + cl, 1);
+    if (cl < 0 || cl >= C) atomicMin(bad, (unsigned long long)(first + i));
+    else if (cl >= c0 && cl < c0 + nc) atomicAdd(count + (size_t)(i % H) * nc + (cl - c0), 1);
   }
 }
 
 // A row's place in its set's logical page order: (first page of its cluster) * 16 + its rank among
 // the cluster's tokens (arrival order).  One CTA per kv head, a warp per run of consecutive tokens
-// with counters of its own in shared memory: count, prefix over the warps, then 32 tokens at a
-// time, the lanes of a cluster ranked by match_any.  Where even one warp's counters exceed shared
-// memory a single warp counts in `run` (global).  tp and place may be the same array: an entry is
-// read by the thread that overwrites it, after every count has been taken.
+// with counters of its own in shared memory, which hold the cluster's next place: count, prefix over the
+// warps, then 32 tokens at a time, the lanes of a cluster ranked by match_any.  Where even one warp's
+// counters exceed shared memory a single warp counts in the clusters' residency words (zero until the
+// prefill is done); these also carry the counts from one chunk of tokens to the next.  tp and place may be
+// the same array: an entry is read by the thread that overwrites it, after every count has been taken.
 // Latency-bound (a warp's steps follow one another): ~30 us for 32768 tokens and 512 clusters,
 // beside 2.6 ms for their rows on the host link.
 constexpr int kPlaceWarps = 16, kPlaceSmem = 160 * 1024;
 __global__ void __launch_bounds__(kPlaceWarps * 32)
-k_cluster_place(const int32_t *tp, int64_t n, int H, int C, const int32_t *__restrict__ base, int32_t *__restrict__ run,
-                int n_warps, int in_smem, int32_t *place) {
+k_cluster_place(DevCtx c, int req, int layer, const int32_t *tp, int64_t n, int C, int n_warps, int in_smem, int first_chunk, int last_chunk,
+                int32_t *place) {
   extern __shared__ int32_t s_run[];
-  const int head = blockIdx.x, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  int32_t *cnt = in_smem ? s_run + (size_t)warp * C : run + (size_t)head * C;
+  const int head = blockIdx.x, H = c.Hkv, set = set_index(c, req, layer, head), warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  int32_t *cnt = s_run + (size_t)warp * C;
   const int64_t per = (n + n_warps - 1) / n_warps, lo = warp < n_warps ? min(n, warp * per) : n, hi = warp < n_warps ? min(n, lo + per) : n;
   const int32_t *mine = tp + head;
+  // the cluster's next place before this chunk (every entry is mapped: the tables have been laid out)
+  auto next_of = [&](int cl) {
+    const MetaEntry *m = first_chunk ? nullptr : meta_at(c, set, cl);
+    const int32_t *o = first_chunk ? off_lookup(c, set, cl) : nullptr;
+    return m ? m->resident : o ? *o * kPageTokens : 0;
+  };
+  auto keep = [&](int cl, int32_t next) { MetaEntry *m = meta_at(c, set, cl); if (m) m->resident = next; else dev_error(c, kErrBounds); };
   if (in_smem) {
-    for (int c = threadIdx.x; c < n_warps * C; c += blockDim.x) s_run[c] = 0;
+    for (int i = threadIdx.x; i < n_warps * C; i += blockDim.x) s_run[i] = 0;
     __syncthreads();
 #pragma unroll 4
     for (int64_t t = lo + lane; t < hi; t += 32) atomicAdd(cnt + mine[(size_t)t * H], 1);
     __syncthreads();
-    for (int c = threadIdx.x; c < C; c += blockDim.x) {
-      int32_t sum = 0;
-      for (int w = 0; w < n_warps; ++w) { const int32_t x = s_run[(size_t)w * C + c]; s_run[(size_t)w * C + c] = sum; sum += x; }
+    for (int cl = threadIdx.x; cl < C; cl += blockDim.x) {
+      int32_t sum = next_of(cl);
+      for (int w = 0; w < n_warps; ++w) { const int32_t x = s_run[(size_t)w * C + cl]; s_run[(size_t)w * C + cl] = sum; sum += x; }
+      if (!first_chunk || !last_chunk) keep(cl, last_chunk ? 0 : sum);
     }
     __syncthreads();
   } else {
-    for (int c = threadIdx.x; c < C; c += blockDim.x) cnt[c] = 0;
+    if (first_chunk)
+      for (int cl = threadIdx.x; cl < C; cl += blockDim.x) keep(cl, next_of(cl));
     __syncthreads();
-    if (warp >= n_warps) return;
   }
   int64_t t = lo + lane;
   int cl = t < hi ? mine[(size_t)t * H] : -1;
@@ -116,27 +126,36 @@ k_cluster_place(const int32_t *tp, int64_t n, int H, int C, const int32_t *__res
     const int64_t t_next = t + 32;
     const int cl_next = t_next < hi ? mine[(size_t)t_next * H] : -1;       // in flight while these 32 are ranked
     const uint32_t same = __match_any_sync(0xffffffffu, cl);
-    const int32_t seen = cl >= 0 ? cnt[cl] : 0;
+    MetaEntry *m = in_smem || cl < 0 ? nullptr : meta_at(c, set, cl);
+    const int32_t next = cl < 0 ? 0 : in_smem ? cnt[cl] : m ? m->resident : 0;
     __syncwarp();
     if (cl >= 0) {
-      place[(size_t)t * H + head] = base[(size_t)head * C + cl] * kPageTokens + seen + __popc(same & ((1u << lane) - 1u));
-      if ((same >> lane) == 1u) cnt[cl] = seen + __popc(same);             // the cluster's last lane
+      place[(size_t)t * H + head] = next + __popc(same & ((1u << lane) - 1u));
+      if ((same >> lane) == 1u) {                                          // the cluster's last lane
+        if (in_smem) cnt[cl] = next + __popc(same); else if (m) m->resident = next + __popc(same);
+      }
     }
     __syncwarp();
     t = t_next;
     cl = cl_next;
   }
+  if (!in_smem && last_chunk) {
+    __syncthreads();
+    for (int cl = threadIdx.x; cl < C; cl += blockDim.x) keep(cl, 0);
+  }
 }
 
-// What follows from the layout, for every kv head's set: Meta-partition entries, the HBM copies of
-// the Partition Offset and CPU page tables (read from the pinned originals) and the set's scalars.
+// What follows from the layout, for every kv head's set: Meta-partition entries of the clusters
+// [c0, c0 + nc), whose counts these are, and with the first of them the HBM copies of the Partition
+// Offset and CPU page tables (read from the pinned originals) and the set's scalars.
 __global__ void __launch_bounds__(256)
-k_cluster_tables(DevCtx c, int req, int layer, int C, int n_pages, int n_tokens, const int32_t *__restrict__ count, int slots) {
+k_cluster_tables(DevCtx c, int req, int layer, int C, int c0, int nc, int n_pages, int n_tokens, const int32_t *__restrict__ count, int slots) {
   const int head = blockIdx.y, set = set_index(c, req, layer, head), e = blockIdx.x * 256 + threadIdx.x;
-  if (e < C) {
-    MetaEntry *m = meta_at(c, set, e);
-    if (m) *m = MetaEntry{count[(size_t)head * C + e], 0}; else dev_error(c, kErrBounds);
+  if (e < nc) {
+    MetaEntry *m = meta_at(c, set, c0 + e);
+    if (m) *m = MetaEntry{count[(size_t)head * nc + e], 0}; else dev_error(c, kErrBounds);
   }
+  if (c0 > 0) return;
   mirror_tables(c, set, e, C, n_pages);
   if (e == 0) {
     SetState *s = c.state + set;
@@ -255,13 +274,15 @@ int launch_append_edge(const DevCtx &c, const AppendEdgeArgs &a, const __nv_bflo
   return 1;
 }
 
-int launch_cluster_count(const int32_t *tp, size_t rows, int H, int C, int32_t *count, unsigned long long *bad, cudaStream_t st) {
+int launch_cluster_count(const int32_t *tp, size_t first, size_t rows, int H, int C, int c0, int nc, int32_t *count, unsigned long long *bad,
+                         cudaStream_t st) {
   const size_t want = (rows + 255) / 256;
-  k_cluster_count<<<(int)(want < 148 * 8 ? want : 148 * 8), 256, 0, st>>>(tp, rows, H, C, count, bad);
+  k_cluster_count<<<(int)(want < 148 * 8 ? want : 148 * 8), 256, 0, st>>>(tp, first, rows, H, C, c0, nc, count, bad);
   return 1;
 }
 
-int launch_cluster_place(const int32_t *tp, int64_t n, int H, int C, const int32_t *base, int32_t *run, int32_t *place, cudaStream_t st) {
+int launch_cluster_place(const DevCtx &c, int req, int layer, const int32_t *tp, int64_t n, int C, bool first_chunk, bool last_chunk, int32_t *place,
+                         cudaStream_t st) {
   // as many warps as have room for their counters; one, counting in global memory, where none has
   int warps = kPlaceSmem / 4 / C;
   const int in_smem = warps >= 1;
@@ -270,13 +291,15 @@ int launch_cluster_place(const int32_t *tp, int64_t n, int H, int C, const int32
   static bool configured_dev[kMaxDevices] = {};
   bool &configured = configured_dev[current_device_slot()];
   if (!configured) { cudaFuncSetAttribute(k_cluster_place, cudaFuncAttributeMaxDynamicSharedMemorySize, kPlaceSmem); configured = true; }
-  k_cluster_place<<<H, kPlaceWarps * 32, smem, st>>>(tp, n, H, C, base, run, warps, in_smem, place);
+  k_cluster_place<<<c.Hkv, kPlaceWarps * 32, smem, st>>>(c, req, layer, tp, n, C, warps, in_smem, first_chunk, last_chunk, place);
   return 1;
 }
 
-int launch_cluster_tables(const DevCtx &c, int req, int layer, int C, int n_pages, int n_tokens, const int32_t *count, int slots, cudaStream_t st) {
-  const int n = C > n_pages ? C : n_pages;
-  k_cluster_tables<<<dim3((n + 255) / 256, c.Hkv), 256, 0, st>>>(c, req, layer, C, n_pages, n_tokens, count, slots);
+int launch_cluster_tables(const DevCtx &c, int req, int layer, int C, int c0, int nc, int n_pages, int n_tokens, const int32_t *count, int slots,
+                          cudaStream_t st) {
+  int n = nc;
+  if (c0 == 0) { n = C > n_pages ? C : n_pages; }
+  k_cluster_tables<<<dim3((n + 255) / 256, c.Hkv), 256, 0, st>>>(c, req, layer, C, c0, nc, n_pages, n_tokens, count, slots);
   return 1;
 }
 

@@ -189,7 +189,7 @@ __device__ __forceinline__ void stores_read() { asm volatile("cp.async.bulk.wait
 // Measured on the Llama-shaped step (64 sets, 396 missed pages): last set's list of missed pages
 // 75-86 us into the step without a limit, 35 us with one; step 112 us without, 106 / 102 / 103 / 107 us
 // with a window of 32 / 64 / 96 / 160 pages.
-constexpr int kLinkWindow = 64, kLinkDone = 32, kLinkPolls = 1 << 20;
+constexpr int kLinkWindow = 64, kLinkDone = 64, kLinkPolls = 1 << 20;
 __device__ __forceinline__ int link_turn(const DevCtx &c, int lane) { return lane == 0 ? atomicAdd(c.link, 1) : 0; }   // lane 0's
 __device__ __forceinline__ void link_close(const DevCtx &c, int lane) { if (lane == 0) atomicAdd(c.link + kLinkDone, 1); }
 __device__ __forceinline__ int link_closed(const DevCtx &c) {
@@ -503,7 +503,7 @@ __device__ __forceinline__ void attn_row(const DevCtx &c, const Batch &bt, const
     }
     if (!listed) {
       int ok = 1;
-      if (lane == 0) ok = flag_wait2(c, c.ready + b, c.tail_ready + b, bt.epoch);
+      if (lane == 0) ok = list_wait(c, c.ready + b, c.tail_ready + b, bt.epoch);
       listed = __shfl_sync(0xffffffffu, ok, 0) != 0;
       __syncwarp();                        // lane 0's acquire comes before every lane's reads of the list
       pages_visible();
@@ -581,7 +581,7 @@ __device__ __forceinline__ void attn_row(const DevCtx &c, const Batch &bt, const
       }
       if (((hosted >> j) & 1u) && !slots_known) {                           // while the page is on its way
         int ok = 1;
-        if (lane == 0) ok = flag_wait(c, c.slots_ready + b, bt.epoch);
+        if (lane == 0) ok = flag_wait(c, c.ready + b, slots_ready(bt.epoch));
         slots_known = __shfl_sync(0xffffffffu, ok, 0) != 0;
         if (!slots_known) { dead = true; break; }                           // reported by the wait
         __syncwarp();                                                       // (as above)
@@ -849,7 +849,6 @@ extern "C" int spin_paged_attention_static(const void *q, const void *page_pool,
   c.ready = nullptr;                                        // plain stream order: no per-set flags
   c.tail_ready = nullptr;
   c.ready1 = nullptr;
-  c.slots_ready = nullptr;
   c.att_part = g_static_partials_addr[dev];
   c.att_ml = reinterpret_cast<float2 *>(c.att_part + (size_t)n_sets * chunks * group * kHeadDim);
   c.att_words = g_static_words_addr[dev];

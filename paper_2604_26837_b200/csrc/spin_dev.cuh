@@ -108,16 +108,16 @@ struct DevCtx {
   int32_t *att_count;           // [b] CTAs of the set that have finished (zero before attention)
   unsigned long long *att_words;   // the same for the allocation-free call (null in a context), with
   uint32_t att_call;            //   the call's number in the upper half of each word
-  int32_t *link;                // turns on the host link: [0] taken, [32] done (words of their own lines)
+  int32_t *link;                // turns on the host link: [0] taken, [64] done (words of their own lines)
   int32_t *sel_count;           // [b] scoring CTAs of the set that have finished (zero between steps)
   int32_t *score_queue;         // next work item of the resident scoring grid (zero between steps)
   int32_t *score_done;          // CTAs of that grid that have left (zero between steps)
   int32_t *scored;              // [b] epoch of the last step whose scores are complete (stand-alone top-k waits on it)
-  int32_t *ready;               // [b] epoch of the last step whose page list is complete (slots of missed pages may be open)
+  int32_t *ready;               // [b] how far the set's step is: 2 x epoch once its page list is complete (slots of missed pages
+                                //   may be open), 1 more once the missed pages have their slots (page_src)
   int32_t *tail_ready;          // [b] epoch of the last step whose appended rows are in the tail page
   unsigned long long *ready1;   // [b] first flag: epoch of the last step whose missed pages are listed (upper half), with the
                                 //   length of the page list and its early descriptors (see first_flag)
-  int32_t *slots_ready;         // [b] epoch of the last step whose missed pages have their slots (page_src)
   int32_t max_chunks;
   int32_t fetch_mode;           // 0: misses are fetched by the attention kernel; 1: by k_fetch
   int32_t evict_exact;          // 1: exact-demand eviction variant (see spin_config)
@@ -276,13 +276,16 @@ __device__ __forceinline__ bool first_flag_wait(const DevCtx &c, const unsigned 
   return false;
 }
 
-// The same for two flags, polled together.
-__device__ __forceinline__ bool flag_wait2(const DevCtx &c, const int32_t *flag0, const int32_t *flag1, int32_t value) {
+// A set's `ready` word: the list is complete; its missed pages have their slots too.
+__device__ __forceinline__ int32_t list_ready(int32_t epoch) { return (int32_t)(2u * (uint32_t)epoch); }
+__device__ __forceinline__ int32_t slots_ready(int32_t epoch) { return (int32_t)(2u * (uint32_t)epoch + 1u); }
+// A complete list and the tail page, polled together.
+__device__ __forceinline__ bool list_wait(const DevCtx &c, const int32_t *ready, const int32_t *tail_ready, int32_t epoch) {
   unsigned pause = 32;
   for (int spin = 0; spin < kFlagWaitPolls; ++spin) {
     int32_t v0, v1;
-    asm volatile("ld.acquire.gpu.global.s32 %0, [%2];\nld.acquire.gpu.global.s32 %1, [%3];" : "=&r"(v0), "=r"(v1) : "l"(flag0), "l"(flag1) : "memory");
-    if (v0 == value && v1 == value) return true;
+    asm volatile("ld.acquire.gpu.global.s32 %0, [%2];\nld.acquire.gpu.global.s32 %1, [%3];" : "=&r"(v0), "=r"(v1) : "l"(ready), "l"(tail_ready) : "memory");
+    if ((v0 & ~1) == list_ready(epoch) && v1 == epoch) return true;
     __nanosleep(pause);
     if (pause < 256) pause <<= 1;
   }
@@ -379,9 +382,12 @@ int launch_append_bulk(const DevCtx &c, int req, int layer, const __nv_bfloat16 
 int launch_append_edge(const DevCtx &c, const AppendEdgeArgs &a, const __nv_bfloat16 *k,
                        const __nv_bfloat16 *v, int n_new, cudaStream_t st, Prof *prof,
                        void *dq = nullptr, const void *sq = nullptr, size_t q_bytes = 0);
-int launch_cluster_count(const int32_t *tp, size_t rows, int H, int C, int32_t *count, unsigned long long *bad, cudaStream_t st);
-int launch_cluster_place(const int32_t *tp, int64_t n, int H, int C, const int32_t *base, int32_t *run, int32_t *place, cudaStream_t st);
-int launch_cluster_tables(const DevCtx &c, int req, int layer, int C, int n_pages, int n_tokens, const int32_t *count, int slots, cudaStream_t st);
+int launch_cluster_count(const int32_t *tp, size_t first, size_t rows, int H, int C, int c0, int nc, int32_t *count, unsigned long long *bad,
+                         cudaStream_t st);
+int launch_cluster_place(const DevCtx &c, int req, int layer, const int32_t *tp, int64_t n, int C, bool first_chunk, bool last_chunk, int32_t *place,
+                         cudaStream_t st);
+int launch_cluster_tables(const DevCtx &c, int req, int layer, int C, int c0, int nc, int n_pages, int n_tokens, const int32_t *count, int slots,
+                          cudaStream_t st);
 int launch_cluster_scatter(const DevCtx &c, int req, int layer, const __nv_bfloat16 *k, const __nv_bfloat16 *v,
                            const int32_t *place, int64_t n_tokens, cudaStream_t st);
 int launch_cluster_scatter_staged(const DevCtx &c, const __nv_bfloat16 *k, const __nv_bfloat16 *v, const int32_t *place,

@@ -1006,8 +1006,7 @@ __device__ __forceinline__ void cache_stage(const DevCtx &c, int b, int set, int
     atomicAdd(&k->bypass_pages, (unsigned long long)sh.bypass_pages);
     // no early list on this path: all flags go up together, and attention may start on this set
     first_flag_publish(c.ready1 + b, first_flag(epoch, total_pages + tail_pages, 0));
-    flag_publish(c.ready + b, epoch);
-    flag_publish(c.slots_ready + b, epoch);
+    flag_publish(c.ready + b, slots_ready(epoch));
   }
 }
 
@@ -1621,7 +1620,7 @@ __device__ __forceinline__ void cache_fast(const DevCtx &c, const Batch &bt, int
   // The list is complete but for the missed pages' slots, which nobody needs before such a page has
   // arrived: attention may go on to the hits while slots are being freed (a step without misses
   // has nothing left to wait for).
-  if (tid == 0 && early) flag_publish(c.ready + b, bt.epoch);
+  if (tid == 0 && early) flag_publish(c.ready + b, list_ready(bt.epoch));
 
   dbg_ts(b, 5);
   // ---- step 3: threshold, eviction, free slots in ascending order (one scan) ----------------
@@ -1784,8 +1783,7 @@ __device__ __forceinline__ void cache_fast(const DevCtx &c, const Batch &bt, int
     c.n_pages[b] = total_pages + tail_pages;
     c.n_parts[b] = np;
     c.state[set].step = t + 1;
-    if (!early) flag_publish(c.ready + b, bt.epoch);
-    flag_publish(c.slots_ready + b, bt.epoch);
+    flag_publish(c.ready + b, slots_ready(bt.epoch));
     // the counters go last: the flag's fence should not have to wait for them
     Counters *kc = c.counters;
     const int miss_pages = sh.admit_pages + sh.bypass_pages;

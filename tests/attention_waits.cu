@@ -34,7 +34,7 @@ void scene(const char *name, int list, int slots, int early, int n_miss, int clo
   c.page_desc = device<int4>(kSets * kStride);
   c.page_src = device<int32_t>(kSets * kStride);
   std::vector<int4> desc(kSets * kStride);
-  std::vector<int32_t> src(kSets * kStride), ready(kSets, list ? kEpoch : 0), tails(kSets, kEpoch), slot(kSets, slots ? kEpoch : 0), link(64, 0);
+  std::vector<int32_t> src(kSets * kStride), ready(kSets, list ? 2 * kEpoch + slots : 0), tails(kSets, kEpoch), link(kLinkDone + 1, 0);
   std::vector<unsigned long long> first(kSets);
   for (int b = 0; b < kSets; ++b) {
     for (int i = 0; i < kList; ++i) {
@@ -45,11 +45,10 @@ void scene(const char *name, int list, int slots, int early, int n_miss, int clo
     first[b] = (unsigned long long)kEpoch << 32 | (unsigned)kList << 12 | (unsigned)early;
   }
   put(c.page_desc, desc); put(c.page_src, src);
-  c.ready = device<int32_t>(kSets); c.tail_ready = device<int32_t>(kSets); c.slots_ready = device<int32_t>(kSets);
+  c.ready = device<int32_t>(kSets); c.tail_ready = device<int32_t>(kSets);
   c.ready1 = device<unsigned long long>(kSets);
-  put(c.ready, ready); put(c.tail_ready, tails); put(c.slots_ready, slot); put(c.ready1, first);
+  put(c.ready, ready); put(c.tail_ready, tails); put(c.ready1, first);
   c.link = device<int32_t>(kLinkDone + 1);
-  link.resize(kLinkDone + 1);
   link[kLinkDone] = closed;
   put(c.link, link);
   c.att_part = device<float>((size_t)kSets * c.max_chunks * kG * (kHeadDim + 2));
@@ -78,7 +77,7 @@ void scene(const char *name, int list, int slots, int early, int n_miss, int clo
   printf("%-40s %s: cuda %d, error bits %u, turns taken %d, closed %d, outputs not zero %d, not written %d\n", name, good ? "ok" : "WRONG", (int)e,
          k.error_bits, link[0], link[kLinkDone] - closed, nonzero, untouched);
   ok_all = ok_all && good;
-  for (void *p : {(void *)c.gpu_pages, (void *)c.page_desc, (void *)c.page_src, (void *)c.ready, (void *)c.tail_ready, (void *)c.slots_ready, (void *)c.ready1,
+  for (void *p : {(void *)c.gpu_pages, (void *)c.page_desc, (void *)c.page_src, (void *)c.ready, (void *)c.tail_ready, (void *)c.ready1,
                   (void *)c.link, (void *)c.att_part, (void *)c.att_count, (void *)c.counters, (void *)q, (void *)out})
     cudaFree(p);
   cudaFreeHost(host);
