@@ -959,10 +959,10 @@ int launch_select(const DevCtx &c, Batch &b, const __nv_bfloat16 *q, const __nv_
   int keys_cap = fuse ? max_cand : 0, tbl_cap = 0;
   size_t smem = 0;
   if (fuse) smem = cache_smem > (size_t)keys_cap * 4 ? cache_smem : (size_t)keys_cap * 4;
+  int max_slots_batch = 0;
   {
     // the low-latency continuation: the keys and the whole GPU page table
     // of a set in shared memory
-    int max_slots_batch = 0;
     for (int i = 0; i < b.n_req; ++i) max_slots_batch = b.slots[i] > max_slots_batch ? b.slots[i] : max_slots_batch;
     const size_t fs = fast_smem_bytes(max_cand, max_slots_batch, c.dir_part, c.dir_slot, c.dir_page, c.max_parts, c.max_pages, 0);
     if (max_slots_batch <= kFastSlots && max_cand <= 16384 && fs <= 100 * 1024) {
@@ -1038,9 +1038,13 @@ int launch_select(const DevCtx &c, Batch &b, const __nv_bfloat16 *q, const __nv_
       return 2;
     }
   }
-  // resident form (grid sized in launch_score_g) when scoring is many waves long
+  // Resident form (grid sized in launch_score_g) when scoring is many waves long and the caches are small
+  // against it, so that attention has pages to bring in meanwhile.  Sets with more than 1024 slots have the
+  // page table's copy beside the staged segment, which leaves fewer CTAs per SM, and few misses: 24 requests of
+  // 20000 tokens with all pages cached 90 us in this form, 77 with a CTA per item; 8 of 60000 108 and 83, with
+  // a cache of 0.3 93 and 74.
   sg.persistent = (!stream && (fuse == 2 || fuse == 3) && c.ready && c.resident_scoring >= 0 &&
-                   (c.resident_scoring == 1 || (fuse == 2 && sg.n_items > 12 * sm_count_of_device()))) ? 1 : 0;
+                   (c.resident_scoring == 1 || (fuse == 2 && max_slots_batch <= 1024 && sg.n_items > 12 * sm_count_of_device()))) ? 1 : 0;
   dim3 grid(sg.n_items);
   if (!stream) b.attn_set_major = sg.persistent;
   if (!stream) {
