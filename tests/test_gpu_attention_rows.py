@@ -13,7 +13,7 @@ pytestmark = pytest.mark.gpu
 @pytest.mark.parametrize("sets,group,pages", [
     (1, 1, 1), (1, 8, 7), (2, 4, 8), (3, 2, 9), (1, 4, 33), (5, 1, 72),   # one CTA; a CTA's remainder; several CTAs
     (64, 4, 129),                                                        # six CTAs per set
-    (449, 1, 129), (450, 1, 140),                                        # one CTA per set: 32 and 35 pages per warp, more CTAs than fit
+    (449, 1, 129), (450, 1, 140),                                        # one CTA per set: up to 33 and 35 pages per warp, more CTAs than fit
     (222, 8, 17), (223, 8, 17),                                          # two CTAs per set, then one
     (2, 1, 600),                                                         # 75 partials: three tiles of the merge
 ])
