@@ -782,8 +782,8 @@ __device__ __align__(256) static float g_static_partials[kStaticPartialFloats];
 // Arrival words, one per set: the size limit admits fewer sets than this (130 floats and a counter each).
 constexpr int kStaticSets = (int)(kStaticPartialFloats / (kHeadDim + 2 + 1)) + 1;
 __device__ static unsigned long long g_static_words[kStaticSets];         // zero between calls (see last_row)
-float *g_static_partials_addr[kMaxDevices] = {};                          // per device, set up once
-unsigned long long *g_static_words_addr[kMaxDevices] = {};
+std::atomic<float *> g_static_partials_addr[kMaxDevices] = {};            // per device, set up by the first call that finds one missing
+std::atomic<unsigned long long *> g_static_words_addr[kMaxDevices] = {};
 std::atomic<uint32_t> g_static_calls{0};
 }  // namespace
 }  // namespace spin
@@ -819,19 +819,20 @@ extern "C" int spin_paged_attention_static(const void *q, const void *page_pool,
     fprintf(stderr, "spin_paged_attention_static: no usable current CUDA device\n");
     return SPIN_ERR_CUDA;
   }
-  if (!g_static_partials_addr[dev]) {
+  float *p = g_static_partials_addr[dev].load(std::memory_order_relaxed);
+  unsigned long long *w = g_static_words_addr[dev].load(std::memory_order_relaxed);
+  if (!p || !w) {
     // In host code the arrays' names are only stand-ins for the symbols: the addresses the
-    // kernels can use have to be asked for, once per device, with that device current.
-    float *p = nullptr;
-    unsigned long long *w = nullptr;
+    // kernels can use have to be asked for, once per device, with that device current (several
+    // threads that do so at once get the same ones).
     cudaError_t e = cudaGetSymbolAddress(reinterpret_cast<void **>(&p), g_static_partials);
     if (e == cudaSuccess) e = cudaGetSymbolAddress(reinterpret_cast<void **>(&w), g_static_words);
     if (e != cudaSuccess || !p || !w) {
       fprintf(stderr, "spin_paged_attention_static: cudaGetSymbolAddress failed: %s\n", cudaGetErrorString(e));
       return SPIN_ERR_CUDA;
     }
-    g_static_words_addr[dev] = w;
-    g_static_partials_addr[dev] = p;
+    g_static_words_addr[dev].store(w, std::memory_order_relaxed);
+    g_static_partials_addr[dev].store(p, std::memory_order_relaxed);
   }
   DevCtx c{};
   c.num_layers = 1; c.Hq = group; c.Hkv = 1; c.G = group;
@@ -849,9 +850,9 @@ extern "C" int spin_paged_attention_static(const void *q, const void *page_pool,
   c.ready = nullptr;                                        // plain stream order: no per-set flags
   c.tail_ready = nullptr;
   c.ready1 = nullptr;
-  c.att_part = g_static_partials_addr[dev];
+  c.att_part = p;
   c.att_ml = reinterpret_cast<float2 *>(c.att_part + (size_t)n_sets * chunks * group * kHeadDim);
-  c.att_words = g_static_words_addr[dev];
+  c.att_words = w;
   c.att_call = g_static_calls.fetch_add(1u, std::memory_order_relaxed) + 1u;
   cudaStream_t st = reinterpret_cast<cudaStream_t>(cuda_stream);
   Batch b{};
