@@ -1035,6 +1035,8 @@ static int reindex_impl(spin_ctx *ctx, int32_t req, int32_t layer, void *cuda_st
     }
   }
   if (ctx->host_page_pool.available() < need) return fail(ctx, SPIN_ERR_OOM_HOST, "out of host pages");
+  // what a fold has always taken, some 127000 clusters; it keeps k_reindex_apply's bit per cluster within
+  // 16 KB of shared memory, beside its entry per tail page
   const size_t stage_bytes = (size_t)std::max<int64_t>(g.stage_tokens, ctx->cfg.max_requests) * H * kRowBytes;
   if ((size_t)H * (C + (C + 31) / 32) * 4 > stage_bytes) return fail(ctx, SPIN_ERR_INVALID, "too many clusters for the staging buffer");
   // 3. The sets' Partition Offset and CPU page tables: clusters in order, each one's pages together,

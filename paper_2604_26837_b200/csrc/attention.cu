@@ -3,14 +3,16 @@
 // CTAs and merged by log-sum-exp.
 //
 // k_attn: a set's page list is dealt out to the warps of its CTAs (4 warps each), page by page in
-// turn, so every warp has its share of the missed pages (which lead the list) and of the hits.
+// turn, so every warp has its share of the missed pages (which lead the list) and of the hits.  Sets
+// have equal shares of the GPU as a rule, lists far above the average more (see attn_rows_of).
 // A warp keeps two pages in flight in shared memory and one accumulator over all its pages; the
 // CTA writes one partial.  A page (8 KiB: 16 K rows, then 16 V rows) is brought in by one
 // instruction, a 512-byte bulk copy (TMA) per lane of half the warp, each pair of rows to its own
 // place at a stride of 528 bytes; a tile takes the even tokens as its rows 0..7 and the odd ones as
 // rows 8..15, so ldmatrix reads 8 rows without a bank conflict.  (256 sets of 56 pages, 8 heads:
 // 24.0 us; with a copy per row, twice as many for the SM's one copy unit, 32; per four rows, at a
-// two-way conflict, 26.5; per page, at an eight-way conflict, 59.)  The page comes from an HBM
+// two-way conflict, 26.5; per page, at an eight-way conflict, 59.  Rounding against each page's maximum,
+// see attend_page, has made the first 24.8 since.)  The page comes from an HBM
 // slot for a hit and straight from pinned host memory for a miss, so the missed pages of the step
 // are on the host link while the hits are being attended from HBM.  A missed page that was
 // admitted to the cache goes from shared memory to its HBM slot by bulk copies too (that is the
@@ -427,7 +429,7 @@ __device__ __forceinline__ void attn_row(const DevCtx &c, const Batch &bt, const
   }
   int np = 0, nm = 0;                      // pages in the set's list; how many of them are early descriptors
   if (c.ready) {
-    // A set raises three flags.  The first says that its missed pages are listed (the leading
+    // A set raises three flags (the last two are one word).  The first says that its missed pages are listed (the leading
     // descriptors, slot still open): a warp requests its first missed page at once, so the
     // pages cross the host link while the cache manager is still busy.  For the hits a warp waits
     // for the second flag (complete list) and for the tail page, for the slot of a page that has

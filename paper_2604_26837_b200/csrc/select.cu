@@ -1008,8 +1008,8 @@ int launch_select(const DevCtx &c, Batch &b, const __nv_bfloat16 *q, const __nv_
   // (query groups of up to four heads: a candidate's block sums then fit into its own row)
   const bool stream = (fuse == 2 || fuse == 3) && c.ready && c.G <= 4 && c.resident_scoring == 2;
   if (stream) {
-    // shared memory of an SM: this kernel's ring beside ONE more CTA, an attention CTA (64 KiB of
-    // pages and its per-warp partials) or a selection CTA (smaller); the selection CTAs, one per
+    // shared memory of an SM: this kernel's ring beside ONE more CTA, an attention CTA (its warps'
+    // stages and a few hundred bytes) or a selection CTA (smaller); the selection CTAs, one per
     // set, take some SMs and the first attention CTAs the others.  1 KiB per CTA is the system's.
     const int attn_smem = kAttnCtaSmem + 4 * 1024;
     int n_stages = 227 * 1024 - attn_smem - 8 * 1024;

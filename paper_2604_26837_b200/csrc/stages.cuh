@@ -1540,7 +1540,7 @@ __device__ __forceinline__ void cache_fast(const DevCtx &c, const Batch &bt, int
   // has been freed.  With the fetch fused into attention those descriptors (slot still open,
   // x = -3) are published now under the set's first flag: the attention CTAs that own them
   // put the pages on the host link while this CTA goes on to promote, evict and admit, and
-  // pick the slot up from page_src once the third flag is set.
+  // pick the slot up from page_src once `ready` says that the slots are known.
   const size_t pl = (size_t)b * (c.max_pages + c.tail_cap);
   int32_t *page_src = c.page_src + pl, *page_slot = c.page_slot + pl;
   int32_t *page_part = c.page_part + pl, *page_pidx = c.page_pidx + pl;
