@@ -413,7 +413,7 @@ __device__ __forceinline__ bool further_row(const DevCtx &c, const Batch &bt, in
 // One row of a set by a CTA of W warps (kAttnWarps; 1 for lists that fit one, which have a single row).
 template <int G, int W>
 __device__ __forceinline__ void attn_row(const DevCtx &c, const Batch &bt, const __nv_bfloat16 *__restrict__ q,
-                                         __nv_bfloat16 *__restrict__ out, uint8_t *smem, int b, int row, int max_rows, int share) {
+                                         __nv_bfloat16 *__restrict__ out, uint8_t *smem, int b, int row, int max_rows, int share, int counted = -1) {
   __shared__ __align__(8) unsigned long long s_bar[W * kWarpStages];
   __shared__ float s_m[W][G], s_l[W][G];
   __shared__ int sh_ok, sh_np, sh_nm, sh_last;
@@ -448,7 +448,7 @@ __device__ __forceinline__ void attn_row(const DevCtx &c, const Batch &bt, const
     pages_visible();
   } else {
     pdl_wait_prev();
-    np = max(0, min(c.n_pages[b], np_most));
+    np = counted >= 0 ? counted : max(0, min(c.n_pages[b], np_most));
     __syncwarp();
   }
   if (row == 0) dbg_ta(b, 10);
@@ -691,9 +691,14 @@ k_attn(DevCtx c, Batch bt, const __nv_bfloat16 *__restrict__ q, __nv_bfloat16 *_
     __shared__ int s_sum[kAttnWarps], s_at[2];
     int b = blockIdx.x % bt.n_req, row = blockIdx.x / bt.n_req;
     pdl_wait_prev();
+    int np = count_of(c, b);                                      // (asked for together with the other counts)
     const int share = share_by_counts(c, bt, s_sum), own = bt.n_req * bt.attn_rows;
-    if ((int)blockIdx.x < own || further_row(c, bt, share, (int)blockIdx.x - own, s_sum, s_at, &b, &row))
-      attn_row<G, W>(c, bt, q, out, smem, b, row, c.max_chunks, share);
+    bool mine = (int)blockIdx.x < own;
+    if (!mine) {
+      mine = further_row(c, bt, share, (int)blockIdx.x - own, s_sum, s_at, &b, &row);
+      if (mine) np = count_of(c, b);
+    }
+    if (mine) attn_row<G, W>(c, bt, q, out, smem, b, row, c.max_chunks, share, np);
   }
   if (blockIdx.x == 0 && blockIdx.y == 0) pdl_wait_prev();
 }
@@ -726,9 +731,11 @@ void launch_attn_g(const DevCtx &c, Batch b, const __nv_bfloat16 *q, __nv_bfloat
   // CTAs each: 35 us instead of 25.  In a decode step the average is the host's estimate, and the grid has
   // rows for the longest list it may meet, at most kExtraCtas of them, which leave at once where they
   // are not needed (~1 ns each).  Where only the device knows the lengths, CTAs take the average from the
-  // counts, and fewer spare ones find out from them what is theirs; looking at the counts costs a call ~1 us
-  // (256 even lists of 56 pages: 26.0 us instead of 25.0), so it is done where a list may leave a CTA more than
-  // 2 kSharePages (445 lists, one of 64 pages and the rest of 8: 19 us without, 22 with).
+  // counts, and fewer spare ones find out from them what is theirs.  That costs a call of even lists 1-2 us,
+  // so it is done where a list may leave a CTA more than 48 pages (72 lists, one of 354 pages and the rest of
+  // 8: 15 us with, 21 without, 17 with a CTA per 8 pages), or 64 where sets have one CTA each: there are so
+  // many of them then that looking costs most (256 lists of 56 pages: 25 us without, 27 with) and gains
+  // least (445 lists, one of 64 and the rest of 8: 19 without, 22 with).
   auto clamp = [](long long x, long long lo, long long hi) { return (int)(x > hi ? hi : x < lo ? lo : x); };
   const int chunks = clamp((max_pages + kCtaPages - 1) / kCtaPages, 1, c.max_chunks);
   b.attn_rows = clamp(resident / n_sets, 1, chunks);
@@ -740,7 +747,7 @@ void launch_attn_g(const DevCtx &c, Batch b, const __nv_bfloat16 *q, __nv_bfloat
     launch_pdl(k_attn<G, 1, false>, b.attn_set_major ? dim3(1, n_sets) : dim3(n_sets, 1), dim3(32), (size_t)kAttnSmem / kAttnWarps, st, 1, c, b, q, out);
     return;
   }
-  if (!c.ready && max_pages > 2 * kSharePages * b.attn_rows) {
+  if (!c.ready && max_pages > (b.attn_rows > 1 ? 3 : 4) * kSharePages / 2 * b.attn_rows) {
     const int own = n_sets * b.attn_rows;
     launch_pdl(k_attn<G, kAttnWarps, true>, dim3(own + own * 2 / 3), dim3(kAttnThreads), (size_t)kAttnSmem, st, 1, c, b, q, out);
     return;

@@ -113,6 +113,7 @@ def _lists(sets, group, pages, counts, seed=5):
     (256, 1, 500, 8, {i: 500 for i in range(100, 256, 2)}), # further rows of many lists
     (64, 1, 500, 9, {0: 500, 63: 65}),                      # 16 rows where six are the rule
     (64, 8, 248, 9, {0: 248, 63: 65}),                      # lists too short for the counts to be looked at
+    (72, 2, 288, 8, {0: 288, 71: 287}), (72, 2, 289, 8, {0: 289, 71: 288}),   # the longest such, one more
     (700, 1, 180, 3, {0: 180, 1: 33, 698: 95, 699: 97}),    # more sets than CTAs at once
     (223, 2, 280, 0, {5: 280}),                             # nothing in the other lists
     (1790, 1, 72, 1, {0: 72, 1789: 33}), (2048, 1, 56, 1, {0: 56, 2047: 33}),   # the most sets that the built-in arrays take with such lists
