@@ -342,6 +342,46 @@ int validate_req_layer(spin_ctx *ctx, int req, int layer) {
   return SPIN_OK;
 }
 
+// Pages per head that a slot of the staging ring takes: a slot is laid out [head][page].
+inline int64_t staged_pages(const spin_ctx *ctx) { return ctx->offload_slot_units / ctx->cfg.num_kv_heads; }
+
+// Host pages for the logical pages [j, j_end) of a set, entered in its CPU page table; false: no segment left.
+bool take_host_pages(spin_ctx *ctx, int set, int64_t j, int64_t j_end) {
+  const Geometry &g = ctx->g;
+  SetHost &S = ctx->sets[(size_t)set];
+  while (j < j_end) {
+    const int64_t end = std::min(j_end, ((j >> g.seg_shift) + 1) << g.seg_shift);
+    const int seg = ensure_seg(ctx, ctx->cpt_segs, S.dir_cpt, ctx->d.dir_cpt + (size_t)set * g.dir_page, j, g.seg_shift);
+    if (seg < 0) return false;
+    int32_t *cpt = ctx->h_cpt_pool + ((size_t)seg << g.seg_shift);
+    for (; j < end; ++j) {
+      const int32_t hp = (int32_t)ctx->host_page_pool.alloc();
+      cpt[j & (g.seg - 1)] = hp;
+      S.host_pages.push_back(hp);
+    }
+  }
+  return true;
+}
+
+// A staged slot (m pages of every head) to the host tier: one copy-engine transfer per
+// run of consecutive host pages.  Pages are handed out in the slot's own order, so the slot is one run as a
+// rule, of several MB: the engine moves 55.7 GB/s in pieces of 8 MB, 47 in pieces of 1 MB (a head's pages
+// of 2048 tokens), 31 in pieces of 256 KB.  (Fragmented host pools mean more and shorter transfers.)
+// hp: the units' host pages, negative where a head has no such page.
+cudaError_t drain_slot(spin_ctx *ctx, const uint8_t *stage, const std::vector<int32_t> &hp) {
+  for (size_t u = 0; u < hp.size();) {
+    size_t len = 1;
+    if (hp[u] >= 0) {
+      while (u + len < hp.size() && hp[u + len] == hp[u] + (int32_t)len) ++len;
+      const cudaError_t e = cudaMemcpyAsync(ctx->h_pages + (size_t)hp[u] * kPageBytes, stage + u * kPageBytes, len * kPageBytes,
+                                            cudaMemcpyDeviceToHost, ctx->offload_stream);
+      if (e != cudaSuccess) return e;
+    }
+    u += len;
+  }
+  return cudaSuccess;
+}
+
 // Host-side Index/Offload bookkeeping of the page-sized kinds for one (request, layer) that
 // grows from n0 to n1 tokens: allocate host pages, fill CPU page table / Partition Offset
 // entries, map the segments the kernels will write.
@@ -356,21 +396,19 @@ int grow_paged(spin_ctx *ctx, int req, int layer, int64_t n1) {
   const int64_t new_pages = j_end - first_new_page + 1;
   if (new_pages > 0 && ctx->host_page_pool.available() < new_pages * ctx->cfg.num_kv_heads)
     return fail(ctx, SPIN_ERR_OOM_HOST, "out of host pages");
-  // segment by segment: the tables' entries of a segment are consecutive in the pinned pools
+  // Host pages in the order in which the staging ring drains them (see staged_pages): what a slot takes of
+  // every head is one run.  Segment by segment: the tables' entries of a segment are consecutive in
+  // the pinned pools.
+  const int64_t per = ctx->offload_slot_units > 0 ? staged_pages(ctx) : new_pages;
+  for (int64_t p = first_new_page; p <= j_end;) {
+    const int64_t p_end = ctx->offload_slot_units > 0 && p < j_end ? std::min(j_end, p + per) : std::min(j_end + 1, p + per);
+    for (int h = 0; h < ctx->cfg.num_kv_heads; ++h)
+      if (!take_host_pages(ctx, set_index(d, req, layer, h), p, p_end)) return fail(ctx, SPIN_ERR_OOM_HOST, "out of CPU page table segments");
+    p = p_end;
+  }
   for (int h = 0; h < ctx->cfg.num_kv_heads; ++h) {
     const int set = set_index(d, req, layer, h);
     SetHost &S = ctx->sets[(size_t)set];
-    for (int64_t j = first_new_page; j <= j_end;) {
-      const int64_t end = std::min(j_end + 1, ((j >> g.seg_shift) + 1) << g.seg_shift);
-      const int seg = ensure_seg(ctx, ctx->cpt_segs, S.dir_cpt, d.dir_cpt + (size_t)set * g.dir_page, j, g.seg_shift);
-      if (seg < 0) return fail(ctx, SPIN_ERR_OOM_HOST, "out of CPU page table segments");
-      int32_t *cpt = ctx->h_cpt_pool + ((size_t)seg << g.seg_shift);
-      for (; j < end; ++j) {
-        const int32_t hp = (int32_t)ctx->host_page_pool.alloc();
-        cpt[j & (g.seg - 1)] = hp;
-        S.host_pages.push_back(hp);
-      }
-    }
     // partitions L.n_partitions .. j_end-1 get indexed by this call
     for (int64_t p = L.n_partitions; p < j_end;) {
       const int64_t end = std::min(j_end, ((p >> g.seg_shift) + 1) << g.seg_shift);
@@ -492,42 +530,24 @@ int append_paged_device(spin_ctx *ctx, int req, int layer, const __nv_bfloat16 *
   const int64_t first = j0 + 1, nb = j_end - first;
   if (ctx->offload_slot_units > 0 && nb > 0) {
     // asynchronous offload: slot by slot through the staging ring (see spin_ctx)
-    const int64_t per = ctx->offload_slot_units / ctx->cfg.num_kv_heads;
+    const int64_t per = staged_pages(ctx);
     for (int64_t p = 0; p < nb; p += per) {
       const int m = (int)std::min<int64_t>(per, nb - p), slot = ctx->offload_next;
       ctx->offload_next = (slot + 1) % spin_ctx::kOffloadSlots;
       if (ctx->slot_used[slot]) CK(cudaStreamWaitEvent(st, ctx->ev_done[slot], 0));     // ring full: wait for the drain
       uint8_t *stage = ctx->offload_stage + (size_t)slot * ctx->offload_slot_units * kPageBytes;
       int32_t *hp = ctx->offload_hp + (size_t)slot * ctx->offload_slot_units;
-      {
-        // the pages' host ids come with the call (head-major like the slot): while copy-engine
-        // transfers own the host link, a kernel's small reads of the pinned CPU page table
-        // would wait behind them
-        std::vector<int32_t> ids((size_t)m * ctx->cfg.num_kv_heads);
-        for (int h = 0; h < ctx->cfg.num_kv_heads; ++h) {
-          const std::vector<int32_t> &hpv = set_of(ctx, req, layer, h).host_pages;
-          for (int i = 0; i < m; ++i) ids[(size_t)h * m + i] = hpv[(size_t)(first + p + i)];
-        }
-        CK(cudaMemcpyAsync(hp, ids.data(), ids.size() * 4, cudaMemcpyHostToDevice, st));   // pageable source: staged before the call returns
-      }
+      // the pages' host ids come with the call (head-major like the slot): while copy-engine
+      // transfers own the host link, a kernel's small reads of the pinned CPU page table
+      // would wait behind them
+      std::vector<int32_t> ids((size_t)m * ctx->cfg.num_kv_heads);
+      for (int h = 0; h < ctx->cfg.num_kv_heads; ++h)
+        std::copy_n(set_of(ctx, req, layer, h).host_pages.begin() + (first + p), m, ids.begin() + (ptrdiff_t)h * m);
+      CK(cudaMemcpyAsync(hp, ids.data(), ids.size() * 4, cudaMemcpyHostToDevice, st));   // pageable source: staged before the call returns
       ctx->launches += launch_append_bulk(ctx->d, req, layer, k, v, (int)(first + p), m, (int)n0, st, &ctx->prof, stage, hp);
       CK(cudaEventRecord(ctx->ev_staged[slot], st));
       CK(cudaStreamWaitEvent(ctx->offload_stream, ctx->ev_staged[slot], 0));
-      // The slot is laid out head-major, the order in which host pages were handed out, so a
-      // head's pages are as a rule one run of consecutive host pages: one copy-engine transfer
-      // per run, no SM involved (a fragmented host pool means more and shorter transfers).
-      const int H = ctx->cfg.num_kv_heads;
-      for (int h = 0; h < H; ++h) {
-        const std::vector<int32_t> &hpv = set_of(ctx, req, layer, h).host_pages;
-        for (int i = 0; i < m;) {
-          int len = 1;
-          while (i + len < m && hpv[(size_t)(first + p + i + len)] == hpv[(size_t)(first + p + i)] + len) ++len;
-          CK(cudaMemcpyAsync(ctx->h_pages + (size_t)hpv[(size_t)(first + p + i)] * kPageBytes,
-                             stage + ((size_t)h * m + i) * kPageBytes, (size_t)len * kPageBytes,
-                             cudaMemcpyDeviceToHost, ctx->offload_stream));
-          i += len;
-        }
-      }
+      CK(drain_slot(ctx, stage, ids));
       CK(cudaEventRecord(ctx->ev_done[slot], ctx->offload_stream));
       ctx->slot_used[slot] = true;
       ctx->offload_last = slot;
@@ -621,6 +641,7 @@ int prefill_clustered_impl(spin_ctx *ctx, int req, int layer, const void *k, con
   if (ctx->host_page_pool.available() < pages_needed) return fail(ctx, SPIN_ERR_OOM_HOST, "out of host pages");
   // 2. the sets' pages, clusters in order, each one's pages together
   int32_t total_pages_max = 0;
+  std::vector<int32_t> n_pages_of((size_t)H);
   for (int h = 0; h < H; ++h) {
     const int set = set_index(d, req, layer, h);
     SetHost &S = ctx->sets[(size_t)set];
@@ -640,20 +661,15 @@ int prefill_clustered_impl(spin_ctx *ctx, int req, int layer, const void *k, con
     for (int c0 = 0; c0 < C; c0 += g.sum_entries)
       if (ensure_seg(ctx, ctx->sum_segs, S.dir_sum, d.dir_sumseg + (size_t)set * g.dir_sum, c0, g.sum_shift) < 0)
         return fail(ctx, SPIN_ERR_OOM_DEVICE, "out of summary segments");
-    for (int32_t j = 0; j < off;) {
-      const int32_t end = std::min<int32_t>(off, ((j >> g.seg_shift) + 1) << g.seg_shift);
-      const int cs = ensure_seg(ctx, ctx->cpt_segs, S.dir_cpt, d.dir_cpt + (size_t)set * g.dir_page, j, g.seg_shift);
-      if (cs < 0) return fail(ctx, SPIN_ERR_OOM_HOST, "out of CPU page table segments");
-      int32_t *cpt = ctx->h_cpt_pool + ((size_t)cs << g.seg_shift);
-      for (; j < end; ++j) {
-        const int32_t hp = (int32_t)ctx->host_page_pool.alloc();
-        cpt[j & (g.seg - 1)] = hp;
-        S.host_pages.push_back(hp);
-      }
-    }
+    n_pages_of[(size_t)h] = off;
     total_pages_max = std::max(total_pages_max, off);
     S.cl_tokens.assign(cnt, cnt + C);
   }
+  const int64_t block = ring ? staged_pages(ctx) : total_pages_max;        // in the order in which a ring drains them
+  for (int64_t p0 = 0; p0 < total_pages_max; p0 += block)
+    for (int h = 0; h < H; ++h)
+      if (!take_host_pages(ctx, set_index(d, req, layer, h), p0, std::min<int64_t>(n_pages_of[(size_t)h], p0 + block)))
+        return fail(ctx, SPIN_ERR_OOM_HOST, "out of CPU page table segments");
   // all heads of a (request, layer) share one tail position: use the largest page count so
   // that tail pages never collide with cluster pages of any head
   for (int h = 0; h < H; ++h) set_of(ctx, req, layer, h).host_pages.resize((size_t)total_pages_max, -1);
@@ -685,7 +701,7 @@ int prefill_clustered_impl(spin_ctx *ctx, int req, int layer, const void *k, con
     // the caller's stream, at HBM speed, range by range of the sets' logical pages; each slot
     // then moves to host memory by copy-engine transfers (one per run of consecutive host
     // pages) on the library's stream, behind this call.
-    const int64_t per = ctx->offload_slot_units / H;
+    const int64_t per = staged_pages(ctx);
     for (int64_t p0 = 0; p0 < total_pages_max; p0 += per) {
       const int m = (int)std::min<int64_t>(per, total_pages_max - p0), slot = ctx->offload_next;
       ctx->offload_next = (slot + 1) % spin_ctx::kOffloadSlots;
@@ -695,18 +711,9 @@ int prefill_clustered_impl(spin_ctx *ctx, int req, int layer, const void *k, con
       ctx->launches += launch_cluster_scatter_staged(d, kd, vd, room.words, (int)n, (int)p0, m, stage, st);
       CK(cudaEventRecord(ctx->ev_staged[slot], st));
       CK(cudaStreamWaitEvent(ctx->offload_stream, ctx->ev_staged[slot], 0));
-      for (int h = 0; h < H; ++h) {
-        const std::vector<int32_t> &hpv = set_of(ctx, req, layer, h).host_pages;
-        for (int i = 0; i < m;) {
-          const int32_t hp0 = hpv[(size_t)(p0 + i)];
-          if (hp0 < 0) { ++i; continue; }                                               // this head has fewer pages
-          int len = 1;
-          while (i + len < m && hpv[(size_t)(p0 + i + len)] == hp0 + len) ++len;
-          CK(cudaMemcpyAsync(ctx->h_pages + (size_t)hp0 * kPageBytes, stage + ((size_t)h * m + i) * kPageBytes,
-                             (size_t)len * kPageBytes, cudaMemcpyDeviceToHost, ctx->offload_stream));
-          i += len;
-        }
-      }
+      std::vector<int32_t> ids((size_t)H * m);
+      for (int h = 0; h < H; ++h) std::copy_n(set_of(ctx, req, layer, h).host_pages.begin() + p0, m, ids.begin() + (ptrdiff_t)h * m);
+      CK(drain_slot(ctx, stage, ids));
       CK(cudaEventRecord(ctx->ev_done[slot], ctx->offload_stream));
       ctx->slot_used[slot] = true;
       ctx->offload_last = slot;
