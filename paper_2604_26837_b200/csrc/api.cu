@@ -38,6 +38,35 @@ struct BitmapPool {
     }
     return -1;
   }
+  // `want` ids at once, lowest first (the caller has seen that they are there), a word of the bitmap at a time.
+  void take(int64_t want, int32_t *out) {
+    in_use += want;
+    for (int64_t w = hint; want > 0; ++w) {
+      uint64_t free = ~bits[(size_t)w];
+      if (free) hint = w;
+      if (free == ~0ull && want >= 64) {
+        for (int b = 0; b < 64; ++b) out[b] = (int32_t)(w * 64 + b);
+        bits[(size_t)w] = ~0ull;
+        out += 64;
+        want -= 64;
+        continue;
+      }
+      for (; free && want > 0; free &= free - 1, --want) *out++ = (int32_t)(w * 64 + __builtin_ctzll(free));
+      bits[(size_t)w] = ~free;                     // what is left of the word's free ids
+    }
+  }
+  void give(const std::vector<int32_t> &ids) {
+    for (size_t i = 0; i < ids.size();) {
+      if (ids[i] < 0 || ids[i] >= n) { ++i; continue; }
+      const int64_t w = ids[i] >> 6;
+      uint64_t m = 0;
+      for (; i < ids.size() && ids[i] >= 0 && ids[i] < n && (ids[i] >> 6) == w; ++i) m |= 1ull << (ids[i] & 63);
+      m &= bits[(size_t)w];
+      bits[(size_t)w] &= ~m;
+      in_use -= __builtin_popcountll(m);
+      hint = std::min(hint, w);
+    }
+  }
   void release(int64_t id) {
     if (id < 0 || id >= n) return;
     uint64_t m = 1ull << (id & 63);
@@ -304,6 +333,16 @@ bool is_device_ptr(const void *p) {
   return at.type == cudaMemoryTypeDevice || at.type == cudaMemoryTypeManaged;
 }
 
+// A call without a stream launches on its context's device, whichever is current.
+struct DeviceGuard {
+  int was = -1;
+  explicit DeviceGuard(int device) {
+    int now = -1;
+    if (cudaGetDevice(&now) == cudaSuccess && now != device && cudaSetDevice(device) == cudaSuccess) was = now;
+  }
+  ~DeviceGuard() { if (was >= 0) cudaSetDevice(was); }
+};
+
 inline SetHost &set_of(spin_ctx *ctx, int req, int layer, int head) {
   return ctx->sets[(size_t)set_index(ctx->d, req, layer, head)];
 }
@@ -354,11 +393,11 @@ bool take_host_pages(spin_ctx *ctx, int set, int64_t j, int64_t j_end) {
     const int seg = ensure_seg(ctx, ctx->cpt_segs, S.dir_cpt, ctx->d.dir_cpt + (size_t)set * g.dir_page, j, g.seg_shift);
     if (seg < 0) return false;
     int32_t *cpt = ctx->h_cpt_pool + ((size_t)seg << g.seg_shift);
-    for (; j < end; ++j) {
-      const int32_t hp = (int32_t)ctx->host_page_pool.alloc();
-      cpt[j & (g.seg - 1)] = hp;
-      S.host_pages.push_back(hp);
-    }
+    const size_t had = S.host_pages.size(), more = (size_t)(end - j);
+    S.host_pages.resize(had + more);
+    ctx->host_page_pool.take((int64_t)more, S.host_pages.data() + had);
+    memcpy(cpt + (j & (g.seg - 1)), S.host_pages.data() + had, more * 4);
+    j = end;
   }
   return true;
 }
@@ -954,19 +993,13 @@ int spin_request_open(spin_ctx *ctx, int64_t slots, int32_t *out_req) {
     return fail(ctx, SPIN_ERR_BUDGET, "budget needs %lld GPU pages, %lld free", (long long)(slots * sets_per_req), (long long)ctx->gpu_page_pool.available());
   if (ctx->gpt_segs.available() < segs_per_set * sets_per_req)
     return fail(ctx, SPIN_ERR_OOM_DEVICE, "out of GPU page table segments");
-  // All sets of a request are consecutive (layer by layer, head by head), so each table's rows go up
-  // in one copy, and the page table segments in one copy per run of consecutive segments.  The
-  // directories of the other tables hold nothing but "unmapped" since spin_create or the last close.
+  // All sets of a request are consecutive (layer by layer, head by head).  The directories of the other
+  // tables hold nothing but "unmapped" since spin_create or the last close.  One kernel writes the
+  // GPU page tables, tail pages and states: what it cannot work out are the runs of physical pages
+  // that the slots get (one per set as a rule) and the segments, which go up like all
+  // directory entries.  Four blocking copies of host-made tables took half of the call's time.
+  const DeviceGuard on(ctx->cfg.device);
   const int set0 = set_index(d, req, 0, 0), n_sets = (int)sets_per_req;
-  std::vector<GptEntry> ent;
-  std::vector<int32_t> dir_gpt((size_t)n_sets * g.dir_slot, -1), tails((size_t)n_sets * g.tail_cap);
-  std::vector<SetState> states((size_t)n_sets);
-  int64_t run_seg = -1;                                     // first segment of the entries collected so far
-  auto upload = [&]() {
-    cudaError_t e = ent.empty() ? cudaSuccess : cudaMemcpy(d.gpt_pool + ((size_t)run_seg << g.seg_shift), ent.data(), ent.size() * sizeof(GptEntry), cudaMemcpyHostToDevice);
-    ent.clear();
-    return e;
-  };
   for (int i = 0; i < n_sets; ++i) {
     const int set = set0 + i;
     SetHost &S = ctx->sets[(size_t)set];
@@ -976,27 +1009,34 @@ int spin_request_open(spin_ctx *ctx, int64_t slots, int32_t *out_req) {
     S.dir_gpt.assign((size_t)g.dir_slot, -1);
     S.dir_cpt.assign((size_t)g.dir_page, -1);
     S.dir_sum.assign((size_t)g.dir_sum, -1);
-    for (int64_t s0 = 0; s0 < slots; s0 += g.seg) {
-      const int64_t seg = ctx->gpt_segs.alloc();
-      S.dir_gpt[(size_t)(s0 >> g.seg_shift)] = (int32_t)seg;
-      dir_gpt[(size_t)i * g.dir_slot + (size_t)(s0 >> g.seg_shift)] = (int32_t)seg;
-      ctx->dir_bytes_in_use += 4;
-      if (!ent.empty() && seg != run_seg + (int64_t)(ent.size() >> g.seg_shift)) CK(upload());
-      if (ent.empty()) run_seg = seg;
-      const int cnt = (int)std::min<int64_t>(g.seg, slots - s0);
-      for (int k = 0; k < g.seg; ++k) {
-        int32_t phys = -1;
-        if (k < cnt) { phys = (int32_t)ctx->gpu_page_pool.alloc(); S.gpu_pages.push_back(phys); }
-        ent.push_back(GptEntry{-1, phys, 0, -1});
-      }
-    }
-    for (int j = 0; j < g.tail_cap; ++j) tails[(size_t)i * g.tail_cap + j] = (int32_t)(ctx->cfg.gpu_cache_pages + (int64_t)set * g.tail_cap + j);
-    states[(size_t)i].slots = (int32_t)slots;
+    for (int64_t s0 = 0; s0 < slots; s0 += g.seg)
+      ensure_seg(ctx, ctx->gpt_segs, S.dir_gpt, d.dir_gpt + (size_t)set * g.dir_slot, s0, g.seg_shift);
+    S.gpu_pages.resize((size_t)slots);
+    ctx->gpu_page_pool.take(slots, S.gpu_pages.data());
   }
-  CK(upload());
-  CK(cudaMemcpy(d.dir_gpt + (size_t)set0 * g.dir_slot, dir_gpt.data(), dir_gpt.size() * 4, cudaMemcpyHostToDevice));
-  CK(cudaMemcpy(d.tail_phys + (size_t)set0 * g.tail_cap, tails.data(), tails.size() * 4, cudaMemcpyHostToDevice));
-  CK(cudaMemcpy(d.state + set0, states.data(), states.size() * sizeof(SetState), cudaMemcpyHostToDevice));
+  launch_dir_update(d, ctx->dir_updates.data(), (int)ctx->dir_updates.size(), nullptr);   // (the count of launches is of those that work for requests)
+  ctx->dir_updates.clear();
+  const int64_t padded = segs_per_set << g.seg_shift;           // entries that a set's segments have
+  OpenRuns runs;
+  runs.n = 0;
+  int64_t from = 0;                                             // entries before this one are on their way
+  for (int i = 0; i < n_sets; ++i) {
+    const std::vector<int32_t> &pages = ctx->sets[(size_t)(set0 + i)].gpu_pages;
+    for (int64_t s = 0; s < slots; ++s) {
+      if (s > 0 && pages[(size_t)s] == pages[(size_t)s - 1] + 1) continue;
+      const int64_t at = i * padded + s;
+      if (runs.n == OpenRuns::kMost) {
+        launch_request_open(d, set0, n_sets, (int)slots, padded, from, at, ctx->cfg.gpu_cache_pages, runs, nullptr);
+        from = at;
+        runs.n = 0;
+      }
+      runs.at[runs.n] = at;
+      runs.page[runs.n++] = pages[(size_t)s];
+    }
+  }
+  launch_request_open(d, set0, n_sets, (int)slots, padded, from, n_sets * padded, ctx->cfg.gpu_cache_pages, runs, nullptr);
+  CK(cudaGetLastError());
+  CK(cudaStreamSynchronize(nullptr));                           // the request may be used on any stream from here on
   RequestHost &R = ctx->reqs[(size_t)req];
   R.open = true;
   R.slots = slots;
@@ -1149,8 +1189,8 @@ int spin_request_close(spin_ctx *ctx, int32_t req) {
     for (int h = 0; h < ctx->cfg.num_kv_heads; ++h) {
       const int set = set_index(d, req, l, h);
       SetHost &S = ctx->sets[(size_t)set];
-      for (int32_t p : S.gpu_pages) ctx->gpu_page_pool.release(p);
-      for (int32_t p : S.host_pages) ctx->host_page_pool.release(p);
+      ctx->gpu_page_pool.give(S.gpu_pages);
+      ctx->host_page_pool.give(S.host_pages);
       auto drop = [&](BitmapPool &pool, std::vector<int32_t> &dir) {
         for (int32_t s : dir) if (s >= 0) { pool.release(s); ctx->dir_bytes_in_use -= 4; }
       };
@@ -1161,14 +1201,10 @@ int spin_request_close(spin_ctx *ctx, int32_t req) {
       drop(ctx->sum_segs, S.dir_sum);
       S = SetHost();
     }
-  // the rows of a request's sets are consecutive in every table
-  const size_t set0 = (size_t)set_index(d, req, 0, 0), n = (size_t)ctx->cfg.num_layers * ctx->cfg.num_kv_heads;
-  CK(cudaMemset(d.dir_gpt + set0 * g.dir_slot, 0xff, n * g.dir_slot * 4));
-  CK(cudaMemset(d.dir_meta + set0 * g.dir_part, 0xff, n * g.dir_part * 4));
-  CK(cudaMemset(d.dir_off + set0 * g.dir_part, 0xff, n * g.dir_part * 4));
-  CK(cudaMemset(d.dir_cpt + set0 * g.dir_page, 0xff, n * g.dir_page * 4));
-  CK(cudaMemset(d.dir_sumseg + set0 * g.dir_sum, 0xff, n * g.dir_sum * 4));
-  CK(cudaMemset(d.state + set0, 0, n * sizeof(SetState)));
+  // the rows of a request's sets are consecutive in every table: one kernel for all (six memsets before)
+  const DeviceGuard on(ctx->cfg.device);
+  launch_request_close(d, set_index(d, req, 0, 0), ctx->cfg.num_layers * ctx->cfg.num_kv_heads, nullptr);
+  CK(cudaGetLastError());
   R = RequestHost();
   return SPIN_OK;
 }
