@@ -20,7 +20,8 @@
 // with fp32 accumulators (the page's 16 tokens resp. 16 channels as M, the query heads as N = 8): at
 // ~4 flop/byte the kernel is HBM/PCIe bound and tensor tiles are used to take instruction issue
 // off the critical path, which is also why the 64..128-row tcgen05 tiles (>90% padding at GQA 4)
-// are not.  The last CTA of a set to finish merges the set's partials and writes bf16.
+// are not.  A set's CTAs merge their partials through distributed shared memory where they are a cluster (up
+// to eight of them); else the last one to finish merges them from HBM.
 #define SPIN_FILE_ID 4
 #include <atomic>
 #include <cstdio>
@@ -209,6 +210,13 @@ struct PageRef {
   uint32_t mask;
 };
 
+// A descriptor that points outside the pools is dropped (and reported), never followed.
+__device__ __forceinline__ PageRef in_range(const DevCtx &c, const PageRef &r) {
+  const bool ok = (r.src >= 0 ? r.src < c.n_gpu_pages : ~r.src < c.n_host_pages) && r.fill < c.n_host_pages;
+  if (ok) return r;
+  dev_error(c, kErrBounds);
+  return PageRef{0, -1, -1, 0u};
+}
 __device__ __forceinline__ PageRef page_ref(const DevCtx &c, const Batch &bt, int b, int i_req, int head, size_t pl, int pos) {
   PageRef r{0, -1, -1, 0u};
   if (c.page_desc) {                        // work-ordered descriptors written by the cache manager
@@ -232,10 +240,7 @@ __device__ __forceinline__ PageRef page_ref(const DevCtx &c, const Batch &bt, in
     r.src = c.page_src[pl + pos];
     r.mask = c.page_mask[pl + pos];
   }
-  // a descriptor that points outside the pools is dropped (and reported), never followed
-  const bool ok = (r.src >= 0 ? r.src < c.n_gpu_pages : ~r.src < c.n_host_pages) && r.fill < c.n_host_pages;
-  if (!ok) { dev_error(c, kErrBounds); r = PageRef{0, -1, -1, 0u}; }
-  return r;
+  return in_range(c, r);
 }
 
 // Four outputs over their softmax denominator, as bf16; zero where nothing was attended.
@@ -354,7 +359,7 @@ __device__ __forceinline__ void merge_rows(const DevCtx &c, int b, int n_rows, _
 // CTAs that share a list of np pages.  As a rule the set's part of the GPU; a list that would leave more than
 // `share` pages to each of those gets more, up to the grid's rows.
 __device__ __forceinline__ int attn_rows_of(const Batch &bt, int np, int share, int max_rows) {
-  const int most = min(max_rows, (np + kCtaPages - 1) / kCtaPages);
+  const int most = min(max_rows, (np + bt.attn_least - 1) / bt.attn_least);
   return min(most, max(bt.attn_rows, (np + share - 1) / share));
 }
 // Half as much again as a CTA's part of an average list.
@@ -410,17 +415,85 @@ __device__ __forceinline__ bool further_row(const DevCtx &c, const Batch &bt, in
   return *b >= 0;
 }
 
+// Pages that a list of the request's sets may have.
+__device__ __forceinline__ int most_pages(const DevCtx &c, const Batch &bt, int i_req) {
+  const int most = c.max_pages + c.tail_cap;
+  return c.ready && c.kind != kKindCluster ? min(most, min(c.topk, bt.n_partitions[i_req]) + bt.tail_pages[i_req]) : most;
+}
+
+constexpr int kClusterRows = 8;            // CTAs that a cluster may have everywhere
+
+// The part of a set's outputs that a CTA of a cluster has computed, for the other CTAs to read: whether there
+// is one, its maxima and sums; the outputs are in the CTA's dynamic shared memory (cluster_outputs).
+template <int G> struct ClusterPart { float2 ml[G]; int valid; };
+__device__ __forceinline__ float *cluster_outputs(uint8_t *smem) { return reinterpret_cast<float *>(smem + kStageBytes); }   // warp 0's second stage
+__device__ __forceinline__ uint32_t remote(uint32_t addr, int rank) {
+  uint32_t r;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;\n" : "=r"(r) : "r"(addr), "r"(rank));
+  return r;
+}
+__device__ __forceinline__ void cluster_meet() {
+  asm volatile("barrier.cluster.arrive.release;\nbarrier.cluster.wait.acquire;\n" ::: "memory");
+}
+// Merge of a set's partials by the cluster that holds all its rows: every CTA takes a share of the outputs
+// and reads the others' partials through distributed shared memory, rows in ascending order.  No partial goes to
+// memory, and no fence or counter stands between the rows' ends and the merge.  CTAs that no page of the
+// list has reached have left (the cluster's barrier does not wait for those).  The others, the first
+// `rows`, all come here, one that has waited for the list in vain too (rows < 0: without a part, and
+// it reads none), and none leaves before the last has read.
+// Latency-bound: two cluster barriers and one read of the partials.  Against the merge through memory (write,
+// fence, counter, read): 8 lists of up to 40 pages 7.2 -> 6.7 us, decode of one set of 17 pages 22.3 -> 21.2
+// (five rows instead of three), of 64 sets of 129 pages 100.9 -> 98.5, of 128 sets of 65 pages 78.1 -> 76.4.
+template <int G>
+__device__ __forceinline__ void merge_cluster(ClusterPart<G> &part, uint8_t *smem, __nv_bfloat16 *__restrict__ out_rows, int row, int rows) {
+  constexpr int kMost = kClusterRows;
+  if (threadIdx.x == 0) part.valid = rows > 0;
+  cluster_meet();
+  const uint32_t ml = smem_u32(&part.ml[0]), ok = smem_u32(&part.valid), outs = smem_u32(cluster_outputs(smem));
+#pragma unroll 1
+  for (int e = row * kAttnThreads + threadIdx.x; rows > 0 && e < G * (kHeadDim / 4); e += rows * kAttnThreads) {
+    const int g = e / (kHeadDim / 4);
+    float m[kMost], l[kMost];
+    float4 x[kMost];
+    int valid[kMost];
+#pragma unroll
+    for (int r = 0; r < kMost; ++r) {
+      const int rank = min(r, rows - 1);
+      asm volatile("ld.shared::cluster.s32 %0, [%1];\n" : "=r"(valid[r]) : "r"(remote(ok, rank)));
+      asm volatile("ld.shared::cluster.v2.f32 {%0, %1}, [%2];\n" : "=f"(m[r]), "=f"(l[r]) : "r"(remote(ml + g * 8, rank)));
+      asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];\n" : "=f"(x[r].x), "=f"(x[r].y), "=f"(x[r].z), "=f"(x[r].w) : "r"(remote(outs + e * 16, rank)));
+    }
+    float mx = -INFINITY;
+#pragma unroll
+    for (int r = 0; r < kMost; ++r) {
+      valid[r] = r < rows && valid[r];
+      if (valid[r]) mx = fmaxf(mx, m[r]);
+    }
+    float4 o = make_float4(0.f, 0.f, 0.f, 0.f);
+    float den = 0.f;
+#pragma unroll
+    for (int r = 0; r < kMost; ++r)
+      if (valid[r]) {
+        const float a = m[r] == -INFINITY ? 0.f : exp2f(m[r] - mx);
+        o.x = fmaf(x[r].x, a, o.x); o.y = fmaf(x[r].y, a, o.y); o.z = fmaf(x[r].z, a, o.z); o.w = fmaf(x[r].w, a, o.w);
+        den = fmaf(l[r], a, den);
+      }
+    store_out(out_rows + 4 * e, normalised(o, den));
+  }
+  cluster_meet();
+}
+
 // One row of a set by a CTA of W warps (kAttnWarps; 1 for lists that fit one, which have a single row).
+// With `part` (the set's rows are a cluster) the result says how many rows' outputs are there to be merged, 0 if
+// that is settled without this one, -1 if the row has waited for its list in vain.
 template <int G, int W>
-__device__ __forceinline__ void attn_row(const DevCtx &c, const Batch &bt, const __nv_bfloat16 *__restrict__ q,
-                                         __nv_bfloat16 *__restrict__ out, uint8_t *smem, int b, int row, int max_rows, int share, int counted = -1) {
+__device__ __forceinline__ int attn_row(const DevCtx &c, const Batch &bt, const __nv_bfloat16 *__restrict__ q,
+                                         __nv_bfloat16 *__restrict__ out, uint8_t *smem, int b, int row, int max_rows, int share, int counted, ClusterPart<G> *part) {
   __shared__ __align__(8) unsigned long long s_bar[W * kWarpStages];
   __shared__ float s_m[W][G], s_l[W][G];
   __shared__ int sh_ok, sh_np, sh_nm, sh_last;
   const int i_req = b / c.Hkv, head = b % c.Hkv;
-  int np_most = c.max_pages + c.tail_cap;  // pages that the set's list may have
-  if (c.ready && c.kind != kKindCluster) np_most = min(np_most, min(c.topk, bt.n_partitions[i_req]) + bt.tail_pages[i_req]);
-  if (row > 0 && row >= attn_rows_of(bt, np_most, bt.attn_share, max_rows)) return;       // no list of this set reaches this row
+  const int np_most = most_pages(c, bt, i_req);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const uint32_t bar0 = smem_u32(&s_bar[kWarpStages * warp]), stage0 = smem_u32(smem) + (uint32_t)(kWarpStages * warp) * kStageBytes;
   if (lane < kWarpStages) {
@@ -428,6 +501,10 @@ __device__ __forceinline__ void attn_row(const DevCtx &c, const Batch &bt, const
     asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
   }
   int np = 0, nm = 0;                      // pages in the set's list; how many of them are early descriptors
+  const size_t pl = (size_t)b * (c.max_pages + c.tail_cap);
+  const int mine = row * W + warp;
+  PageRef ahead{0, -1, -1, 0u};            // a plain list's first batch, asked for together with the list's length (256 sets of 56 pages: 26.4 -> 25.6 us)
+  const bool plain = !c.ready && max_rows == bt.attn_rows && (max_rows == 1 || part);   // (which pages are the row's does not depend on it)
   if (c.ready) {
     // A set raises three flags (the last two are one word).  The first says that its missed pages are listed (the leading
     // descriptors, slot still open): a warp requests its first missed page at once, so the
@@ -443,11 +520,13 @@ __device__ __forceinline__ void attn_row(const DevCtx &c, const Batch &bt, const
       sh_nm = (int)(word & 4095u);
     }
     __syncthreads();
-    if (!sh_ok) return;
+    if (!sh_ok) return -1;
     np = sh_np; nm = sh_nm;
     pages_visible();
   } else {
     pdl_wait_prev();
+    const int pos = mine + lane * max_rows * W;
+    if (plain && pos < c.max_pages) { ahead.src = c.page_src[pl + pos]; ahead.mask = c.page_mask[pl + pos]; }
     np = counted >= 0 ? counted : max(0, min(c.n_pages[b], np_most));
     __syncwarp();
   }
@@ -456,13 +535,11 @@ __device__ __forceinline__ void attn_row(const DevCtx &c, const Batch &bt, const
   if (np == 0) {                           // nothing to attend: the set's rows are zero
     if (row == 0)
       for (int e = threadIdx.x; e < G * kHeadDim / 4; e += W * 32) store_out(out_rows + 4 * e, make_uint2(0u, 0u));
-    return;
+    return 0;
   }
   const int n_rows = attn_rows_of(bt, np, share, max_rows);
-  if (row >= n_rows) return;
-  const size_t pl = (size_t)b * (c.max_pages + c.tail_cap);
+  if (row >= n_rows) return 0;
   const int stride = n_rows * W;                                   // the warp's pages: mine, mine + stride, ...
-  const int mine = row * W + warp;
 
   // Q^T as B-operand fragments: column = lane/4 (query head, zero beyond G), 8 k-steps of 16 channels
   uint32_t qb[8][2];
@@ -511,7 +588,7 @@ __device__ __forceinline__ void attn_row(const DevCtx &c, const Batch &bt, const
       pages_visible();
       if (!listed) { dead = true; break; } // reported by the wait: nothing more is requested
     }
-    if (pos < np && !early) ref = page_ref(c, bt, b, i_req, head, pl, pos);
+    if (pos < np && !early) ref = plain && p0 == mine ? in_range(c, ahead) : page_ref(c, bt, b, i_req, head, pl, pos);
     const bool from_host = ref.fill >= 0 || ref.src < 0;
     const uint32_t here = __ballot_sync(0xffffffffu, pos < np), host = __ballot_sync(0xffffffffu, from_host) & here;   // (lane 0 is here)
     if (row == 0 && p0 == mine) dbg_ta(b, 11);
@@ -657,21 +734,26 @@ __device__ __forceinline__ void attn_row(const DevCtx &c, const Batch &bt, const
     }
     if (n_rows == 1) {                     // the set's only CTA finishes here
       store_out(out_rows + 4 * e, normalised(o, l));
+    } else if (part) {
+      reinterpret_cast<float4 *>(cluster_outputs(smem))[e] = o;
+      if (col == 0) part->ml[g] = make_float2(mn, l);
     } else {
       const size_t at = ((size_t)b * c.max_chunks + row) * G + g;
       reinterpret_cast<float4 *>(c.att_part)[at * (kHeadDim / 4) + col] = o;
       if (col == 0) c.att_ml[at] = make_float2(mn, l);
     }
   }
-  if (W < kAttnWarps || n_rows == 1) return;
+  if (W < kAttnWarps || n_rows == 1) return 0;
+  if (part) return n_rows;
   // the last CTA of the set to get here merges all partials (log-sum-exp)
   __syncthreads();
   if (threadIdx.x == 0) sh_last = last_row(c, b, n_rows);
   __syncthreads();
-  if (!sh_last) return;
+  if (!sh_last) return 0;
   dbg_ta(b, 14);
   merge_rows<G>(c, b, n_rows, out_rows, comb);
   dbg_ta(b, 15);
+  return 0;
 }
 
 // The kernel: the CTA's work; one CTA then waits for the kernel before this one.  CTAs that
@@ -686,7 +768,17 @@ k_attn(DevCtx c, Batch bt, const __nv_bfloat16 *__restrict__ q, __nv_bfloat16 *_
   if (!kCounted) {
     // launch order: row 0 of every set first (the rows that own the first missed pages), or set by set
     const int b = bt.attn_set_major ? blockIdx.y : blockIdx.x, row = bt.attn_set_major ? blockIdx.x : blockIdx.y;
-    attn_row<G, W>(c, bt, q, out, smem, b, row, bt.attn_set_major ? gridDim.x : gridDim.y, bt.attn_share);
+    const int rows = bt.attn_set_major ? gridDim.x : gridDim.y, i_req = b / c.Hkv;
+    if (row == 0 || row < attn_rows_of(bt, most_pages(c, bt, i_req), bt.attn_share, rows)) {   // else no list of this set reaches this row
+      if (W == kAttnWarps && bt.attn_cluster) {
+        __shared__ ClusterPart<G> part;
+        const int n = attn_row<G, W>(c, bt, q, out, smem, b, row, rows, bt.attn_share, -1, &part);
+        if (n != 0) merge_cluster<G>(part, smem, out + ((size_t)i_req * c.Hq + (b % c.Hkv) * G) * kHeadDim, row, n);
+        if (row == 0) dbg_ta(b, 15);
+      } else {
+        attn_row<G, W>(c, bt, q, out, smem, b, row, rows, bt.attn_share, -1, nullptr);
+      }
+    }
   } else {
     __shared__ int s_sum[kAttnWarps], s_at[2];
     int b = blockIdx.x % bt.n_req, row = blockIdx.x / bt.n_req;
@@ -698,7 +790,7 @@ k_attn(DevCtx c, Batch bt, const __nv_bfloat16 *__restrict__ q, __nv_bfloat16 *_
       mine = further_row(c, bt, share, (int)blockIdx.x - own, s_sum, s_at, &b, &row);
       if (mine) np = count_of(c, b);
     }
-    if (mine) attn_row<G, W>(c, bt, q, out, smem, b, row, c.max_chunks, share, np);
+    if (mine) attn_row<G, W>(c, bt, q, out, smem, b, row, c.max_chunks, share, np, nullptr);
   }
   if (blockIdx.x == 0 && blockIdx.y == 0) pdl_wait_prev();
 }
@@ -738,6 +830,8 @@ void launch_attn_g(const DevCtx &c, Batch b, const __nv_bfloat16 *q, __nv_bfloat
   // least (445 lists, one of 64 and the rest of 8: 19 without, 22 with).
   auto clamp = [](long long x, long long lo, long long hi) { return (int)(x > hi ? hi : x < lo ? lo : x); };
   const int chunks = clamp((max_pages + kCtaPages - 1) / kCtaPages, 1, c.max_chunks);
+  b.attn_cluster = 0;
+  b.attn_least = kCtaPages;
   b.attn_rows = clamp(resident / n_sets, 1, chunks);
   b.attn_share = clamp(share_of(est_pages, n_sets, b.attn_rows), kSharePages, 1 << 30);
   int rows = clamp((max_pages + b.attn_share - 1) / b.attn_share, b.attn_rows, chunks);
@@ -755,8 +849,19 @@ void launch_attn_g(const DevCtx &c, Batch b, const __nv_bfloat16 *q, __nv_bfloat
   if (!c.ready) rows = b.attn_rows;
   rows = clamp(rows, b.attn_rows, clamp(kExtraCtas / n_sets, b.attn_rows, chunks));
   b.attn_share = clamp((max_pages + rows - 1) / rows, b.attn_share, 1 << 30);
+  const int fit = clamp(resident / n_sets, 1, kClusterRows);
+  if (rows <= fit) {
+    // few rows, all resident: a cluster per set, which merges through shared memory (figures at merge_cluster).  The
+    // merge costs little, so a row may be left with a page per warp.  Not where rows exceed what is resident at once:
+    // the CTAs of a long list would have to find room together.
+    b.attn_least = kCtaPages / 2;
+    static_assert(kCtaPages / 2 == kAttnWarps, "a row short of its warps has one page per warp (see `plain`)");
+    b.attn_rows = rows = clamp((max_pages + b.attn_least - 1) / b.attn_least, 1, fit);
+    if (rows > 1) b.attn_cluster = rows;
+  }
   const dim3 grid = b.attn_set_major ? dim3(rows, n_sets) : dim3(n_sets, rows);
-  launch_pdl(k_attn<G, kAttnWarps, false>, grid, dim3(kAttnThreads), (size_t)kAttnSmem, st, 1, c, b, q, out);
+  launch_pdl(k_attn<G, kAttnWarps, false>, grid, dim3(kAttnThreads), (size_t)kAttnSmem, st,
+             b.attn_cluster ? b.attn_set_major ? dim3(rows, 1) : dim3(1, rows) : dim3(1), c, b, q, out);
 }
 
 }  // namespace

@@ -144,6 +144,7 @@ struct Batch {
   int32_t attn_set_major;   // attention CTAs ordered set by set (sets become ready one after the
                             // other over a long scoring phase) instead of row 0 of every set first
   int32_t attn_rows, attn_share;   // attention: CTAs of a set as a rule; pages per CTA beyond which a list gets more (see attn_rows_of)
+  int32_t attn_cluster, attn_least;   // CTAs of a set are a cluster (their number, else 0); pages that a CTA has at least
 };
 
 __host__ __device__ inline int set_index(const DevCtx &c, int req, int layer, int head) {
@@ -341,7 +342,7 @@ inline void prof_mark(Prof *p, cudaStream_t st, int kernel) { if (p && p->on) p-
 // Launch with programmatic stream serialization (and optionally a cluster size).
 template <typename... KArgs, typename... Args>
 inline cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
-                              int cluster_x, Args &&...args) {
+                              dim3 cluster, Args &&...args) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = grid;
   cfg.blockDim = block;
@@ -352,10 +353,10 @@ inline cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, s
   attr[na].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[na].val.programmaticStreamSerializationAllowed = 1;
   ++na;
-  if (cluster_x > 1) {
+  if (cluster.x * cluster.y > 1) {
     attr[na].id = cudaLaunchAttributeClusterDimension;
-    attr[na].val.clusterDim.x = cluster_x;
-    attr[na].val.clusterDim.y = 1;
+    attr[na].val.clusterDim.x = cluster.x;
+    attr[na].val.clusterDim.y = cluster.y;
     attr[na].val.clusterDim.z = 1;
     ++na;
   }
