@@ -1423,11 +1423,12 @@ static int step_impl(spin_ctx *ctx, int32_t layer, const int32_t *req_ids, int32
       ctx->launches += launch_append_edge(ctx->d, a, kk, vv, 1, st, &ctx->prof, ctx->stage_q, qc == 1 ? q_alias : nullptr, qbytes);
     }
   }
-  int64_t max_cand = 0, max_pages = 0, est_pages = 0;
+  int64_t max_cand = 0, max_pages = 0, est_pages = 0, cands = 0;
   for (int i = 0; i < n_req; ++i) {
     LayerHost &L = ctx->reqs[(size_t)req_ids[i]].layers[(size_t)layer];
     const int64_t cand = ctx->cfg.partition_kind == SPIN_PART_TOKEN_DOT ? (int64_t)L.n_partitions * kPageTokens : L.n_partitions;
     max_cand = std::max(max_cand, cand);
+    cands += cand * ctx->cfg.num_kv_heads;
     int64_t pages = cluster ? ctx->g.max_pages : std::min<int64_t>(ctx->cfg.topk, L.n_partitions);
     max_pages = std::max(max_pages, pages + L.tail_pages);
     // the clusters' average size is all the host knows of what topk of them will hold
@@ -1452,6 +1453,7 @@ static int step_impl(spin_ctx *ctx, int32_t layer, const int32_t *req_ids, int32
   prof_mark(&ctx->prof, st, -1);
   b.epoch = ++ctx->epoch;
   b.append_in_grid = in_grid ? 1 : 0;
+  b.read_once = streams_much((double)cands * ctx->g.sum_entry_bytes + (double)est_pages * kPageBytes);
   ctx->launches += launch_select(ctx->d, b, qd, kk, vv, (int)max_cand, st, &ctx->prof);
   ctx->launches += launch_fetch(ctx->d, st, ctx->sm_count, &ctx->prof);
   ctx->launches += launch_attention(ctx->d, b, qd, od, (int)max_pages, est_pages, st, &ctx->prof);

@@ -78,12 +78,12 @@ __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
 }
 
 // One warp requests one page: lane i copies pair i of its rows; the stage's mbarrier counts the bytes.
-__device__ __forceinline__ void request_page(uint32_t sdst, uint32_t bar, const uint8_t *src, int lane) {
+__device__ __forceinline__ void request_page(uint32_t sdst, uint32_t bar, const uint8_t *src, int lane, uint64_t policy) {
   if (lane == 0) asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n" ::"r"(bar), "r"(kPageBytes) : "memory");
   __syncwarp();
   if (lane < kPairs)
-    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];\n"
-                 ::"r"(sdst + lane * kPairStride), "l"(src + lane * kPairBytes), "r"(kPairBytes), "r"(bar) : "memory");
+    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint [%0], [%1], %2, [%3], %4;\n"
+                 ::"r"(sdst + lane * kPairStride), "l"(src + lane * kPairBytes), "r"(kPairBytes), "r"(bar), "l"(policy) : "memory");
 }
 // Pages that other SMs have written with ordinary stores and announced by a flag may now be read by
 // bulk copies.
@@ -541,6 +541,7 @@ __device__ __forceinline__ int attn_row(const DevCtx &c, const Batch &bt, const 
   if (row >= n_rows) return 0;
   const int stride = n_rows * W;                                   // the warp's pages: mine, mine + stride, ...
 
+  const uint64_t policy = stream_policy(bt.read_once);
   // Q^T as B-operand fragments: column = lane/4 (query head, zero beyond G), 8 k-steps of 16 channels
   uint32_t qb[8][2];
   WarpAcc acc;
@@ -561,7 +562,7 @@ __device__ __forceinline__ int attn_row(const DevCtx &c, const Batch &bt, const 
     PageRef ref{0, -1, -1, 0u};
     auto request = [&](int stage, int j) {
       const int src = __shfl_sync(0xffffffffu, ref.src, j), fill = __shfl_sync(0xffffffffu, ref.fill, j);
-      request_page(stage0 + stage * kStageBytes, bar0 + 8 * stage, fill >= 0 ? c.host_pages + (size_t)fill * kPageBytes : page_ptr(c, src), lane);
+      request_page(stage0 + stage * kStageBytes, bar0 + 8 * stage, fill >= 0 ? c.host_pages + (size_t)fill * kPageBytes : page_ptr(c, src), lane, policy);
     };
     // a missed page is requested as soon as it is known (early pages lead the list: lane 0's is one of
     // them): its turn, its descriptor and the count of closed turns are asked for together
@@ -971,6 +972,7 @@ extern "C" int spin_paged_attention_static(const void *q, const void *page_pool,
   cudaStream_t st = reinterpret_cast<cudaStream_t>(cuda_stream);
   Batch b{};
   b.n_req = n_sets;
+  b.read_once = streams_much((double)n_sets * list_stride * kPageBytes);
   launch_attention(c, b, reinterpret_cast<const __nv_bfloat16 *>(q), reinterpret_cast<__nv_bfloat16 *>(out),
                    list_stride, 0, st, nullptr);
   const cudaError_t e = cudaGetLastError();

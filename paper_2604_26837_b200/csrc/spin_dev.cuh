@@ -144,6 +144,7 @@ struct Batch {
   int32_t attn_set_major;   // attention CTAs ordered set by set (sets become ready one after the
                             // other over a long scoring phase) instead of row 0 of every set first
   int32_t attn_rows, attn_share;   // attention: CTAs of a set as a rule; pages per CTA beyond which a list gets more (see attn_rows_of)
+  int32_t read_once;        // this step streams through more than stays in L2 (see stream_policy)
   int32_t attn_cluster, attn_least;   // CTAs of a set are a cluster (their number, else 0); pages that a CTA has at least
 };
 
@@ -223,6 +224,20 @@ __device__ __forceinline__ uint8_t *summary_at(const DevCtx &c, int set, int e) 
 // another kernel touches.
 __device__ __forceinline__ void pdl_launch_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void pdl_wait_prev() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
+// The L2 policy of what a step streams through: summaries and pages.  Where there is much of it (Batch::read_once) they are first
+// to leave L2 again, so that what every step comes back for stays: the kernels' code (a set's
+// continuation runs through 30 KB of it once per launch), page tables, directories.  Three contexts in turn, us:
+// 64 sets of 2048 pages 96.5 -> 93.4, 4 sets of 65536 tokens 134.9 -> 131.9, 128 sets with all pages in HBM 75.8 -> 72.5,
+// 256 plain lists of 56 pages 25.7 -> 25.0.
+__device__ __forceinline__ uint64_t stream_policy(int read_once) {
+  uint64_t first, normal;
+  asm("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(first));
+  asm("createpolicy.fractional.L2::evict_normal.b64 %0, 1.0;" : "=l"(normal));
+  return read_once ? first : normal;
+}
+// ... a quarter of L2.  (One request, 8 sets of 2048 pages, 17 MB: 35.8 us as it is, 36.3 with pages and summaries leaving first.)
+inline int streams_much(double bytes) { return bytes > 32e6 ? 1 : 0; }
 
 // Per-set flags that let the attention kernel start on a set as soon as that set's page list
 // is complete, while the scoring kernel is still working on other sets.  The producer is
