@@ -10,12 +10,26 @@ namespace spin {
 
 namespace {
 
+// The HBM copies of the CPU page table entries of pages [first_page, first_page + n), from the pinned originals, in
+// front of the kernel below: its own small reads of those would cross the link against its writes, and wait
+// behind them.  32768 tokens of 8 heads: 3001 -> 2864 us with the first step; calls of 512 tokens 622 -> 603 for
+// 4100.  Short calls would pay more for the launch than it gives (128 tokens of 8 heads, 56 pages: 924 -> 1000;
+// 256 tokens, 120 pages: no difference), so it is for kMirrorPages of all heads together.
+constexpr int kMirrorPages = 192;
+__global__ void __launch_bounds__(256)
+k_mirror_pages(DevCtx c, int req, int layer, int first_page, int n) {
+  const int e = blockIdx.x * 256 + threadIdx.x, set = set_index(c, req, layer, blockIdx.y);
+  if (e >= n) return;
+  const int32_t *hp = cpt_at(c, set, first_page + e);
+  if (hp) cpt_mirror_set(c, set, first_page + e, *hp); else dev_error(c, kErrBounds);
+}
+
 // Pages completely covered by this call's tokens that are not the newest page: all 16 rows
 // come from the input; the page is written to the host tier and indexed.
 __global__ void __launch_bounds__(256)
 k_append_bulk(DevCtx c, int req, int layer, const __nv_bfloat16 *__restrict__ k,
               const __nv_bfloat16 *__restrict__ v, int first_page, int first_token_of_call,
-              uint8_t *__restrict__ stage, const int32_t *__restrict__ stage_hp) {
+              uint8_t *__restrict__ stage, const int32_t *__restrict__ stage_hp, int mirrored) {
   __shared__ __align__(16) __nv_bfloat16 krows[kPageTokens][kHeadDim];
   const int head = blockIdx.y, page = first_page + blockIdx.x, tid = threadIdx.x;
   const int set = set_index(c, req, layer, head);
@@ -26,15 +40,16 @@ k_append_bulk(DevCtx c, int req, int layer, const __nv_bfloat16 *__restrict__ k,
   uint4 vv = ld16(reinterpret_cast<const uint8_t *>(v) + in_off);
   const IndexPlace at = index_place(c, set, page);
   const size_t unit = (size_t)head * gridDim.x + blockIdx.x;        // head-major, as host pages are handed out
+  const bool ahead = !stage && mirrored;
   int32_t host_page;
   if (stage) {
     host_page = stage_hp[unit];
   } else {
-    const int32_t *hp = cpt_at(c, set, page);
+    const int32_t *hp = ahead ? cpt_lookup(c, set, page) : cpt_at(c, set, page);
     if (!hp) { if (tid == 0) dev_error(c, 1u); return; }
     host_page = *hp;
   }
-  if (tid == 0) cpt_mirror_set(c, set, page, host_page);
+  if (!ahead && tid == 0) cpt_mirror_set(c, set, page, host_page);
   // Offload: straight to the page's place in pinned host memory, or -- asynchronous offload --
   // into an HBM staging slot from which copy-engine transfers move it on the library's own stream
   uint8_t *dst = c.host_pages + (size_t)host_page * kPageBytes + r * kRowBytes + piece * 16;
@@ -314,9 +329,11 @@ int launch_append_bulk(const DevCtx &c, int req, int layer, const __nv_bfloat16 
                        const __nv_bfloat16 *v, int first_page, int n_pages, int first_token_of_call,
                        cudaStream_t st, Prof *prof, uint8_t *stage, const int32_t *stage_hp) {
   if (n_pages <= 0) return 0;
-  k_append_bulk<<<dim3(n_pages, c.Hkv), 256, 0, st>>>(c, req, layer, k, v, first_page, first_token_of_call, stage, stage_hp);
+  const bool mirrored = !stage && c.cpt_mirror && n_pages * c.Hkv >= kMirrorPages;
+  if (mirrored) k_mirror_pages<<<dim3((n_pages + 255) / 256, c.Hkv), 256, 0, st>>>(c, req, layer, first_page, n_pages);
+  k_append_bulk<<<dim3(n_pages, c.Hkv), 256, 0, st>>>(c, req, layer, k, v, first_page, first_token_of_call, stage, stage_hp, mirrored);
   prof_mark(prof, st, kProfAppend);
-  return 1;
+  return mirrored ? 2 : 1;
 }
 
 int launch_append_edge(const DevCtx &c, const AppendEdgeArgs &a, const __nv_bfloat16 *k,
