@@ -799,8 +799,9 @@ k_attn(DevCtx c, Batch bt, const __nv_bfloat16 *__restrict__ q, __nv_bfloat16 *_
 constexpr int kSharePages = 32, kExtraCtas = 2048;
 template <int G>
 void launch_attn_g(const DevCtx &c, Batch b, const __nv_bfloat16 *q, __nv_bfloat16 *out, int n_sets, int max_pages, long long est_pages, cudaStream_t st) {
-  static int resident_dev[kMaxDevices] = {};
+  static int resident_dev[kMaxDevices] = {}, clusters_dev[kMaxDevices][kClusterRows + 1] = {};
   int &resident = resident_dev[current_device_slot()];
+  int (&clusters)[kClusterRows + 1] = clusters_dev[current_device_slot()];     // how many clusters of so many CTAs the GPU holds at once
   if (!resident) {
     for (auto kernel : {k_attn<G, kAttnWarps, false>, k_attn<G, kAttnWarps, true>, k_attn<G, 1, false>}) {
       cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kAttnSmem);
@@ -810,6 +811,22 @@ void launch_attn_g(const DevCtx &c, Batch b, const __nv_bfloat16 *q, __nv_bfloat
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_attn<G, kAttnWarps, false>, kAttnThreads, kAttnSmem);
+    for (int r = 2; r <= kClusterRows; ++r) {
+      cudaLaunchAttribute attr[1];
+      attr[0].id = cudaLaunchAttributeClusterDimension;
+      attr[0].val.clusterDim.x = 1;
+      attr[0].val.clusterDim.y = r;
+      attr[0].val.clusterDim.z = 1;
+      cudaLaunchConfig_t cfg = {};
+      cfg.gridDim = dim3(1, r);
+      cfg.blockDim = dim3(kAttnThreads);
+      cfg.dynamicSmemBytes = kAttnSmem;
+      cfg.attrs = attr;
+      cfg.numAttrs = 1;
+      int n = 0;
+      if (cudaOccupancyMaxActiveClusters(&n, k_attn<G, kAttnWarps, false>, &cfg) != cudaSuccess) { cudaGetLastError(); n = 0; }
+      clusters[r] = n;
+    }
     resident = sms * per_sm > 0 ? sms * per_sm : 148;
   }
   // As many CTAs per set as the GPU holds at once (444), and at least 8 pages for each: every CTA is
@@ -850,8 +867,13 @@ void launch_attn_g(const DevCtx &c, Batch b, const __nv_bfloat16 *q, __nv_bfloat
   if (!c.ready) rows = b.attn_rows;
   rows = clamp(rows, b.attn_rows, clamp(kExtraCtas / n_sets, b.attn_rows, chunks));
   b.attn_share = clamp((max_pages + rows - 1) / rows, b.attn_share, 1 << 30);
-  const int fit = clamp(resident / n_sets, 1, kClusterRows);
-  if (rows <= fit) {
+  // A cluster's CTAs share a GPC, whose room is not a multiple of every size: as many CTAs per set as leave all clusters
+  // resident at once (a second wave costs a drawn batch of plain lists 18.3 -> 22.5 us), and no cluster where
+  // that is less than three quarters of the CTAs that the set has without one.
+  const int most = clamp(resident / n_sets, 1, kClusterRows);
+  int fit = clamp((max_pages + kCtaPages / 2 - 1) / (kCtaPages / 2), 1, most);
+  while (fit > 1 && clusters[fit] < n_sets) --fit;
+  if (rows <= most && 4 * fit >= 3 * rows) {
     // few rows, all resident: a cluster per set, which merges through shared memory (figures at merge_cluster).  The
     // merge costs little, so a row may be left with a page per warp.  Not where rows exceed what is resident at once:
     // the CTAs of a long list would have to find room together.
