@@ -868,12 +868,14 @@ void launch_attn_g(const DevCtx &c, Batch b, const __nv_bfloat16 *q, __nv_bfloat
   rows = clamp(rows, b.attn_rows, clamp(kExtraCtas / n_sets, b.attn_rows, chunks));
   b.attn_share = clamp((max_pages + rows - 1) / rows, b.attn_share, 1 << 30);
   // A cluster's CTAs share a GPC, whose room is not a multiple of every size: as many CTAs per set as leave all clusters
-  // resident at once (a second wave costs a drawn batch of plain lists 18.3 -> 22.5 us), and no cluster where
-  // that is less than three quarters of the CTAs that the set has without one.
+  // resident at once (111 lists of 84 pages: 25.6 us with a second wave, 17.8 without), and no cluster where
+  // that gives a warp over an eighth more pages than it has without one (55 lists of 60 pages, seven CTAs instead of eight: 10.1
+  // instead of 9.0).
   const int most = clamp(resident / n_sets, 1, kClusterRows);
   int fit = clamp((max_pages + kCtaPages / 2 - 1) / (kCtaPages / 2), 1, most);
   while (fit > 1 && clusters[fit] < n_sets) --fit;
-  if (rows <= most && 4 * fit >= 3 * rows) {
+  auto warp_pages = [&](int r) { return (max_pages + r * kAttnWarps - 1) / (r * kAttnWarps); };
+  if (rows <= most && 8 * warp_pages(fit) <= 9 * warp_pages(rows)) {
     // few rows, all resident: a cluster per set, which merges through shared memory (figures at merge_cluster).  The
     // merge costs little, so a row may be left with a page per warp.  Not where rows exceed what is resident at once:
     // the CTAs of a long list would have to find room together.
