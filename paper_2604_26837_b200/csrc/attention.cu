@@ -440,7 +440,8 @@ __device__ __forceinline__ void cluster_meet() {
 // memory, and no fence or counter stands between the rows' ends and the merge.  CTAs that no page of the
 // list has reached have left (the cluster's barrier does not wait for those).  The others, the first
 // `rows`, all come here, one that has waited for the list in vain too (rows < 0: without a part, and
-// it reads none), and none leaves before the last has read.
+// it reads none), and none leaves before the last has read.  Where a part is missing nothing is written: the
+// outputs of a set whose list has not come to all its rows stay as they were.
 // Latency-bound: two cluster barriers and one read of the partials.  Against the merge through memory (write,
 // fence, counter, read): 8 lists of up to 40 pages 7.2 -> 6.7 us, decode of one set of 17 pages 22.3 -> 21.2
 // (five rows instead of three), of 64 sets of 129 pages 100.9 -> 98.5, of 128 sets of 65 pages 78.1 -> 76.4.
@@ -464,21 +465,22 @@ __device__ __forceinline__ void merge_cluster(ClusterPart<G> &part, uint8_t *sme
       asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];\n" : "=f"(x[r].x), "=f"(x[r].y), "=f"(x[r].z), "=f"(x[r].w) : "r"(remote(outs + e * 16, rank)));
     }
     float mx = -INFINITY;
+    bool whole = true;
 #pragma unroll
     for (int r = 0; r < kMost; ++r) {
-      valid[r] = r < rows && valid[r];
-      if (valid[r]) mx = fmaxf(mx, m[r]);
+      whole = whole && valid[r];
+      if (r < rows) mx = fmaxf(mx, m[r]);
     }
     float4 o = make_float4(0.f, 0.f, 0.f, 0.f);
     float den = 0.f;
 #pragma unroll
     for (int r = 0; r < kMost; ++r)
-      if (valid[r]) {
+      if (r < rows) {
         const float a = m[r] == -INFINITY ? 0.f : exp2f(m[r] - mx);
         o.x = fmaf(x[r].x, a, o.x); o.y = fmaf(x[r].y, a, o.y); o.z = fmaf(x[r].z, a, o.z); o.w = fmaf(x[r].w, a, o.w);
         den = fmaf(l[r], a, den);
       }
-    store_out(out_rows + 4 * e, normalised(o, den));
+    if (whole) store_out(out_rows + 4 * e, normalised(o, den));
   }
   cluster_meet();
 }

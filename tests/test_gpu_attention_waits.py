@@ -1,5 +1,5 @@
 """Attention whose flags, turns on the host link or pages do not come: every wait ends, says so, leaves no turn open and
-no copy behind, and the outputs are written."""
+no copy behind, and the outputs are written, or left as they were where a set's first flag does not come to all its rows."""
 import os
 import subprocess
 
