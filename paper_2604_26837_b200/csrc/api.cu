@@ -373,6 +373,25 @@ void flush_dirs(spin_ctx *ctx, cudaStream_t st) {
   ctx->dir_updates.clear();
 }
 
+// Everything the sets of a request hold goes back to its pool.
+void give_back(spin_ctx *ctx, int req) {
+  for (int l = 0; l < ctx->cfg.num_layers; ++l)
+    for (int h = 0; h < ctx->cfg.num_kv_heads; ++h) {
+      SetHost &S = set_of(ctx, req, l, h);
+      ctx->gpu_page_pool.give(S.gpu_pages);
+      ctx->host_page_pool.give(S.host_pages);
+      auto drop = [&](BitmapPool &pool, std::vector<int32_t> &dir) {
+        for (int32_t s : dir) if (s >= 0) { pool.release(s); ctx->dir_bytes_in_use -= 4; }
+      };
+      drop(ctx->gpt_segs, S.dir_gpt);
+      drop(ctx->meta_segs, S.dir_meta);
+      drop(ctx->off_segs, S.dir_off);
+      drop(ctx->cpt_segs, S.dir_cpt);
+      drop(ctx->sum_segs, S.dir_sum);
+      S = SetHost();
+    }
+}
+
 int validate_req_layer(spin_ctx *ctx, int req, int layer) {
   if (!ctx) return SPIN_ERR_INVALID;
   if (req < 0 || req >= ctx->cfg.max_requests) return fail(ctx, SPIN_ERR_INVALID, "request id %d out of range", req);
@@ -1014,19 +1033,20 @@ int spin_request_open(spin_ctx *ctx, int64_t slots, int32_t *out_req) {
     S.gpu_pages.resize((size_t)slots);
     ctx->gpu_page_pool.take(slots, S.gpu_pages.data());
   }
-  launch_dir_update(d, ctx->dir_updates.data(), (int)ctx->dir_updates.size(), nullptr);   // (the count of launches is of those that work for requests)
+  cudaError_t e = cudaSuccess;
+  launch_dir_update(d, ctx->dir_updates.data(), (int)ctx->dir_updates.size(), nullptr, &e);   // (the count of launches is of those that work for requests)
   ctx->dir_updates.clear();
   const int64_t padded = segs_per_set << g.seg_shift;           // entries that a set's segments have
   OpenRuns runs;
   runs.n = 0;
   int64_t from = 0;                                             // entries before this one are on their way
-  for (int i = 0; i < n_sets; ++i) {
+  for (int i = 0; i < n_sets && e == cudaSuccess; ++i) {
     const std::vector<int32_t> &pages = ctx->sets[(size_t)(set0 + i)].gpu_pages;
-    for (int64_t s = 0; s < slots; ++s) {
+    for (int64_t s = 0; s < slots && e == cudaSuccess; ++s) {
       if (s > 0 && pages[(size_t)s] == pages[(size_t)s - 1] + 1) continue;
       const int64_t at = i * padded + s;
       if (runs.n == OpenRuns::kMost) {
-        launch_request_open(d, set0, n_sets, (int)slots, padded, from, at, ctx->cfg.gpu_cache_pages, runs, nullptr);
+        e = launch_request_open(d, set0, n_sets, (int)slots, padded, from, at, ctx->cfg.gpu_cache_pages, runs, nullptr);
         from = at;
         runs.n = 0;
       }
@@ -1034,9 +1054,13 @@ int spin_request_open(spin_ctx *ctx, int64_t slots, int32_t *out_req) {
       runs.page[runs.n++] = pages[(size_t)s];
     }
   }
-  launch_request_open(d, set0, n_sets, (int)slots, padded, from, n_sets * padded, ctx->cfg.gpu_cache_pages, runs, nullptr);
-  CK(cudaGetLastError());
-  CK(cudaStreamSynchronize(nullptr));                           // the request may be used on any stream from here on
+  if (e == cudaSuccess) e = launch_request_open(d, set0, n_sets, (int)slots, padded, from, n_sets * padded, ctx->cfg.gpu_cache_pages, runs, nullptr);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(nullptr);     // the request may be used on any stream from here on
+  if (e != cudaSuccess) {
+    give_back(ctx, req);
+    launch_request_close(d, set0, n_sets, nullptr);             // what has been mapped on the device
+    return fail(ctx, SPIN_ERR_CUDA, "opening a request failed: %s", cudaGetErrorString(e));
+  }
   RequestHost &R = ctx->reqs[(size_t)req];
   R.open = true;
   R.slots = slots;
@@ -1182,30 +1206,14 @@ int spin_request_close(spin_ctx *ctx, int32_t req) {
   if (req < 0 || req >= ctx->cfg.max_requests) return fail(ctx, SPIN_ERR_INVALID, "request id %d out of range", req);
   RequestHost &R = ctx->reqs[(size_t)req];
   if (!R.open) return fail(ctx, SPIN_ERR_STATE, "request %d is not open", req);
-  const Geometry &g = ctx->g;
   const DevCtx &d = ctx->d;
   if (ctx->offload_stream) CK(cudaStreamSynchronize(ctx->offload_stream));   // its pages may still be on their way
-  for (int l = 0; l < ctx->cfg.num_layers; ++l)
-    for (int h = 0; h < ctx->cfg.num_kv_heads; ++h) {
-      const int set = set_index(d, req, l, h);
-      SetHost &S = ctx->sets[(size_t)set];
-      ctx->gpu_page_pool.give(S.gpu_pages);
-      ctx->host_page_pool.give(S.host_pages);
-      auto drop = [&](BitmapPool &pool, std::vector<int32_t> &dir) {
-        for (int32_t s : dir) if (s >= 0) { pool.release(s); ctx->dir_bytes_in_use -= 4; }
-      };
-      drop(ctx->gpt_segs, S.dir_gpt);
-      drop(ctx->meta_segs, S.dir_meta);
-      drop(ctx->off_segs, S.dir_off);
-      drop(ctx->cpt_segs, S.dir_cpt);
-      drop(ctx->sum_segs, S.dir_sum);
-      S = SetHost();
-    }
-  // the rows of a request's sets are consecutive in every table: one kernel for all (six memsets before)
-  const DeviceGuard on(ctx->cfg.device);
-  launch_request_close(d, set_index(d, req, 0, 0), ctx->cfg.num_layers * ctx->cfg.num_kv_heads, nullptr);
-  CK(cudaGetLastError());
+  give_back(ctx, req);
   R = RequestHost();
+  // the rows of a request's sets are consecutive in every table: one kernel for all
+  const DeviceGuard on(ctx->cfg.device);
+  const cudaError_t e = launch_request_close(d, set_index(d, req, 0, 0), ctx->cfg.num_layers * ctx->cfg.num_kv_heads, nullptr);
+  if (e != cudaSuccess) return fail(ctx, SPIN_ERR_CUDA, "closing request %d failed: %s", req, cudaGetErrorString(e));
   return SPIN_OK;
 }
 

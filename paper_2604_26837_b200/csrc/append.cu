@@ -301,26 +301,25 @@ static int grid_of(int64_t threads) {
   return (int)(ctas < 1 ? 1 : ctas < 148 * 8 ? ctas : 148 * 8);
 }
 
-int launch_request_open(const DevCtx &c, int set0, int n_sets, int slots, int64_t padded, int64_t from, int64_t to, int64_t first_tail,
-                        const OpenRuns &runs, cudaStream_t st) {
+cudaError_t launch_request_open(const DevCtx &c, int set0, int n_sets, int slots, int64_t padded, int64_t from, int64_t to, int64_t first_tail,
+                                const OpenRuns &runs, cudaStream_t st) {
   const int64_t tails = (int64_t)n_sets * c.tail_cap;
-  k_request_open<<<grid_of(to - from > tails ? to - from : tails), 256, 0, st>>>(c, set0, n_sets, slots, padded, from, to, first_tail, runs);
-  return 1;
+  return launch_plain(k_request_open, grid_of(to - from > tails ? to - from : tails), 256, st, c, set0, n_sets, slots, padded, from, to, first_tail, runs);
 }
 
-int launch_request_close(const DevCtx &c, int set0, int n_sets, cudaStream_t st) {
+cudaError_t launch_request_close(const DevCtx &c, int set0, int n_sets, cudaStream_t st) {
   const int most = c.dir_sum > c.dir_part ? c.dir_sum : c.dir_part;
-  k_request_close<<<grid_of((int64_t)n_sets * (most > c.dir_page ? most : c.dir_page)), 256, 0, st>>>(c, set0, n_sets);
-  return 1;
+  return launch_plain(k_request_close, grid_of((int64_t)n_sets * (most > c.dir_page ? most : c.dir_page)), 256, st, c, set0, n_sets);
 }
 
-int launch_dir_update(const DevCtx &c, const DirUpdate *u, int n, cudaStream_t st) {
+int launch_dir_update(const DevCtx &c, const DirUpdate *u, int n, cudaStream_t st, cudaError_t *status) {
   int launched = 0;
   for (int i = 0; i < n; i += kDirBatch, ++launched) {
     DirBatch a;
     a.n = n - i < kDirBatch ? n - i : kDirBatch;
     for (int j = 0; j < a.n; ++j) { a.at[j] = u[i + j].at; a.value[j] = u[i + j].value; }
-    k_dir_update<<<1, 256, 0, st>>>(c.dir_meta, a);
+    const cudaError_t e = launch_plain(k_dir_update, 1, 256, st, c.dir_meta, a);
+    if (status && *status == cudaSuccess) *status = e;
   }
   return launched;
 }
