@@ -333,7 +333,7 @@ bool is_device_ptr(const void *p) {
   return at.type == cudaMemoryTypeDevice || at.type == cudaMemoryTypeManaged;
 }
 
-// A call without a stream launches on its context's device, whichever is current.
+// A call without a stream launches on its context's device, and waits for that one, whichever is current.
 struct DeviceGuard {
   int was = -1;
   explicit DeviceGuard(int device) {
@@ -831,6 +831,7 @@ extern "C" {
 
 int spin_profile(spin_ctx *ctx, int32_t enable) {
   if (!ctx) return SPIN_ERR_INVALID;
+  const DeviceGuard on(ctx->cfg.device);
   CK(cudaDeviceSynchronize());
   ctx->prof.on = enable != 0;
   ctx->prof.used = 0;
@@ -840,6 +841,7 @@ int spin_profile(spin_ctx *ctx, int32_t enable) {
 int spin_profile_read(spin_ctx *ctx, spin_profile_t *out) {
   if (!ctx || !out) return SPIN_ERR_INVALID;
   if (out->struct_size != sizeof(spin_profile_t)) return fail(ctx, SPIN_ERR_INVALID, "spin_profile_t.struct_size mismatch");
+  const DeviceGuard on(ctx->cfg.device);
   CK(cudaDeviceSynchronize());
   out->n_kernels = kProfKernels;
   for (int i = 0; i < 8; ++i) { out->launches[i] = 0; out->ms[i] = 0.0; }
@@ -983,6 +985,7 @@ int spin_create(const spin_config *cfg, spin_ctx **out) {
 
 int spin_destroy(spin_ctx *ctx) {
   if (!ctx) return SPIN_ERR_INVALID;
+  const DeviceGuard on(ctx->cfg.device);
   cudaDeviceSynchronize();
   if (ctx->prof.ev) {
     for (size_t i = 0; i < Prof::kMaxMarks; ++i) cudaEventDestroy(ctx->prof.ev[i]);
@@ -1228,6 +1231,7 @@ int spin_set_budget(spin_ctx *ctx, int32_t req, int64_t slots) {
   const int64_t old = R.slots;
   if (slots == old) return SPIN_OK;
   const int64_t sets_per_req = (int64_t)ctx->cfg.num_layers * ctx->cfg.num_kv_heads;
+  const DeviceGuard on(ctx->cfg.device);
   CK(cudaDeviceSynchronize());
   if (slots < old) {
     // reclaim the tail of every set's GPU page table on the device, then give the pages and
@@ -1487,6 +1491,7 @@ int spin_decode_step_append(spin_ctx *ctx, int32_t layer, const int32_t *req_ids
 int spin_stats(spin_ctx *ctx, spin_stats_t *out) {
   if (!ctx || !out) return SPIN_ERR_INVALID;
   if (out->struct_size != sizeof(spin_stats_t)) return fail(ctx, SPIN_ERR_INVALID, "spin_stats_t.struct_size mismatch");
+  const DeviceGuard on(ctx->cfg.device);
   CK(cudaDeviceSynchronize());
   Counters c{};
   CK(cudaMemcpy(&c, ctx->d.counters, sizeof c, cudaMemcpyDeviceToHost));
@@ -1548,6 +1553,7 @@ int spin_debug_dump(spin_ctx *ctx, int32_t req, int32_t layer, int32_t kv_head, 
   if (rc) return rc;
   if (!o || o->struct_size != sizeof(spin_dump_t)) return fail(ctx, SPIN_ERR_INVALID, "bad spin_dump_t");
   if (kv_head < 0 || kv_head >= ctx->cfg.num_kv_heads) return fail(ctx, SPIN_ERR_INVALID, "kv_head out of range");
+  const DeviceGuard on(ctx->cfg.device);
   CK(cudaDeviceSynchronize());
   const Geometry &g = ctx->g;
   const DevCtx &d = ctx->d;
@@ -1633,6 +1639,7 @@ int spin_debug_read_page(spin_ctx *ctx, int32_t req, int32_t layer, int32_t kv_h
   int rc = validate_req_layer(ctx, req, layer);
   if (rc) return rc;
   if (!out || kv_head < 0 || kv_head >= ctx->cfg.num_kv_heads) return fail(ctx, SPIN_ERR_INVALID, "bad arguments");
+  const DeviceGuard on(ctx->cfg.device);
   CK(cudaDeviceSynchronize());
   const Geometry &g = ctx->g;
   const DevCtx &d = ctx->d;

@@ -92,3 +92,24 @@ assert lib.spin_request_close(h, 0) == 6 and in_use(h) == (0, 0)
 assert lib.spin_request_close(h, 0) == 2                           # not open any more
 assert opened(h, 64) == (0, 0)
 """)
+
+
+def test_calls_without_a_stream_work_on_the_contexts_device(stand_in):
+    # a context of the second device, the first one current
+    stand_in("""
+h = context(device=1)
+cuda.cudaSetDevice(0)
+before = cuda.stand_in_launches(1)
+assert opened(h, 64) == (0, 0)
+for slots in (32, 48):                                             # a kernel reclaims what a smaller budget gives up
+    assert lib.spin_set_budget(h, 0, slots) == 0
+assert in_use(h)[0] == 4 * 48
+page = (C.c_uint8 * 8192)()
+assert lib.spin_debug_read_page(h, 0, 0, 0, 0, 0, 0, page) == 0
+assert lib.spin_profile(h, 0) == 0
+assert lib.spin_request_close(h, 0) == 0 and lib.spin_destroy(h) == 0
+d = C.c_int(-1)
+cuda.cudaGetDevice(C.byref(d))
+assert d.value == 0 and cuda.stand_in_launches(0) == 0 and cuda.stand_in_launches(1) - before == 4
+assert cuda.stand_in_synced(0) == 0 and cuda.stand_in_synced(1) > 0
+""")
