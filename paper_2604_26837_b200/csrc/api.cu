@@ -392,6 +392,24 @@ void give_back(spin_ctx *ctx, int req) {
     }
 }
 
+// The directories and scalars of a request's sets on the device: nothing mapped, nothing there.  The rows of a request's sets are
+// consecutive in every table.  (One kernel for all takes the caller 7 us less than these, but it waits for room on
+// the SMs like any other, and the next request that opens waits behind it: see spin_request_open.)
+cudaError_t unmap_request(spin_ctx *ctx, int req) {
+  const Geometry &g = ctx->g;
+  const DevCtx &d = ctx->d;
+  const size_t set0 = (size_t)set_index(d, req, 0, 0), n = (size_t)ctx->cfg.num_layers * ctx->cfg.num_kv_heads;
+  cudaError_t e = cudaSuccess;
+  auto fill = [&](void *p, int v, size_t bytes) { if (e == cudaSuccess) e = cudaMemsetAsync(p, v, bytes, nullptr); };
+  fill(d.dir_gpt + set0 * g.dir_slot, 0xff, n * g.dir_slot * 4);
+  fill(d.dir_meta + set0 * g.dir_part, 0xff, n * g.dir_part * 4);
+  fill(d.dir_off + set0 * g.dir_part, 0xff, n * g.dir_part * 4);
+  fill(d.dir_cpt + set0 * g.dir_page, 0xff, n * g.dir_page * 4);
+  fill(d.dir_sumseg + set0 * g.dir_sum, 0xff, n * g.dir_sum * 4);
+  fill(d.state + set0, 0, n * sizeof(SetState));
+  return e;
+}
+
 int validate_req_layer(spin_ctx *ctx, int req, int layer) {
   if (!ctx) return SPIN_ERR_INVALID;
   if (req < 0 || req >= ctx->cfg.max_requests) return fail(ctx, SPIN_ERR_INVALID, "request id %d out of range", req);
@@ -1015,14 +1033,22 @@ int spin_request_open(spin_ctx *ctx, int64_t slots, int32_t *out_req) {
     return fail(ctx, SPIN_ERR_BUDGET, "budget needs %lld GPU pages, %lld free", (long long)(slots * sets_per_req), (long long)ctx->gpu_page_pool.available());
   if (ctx->gpt_segs.available() < segs_per_set * sets_per_req)
     return fail(ctx, SPIN_ERR_OOM_DEVICE, "out of GPU page table segments");
-  // All sets of a request are consecutive (layer by layer, head by head).  The directories of the other
-  // tables hold nothing but "unmapped" since spin_create or the last close.  One kernel writes the
-  // GPU page tables, tail pages and states: what it cannot work out are the runs of physical pages
-  // that the slots get (one per set as a rule) and the segments, which go up like all
-  // directory entries.  Four blocking copies of host-made tables took half of the call's time.
+  // All sets of a request are consecutive (layer by layer, head by head), so each table's rows go up
+  // in one copy, and the page table segments in one copy per run of consecutive segments.  The
+  // directories of the other tables hold nothing but "unmapped" since spin_create or the last close.
+  // Copies, not a kernel: a kernel waits for room on the SMs, which decode steps on other streams fill (attention
+  // leaves no registers, and the next step's scoring CTAs take the rest), and the caller with it.  512 slots of 8 sets, us, with a
+  // kernel and with copies: beside steps of 6 requests of up to 131072 tokens 512 and 92 (with another request closed just
+  // before 1063 and 131), of 16 of 32768 200 and 92; with the GPU idle 26 and 55, 64 slots of one set 23 and 18.
   const DeviceGuard on(ctx->cfg.device);
   const int set0 = set_index(d, req, 0, 0), n_sets = (int)sets_per_req;
-  for (int i = 0; i < n_sets; ++i) {
+  std::vector<int32_t> dir_gpt((size_t)n_sets * g.dir_slot, -1), tails((size_t)n_sets * g.tail_cap);
+  std::vector<SetState> states((size_t)n_sets);
+  std::vector<GptEntry> entries((size_t)(segs_per_set * n_sets) << g.seg_shift, GptEntry{-1, -1, 0, -1});
+  std::vector<int32_t> segs;                                    // the segments behind them
+  segs.reserve((size_t)(segs_per_set * n_sets));
+  GptEntry *to = entries.data();
+  for (int i = 0; i < n_sets; ++i, to += segs_per_set << g.seg_shift) {
     const int set = set0 + i;
     SetHost &S = ctx->sets[(size_t)set];
     S = SetHost();
@@ -1031,37 +1057,34 @@ int spin_request_open(spin_ctx *ctx, int64_t slots, int32_t *out_req) {
     S.dir_gpt.assign((size_t)g.dir_slot, -1);
     S.dir_cpt.assign((size_t)g.dir_page, -1);
     S.dir_sum.assign((size_t)g.dir_sum, -1);
-    for (int64_t s0 = 0; s0 < slots; s0 += g.seg)
-      ensure_seg(ctx, ctx->gpt_segs, S.dir_gpt, d.dir_gpt + (size_t)set * g.dir_slot, s0, g.seg_shift);
+    for (int64_t j = 0; j < segs_per_set; ++j) {
+      segs.push_back((int32_t)ctx->gpt_segs.alloc());
+      S.dir_gpt[(size_t)j] = dir_gpt[(size_t)i * g.dir_slot + (size_t)j] = segs.back();
+      ctx->dir_bytes_in_use += 4;
+    }
     S.gpu_pages.resize((size_t)slots);
     ctx->gpu_page_pool.take(slots, S.gpu_pages.data());
+    for (int64_t s = 0; s < slots; ++s) to[s].phys = S.gpu_pages[(size_t)s];
+    for (int j = 0; j < g.tail_cap; ++j) tails[(size_t)i * g.tail_cap + j] = (int32_t)(ctx->cfg.gpu_cache_pages + (int64_t)set * g.tail_cap + j);
+    states[(size_t)i].slots = (int32_t)slots;
   }
   cudaError_t e = cudaSuccess;
-  launch_dir_update(d, ctx->dir_updates.data(), (int)ctx->dir_updates.size(), nullptr, &e);   // (the count of launches is of those that work for requests)
-  ctx->dir_updates.clear();
-  const int64_t padded = segs_per_set << g.seg_shift;           // entries that a set's segments have
-  OpenRuns runs;
-  runs.n = 0;
-  int64_t from = 0;                                             // entries before this one are on their way
-  for (int i = 0; i < n_sets && e == cudaSuccess; ++i) {
-    const std::vector<int32_t> &pages = ctx->sets[(size_t)(set0 + i)].gpu_pages;
-    for (int64_t s = 0; s < slots && e == cudaSuccess; ++s) {
-      if (s > 0 && pages[(size_t)s] == pages[(size_t)s - 1] + 1) continue;
-      const int64_t at = i * padded + s;
-      if (runs.n == OpenRuns::kMost) {
-        e = launch_request_open(d, set0, n_sets, (int)slots, padded, from, at, ctx->cfg.gpu_cache_pages, runs, nullptr);
-        from = at;
-        runs.n = 0;
-      }
-      runs.at[runs.n] = at;
-      runs.page[runs.n++] = pages[(size_t)s];
-    }
+  auto put = [&](void *dst, const void *src, size_t bytes) {
+    if (e == cudaSuccess && bytes > 0) e = cudaMemcpyAsync(dst, src, bytes, cudaMemcpyHostToDevice, nullptr);
+  };
+  for (size_t j = 0; j < segs.size();) {
+    size_t len = 1;
+    while (j + len < segs.size() && segs[j + len] == segs[j] + (int32_t)len) ++len;
+    put(d.gpt_pool + ((size_t)segs[j] << g.seg_shift), entries.data() + (j << g.seg_shift), (len << g.seg_shift) * sizeof(GptEntry));
+    j += len;
   }
-  if (e == cudaSuccess) e = launch_request_open(d, set0, n_sets, (int)slots, padded, from, n_sets * padded, ctx->cfg.gpu_cache_pages, runs, nullptr);
+  put(d.dir_gpt + (size_t)set0 * g.dir_slot, dir_gpt.data(), dir_gpt.size() * 4);
+  put(d.tail_phys + (size_t)set0 * g.tail_cap, tails.data(), tails.size() * 4);
+  put(d.state + set0, states.data(), states.size() * sizeof(SetState));
   if (e == cudaSuccess) e = cudaStreamSynchronize(nullptr);     // the request may be used on any stream from here on
   if (e != cudaSuccess) {
     give_back(ctx, req);
-    launch_request_close(d, set0, n_sets, nullptr);             // what has been mapped on the device
+    unmap_request(ctx, req);                                    // what has been mapped on the device
     return fail(ctx, SPIN_ERR_CUDA, "opening a request failed: %s", cudaGetErrorString(e));
   }
   RequestHost &R = ctx->reqs[(size_t)req];
@@ -1209,13 +1232,11 @@ int spin_request_close(spin_ctx *ctx, int32_t req) {
   if (req < 0 || req >= ctx->cfg.max_requests) return fail(ctx, SPIN_ERR_INVALID, "request id %d out of range", req);
   RequestHost &R = ctx->reqs[(size_t)req];
   if (!R.open) return fail(ctx, SPIN_ERR_STATE, "request %d is not open", req);
-  const DevCtx &d = ctx->d;
   if (ctx->offload_stream) CK(cudaStreamSynchronize(ctx->offload_stream));   // its pages may still be on their way
   give_back(ctx, req);
   R = RequestHost();
-  // the rows of a request's sets are consecutive in every table: one kernel for all
   const DeviceGuard on(ctx->cfg.device);
-  const cudaError_t e = launch_request_close(d, set_index(d, req, 0, 0), ctx->cfg.num_layers * ctx->cfg.num_kv_heads, nullptr);
+  const cudaError_t e = unmap_request(ctx, req);
   if (e != cudaSuccess) return fail(ctx, SPIN_ERR_CUDA, "closing request %d failed: %s", req, cudaGetErrorString(e));
   return SPIN_OK;
 }

@@ -241,43 +241,6 @@ k_dir_update(int32_t *__restrict__ dirs, const __grid_constant__ DirBatch a) {
   for (int i = threadIdx.x; i < a.n; i += 256) dirs[a.at[i]] = a.value[i];
 }
 
-// A new request's GPU page tables, entries [from, to) of its sets' (all free: the physical page, no owner);
-// with the first of them the tail pages and scalars of its sets.
-__global__ void __launch_bounds__(256)
-k_request_open(DevCtx c, int set0, int n_sets, int slots, int64_t padded, int64_t from, int64_t to, int64_t first_tail, const __grid_constant__ OpenRuns runs) {
-  const int64_t i0 = (int64_t)blockIdx.x * 256 + threadIdx.x, step = (int64_t)gridDim.x * 256;
-  for (int64_t e = from + i0; e < to; e += step) {
-    const int i = (int)(e / padded), s = (int)(e - i * padded);
-    int lo = 0, hi = runs.n;                             // the run that holds e
-    while (hi - lo > 1) {
-      const int mid = (lo + hi) >> 1;
-      if (runs.at[mid] <= e) lo = mid; else hi = mid;
-    }
-    GptEntry *to_entry = gpt_at(c, set0 + i, s);
-    if (to_entry) *to_entry = GptEntry{-1, s < slots ? runs.page[lo] + (int32_t)(e - runs.at[lo]) : -1, 0, -1};
-    else dev_error(c, kErrBounds);
-  }
-  if (from > 0) return;
-  for (int64_t j = i0; j < (int64_t)n_sets * c.tail_cap; j += step)
-    c.tail_phys[(size_t)set0 * c.tail_cap + j] = (int32_t)(first_tail + (int64_t)set0 * c.tail_cap + j);
-  for (int64_t i = i0; i < n_sets; i += step) c.state[set0 + i] = SetState{0, 0, 0, 0, 0, 0, 0, slots};
-}
-
-// The directories and scalars of a closed request's sets: nothing mapped, nothing there.
-__global__ void __launch_bounds__(256)
-k_request_close(DevCtx c, int set0, int n_sets) {
-  const size_t i0 = (size_t)blockIdx.x * 256 + threadIdx.x, step = (size_t)gridDim.x * 256;
-  auto unmap = [&](int32_t *dir, int per_set) {
-    for (size_t i = i0; i < (size_t)n_sets * per_set; i += step) dir[(size_t)set0 * per_set + i] = -1;
-  };
-  unmap(c.dir_gpt, c.dir_slot);
-  unmap(c.dir_meta, c.dir_part);
-  unmap(c.dir_off, c.dir_part);
-  unmap(c.dir_cpt, c.dir_page);
-  unmap(c.dir_sumseg, c.dir_sum);
-  for (size_t i = i0; i < (size_t)n_sets; i += step) c.state[set0 + i] = SetState{};
-}
-
 // A step's queries that live in pinned host memory are brought into the staging buffer by a small
 // kernel of zero-copy reads instead of a copy-engine transfer.
 __global__ void __launch_bounds__(256)
@@ -296,30 +259,13 @@ int launch_stage_in(void *dq, const void *sq, size_t q_bytes, cudaStream_t st) {
   return 1;
 }
 
-static int grid_of(int64_t threads) {
-  const int64_t ctas = (threads + 255) / 256;
-  return (int)(ctas < 1 ? 1 : ctas < 148 * 8 ? ctas : 148 * 8);
-}
-
-cudaError_t launch_request_open(const DevCtx &c, int set0, int n_sets, int slots, int64_t padded, int64_t from, int64_t to, int64_t first_tail,
-                                const OpenRuns &runs, cudaStream_t st) {
-  const int64_t tails = (int64_t)n_sets * c.tail_cap;
-  return launch_plain(k_request_open, grid_of(to - from > tails ? to - from : tails), 256, st, c, set0, n_sets, slots, padded, from, to, first_tail, runs);
-}
-
-cudaError_t launch_request_close(const DevCtx &c, int set0, int n_sets, cudaStream_t st) {
-  const int most = c.dir_sum > c.dir_part ? c.dir_sum : c.dir_part;
-  return launch_plain(k_request_close, grid_of((int64_t)n_sets * (most > c.dir_page ? most : c.dir_page)), 256, st, c, set0, n_sets);
-}
-
-int launch_dir_update(const DevCtx &c, const DirUpdate *u, int n, cudaStream_t st, cudaError_t *status) {
+int launch_dir_update(const DevCtx &c, const DirUpdate *u, int n, cudaStream_t st) {
   int launched = 0;
   for (int i = 0; i < n; i += kDirBatch, ++launched) {
     DirBatch a;
     a.n = n - i < kDirBatch ? n - i : kDirBatch;
     for (int j = 0; j < a.n; ++j) { a.at[j] = u[i + j].at; a.value[j] = u[i + j].value; }
-    const cudaError_t e = launch_plain(k_dir_update, 1, 256, st, c.dir_meta, a);
-    if (status && *status == cudaSuccess) *status = e;
+    k_dir_update<<<1, 256, 0, st>>>(c.dir_meta, a);
   }
   return launched;
 }

@@ -380,18 +380,7 @@ inline cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, s
   return cudaLaunchKernelEx(&cfg, kernel, KArgs(args)...);
 }
 
-// A plain launch that returns its own status: what cudaGetLastError says after <<<>>> may be an error that some other
-// call of the thread has left behind.
-template <typename... KArgs, typename... Args>
-inline cudaError_t launch_plain(void (*kernel)(KArgs...), dim3 grid, dim3 block, cudaStream_t st, Args &&...args) {
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = grid;
-  cfg.blockDim = block;
-  cfg.stream = st;
-  return cudaLaunchKernelEx(&cfg, kernel, KArgs(args)...);
-}
-
-// ---- kernel launchers (each returns the number of kernels it launched, or the launch's status) -----------------
+// ---- kernel launchers (each returns the number of kernels it launched) -----------------
 struct AppendEdgeArgs {     // one (request) per entry; all its kv heads are processed
   int32_t n_req, layer;
   int32_t req[kMaxBatch];
@@ -402,18 +391,7 @@ struct AppendEdgeArgs {     // one (request) per entry; all its kv heads are pro
 // tokens each and 16-entry segments have 3.4e9 words of directories.
 struct DirUpdate { int64_t at; int32_t value; };
 inline DirUpdate dir_update(const int32_t *dirs, const int32_t *entry, int32_t value) { return DirUpdate{(int64_t)(entry - dirs), value}; }
-// Runs of consecutive physical pages behind a new request's slots; `at` counts the entries of its sets' page
-// tables, set by set, whole segments each.
-struct OpenRuns {
-  static constexpr int kMost = 200;
-  int64_t at[kMost];
-  int32_t page[kMost];
-  int32_t n;
-};
-cudaError_t launch_request_open(const DevCtx &c, int set0, int n_sets, int slots, int64_t padded, int64_t from, int64_t to, int64_t first_tail,
-                                const OpenRuns &runs, cudaStream_t st);
-cudaError_t launch_request_close(const DevCtx &c, int set0, int n_sets, cudaStream_t st);
-int launch_dir_update(const DevCtx &c, const DirUpdate *u, int n, cudaStream_t st, cudaError_t *status = nullptr);   // status: the first launch that failed
+int launch_dir_update(const DevCtx &c, const DirUpdate *u, int n, cudaStream_t st);
 int launch_append_bulk(const DevCtx &c, int req, int layer, const __nv_bfloat16 *k,
                        const __nv_bfloat16 *v, int first_page, int n_pages, int first_token_of_call,
                        cudaStream_t st, Prof *prof, uint8_t *stage = nullptr, const int32_t *stage_hp = nullptr);

@@ -1,6 +1,6 @@
 /* A CUDA runtime without a device, for the host side of the library: host memory is real, device memory an
  * address range that nothing touches, kernels do not run.  It notes the device each kernel was launched on, keeps the
- * runtime's last error as the real one does, and makes the launch fail whose turn the test says. */
+ * runtime's last error as the real one does, and makes the launch, asynchronous copy or fill fail whose turn the test says. */
 #include <stddef.h>
 #include <stdlib.h>
 #include <string.h>
@@ -8,7 +8,7 @@
 #define API __attribute__((visibility("default")))
 typedef int err;
 enum { kDevices = 2, kLaunchFailed = 719, kBadDevice = 101 };
-static int current, last, fail_in = -1, launches, on_device[kDevices], synced_device[kDevices];
+static int current, last, fail_in = -1, on_device[kDevices], synced_device[kDevices];
 
 static err status(err e) { if (e) last = e; return e; }
 API err cudaGetLastError(void) { err e = last; last = 0; return e; }
@@ -29,21 +29,21 @@ API err cudaHostAlloc(void **p, size_t n, unsigned f) { (void)f; *p = malloc(n);
 API err cudaFreeHost(void *p) { free(p); return 0; }
 API err cudaHostGetDevicePointer(void **d, void *h, unsigned f) { (void)f; *d = h; return 0; }
 API err cudaMemset(void *p, int v, size_t n) { (void)p; (void)v; (void)n; return 0; }
-API err cudaMemsetAsync(void *p, int v, size_t n, void *s) { (void)p; (void)v; (void)n; (void)s; return 0; }
 /* device to host: zeros */
 API err cudaMemcpy(void *d, const void *s, size_t n, int kind) { (void)s; if (kind == 2) memset(d, 0, n); return 0; }
-API err cudaMemcpyAsync(void *d, const void *s, size_t n, int kind, void *st) { (void)st; return cudaMemcpy(d, s, n, kind); }
+static err turn(void) { return fail_in >= 0 && fail_in-- == 0 ? status(kLaunchFailed) : 0; }
+API err cudaMemcpyAsync(void *d, const void *s, size_t n, int kind, void *st) { (void)st; cudaMemcpy(d, s, n, kind); return turn(); }
+API err cudaMemsetAsync(void *p, int v, size_t n, void *s) { (void)p; (void)v; (void)n; (void)s; return turn(); }
 API err cudaFuncSetAttribute(const void *f, int a, int v) { (void)f; (void)a; (void)v; return 0; }
 static err launch(void) {
-  ++launches;
   ++on_device[current];
-  return fail_in >= 0 && fail_in-- == 0 ? status(kLaunchFailed) : 0;
+  return turn();
 }
 API err cudaLaunchKernel(const void *f, ...) { (void)f; return launch(); }
 API err cudaLaunchKernelExC(const void *c, const void *f, void **a) { (void)c; (void)f; (void)a; return launch(); }
 
 /* for the test */
-API void stand_in_fail(int in) { fail_in = in; }             /* the launch after so many more fails */
+API void stand_in_fail(int in) { fail_in = in; }             /* the launch, copy or fill after so many more fails */
 API void stand_in_stale(int e) { last = e; }                 /* an error that some other call has left behind */
 API int stand_in_launches(int device) { return on_device[device]; }
 API int stand_in_synced(int device) { return synced_device[device]; }

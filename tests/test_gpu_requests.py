@@ -1,5 +1,9 @@
 """Requests that open in page pools which earlier ones have left in pieces: hundreds of runs of physical pages, sets whose
 slots end within a table segment, slots in none; and prefills through the staging ring into a host pool in pieces."""
+import ctypes
+import os
+import subprocess
+
 import pytest
 import torch
 
@@ -60,3 +64,26 @@ def test_requests_in_pools_in_pieces(slots, segment_entries, ring):
         assert torch.equal(again, out)
         s.close()
     assert torch.equal(got[0][0], got[1][0]) and got[0][1:] == got[1][1:]
+
+
+def test_requests_come_and_go_while_the_sms_are_full(tmp_path):
+    # beside work that fills every SM for a while, as decode steps on other streams do
+    import paper_2604_26837_b200 as P
+    from paper_2604_26837_b200 import build
+    so = tmp_path / "full.so"
+    subprocess.check_call([build._nvcc(), "-O2", "-std=c++17", "-gencode", "arch=compute_100a,code=sm_100a", "-shared", "-Xcompiler", "-fPIC",
+                           os.path.join(os.path.dirname(os.path.abspath(__file__)), "full_sms.cu"), "-o", str(so)])
+    full = ctypes.CDLL(str(so))
+    s = _context(P, num_layers=1)
+    s.request_close(s.request_open(500))                       # (first calls load what they need)
+    for slots in (40, 1000):
+        r = s.request_open(500)
+        torch.cuda.synchronize()
+        assert full.fill(100) == 1
+        s.request_close(r)
+        r = s.request_open(slots)
+        assert full.still_full() == 1
+        torch.cuda.synchronize()
+        assert s.stats()["gpu_pages_in_use"] == 2 * slots
+        s.request_close(r)
+    s.close()
