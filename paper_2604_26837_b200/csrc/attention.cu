@@ -25,8 +25,10 @@
 #define SPIN_FILE_ID 4
 #include <atomic>
 #include <cstdio>
+#include <mutex>
 
 #include "../../include/spin.h"
+#include "attention_plan.cuh"
 #include "spin_dev.cuh"
 
 namespace spin {
@@ -40,14 +42,12 @@ __device__ __forceinline__ void dbg_ta(int, int) {}
 
 namespace {
 
-constexpr int kAttnWarps = 4, kAttnThreads = kAttnWarps * 32;
+constexpr int kAttnThreads = kAttnWarps * 32;
 constexpr int kPairs = kPageTokens, kPairBytes = 2 * kRowBytes;   // pairs of rows of a page: 8 of K, 8 of V
 constexpr int kPairStride = kPairBytes + 16;               // 8 pairs' 16-byte pieces fall into 8 bank groups
 constexpr int kStageBytes = kPairs * kPairStride;
-constexpr int kWarpStages = 2;
 constexpr int kAttnSmem = kAttnWarps * kWarpStages * kStageBytes;
 static_assert(kAttnSmem == kAttnCtaSmem, "what the scoring launcher leaves room for");
-constexpr int kCtaPages = kChunkPages;                     // a set of n pages is split over at most ceil(n / 8) CTAs
 constexpr int kCombStride = kHeadDim + 4;                  // floats of a head's row in the warps' exchange area
 
 __device__ __forceinline__ uint32_t smem_u32(const void *p) {
@@ -362,10 +362,6 @@ __device__ __forceinline__ int attn_rows_of(const Batch &bt, int np, int share, 
   const int most = min(max_rows, (np + bt.attn_least - 1) / bt.attn_least);
   return min(most, max(bt.attn_rows, (np + share - 1) / share));
 }
-// Half as much again as a CTA's part of an average list.
-__host__ __device__ inline long long share_of(long long pages, long long n_sets, int rows) {
-  return (3 * pages + 2 * n_sets * rows - 1) / (2 * n_sets * rows);
-}
 
 // Lists whose lengths only the device knows (a set per request): every CTA takes the average from all
 // counts.  With half as much again as the average for a share, the further rows of all long lists
@@ -420,8 +416,6 @@ __device__ __forceinline__ int most_pages(const DevCtx &c, const Batch &bt, int 
   const int most = c.max_pages + c.tail_cap;
   return c.ready && c.kind != kKindCluster ? min(most, min(c.topk, bt.n_partitions[i_req]) + bt.tail_pages[i_req]) : most;
 }
-
-constexpr int kClusterRows = 8;            // CTAs that a cluster may have everywhere
 
 // The part of a set's outputs that a CTA of a cluster has computed, for the other CTAs to read: whether there
 // is one, its maxima and sums; the outputs are in the CTA's dynamic shared memory (cluster_outputs).
@@ -798,17 +792,18 @@ k_attn(DevCtx c, Batch bt, const __nv_bfloat16 *__restrict__ q, __nv_bfloat16 *_
   if (blockIdx.x == 0 && blockIdx.y == 0) pdl_wait_prev();
 }
 
-constexpr int kSharePages = 32, kExtraCtas = 2048;
+// Set up and asked for once per device, by the first call that launches there.
 template <int G>
-void launch_attn_g(const DevCtx &c, Batch b, const __nv_bfloat16 *q, __nv_bfloat16 *out, int n_sets, int max_pages, long long est_pages, cudaStream_t st) {
-  static int resident_dev[kMaxDevices] = {}, clusters_dev[kMaxDevices][kClusterRows + 1] = {};
-  int &resident = resident_dev[current_device_slot()];
-  int (&clusters)[kClusterRows + 1] = clusters_dev[current_device_slot()];     // how many clusters of so many CTAs the GPU holds at once
-  if (!resident) {
+const AttnGpu &attn_gpu() {
+  static AttnGpu gpus[kMaxDevices] = {};
+  static std::once_flag once[kMaxDevices];
+  const int slot = current_device_slot();
+  std::call_once(once[slot], [slot] {
     for (auto kernel : {k_attn<G, kAttnWarps, false>, k_attn<G, kAttnWarps, true>, k_attn<G, 1, false>}) {
       cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kAttnSmem);
       cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
     }
+    AttnGpu &gpu = gpus[slot];
     int dev = 0, sms = 0, per_sm = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
@@ -827,68 +822,29 @@ void launch_attn_g(const DevCtx &c, Batch b, const __nv_bfloat16 *q, __nv_bfloat
       cfg.numAttrs = 1;
       int n = 0;
       if (cudaOccupancyMaxActiveClusters(&n, k_attn<G, kAttnWarps, false>, &cfg) != cudaSuccess) { cudaGetLastError(); n = 0; }
-      clusters[r] = n;
+      gpu.clusters[r] = n;
     }
-    resident = sms * per_sm > 0 ? sms * per_sm : 148;
+    gpu.resident = sms * per_sm > 0 ? sms * per_sm : 148;
+  });
+  return gpus[slot];
+}
+
+template <int G>
+void launch_attn_g(const DevCtx &c, Batch b, const __nv_bfloat16 *q, __nv_bfloat16 *out, int n_sets, int max_pages, long long est_pages, cudaStream_t st) {
+  const AttnPlan p = attn_plan(attn_gpu<G>(), c.ready != nullptr, n_sets, max_pages, est_pages, c.max_chunks);
+  b.attn_rows = p.own;
+  b.attn_least = p.least;
+  b.attn_share = p.share;
+  b.attn_cluster = p.cluster;
+  const dim3 grid = b.attn_set_major ? dim3(p.rows, n_sets) : dim3(n_sets, p.rows);
+  if (p.form == kAttnWarp) {
+    launch_pdl(k_attn<G, 1, false>, grid, dim3(32), (size_t)kAttnSmem / kAttnWarps, st, 1, c, b, q, out);
+  } else if (p.form == kAttnCounted) {
+    launch_pdl(k_attn<G, kAttnWarps, true>, dim3(p.rows), dim3(kAttnThreads), (size_t)kAttnSmem, st, 1, c, b, q, out);
+  } else {
+    launch_pdl(k_attn<G, kAttnWarps, false>, grid, dim3(kAttnThreads), (size_t)kAttnSmem, st,
+               p.cluster ? b.attn_set_major ? dim3(p.rows, 1) : dim3(1, p.rows) : dim3(1), c, b, q, out);
   }
-  // As many CTAs per set as the GPU holds at once (444), and at least 8 pages for each: every CTA is
-  // resident, its pages stream through its stages, and CTAs share HBM by what they have in flight,
-  // so equal shares end together.  256 sets of 56 pages, 8 heads: 57.7 us with a CTA per 8 pages
-  // (four waves), 24 us with one CTA per set; 128 sets of 65 pages: lists complete to merged
-  // 34 us -> 17 us.
-  // Lists are not always equal.  One that leaves a CTA more than kSharePages and more than half as much
-  // again as the average list does is split further (256 lists, one of 500 pages and the rest of 8: 128 us
-  // without that, 17 with, 31 with a CTA per 8 pages; decode, 32 requests x 8 heads, one of 8192 tokens
-  // and the rest of 130: 152 us, 46, 74).  Below that a further split only costs: 256 lists of 56 pages, two
-  // CTAs each: 35 us instead of 25.  In a decode step the average is the host's estimate, and the grid has
-  // rows for the longest list it may meet, at most kExtraCtas of them, which leave at once where they
-  // are not needed (~1 ns each).  Where only the device knows the lengths, CTAs take the average from the
-  // counts, and fewer spare ones find out from them what is theirs.  That costs a call of even lists 1-2 us,
-  // so it is done where a list may leave a CTA more than 48 pages (72 lists, one of 354 pages and the rest of
-  // 8: 15 us with, 21 without, 17 with a CTA per 8 pages), or 64 where sets have one CTA each: there are so
-  // many of them then that looking costs most (256 lists of 56 pages: 25 us without, 27 with) and gains
-  // least (445 lists, one of 64 and the rest of 8: 19 without, 22 with).
-  auto clamp = [](long long x, long long lo, long long hi) { return (int)(x > hi ? hi : x < lo ? lo : x); };
-  const int chunks = clamp((max_pages + kCtaPages - 1) / kCtaPages, 1, c.max_chunks);
-  b.attn_cluster = 0;
-  b.attn_least = kCtaPages;
-  b.attn_rows = clamp(resident / n_sets, 1, chunks);
-  b.attn_share = clamp(share_of(est_pages, n_sets, b.attn_rows), kSharePages, 1 << 30);
-  int rows = clamp((max_pages + b.attn_share - 1) / b.attn_share, b.attn_rows, chunks);
-  // More sets than the GPU holds CTAs, and lists of one page or two per stage: a CTA of one warp each,
-  // four times as many at once.  (16000 lists of one page: 134 us with four warps, 41 with one.)
-  if (max_pages <= 2 * kWarpStages && n_sets > resident) {
-    launch_pdl(k_attn<G, 1, false>, b.attn_set_major ? dim3(1, n_sets) : dim3(n_sets, 1), dim3(32), (size_t)kAttnSmem / kAttnWarps, st, 1, c, b, q, out);
-    return;
-  }
-  if (!c.ready && max_pages > (b.attn_rows > 1 ? 3 : 4) * kSharePages / 2 * b.attn_rows) {
-    const int own = n_sets * b.attn_rows;
-    launch_pdl(k_attn<G, kAttnWarps, true>, dim3(own + own * 2 / 3), dim3(kAttnThreads), (size_t)kAttnSmem, st, 1, c, b, q, out);
-    return;
-  }
-  if (!c.ready) rows = b.attn_rows;
-  rows = clamp(rows, b.attn_rows, clamp(kExtraCtas / n_sets, b.attn_rows, chunks));
-  b.attn_share = clamp((max_pages + rows - 1) / rows, b.attn_share, 1 << 30);
-  // A cluster's CTAs share a GPC, whose room is not a multiple of every size: as many CTAs per set as leave all clusters
-  // resident at once (111 lists of 84 pages: 25.6 us with a second wave, 17.8 without), and no cluster where
-  // that gives a warp over an eighth more pages than it has without one (55 lists of 60 pages, seven CTAs instead of eight: 10.1
-  // instead of 9.0).
-  const int most = clamp(resident / n_sets, 1, kClusterRows);
-  int fit = clamp((max_pages + kCtaPages / 2 - 1) / (kCtaPages / 2), 1, most);
-  while (fit > 1 && clusters[fit] < n_sets) --fit;
-  auto warp_pages = [&](int r) { return (max_pages + r * kAttnWarps - 1) / (r * kAttnWarps); };
-  if (rows <= most && 8 * warp_pages(fit) <= 9 * warp_pages(rows)) {
-    // few rows, all resident: a cluster per set, which merges through shared memory (figures at merge_cluster).  The
-    // merge costs little, so a row may be left with a page per warp.  Not where rows exceed what is resident at once:
-    // the CTAs of a long list would have to find room together.
-    b.attn_least = kCtaPages / 2;
-    static_assert(kCtaPages / 2 == kAttnWarps, "a row short of its warps has one page per warp (see `plain`)");
-    b.attn_rows = rows = clamp((max_pages + b.attn_least - 1) / b.attn_least, 1, fit);
-    if (rows > 1) b.attn_cluster = rows;
-  }
-  const dim3 grid = b.attn_set_major ? dim3(rows, n_sets) : dim3(n_sets, rows);
-  launch_pdl(k_attn<G, kAttnWarps, false>, grid, dim3(kAttnThreads), (size_t)kAttnSmem, st,
-             b.attn_cluster ? b.attn_set_major ? dim3(rows, 1) : dim3(1, rows) : dim3(1), c, b, q, out);
 }
 
 }  // namespace
