@@ -831,7 +831,7 @@ const AttnGpu &attn_gpu() {
 
 template <int G>
 void launch_attn_g(const DevCtx &c, Batch b, const __nv_bfloat16 *q, __nv_bfloat16 *out, int n_sets, int max_pages, long long est_pages, cudaStream_t st) {
-  const AttnPlan p = attn_plan(attn_gpu<G>(), c.ready != nullptr, n_sets, max_pages, est_pages, c.max_chunks);
+  const AttnPlan p = attn_plan(attn_gpu<G>(), c.ready != nullptr, b.attn_set_major != 0, n_sets, max_pages, est_pages, c.max_chunks);
   b.attn_rows = p.own;
   b.attn_least = p.least;
   b.attn_share = p.share;

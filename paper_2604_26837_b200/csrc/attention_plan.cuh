@@ -54,7 +54,8 @@ inline int clusters_at_once(const AttnGpu &gpu, int r) { return r < 2 ? gpu.resi
 // many of them then that looking costs most (256 lists of 56 pages: 25 us without, 27 with) and gains
 // least (445 lists, one of 64 and the rest of 8: 19 without, 22 with).
 // decode: lists of a decode step (est_pages of all of them together, about), else plain lists of up to max_pages.
-inline AttnPlan attn_plan(const AttnGpu &gpu, bool decode, int n_sets, int max_pages, long long est_pages, int max_chunks) {
+// beside_scoring: CTAs move in one by one while a scoring grid still holds the SMs (Batch::attn_set_major).
+inline AttnPlan attn_plan(const AttnGpu &gpu, bool decode, bool beside_scoring, int n_sets, int max_pages, long long est_pages, int max_chunks) {
   auto clamp = [](long long x, long long lo, long long hi) { return (int)(x > hi ? hi : x < lo ? lo : x); };
   const int chunks = clamp((max_pages + kCtaPages - 1) / kCtaPages, 1, max_chunks);
   AttnPlan p;
@@ -81,12 +82,14 @@ inline AttnPlan attn_plan(const AttnGpu &gpu, bool decode, int n_sets, int max_p
   // resident at once, and no cluster where that gives a warp over an eighth more pages than it has without
   // one: 16 numbers of lists from 19 to 222 of 17 to 96 pages, the better of both within 4 % (55 lists of 60 pages,
   // seven CTAs in a cluster 9.9 us, eight without 9.0; 64 of 48, six 8.6 and 9.0).  Not where rows exceed what is resident at
-  // once: the CTAs of a long list would have to find room together.
+  // once: the CTAs of a long list would have to find room together.  Nor beside a scoring grid that leaves room for one
+  // CTA here and there: a cluster waits for room for all of its own in one GPC (8 requests of 131072 tokens, 8 heads, 64
+  // pages and 163 slots per set: 206 us in clusters of six, 202 without; of 128 pages and 1024 slots 155 and 155).
   const int most = clamp(gpu.resident / n_sets, 1, kClusterRows);
   int fit = clamp((max_pages + kClusterPages - 1) / kClusterPages, 1, most);
   while (fit > 1 && clusters_at_once(gpu, fit) < n_sets) --fit;
   auto warp_pages = [&](int r) { return (max_pages + r * kAttnWarps - 1) / (r * kAttnWarps); };
-  if (p.rows <= most && 8 * warp_pages(fit) <= 9 * warp_pages(p.rows)) {
+  if (!beside_scoring && p.rows <= most && 8 * warp_pages(fit) <= 9 * warp_pages(p.rows)) {
     p.least = kClusterPages;
     p.own = p.rows = fit;
     if (p.rows > 1) p.cluster = p.rows;

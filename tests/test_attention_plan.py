@@ -16,8 +16,8 @@ def plans(tmp_path_factory):
     subprocess.check_call([build._nvcc(), "-std=c++17", "-gencode", "arch=compute_100a,code=sm_100a", "-I", build.CSRC,
                            os.path.join(HERE, "attention_plan.cu"), "-o", exe])
 
-    def ask(*args):
-        text = "".join("%d %d %d %d\n" % (decode, sets, pages, (pages + 7) // 8) for decode, sets, pages in args)
+    def ask(*args, beside=0):
+        text = "".join("%d %d %d %d %d\n" % (decode, beside, sets, pages, (pages + 7) // 8) for decode, sets, pages in args)
         out = subprocess.run([exe], input=text, capture_output=True, text=True, check=True).stdout
         return [tuple(map(int, line.split())) for line in out.splitlines()]
     ask.exe = exe
@@ -39,3 +39,10 @@ def test_clusters_leave_a_margin(plans):
 def test_plain_lists(plans):
     got = plans((0, 1, 4), (0, 16000, 1), (0, 256, 56), (0, 72, 354), (0, 148, 33), (0, 8, 80))
     assert got == [(ROWS, 1, 0), (WARP, 1, 0), (ROWS, 1, 0), (COUNTED, 720, 0), (ROWS, 3, 0), (ROWS, 10, 0)]
+
+
+def test_decode_steps_beside_a_scoring_grid(plans):
+    # single CTAs find room there before clusters do
+    steps = (1, 64, 65), (1, 64, 129), (1, 32, 33), (1, 8, 17)
+    assert [g[1:] for g in plans(*steps)] == [(6, 6), (6, 6), (8, 8), (5, 5)]
+    assert [g[1:] for g in plans(*steps, beside=1)] == [(6, 0), (6, 0), (5, 0), (3, 0)]
