@@ -480,9 +480,10 @@ __device__ __forceinline__ void merge_cluster(ClusterPart<G> &part, uint8_t *sme
 }
 
 // One row of a set by a CTA of W warps (kAttnWarps; 1 for lists that fit one, which have a single row).
-// With `part` (the set's rows are a cluster) the result says how many rows' outputs are there to be merged, 0 if
-// that is settled without this one, -1 if the row has waited for its list in vain.
-template <int G, int W>
+// kTogether: the set has a single row, or its rows are a cluster, which leave their outputs in `part`.  The result says
+// how many rows' outputs are there to be merged, 0 if that is settled without this one, -1 if the row has waited for its
+// list in vain.
+template <int G, int W, bool kTogether>
 __device__ __forceinline__ int attn_row(const DevCtx &c, const Batch &bt, const __nv_bfloat16 *__restrict__ q,
                                          __nv_bfloat16 *__restrict__ out, uint8_t *smem, int b, int row, int max_rows, int share, int counted, ClusterPart<G> *part) {
   __shared__ __align__(8) unsigned long long s_bar[W * kWarpStages];
@@ -500,7 +501,7 @@ __device__ __forceinline__ int attn_row(const DevCtx &c, const Batch &bt, const 
   const size_t pl = (size_t)b * (c.max_pages + c.tail_cap);
   const int mine = row * W + warp;
   PageRef ahead{0, -1, -1, 0u};            // a plain list's first batch, asked for together with the list's length (256 sets of 56 pages: 26.4 -> 25.6 us)
-  const bool plain = !c.ready && max_rows == bt.attn_rows && (max_rows == 1 || part);   // (which pages are the row's does not depend on it)
+  const bool plain = kTogether && !c.ready;   // (which pages are the row's does not depend on it)
   if (c.ready) {
     // A set raises three flags (the last two are one word).  The first says that its missed pages are listed (the leading
     // descriptors, slot still open): a warp requests its first missed page at once, so the
@@ -731,7 +732,7 @@ __device__ __forceinline__ int attn_row(const DevCtx &c, const Batch &bt, const 
     }
     if (n_rows == 1) {                     // the set's only CTA finishes here
       store_out(out_rows + 4 * e, normalised(o, l));
-    } else if (part) {
+    } else if (kTogether) {
       reinterpret_cast<float4 *>(cluster_outputs(smem))[e] = o;
       if (col == 0) part->ml[g] = make_float2(mn, l);
     } else {
@@ -741,7 +742,7 @@ __device__ __forceinline__ int attn_row(const DevCtx &c, const Batch &bt, const 
     }
   }
   if (W < kAttnWarps || n_rows == 1) return 0;
-  if (part) return n_rows;
+  if (kTogether) return n_rows;
   // the last CTA of the set to get here merges all partials (log-sum-exp)
   __syncthreads();
   if (threadIdx.x == 0) sh_last = last_row(c, b, n_rows);
@@ -757,23 +758,27 @@ __device__ __forceinline__ int attn_row(const DevCtx &c, const Batch &bt, const 
 // go by the per-set flags never wait for the scoring kernel as a whole; with one CTA doing so
 // before it exits, this grid cannot complete ahead of that one, and whatever the stream runs
 // next (the next step's scoring kernel waits for this grid) comes after all of its writes.
-template <int G, int W, bool kCounted>
+// Three forms, each a kernel of its own, since code for the others costs one that does not need it.  us, in one kernel and
+// apart: decode, 8 sets of 65 pages, through memory 24.7 and 24.1, 32 sets 28.2 and 27.6; 104 shapes of plain lists (84 to 148 of 21
+// to 44 pages), clusters or through memory, 1 % in all.
+enum AttnKernel { kTogether, kByMemory, kByCounts };
+template <int G, int W, AttnKernel kKernel>
 __global__ void __launch_bounds__(W * 32, 3 * kAttnWarps / W)
 k_attn(DevCtx c, Batch bt, const __nv_bfloat16 *__restrict__ q, __nv_bfloat16 *__restrict__ out) {
   extern __shared__ __align__(128) uint8_t smem[];                // [warps][2] staged pages
   pdl_launch_next();
-  if (!kCounted) {
+  if (kKernel != kByCounts) {
     // launch order: row 0 of every set first (the rows that own the first missed pages), or set by set
     const int b = bt.attn_set_major ? blockIdx.y : blockIdx.x, row = bt.attn_set_major ? blockIdx.x : blockIdx.y;
     const int rows = bt.attn_set_major ? gridDim.x : gridDim.y, i_req = b / c.Hkv;
     if (row == 0 || row < attn_rows_of(bt, most_pages(c, bt, i_req), bt.attn_share, rows)) {   // else no list of this set reaches this row
-      if (W == kAttnWarps && bt.attn_cluster) {
+      if (kKernel == kTogether && W == kAttnWarps) {
         __shared__ ClusterPart<G> part;
-        const int n = attn_row<G, W>(c, bt, q, out, smem, b, row, rows, bt.attn_share, -1, &part);
-        if (n != 0) merge_cluster<G>(part, smem, out + ((size_t)i_req * c.Hq + (b % c.Hkv) * G) * kHeadDim, row, n);
+        const int n = attn_row<G, W, true>(c, bt, q, out, smem, b, row, rows, bt.attn_share, -1, &part);
+        if (n != 0 && bt.attn_cluster) merge_cluster<G>(part, smem, out + ((size_t)i_req * c.Hq + (b % c.Hkv) * G) * kHeadDim, row, n);
         if (row == 0) dbg_ta(b, 15);
       } else {
-        attn_row<G, W>(c, bt, q, out, smem, b, row, rows, bt.attn_share, -1, nullptr);
+        attn_row<G, W, kKernel == kTogether>(c, bt, q, out, smem, b, row, rows, bt.attn_share, -1, nullptr);
       }
     }
   } else {
@@ -787,7 +792,7 @@ k_attn(DevCtx c, Batch bt, const __nv_bfloat16 *__restrict__ q, __nv_bfloat16 *_
       mine = further_row(c, bt, share, (int)blockIdx.x - own, s_sum, s_at, &b, &row);
       if (mine) np = count_of(c, b);
     }
-    if (mine) attn_row<G, W>(c, bt, q, out, smem, b, row, c.max_chunks, share, np, nullptr);
+    if (mine) attn_row<G, W, false>(c, bt, q, out, smem, b, row, c.max_chunks, share, np, nullptr);
   }
   if (blockIdx.x == 0 && blockIdx.y == 0) pdl_wait_prev();
 }
@@ -799,7 +804,7 @@ const AttnGpu &attn_gpu() {
   static std::once_flag once[kMaxDevices];
   const int slot = current_device_slot();
   std::call_once(once[slot], [slot] {
-    for (auto kernel : {k_attn<G, kAttnWarps, false>, k_attn<G, kAttnWarps, true>, k_attn<G, 1, false>}) {
+    for (auto kernel : {k_attn<G, kAttnWarps, kTogether>, k_attn<G, kAttnWarps, kByMemory>, k_attn<G, kAttnWarps, kByCounts>, k_attn<G, 1, kTogether>}) {
       cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kAttnSmem);
       cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
     }
@@ -807,7 +812,7 @@ const AttnGpu &attn_gpu() {
     int dev = 0, sms = 0, per_sm = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_attn<G, kAttnWarps, false>, kAttnThreads, kAttnSmem);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_attn<G, kAttnWarps, kByMemory>, kAttnThreads, kAttnSmem);
     for (int r = 2; r <= kClusterRows; ++r) {
       cudaLaunchAttribute attr[1];
       attr[0].id = cudaLaunchAttributeClusterDimension;
@@ -821,7 +826,7 @@ const AttnGpu &attn_gpu() {
       cfg.attrs = attr;
       cfg.numAttrs = 1;
       int n = 0;
-      if (cudaOccupancyMaxActiveClusters(&n, k_attn<G, kAttnWarps, false>, &cfg) != cudaSuccess) { cudaGetLastError(); n = 0; }
+      if (cudaOccupancyMaxActiveClusters(&n, k_attn<G, kAttnWarps, kTogether>, &cfg) != cudaSuccess) { cudaGetLastError(); n = 0; }
       gpu.clusters[r] = n;
     }
     gpu.resident = sms * per_sm > 0 ? sms * per_sm : 148;
@@ -838,11 +843,13 @@ void launch_attn_g(const DevCtx &c, Batch b, const __nv_bfloat16 *q, __nv_bfloat
   b.attn_cluster = p.cluster;
   const dim3 grid = b.attn_set_major ? dim3(p.rows, n_sets) : dim3(n_sets, p.rows);
   if (p.form == kAttnWarp) {
-    launch_pdl(k_attn<G, 1, false>, grid, dim3(32), (size_t)kAttnSmem / kAttnWarps, st, 1, c, b, q, out);
+    launch_pdl(k_attn<G, 1, kTogether>, grid, dim3(32), (size_t)kAttnSmem / kAttnWarps, st, 1, c, b, q, out);
   } else if (p.form == kAttnCounted) {
-    launch_pdl(k_attn<G, kAttnWarps, true>, dim3(p.rows), dim3(kAttnThreads), (size_t)kAttnSmem, st, 1, c, b, q, out);
+    launch_pdl(k_attn<G, kAttnWarps, kByCounts>, dim3(p.rows), dim3(kAttnThreads), (size_t)kAttnSmem, st, 1, c, b, q, out);
+  } else if (p.rows > 1 && !p.cluster) {
+    launch_pdl(k_attn<G, kAttnWarps, kByMemory>, grid, dim3(kAttnThreads), (size_t)kAttnSmem, st, 1, c, b, q, out);
   } else {
-    launch_pdl(k_attn<G, kAttnWarps, false>, grid, dim3(kAttnThreads), (size_t)kAttnSmem, st,
+    launch_pdl(k_attn<G, kAttnWarps, kTogether>, grid, dim3(kAttnThreads), (size_t)kAttnSmem, st,
                p.cluster ? b.attn_set_major ? dim3(p.rows, 1) : dim3(1, p.rows) : dim3(1), c, b, q, out);
   }
 }
