@@ -1486,7 +1486,7 @@ static int step_impl(spin_ctx *ctx, int32_t layer, const int32_t *req_ids, int32
   prof_mark(&ctx->prof, st, -1);
   b.epoch = ++ctx->epoch;
   b.append_in_grid = in_grid ? 1 : 0;
-  b.read_once = streams_much((double)cands * ctx->g.sum_entry_bytes + (double)est_pages * kPageBytes);
+  b.read_once = step_reads_once(ctx->d.kind, (double)cands * ctx->g.sum_entry_bytes, (double)est_pages * kPageBytes);
   ctx->launches += launch_select(ctx->d, b, qd, kk, vv, (int)max_cand, st, &ctx->prof);
   ctx->launches += launch_fetch(ctx->d, st, ctx->sm_count, &ctx->prof);
   ctx->launches += launch_attention(ctx->d, b, qd, od, (int)max_pages, est_pages, st, &ctx->prof);

@@ -538,7 +538,7 @@ __device__ __forceinline__ int attn_row(const DevCtx &c, const Batch &bt, const 
   if (row >= n_rows) return 0;
   const int stride = n_rows * W;                                   // the warp's pages: mine, mine + stride, ...
 
-  const uint64_t policy = stream_policy(bt.read_once);
+  const uint64_t policy = stream_policy(bt.read_once & kOncePages);
   // Q^T as B-operand fragments: column = lane/4 (query head, zero beyond G), 8 k-steps of 16 channels
   uint32_t qb[8][2];
   WarpAcc acc;
@@ -961,7 +961,7 @@ extern "C" int spin_paged_attention_static(const void *q, const void *page_pool,
   cudaStream_t st = reinterpret_cast<cudaStream_t>(cuda_stream);
   Batch b{};
   b.n_req = n_sets;
-  b.read_once = streams_much((double)n_sets * list_stride * kPageBytes);
+  b.read_once = lists_read_once((double)n_sets * list_stride * kPageBytes);
   launch_attention(c, b, reinterpret_cast<const __nv_bfloat16 *>(q), reinterpret_cast<__nv_bfloat16 *>(out),
                    list_stride, 0, st, nullptr);
   const cudaError_t e = cudaGetLastError();

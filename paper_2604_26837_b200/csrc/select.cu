@@ -193,7 +193,7 @@ __device__ __forceinline__ void score_item(const DevCtx &c, const Batch &bt, con
         const uint32_t dst = (uint32_t)__cvta_generic_to_shared(dyn_smem + (size_t)first * kEntry);
         asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n" ::"r"(bar), "r"(bytes) : "memory");
         asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint [%0], [%1], %2, [%3], %4;\n"
-                     ::"r"(dst), "l"(gseg + (size_t)first * kEntry), "r"(bytes), "r"(bar), "l"(stream_policy(bt.read_once)) : "memory");
+                     ::"r"(dst), "l"(gseg + (size_t)first * kEntry), "r"(bytes), "r"(bar), "l"(stream_policy(bt.read_once & kOnceSummaries)) : "memory");
       }
     }
   }

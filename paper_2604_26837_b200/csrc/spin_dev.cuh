@@ -21,6 +21,7 @@ constexpr int kMaxBuckets = 64;
 
 enum : int { kKindPage = 0, kKindToken = 1, kKindCluster = 2, kKindPageMean = 3 };
 // sticky device error bits (same values as SPIN_DEV_ERR_* of the public header)
+enum : int { kOnceSummaries = 1, kOncePages = 2 };
 constexpr unsigned kErrBounds = 1u, kErrPageList = 2u, kErrTimeout = 4u, kErrState = 8u;
 constexpr int kChunkPages = 8;                              // a set of n pages has room for ceil(n / 8) attention partials
 constexpr int kAttnCtaSmem = 8 * kPageTokens * (2 * kRowBytes + 16);   // staged pages of an attention CTA
@@ -144,7 +145,7 @@ struct Batch {
   int32_t attn_set_major;   // attention CTAs ordered set by set (sets become ready one after the
                             // other over a long scoring phase) instead of row 0 of every set first
   int32_t attn_rows, attn_share;   // attention: CTAs of a set as a rule; pages per CTA beyond which a list gets more (see attn_rows_of)
-  int32_t read_once;        // this step streams through more than stays in L2 (see stream_policy)
+  int32_t read_once;        // what leaves L2 first, kOnceSummaries | kOncePages (see step_reads_once, lists_read_once)
   int32_t attn_cluster, attn_least;   // CTAs of a set are a cluster (their number, else 0); pages that a CTA has at least
 };
 
@@ -225,19 +226,36 @@ __device__ __forceinline__ uint8_t *summary_at(const DevCtx &c, int set, int e) 
 __device__ __forceinline__ void pdl_launch_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void pdl_wait_prev() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
-// The L2 policy of what a step streams through: summaries and pages.  Where there is much of it (Batch::read_once) they are first
-// to leave L2 again, so that what every step comes back for stays: the kernels' code (a set's
-// continuation runs through 30 KB of it once per launch), page tables, directories.  Three contexts in turn, us:
-// 64 sets of 2048 pages 96.5 -> 93.4, 4 sets of 65536 tokens 134.9 -> 131.9, 128 sets with all pages in HBM 75.8 -> 72.5,
-// 256 plain lists of 56 pages 25.7 -> 25.0.
-__device__ __forceinline__ uint64_t stream_policy(int read_once) {
+// The L2 policy of what a call streams through.  Where there is much of it, it is first to leave L2 again, so that what every
+// step comes back for stays: the kernels' code (a set's continuation runs through 30 KB of it once per launch), page
+// tables, directories.
+__device__ __forceinline__ uint64_t stream_policy(bool read_once) {
   uint64_t first, normal;
   asm("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(first));
   asm("createpolicy.fractional.L2::evict_normal.b64 %0, 1.0;" : "=l"(normal));
   return read_once ? first : normal;
 }
-// ... a quarter of L2.  (One request, 8 sets of 2048 pages, 17 MB: 35.8 us as it is, 36.3 with pages and summaries leaving first.)
-inline int streams_much(double bytes) { return bytes > 32e6 ? 1 : 0; }
+// More than this does not stay in L2 (126 MB) until it is read again.
+constexpr double kStaysInL2 = 85e6;
+// A decode step: its pages, where they and the summaries are more than a quarter of L2; its summaries where they are most of it
+// (token granularity) or more than stays.  Steps on three contexts in turn and on the same one again, us, with no policy, for
+// the pages, for both:
+//   64 sets of 2048 candidates, 129 pages (134 MB)   96.7 94.7 95.9   95.2 91.1 93.7
+//   64 sets of 512, 65 pages (50 MB)                 37.6 35.8 36.9   33.9 34.4 36.2
+//   128 sets of 250, 33 pages (50 MB)                36.1 34.0 35.1   33.2 33.7 35.1
+//   128 sets of up to 375 mean keys, 65 pages (76)   50.3 44.9 45.8   45.5 45.4 46.3
+//   4 sets of 65536 tokens (67 MB of summaries)     133.6 133.4 130.6  128.0 128.8 130.0
+// 64 sets of 8192 candidates (268 MB of summaries), 257 pages: 1275 for the pages, 1271 for both.  8 sets of 2048 pages (17 MB): 35.8 with
+// none, 36.3 with both.
+inline int step_reads_once(int kind, double summaries, double pages) {
+  if (summaries + pages <= 32e6) return 0;
+  return kOncePages | (kind == kKindToken || summaries > kStaysInL2 ? kOnceSummaries : 0);
+}
+// Plain lists: where they do not stay.  Lists that do are found in L2 by the next call on them, which the policy spoils: the same lists
+// again, us, without and with it, 444 of 10 pages (36 MB) 7.1 and 8.2, 1024 of 8 (67 MB) 15.2 and 19.4, 256 of 40 (84 MB)
+// 17.1 and 18.6, 222 of 48 (87 MB) 15.3 and 14.6, 148 of 80 (97 MB) 18.4 and 16.9; three such sets of lists in turn 9.3 and 9.0, 20.3
+// and 19.4, 18.6 and 18.6.
+inline int lists_read_once(double pages) { return pages > kStaysInL2 ? kOncePages : 0; }
 
 // Per-set flags that let the attention kernel start on a set as soon as that set's page list
 // is complete, while the scoring kernel is still working on other sets.  The producer is
