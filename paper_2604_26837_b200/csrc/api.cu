@@ -392,21 +392,20 @@ void give_back(spin_ctx *ctx, int req) {
     }
 }
 
-// The directories and scalars of a request's sets on the device: nothing mapped, nothing there.  The rows of a request's sets are
-// consecutive in every table.  (One kernel for all takes the caller 7 us less than these, but it waits for room on
-// the SMs like any other, and the next request that opens waits behind it: see spin_request_open.)
+// The directories of a request's sets on the device: nothing mapped.  The rows of a request's sets are consecutive in every table,
+// and those that opening a request writes whole need no filling.  (One kernel for all takes the caller 7 us less than a fill
+// each, but it waits for room on the SMs like any other, and the next request that opens waits behind it: see
+// spin_request_open.)
 cudaError_t unmap_request(spin_ctx *ctx, int req) {
   const Geometry &g = ctx->g;
   const DevCtx &d = ctx->d;
   const size_t set0 = (size_t)set_index(d, req, 0, 0), n = (size_t)ctx->cfg.num_layers * ctx->cfg.num_kv_heads;
   cudaError_t e = cudaSuccess;
-  auto fill = [&](void *p, int v, size_t bytes) { if (e == cudaSuccess) e = cudaMemsetAsync(p, v, bytes, nullptr); };
-  fill(d.dir_gpt + set0 * g.dir_slot, 0xff, n * g.dir_slot * 4);
-  fill(d.dir_meta + set0 * g.dir_part, 0xff, n * g.dir_part * 4);
-  fill(d.dir_off + set0 * g.dir_part, 0xff, n * g.dir_part * 4);
-  fill(d.dir_cpt + set0 * g.dir_page, 0xff, n * g.dir_page * 4);
-  fill(d.dir_sumseg + set0 * g.dir_sum, 0xff, n * g.dir_sum * 4);
-  fill(d.state + set0, 0, n * sizeof(SetState));
+  auto unmap = [&](int32_t *dir, int per_set) { if (e == cudaSuccess) e = cudaMemsetAsync(dir + set0 * per_set, 0xff, n * per_set * 4, nullptr); };
+  unmap(d.dir_meta, g.dir_part);
+  unmap(d.dir_off, g.dir_part);
+  unmap(d.dir_cpt, g.dir_page);
+  unmap(d.dir_sumseg, g.dir_sum);
   return e;
 }
 
@@ -978,6 +977,10 @@ int spin_create(const spin_config *cfg, spin_ctx **out) {
   fill(d.n_pages, 0, (size_t)g.max_batch_sets * 4);
   fill(d.n_parts, 0, (size_t)g.max_batch_sets * 4);
   fill(d.n_sel, 0, (size_t)g.max_batch_sets * 4);
+  // a set's tail pages lie behind the cache slots' pages
+  std::vector<int32_t> tails((size_t)g.n_sets * g.tail_cap);
+  for (size_t i = 0; i < tails.size(); ++i) tails[i] = (int32_t)(cfg->gpu_cache_pages + (int64_t)i);
+  if ((e = cudaMemcpy(d.tail_phys, tails.data(), tails.size() * 4, cudaMemcpyHostToDevice)) != cudaSuccess) return cuda_fail("cudaMemcpy", e);
   if (d.evict_trace) fill(d.evict_trace, 0xff, (size_t)g.n_sets * g.max_slots * 8);
   if ((e = cudaDeviceSynchronize()) != cudaSuccess) return cuda_fail("cudaDeviceSynchronize", e);
   if (ctx->offload_slot_units > 0) {
@@ -1035,14 +1038,15 @@ int spin_request_open(spin_ctx *ctx, int64_t slots, int32_t *out_req) {
     return fail(ctx, SPIN_ERR_OOM_DEVICE, "out of GPU page table segments");
   // All sets of a request are consecutive (layer by layer, head by head), so each table's rows go up
   // in one copy, and the page table segments in one copy per run of consecutive segments.  The
-  // directories of the other tables hold nothing but "unmapped" since spin_create or the last close.
+  // directories of the other tables hold nothing but "unmapped" since spin_create or the last close,
+  // and a set's tail pages are its own for good (a fold of the tail turns their order).
   // Copies, not a kernel: a kernel waits for room on the SMs, which decode steps on other streams fill (attention
   // leaves no registers, and the next step's scoring CTAs take the rest), and the caller with it.  512 slots of 8 sets, us, with a
   // kernel and with copies: beside steps of 6 requests of up to 131072 tokens 512 and 92 (with another request closed just
   // before 1063 and 131), of 16 of 32768 200 and 92; with the GPU idle 26 and 55, 64 slots of one set 23 and 18.
   const DeviceGuard on(ctx->cfg.device);
   const int set0 = set_index(d, req, 0, 0), n_sets = (int)sets_per_req;
-  std::vector<int32_t> dir_gpt((size_t)n_sets * g.dir_slot, -1), tails((size_t)n_sets * g.tail_cap);
+  std::vector<int32_t> dir_gpt((size_t)n_sets * g.dir_slot, -1);
   std::vector<SetState> states((size_t)n_sets);
   std::vector<GptEntry> entries((size_t)(segs_per_set * n_sets) << g.seg_shift, GptEntry{-1, -1, 0, -1});
   std::vector<int32_t> segs;                                    // the segments behind them
@@ -1065,7 +1069,6 @@ int spin_request_open(spin_ctx *ctx, int64_t slots, int32_t *out_req) {
     S.gpu_pages.resize((size_t)slots);
     ctx->gpu_page_pool.take(slots, S.gpu_pages.data());
     for (int64_t s = 0; s < slots; ++s) to[s].phys = S.gpu_pages[(size_t)s];
-    for (int j = 0; j < g.tail_cap; ++j) tails[(size_t)i * g.tail_cap + j] = (int32_t)(ctx->cfg.gpu_cache_pages + (int64_t)set * g.tail_cap + j);
     states[(size_t)i].slots = (int32_t)slots;
   }
   cudaError_t e = cudaSuccess;
@@ -1079,7 +1082,6 @@ int spin_request_open(spin_ctx *ctx, int64_t slots, int32_t *out_req) {
     j += len;
   }
   put(d.dir_gpt + (size_t)set0 * g.dir_slot, dir_gpt.data(), dir_gpt.size() * 4);
-  put(d.tail_phys + (size_t)set0 * g.tail_cap, tails.data(), tails.size() * 4);
   put(d.state + set0, states.data(), states.size() * sizeof(SetState));
   if (e == cudaSuccess) e = cudaStreamSynchronize(nullptr);     // the request may be used on any stream from here on
   if (e != cudaSuccess) {

@@ -64,7 +64,7 @@ assert cuda.cudaGetLastError() == 101
 def test_open_that_fails_holds_nothing(stand_in):
     # any of its copies, segments together or (every second one taken) in pieces
     stand_in("""
-for turn in range(4):
+for turn in range(3):
     h = context()
     cuda.stand_in_fail(turn)
     assert opened(h, 64)[0] == 6 and in_use(h) == (0, 0)
@@ -75,7 +75,7 @@ for r in range(4):
     assert opened(h, 16) == (0, r)
 assert lib.spin_request_close(h, 0) == 0 and lib.spin_request_close(h, 2) == 0
 held = in_use(h)
-for turn in range(5):
+for turn in range(4):
     cuda.stand_in_fail(turn)
     assert opened(h, 48)[0] == 6 and in_use(h) == held
 assert opened(h, 48) == (0, 0)
