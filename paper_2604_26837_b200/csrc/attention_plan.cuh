@@ -33,8 +33,12 @@ __host__ __device__ inline long long share_of(long long pages, long long n_sets,
 // Clusters of r CTAs that the GPU holds without some waiting for room.  What cudaOccupancyMaxActiveClusters says needs every
 // GPC packed perfectly, which the hardware does not do: the last few start when others have ended.  Lists of 24
 // pages, us: 142 in clusters of three, as many as it says, 11.9, merged through memory 9.0; 138 8.9 and 9.0; 104 in
-// clusters of four 9.1 and 9.0, 103 8.6 and 9.0; 82 in clusters of five 10.0 and 8.9, 80 8.5 and 8.8.  Pairs always fit.
-inline int clusters_at_once(const AttnGpu &gpu, int r) { return r < 2 ? gpu.resident : gpu.clusters[r] - (r > 2 ? gpu.clusters[r] / 32 : 0); }
+// clusters of four 9.1 and 9.0, 103 8.6 and 9.0; 82 in clusters of five 10.0 and 8.9, 80 8.5 and 8.8; 71 of six 8.9 and 8.7, 69 7.8
+// and 8.7.  Pairs always fit, and clusters of seven and eight leave room in every GPC anyway (56 of seven 7.4 and 8.8, 48
+// of eight, 33 pages, 7.9 and 8.7).
+inline int clusters_at_once(const AttnGpu &gpu, int r) {
+  return r < 2 ? gpu.resident : gpu.clusters[r] - (r > 2 && r < 7 ? gpu.clusters[r] / 32 : 0);
+}
 
 // As many CTAs per set as the GPU holds at once (444), and at least 8 pages for each: every CTA is
 // resident, its pages stream through its stages, and CTAs share HBM by what they have in flight,

@@ -5,6 +5,8 @@ import subprocess
 
 import pytest
 
+from test_gpu_cluster_merge import SHAPES
+
 HERE = os.path.dirname(os.path.abspath(__file__))
 WARP, COUNTED, ROWS = 0, 1, 2
 
@@ -31,8 +33,8 @@ def test_every_plan(plans):
 
 def test_clusters_leave_a_margin(plans):
     # as many sets as the runtime says that clusters fit, and the most that are there at once
-    got = plans((0, 142, 24), (0, 138, 24), (0, 104, 24), (0, 101, 24), (0, 82, 40), (0, 80, 40), (0, 71, 40), (0, 69, 40), (0, 56, 28), (0, 55, 28),
-                (0, 222, 40), (0, 48, 29), (0, 47, 29))
+    got = plans((0, 142, 24), (0, 138, 24), (0, 104, 24), (0, 101, 24), (0, 82, 40), (0, 80, 40), (0, 71, 40), (0, 69, 40), (0, 57, 28), (0, 56, 28),
+                (0, 222, 40), (0, 49, 29), (0, 48, 29))
     assert [g[2] for g in got] == [0, 3, 3, 4, 0, 5, 5, 6, 6, 7, 2, 7, 8]
 
 
@@ -46,3 +48,10 @@ def test_decode_steps_beside_a_scoring_grid(plans):
     steps = (1, 64, 65), (1, 64, 129), (1, 32, 33), (1, 8, 17)
     assert [g[1:] for g in plans(*steps)] == [(6, 6), (6, 6), (8, 8), (5, 5)]
     assert [g[1:] for g in plans(*steps, beside=1)] == [(6, 0), (6, 0), (5, 0), (3, 0)]
+
+
+def test_what_the_cluster_tests_run(plans):
+    assert [g[2] for g in plans(*((0, sets, pages) for sets, _, pages, _ in SHAPES))] == [cluster for *_, cluster in SHAPES]
+    assert {cluster for *_, cluster in SHAPES} == {0, 2, 3, 4, 5, 6, 7, 8}
+    # its decode steps: five requests of 8, 4 and 2 kv heads
+    assert [g[2] for g in plans((1, 40, 41), (1, 20, 61), (1, 10, 41))] == [8, 8, 8]

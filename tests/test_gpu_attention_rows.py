@@ -1,7 +1,7 @@
 """Paged attention at the edges of its work split, against float64 attention over the same rows.
 
 A set's pages are dealt out to the warps of its CTAs: as many CTAs as the GPU holds at once, at least
-eight pages for each, a lane per page in batches of 32 pages per warp, two pages of a warp in flight.
+eight pages for each (four where they are a cluster), a lane per page in batches of 32 pages per warp, two pages of a warp in flight.
 """
 import numpy as np
 import pytest
