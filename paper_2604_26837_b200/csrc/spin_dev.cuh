@@ -235,27 +235,25 @@ __device__ __forceinline__ uint64_t stream_policy(bool read_once) {
   asm("createpolicy.fractional.L2::evict_normal.b64 %0, 1.0;" : "=l"(normal));
   return read_once ? first : normal;
 }
-// More than this does not stay in L2 (126 MB) until it is read again.
-constexpr double kStaysInL2 = 85e6;
-// A decode step: its pages, where they and the summaries are more than a quarter of L2; its summaries where they are most of it
-// (token granularity) or more than stays.  Steps on three contexts in turn and on the same one again, us, with no policy, for
-// the pages, for both:
-//   64 sets of 2048 candidates, 129 pages (134 MB)   96.7 94.7 95.9   95.2 91.1 93.7
-//   64 sets of 512, 65 pages (50 MB)                 37.6 35.8 36.9   33.9 34.4 36.2
+// A decode step: its pages, where they and the summaries are more than a quarter of L2; its summaries too where L2 (126 MB) does
+// not hold both, and in token granularity, where there are few pages.  Steps on three contexts in turn and on the same one
+// again, us, with no policy, for the pages, for both:
+//   64 sets of 512 candidates, 65 pages (50 MB)      37.6 35.8 36.9   33.9 34.4 36.2
 //   128 sets of 250, 33 pages (50 MB)                36.1 34.0 35.1   33.2 33.7 35.1
 //   128 sets of up to 375 mean keys, 65 pages (76)   50.3 44.9 45.8   45.5 45.4 46.3
 //   4 sets of 65536 tokens (67 MB of summaries)     133.6 133.4 130.6  128.0 128.8 130.0
-// 64 sets of 8192 candidates (268 MB of summaries), 257 pages: 1275 for the pages, 1271 for both.  8 sets of 2048 pages (17 MB): 35.8 with
-// none, 36.3 with both.
+//   64 sets of 2048, 129 pages (134 MB)              96.7 94.7 95.9   95.2 91.1 93.7, on another GPU in turn - 99.6 98.8
+// For the pages and for both: 48 sets of 512 to 8192 candidates, 257 pages (177 MB) 1143 and 1136, 64 sets of 8192 (403 MB) 1275
+// and 1271.  8 sets of 2048 (17 MB): 35.8 with none, 36.3 with both.
 inline int step_reads_once(int kind, double summaries, double pages) {
-  if (summaries + pages <= 32e6) return 0;
-  return kOncePages | (kind == kKindToken || summaries > kStaysInL2 ? kOnceSummaries : 0);
+  const double all = summaries + pages;
+  return all <= 32e6 ? 0 : kOncePages | (kind == kKindToken || all > 110e6 ? kOnceSummaries : 0);
 }
 // Plain lists: where they do not stay.  Lists that do are found in L2 by the next call on them, which the policy spoils: the same lists
 // again, us, without and with it, 444 of 10 pages (36 MB) 7.1 and 8.2, 1024 of 8 (67 MB) 15.2 and 19.4, 256 of 40 (84 MB)
 // 17.1 and 18.6, 222 of 48 (87 MB) 15.3 and 14.6, 148 of 80 (97 MB) 18.4 and 16.9; three such sets of lists in turn 9.3 and 9.0, 20.3
 // and 19.4, 18.6 and 18.6.
-inline int lists_read_once(double pages) { return pages > kStaysInL2 ? kOncePages : 0; }
+inline int lists_read_once(double pages) { return pages > 85e6 ? kOncePages : 0; }
 
 // Per-set flags that let the attention kernel start on a set as soon as that set's page list
 // is complete, while the scoring kernel is still working on other sets.  The producer is

@@ -38,5 +38,5 @@ def test_plain_lists(ask):
 def test_decode_steps(ask):
     assert ask(PAGE, 8.4e6, 8.5e6) == 0
     assert ask(PAGE, 17e6, 34e6) == PAGES and ask(MEAN, 8.7e6, 68e6) == PAGES and ask(CLUSTER, 4e6, 60e6) == PAGES
-    assert ask(PAGE, 67e6, 67e6) == PAGES and ask(PAGE, 268e6, 135e6) == PAGES | SUMMARIES
+    assert ask(PAGE, 25e6, 67e6) == PAGES and ask(PAGE, 67e6, 67e6) == PAGES | SUMMARIES
     assert ask(TOKEN, 67e6, 10e6) == PAGES | SUMMARIES and ask(TOKEN, 10e6, 10e6) == 0
