@@ -6,7 +6,7 @@
 // turn, so every warp has its share of the missed pages (which lead the list) and of the hits.  Sets
 // have equal shares of the GPU as a rule, lists far above the average more (see attn_rows_of).
 // A warp keeps two pages in flight in shared memory and one accumulator over all its pages; the
-// CTA writes one partial.  A page (8 KiB: 16 K rows, then 16 V rows) is brought in by one
+// CTA has one partial.  A page (8 KiB: 16 K rows, then 16 V rows) is brought in by one
 // instruction, a 512-byte bulk copy (TMA) per lane of half the warp, each pair of rows to its own
 // place at a stride of 528 bytes; a tile takes the even tokens as its rows 0..7 and the odd ones as
 // rows 8..15, so ldmatrix reads 8 rows without a bank conflict.  (256 sets of 56 pages, 8 heads:
@@ -77,13 +77,19 @@ __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
   return *reinterpret_cast<uint32_t *>(&v);
 }
 
-// One warp requests one page: lane i copies pair i of its rows; the stage's mbarrier counts the bytes.
+// One warp requests one page: lane i copies pair i of its rows; the stage's mbarrier counts the bytes.  kOnce: the page is to
+// leave L2 first (policy).  The copy without a policy is an instruction of its own, since a normal policy costs 1 % (104 shapes of
+// plain lists, geometric mean 1.3 %).
+template <bool kOnce>
 __device__ __forceinline__ void request_page(uint32_t sdst, uint32_t bar, const uint8_t *src, int lane, uint64_t policy) {
   if (lane == 0) asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n" ::"r"(bar), "r"(kPageBytes) : "memory");
   __syncwarp();
-  if (lane < kPairs)
+  if (kOnce && lane < kPairs)
     asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint [%0], [%1], %2, [%3], %4;\n"
                  ::"r"(sdst + lane * kPairStride), "l"(src + lane * kPairBytes), "r"(kPairBytes), "r"(bar), "l"(policy) : "memory");
+  if (!kOnce && lane < kPairs)
+    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];\n"
+                 ::"r"(sdst + lane * kPairStride), "l"(src + lane * kPairBytes), "r"(kPairBytes), "r"(bar) : "memory");
 }
 // Pages that other SMs have written with ordinary stores and announced by a flag may now be read by
 // bulk copies.
@@ -429,8 +435,9 @@ __device__ __forceinline__ uint32_t remote(uint32_t addr, int rank) {
 __device__ __forceinline__ void cluster_meet() {
   asm volatile("barrier.cluster.arrive.release;\nbarrier.cluster.wait.acquire;\n" ::: "memory");
 }
-// Merge of a set's partials by the cluster that holds all its rows: every CTA takes a share of the outputs
-// and reads the others' partials through distributed shared memory, rows in ascending order.  No partial goes to
+// Merge of a set's partials by the cluster that holds all its rows: the first CTA (with eight heads the second too; a thread
+// has four outputs of a head) reads the others' partials through distributed shared memory, rows in ascending order, always eight
+// of them in flight together, the last row's again where the cluster is smaller.  No partial goes to
 // memory, and no fence or counter stands between the rows' ends and the merge.  CTAs that no page of the
 // list has reached have left (the cluster's barrier does not wait for those).  The others, the first
 // `rows`, all come here, one that has waited for the list in vain too (rows < 0: without a part, and
@@ -483,7 +490,7 @@ __device__ __forceinline__ void merge_cluster(ClusterPart<G> &part, uint8_t *sme
 // kTogether: the set has a single row, or its rows are a cluster, which leave their outputs in `part`.  The result says
 // how many rows' outputs are there to be merged, 0 if that is settled without this one, -1 if the row has waited for its
 // list in vain.
-template <int G, int W, bool kTogether>
+template <int G, int W, bool kTogether, bool kOnce>
 __device__ __forceinline__ int attn_row(const DevCtx &c, const Batch &bt, const __nv_bfloat16 *__restrict__ q,
                                          __nv_bfloat16 *__restrict__ out, uint8_t *smem, int b, int row, int max_rows, int share, int counted, ClusterPart<G> *part) {
   __shared__ __align__(8) unsigned long long s_bar[W * kWarpStages];
@@ -538,7 +545,7 @@ __device__ __forceinline__ int attn_row(const DevCtx &c, const Batch &bt, const 
   if (row >= n_rows) return 0;
   const int stride = n_rows * W;                                   // the warp's pages: mine, mine + stride, ...
 
-  const uint64_t policy = stream_policy(bt.read_once & kOncePages);
+  const uint64_t policy = kOnce ? stream_policy(true) : 0ull;
   // Q^T as B-operand fragments: column = lane/4 (query head, zero beyond G), 8 k-steps of 16 channels
   uint32_t qb[8][2];
   WarpAcc acc;
@@ -559,7 +566,7 @@ __device__ __forceinline__ int attn_row(const DevCtx &c, const Batch &bt, const 
     PageRef ref{0, -1, -1, 0u};
     auto request = [&](int stage, int j) {
       const int src = __shfl_sync(0xffffffffu, ref.src, j), fill = __shfl_sync(0xffffffffu, ref.fill, j);
-      request_page(stage0 + stage * kStageBytes, bar0 + 8 * stage, fill >= 0 ? c.host_pages + (size_t)fill * kPageBytes : page_ptr(c, src), lane, policy);
+      request_page<kOnce>(stage0 + stage * kStageBytes, bar0 + 8 * stage, fill >= 0 ? c.host_pages + (size_t)fill * kPageBytes : page_ptr(c, src), lane, policy);
     };
     // a missed page is requested as soon as it is known (early pages lead the list: lane 0's is one of
     // them): its turn, its descriptor and the count of closed turns are asked for together
@@ -762,7 +769,7 @@ __device__ __forceinline__ int attn_row(const DevCtx &c, const Batch &bt, const 
 // apart: decode, 8 sets of 65 pages, through memory 24.7 and 24.1, 32 sets 28.2 and 27.6; 104 shapes of plain lists (84 to 148 of 21
 // to 44 pages), clusters or through memory, 1 % in all.
 enum AttnKernel { kTogether, kByMemory, kByCounts };
-template <int G, int W, AttnKernel kKernel>
+template <int G, int W, AttnKernel kKernel, bool kOnce>
 __global__ void __launch_bounds__(W * 32, 3 * kAttnWarps / W)
 k_attn(DevCtx c, Batch bt, const __nv_bfloat16 *__restrict__ q, __nv_bfloat16 *__restrict__ out) {
   extern __shared__ __align__(128) uint8_t smem[];                // [warps][2] staged pages
@@ -774,11 +781,11 @@ k_attn(DevCtx c, Batch bt, const __nv_bfloat16 *__restrict__ q, __nv_bfloat16 *_
     if (row == 0 || row < attn_rows_of(bt, most_pages(c, bt, i_req), bt.attn_share, rows)) {   // else no list of this set reaches this row
       if (kKernel == kTogether && W == kAttnWarps) {
         __shared__ ClusterPart<G> part;
-        const int n = attn_row<G, W, true>(c, bt, q, out, smem, b, row, rows, bt.attn_share, -1, &part);
+        const int n = attn_row<G, W, true, kOnce>(c, bt, q, out, smem, b, row, rows, bt.attn_share, -1, &part);
         if (n != 0 && bt.attn_cluster) merge_cluster<G>(part, smem, out + ((size_t)i_req * c.Hq + (b % c.Hkv) * G) * kHeadDim, row, n);
         if (row == 0) dbg_ta(b, 15);
       } else {
-        attn_row<G, W, kKernel == kTogether>(c, bt, q, out, smem, b, row, rows, bt.attn_share, -1, nullptr);
+        attn_row<G, W, kKernel == kTogether, kOnce>(c, bt, q, out, smem, b, row, rows, bt.attn_share, -1, nullptr);
       }
     }
   } else {
@@ -792,7 +799,7 @@ k_attn(DevCtx c, Batch bt, const __nv_bfloat16 *__restrict__ q, __nv_bfloat16 *_
       mine = further_row(c, bt, share, (int)blockIdx.x - own, s_sum, s_at, &b, &row);
       if (mine) np = count_of(c, b);
     }
-    if (mine) attn_row<G, W, false>(c, bt, q, out, smem, b, row, c.max_chunks, share, np, nullptr);
+    if (mine) attn_row<G, W, false, kOnce>(c, bt, q, out, smem, b, row, c.max_chunks, share, np, nullptr);
   }
   if (blockIdx.x == 0 && blockIdx.y == 0) pdl_wait_prev();
 }
@@ -804,7 +811,9 @@ const AttnGpu &attn_gpu() {
   static std::once_flag once[kMaxDevices];
   const int slot = current_device_slot();
   std::call_once(once[slot], [slot] {
-    for (auto kernel : {k_attn<G, kAttnWarps, kTogether>, k_attn<G, kAttnWarps, kByMemory>, k_attn<G, kAttnWarps, kByCounts>, k_attn<G, 1, kTogether>}) {
+    for (auto kernel : {k_attn<G, kAttnWarps, kTogether, false>, k_attn<G, kAttnWarps, kByMemory, false>, k_attn<G, kAttnWarps, kByCounts, false>,
+                        k_attn<G, 1, kTogether, false>, k_attn<G, kAttnWarps, kTogether, true>, k_attn<G, kAttnWarps, kByMemory, true>,
+                        k_attn<G, kAttnWarps, kByCounts, true>, k_attn<G, 1, kTogether, true>}) {
       cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kAttnSmem);
       cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
     }
@@ -812,7 +821,7 @@ const AttnGpu &attn_gpu() {
     int dev = 0, sms = 0, per_sm = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_attn<G, kAttnWarps, kByMemory>, kAttnThreads, kAttnSmem);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_attn<G, kAttnWarps, kByMemory, false>, kAttnThreads, kAttnSmem);
     for (int r = 2; r <= kClusterRows; ++r) {
       cudaLaunchAttribute attr[1];
       attr[0].id = cudaLaunchAttributeClusterDimension;
@@ -826,12 +835,27 @@ const AttnGpu &attn_gpu() {
       cfg.attrs = attr;
       cfg.numAttrs = 1;
       int n = 0;
-      if (cudaOccupancyMaxActiveClusters(&n, k_attn<G, kAttnWarps, kTogether>, &cfg) != cudaSuccess) { cudaGetLastError(); n = 0; }
+      if (cudaOccupancyMaxActiveClusters(&n, k_attn<G, kAttnWarps, kTogether, false>, &cfg) != cudaSuccess) { cudaGetLastError(); n = 0; }
       gpu.clusters[r] = n;
     }
     gpu.resident = sms * per_sm > 0 ? sms * per_sm : 148;
   });
   return gpus[slot];
+}
+
+template <int G, bool kOnce>
+void launch_plan(const DevCtx &c, const Batch &b, const AttnPlan &p, const __nv_bfloat16 *q, __nv_bfloat16 *out, int n_sets, cudaStream_t st) {
+  const dim3 grid = b.attn_set_major ? dim3(p.rows, n_sets) : dim3(n_sets, p.rows);
+  if (p.form == kAttnWarp) {
+    launch_pdl(k_attn<G, 1, kTogether, kOnce>, grid, dim3(32), (size_t)kAttnSmem / kAttnWarps, st, 1, c, b, q, out);
+  } else if (p.form == kAttnCounted) {
+    launch_pdl(k_attn<G, kAttnWarps, kByCounts, kOnce>, dim3(p.rows), dim3(kAttnThreads), (size_t)kAttnSmem, st, 1, c, b, q, out);
+  } else if (p.rows > 1 && !p.cluster) {
+    launch_pdl(k_attn<G, kAttnWarps, kByMemory, kOnce>, grid, dim3(kAttnThreads), (size_t)kAttnSmem, st, 1, c, b, q, out);
+  } else {
+    launch_pdl(k_attn<G, kAttnWarps, kTogether, kOnce>, grid, dim3(kAttnThreads), (size_t)kAttnSmem, st,
+               p.cluster ? b.attn_set_major ? dim3(p.rows, 1) : dim3(1, p.rows) : dim3(1), c, b, q, out);
+  }
 }
 
 template <int G>
@@ -841,17 +865,8 @@ void launch_attn_g(const DevCtx &c, Batch b, const __nv_bfloat16 *q, __nv_bfloat
   b.attn_least = p.least;
   b.attn_share = p.share;
   b.attn_cluster = p.cluster;
-  const dim3 grid = b.attn_set_major ? dim3(p.rows, n_sets) : dim3(n_sets, p.rows);
-  if (p.form == kAttnWarp) {
-    launch_pdl(k_attn<G, 1, kTogether>, grid, dim3(32), (size_t)kAttnSmem / kAttnWarps, st, 1, c, b, q, out);
-  } else if (p.form == kAttnCounted) {
-    launch_pdl(k_attn<G, kAttnWarps, kByCounts>, dim3(p.rows), dim3(kAttnThreads), (size_t)kAttnSmem, st, 1, c, b, q, out);
-  } else if (p.rows > 1 && !p.cluster) {
-    launch_pdl(k_attn<G, kAttnWarps, kByMemory>, grid, dim3(kAttnThreads), (size_t)kAttnSmem, st, 1, c, b, q, out);
-  } else {
-    launch_pdl(k_attn<G, kAttnWarps, kTogether>, grid, dim3(kAttnThreads), (size_t)kAttnSmem, st,
-               p.cluster ? b.attn_set_major ? dim3(p.rows, 1) : dim3(1, p.rows) : dim3(1), c, b, q, out);
-  }
+  if (b.read_once & kOncePages) launch_plan<G, true>(c, b, p, q, out, n_sets, st);
+  else launch_plan<G, false>(c, b, p, q, out, n_sets, st);
 }
 
 }  // namespace
