@@ -393,9 +393,8 @@ void give_back(spin_ctx *ctx, int req) {
 }
 
 // The directories of a request's sets on the device: nothing mapped.  The rows of a request's sets are consecutive in every table,
-// and those that opening a request writes whole need no filling.  (One kernel for all takes the caller 7 us less than a fill
-// each, but it waits for room on the SMs like any other, and the next request that opens waits behind it: see
-// spin_request_open.)
+// and those that opening a request writes whole need no filling.  (One kernel for all takes the caller as long, but it waits for
+// room on the SMs like any other, and the next request that opens waits behind it: see spin_request_open.)
 cudaError_t unmap_request(spin_ctx *ctx, int req) {
   const Geometry &g = ctx->g;
   const DevCtx &d = ctx->d;
@@ -1041,9 +1040,9 @@ int spin_request_open(spin_ctx *ctx, int64_t slots, int32_t *out_req) {
   // directories of the other tables hold nothing but "unmapped" since spin_create or the last close,
   // and a set's tail pages are its own for good (a fold of the tail turns their order).
   // Copies, not a kernel: a kernel waits for room on the SMs, which decode steps on other streams fill (attention
-  // leaves no registers, and the next step's scoring CTAs take the rest), and the caller with it.  512 slots of 8 sets, us, with a
-  // kernel and with copies: beside steps of 6 requests of up to 131072 tokens 512 and 92 (with another request closed just
-  // before 1063 and 131), of 16 of 32768 200 and 92; with the GPU idle 26 and 55, 64 slots of one set 23 and 18.
+  // leaves no registers, and the next step's scoring CTAs take the rest), and the caller with it.  512 slots of 8 sets, us, with
+  // a kernel and with copies: beside steps of 6 requests of up to 131072 tokens 512 and 82 (with another request closed just
+  // before 1063 and 105), of 16 of 32768 200 and 82; with the GPU idle 26 and 55, 64 slots of one set 23 and 17.
   const DeviceGuard on(ctx->cfg.device);
   const int set0 = set_index(d, req, 0, 0), n_sets = (int)sets_per_req;
   std::vector<int32_t> dir_gpt((size_t)n_sets * g.dir_slot, -1);

@@ -78,8 +78,8 @@ __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
 }
 
 // One warp requests one page: lane i copies pair i of its rows; the stage's mbarrier counts the bytes.  kOnce: the page is to
-// leave L2 first (policy).  The copy without a policy is an instruction of its own, since a normal policy costs 1 % (104 shapes of
-// plain lists, geometric mean 1.3 %).
+// leave L2 first (policy).  The copy without a policy is an instruction of its own, since a normal policy costs plain lists 1 %
+// (104 shapes, geometric mean).
 template <bool kOnce>
 __device__ __forceinline__ void request_page(uint32_t sdst, uint32_t bar, const uint8_t *src, int lane, uint64_t policy) {
   if (lane == 0) asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n" ::"r"(bar), "r"(kPageBytes) : "memory");
