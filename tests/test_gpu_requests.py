@@ -79,7 +79,7 @@ def test_requests_come_and_go_while_the_sms_are_full(tmp_path):
     for slots in (40, 1000):
         r = s.request_open(500)
         torch.cuda.synchronize()
-        assert full.fill(100) == 1
+        assert full.fill(400) == 1
         s.request_close(r)
         r = s.request_open(slots)
         assert full.still_full() == 1
